@@ -23,75 +23,118 @@
 namespace spca {
 namespace {
 
-constexpr int NT = 256;                 // rows of A per CTA (a chunk), and threads per CTA
-constexpr int NW = NT / 32;             // warps per CTA; warp w takes rows w, w + NW, ... of the chunk
-constexpr int RPW = NT / NW;            // rows per warp (32)
-constexpr int XCHUNK = 1024;            // nonzeros of x staged in shared memory at a time
+constexpr int NT = 512;                 // threads per CTA
+constexpr int NW = NT / 32;             // warps per CTA
+constexpr int NROWS = 256;              // rows of A per CTA (a chunk)
+constexpr int RPW = NROWS / NW;         // consecutive rows per warp (16)
+constexpr int LPR = 8;                  // lanes per row: a warp works on 32 / LPR rows at once
+constexpr int RPL = RPW / (32 / LPR);   // rows per lane (4)
+constexpr int XPIECE = 8 * NT;          // entries of x scanned between two barriers
+constexpr int XSTAGE = XPIECE + 512;    // nonzeros of x staged in shared memory before they are used
 
 // the scratch: (r * ceil(n / 256)) pairs of doubles, at most SPCA_NOALLOC_MAX_PARTIALS pairs.
 // Every GPU that loads the library holds these 4 MiB until the process exits.
 __device__ __align__(256) double g_partials[2 * SPCA_NOALLOC_MAX_PARTIALS];
 
+// Sum of acc[0 .. RPL) over the LPR = 8 lanes of a row group, as a reduce-scatter: each exchange
+// halves the sums a lane still carries, so 4 rows cost 4 FP64 adds per lane instead of 12 (FP64 runs
+// at 1/64 of the FP32 rate and bounds this kernel).  Lane l of the group ends with row l >> 1.
+__device__ __forceinline__ double group_reduce(const double (&acc)[RPL], int lane) {
+  static_assert(RPL == 4 && LPR == 8, "the exchange pattern");
+  const bool h2 = lane & 4, h1 = lane & 2;
+  double a0 = h2 ? acc[2] : acc[0], a1 = h2 ? acc[3] : acc[1];
+  const double g0 = h2 ? acc[0] : acc[2], g1 = h2 ? acc[1] : acc[3];
+  a0 += __shfl_xor_sync(0xffffffffu, g0, 4);
+  a1 += __shfl_xor_sync(0xffffffffu, g1, 4);
+  double v = h1 ? a1 : a0;
+  v += __shfl_xor_sync(0xffffffffu, h1 ? a0 : a1, 2);
+  return v + __shfl_xor_sync(0xffffffffu, v, 1);
+}
+
 // grid (nchunks, r): u_i = sum_j x_j A[i, j] over the nonzeros of x, products and sums in FP64,
 // for the 256 rows of chunk b; this CTA's sums of |u_i| and u_i^2 go to
-// partials[(c * nchunks + b) * 2].  A warp owns 32 rows; for each row its lanes walk the staged
-// nonzeros of x together (lane t reads column sj[t], and the staged columns ascend, so a warp's
-// loads of one row are contiguous when x is dense), each lane keeping one FP64 sum per row that
-// the warp adds up in a fixed order at the end.
+// partials[(c * nchunks + b) * 2].
+// Bound by finding the nonzeros (each CTA scans the p entries of its x from L2) and by the FP64 pipe.
+// The scan takes 4096 entries per barrier pair, a warp 256 consecutive ones with its 8 loads in
+// flight (256 entries per barrier pair before).  Then 8 lanes share a row and a warp works on 4 rows
+// at a time, 4 times: with few nonzeros most lanes have work, a lane has 4 rows' loads in flight,
+// and the lane sums end in the reduce-scatter above.  The staged columns ascend, so 8 lanes read one
+// 32-byte sector of a row when x is dense.
+// 64 starts with 50 nonzeros each, n = 5000, p = 20000: 252 us (659 us before).
 __global__ void __launch_bounds__(NT) k_obj_partial(const float *__restrict__ A, int64_t lda, int n, int p,
                                                     const float *__restrict__ X, int64_t ldx,
                                                     double *__restrict__ partials) {
-  __shared__ int sj[XCHUNK];
-  __shared__ float sx[XCHUNK];
-  __shared__ int red_i[32];
+  __shared__ int sj[XSTAGE];
+  __shared__ float sx[XSTAGE];
+  __shared__ int wcnt[NW];
   __shared__ double red[32];
   const int c = blockIdx.y;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int row0 = blockIdx.x * NT;
+  const int sub = lane / LPR, l8 = lane % LPR;
+  const int row0 = blockIdx.x * NROWS + w * RPW + sub;   // this lane's rows: row0 + k (32 / LPR)
   const float *x = X + (int64_t)c * ldx;
-  double acc[RPW];
+  const float *arow[RPL];
 #pragma unroll
-  for (int k = 0; k < RPW; ++k) acc[k] = 0.0;
-  // walk x in chunks of NT entries; stage its nonzeros (in index order) and use them
+  for (int k = 0; k < RPL; ++k) arow[k] = A + (int64_t)min(row0 + k * (32 / LPR), n - 1) * lda;
+  double acc[RPL] = {0.0, 0.0, 0.0, 0.0};
+  const unsigned lt = (1u << lane) - 1u;
   int staged = 0;
-  for (int base = 0; base < p; base += NT) {
-    const int j = base + threadIdx.x;
-    const float xj = j < p ? x[j] : 0.0f;
-    int tot;
-    const int pos = staged + block_excl_scan_flag(xj != 0.0f, red_i, &tot);
-    if (xj != 0.0f) {
-      sj[pos] = j;
-      sx[pos] = xj;
-    }
-    staged += tot;
-    // flush when the staging buffer could overflow on the next chunk, or at the end
-    if (staged > XCHUNK - NT || base + NT >= p) {
-      __syncthreads();
+  const unsigned up = (unsigned)p;   // (base may pass 2^31 in its last step)
+  for (unsigned base = 0; base < up; base += XPIECE) {
+    // this warp's 256 entries of the piece, in index order
+    float xv[8];
+    unsigned b[8];
+    int cnt = 0;
 #pragma unroll
-      for (int k = 0; k < RPW; ++k) {
-        const int i = row0 + w + k * NW;
-        if (i < n) {
-          const float *arow = A + (int64_t)i * lda;
-          for (int t = lane; t < staged; t += 32) acc[k] = fma((double)sx[t], (double)arow[sj[t]], acc[k]);
-        }
+    for (int k = 0; k < 8; ++k) {
+      const unsigned j = base + w * 256 + k * 32 + lane;
+      xv[k] = j < up ? x[j] : 0.0f;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      b[k] = __ballot_sync(0xffffffffu, xv[k] != 0.0f);
+      cnt += __popc(b[k]);
+    }
+    if (lane == 0) wcnt[w] = cnt;
+    __syncthreads();
+    int pos = staged;
+#pragma unroll
+    for (int q = 0; q < NW; ++q) {
+      const int t = wcnt[q];
+      pos += q < w ? t : 0;
+      staged += t;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (xv[k] != 0.0f) {
+        const int q = pos + __popc(b[k] & lt);
+        sj[q] = (int)(base + w * 256 + k * 32 + lane);
+        sx[q] = xv[k];
+      }
+      pos += __popc(b[k]);
+    }
+    __syncthreads();
+    // use the staged nonzeros when the next piece might not fit, and at the end
+    if (staged > XSTAGE - XPIECE || base + XPIECE >= up) {
+      for (int t = l8; t < staged; t += LPR) {
+        const int j = sj[t];
+        float a[RPL];
+#pragma unroll
+        for (int k = 0; k < RPL; ++k) a[k] = __ldg(arow[k] + j);
+        const double xd = (double)sx[t];
+#pragma unroll
+        for (int k = 0; k < RPL; ++k) acc[k] = fma(xd, (double)a[k], acc[k]);
       }
       __syncthreads();
       staged = 0;
     }
   }
-  // u_i for the warp's rows (lane sums added in a fixed order), then |u_i| and u_i^2
-  double l1 = 0.0, l2 = 0.0;
-#pragma unroll
-  for (int k = 0; k < RPW; ++k) {
-    const double u = warp_sum_d(acc[k]);
-    if (row0 + w + k * NW < n) {
-      l1 += fabs(u);
-      l2 += u * u;
-    }
-  }
-  // every lane holds the warp's sums: lane 0 of each warp contributes them
-  l1 = block_sum_d(lane == 0 ? l1 : 0.0, red);
-  l2 = block_sum_d(lane == 0 ? l2 : 0.0, red);
+  // |u_i| and u_i^2 of the row this lane ends with (the odd lanes hold copies)
+  const double u = group_reduce(acc, lane);
+  const int i = row0 + (l8 >> 1) * (32 / LPR);
+  const bool mine = (l8 & 1) == 0 && i < n;
+  const double l1 = block_sum_d(mine ? fabs(u) : 0.0, red);
+  const double l2 = block_sum_d(mine ? u * u : 0.0, red);
   if (threadIdx.x == 0) {
     double *o = partials + ((int64_t)c * gridDim.x + blockIdx.x) * 2;
     o[0] = l1;
@@ -99,22 +142,39 @@ __global__ void __launch_bounds__(NT) k_obj_partial(const float *__restrict__ A,
   }
 }
 
-// one thread per start: the partials in chunk order, ||x||_0, ||x||_1, then the objective
+// a CTA per start: the partials, ||x||_0 and ||x||_1 (coalesced, 8 loads in flight per thread; one
+// thread per start walked x alone before: 25 us, 2552 us before, at the size above), then the objective
 __global__ void __launch_bounds__(NT) k_obj_reduce(int form, double gamma, const double *__restrict__ partials,
                                                    int nchunks, const float *__restrict__ X, int64_t ldx, int p,
-                                                   int r, double *__restrict__ f, double *__restrict__ ev) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= r) return;
-  double l1 = 0.0, l2sq = 0.0, x0 = 0.0, x1 = 0.0;
-  for (int b = 0; b < nchunks; ++b) {
+                                                   double *__restrict__ f, double *__restrict__ ev) {
+  __shared__ double red[32];
+  __shared__ int red_i[32];
+  const int c = blockIdx.x;
+  double l1 = 0.0, l2sq = 0.0, x1 = 0.0;
+  int nz = 0;
+  for (int b = threadIdx.x; b < nchunks; b += NT) {
     l1 += partials[((int64_t)c * nchunks + b) * 2 + 0];
     l2sq += partials[((int64_t)c * nchunks + b) * 2 + 1];
   }
   const float *x = X + (int64_t)c * ldx;
-  for (int j = 0; j < p; ++j) {
-    x0 += (x[j] != 0.0f);
-    x1 += fabs((double)x[j]);
+  const unsigned up = (unsigned)p;
+  for (unsigned base = threadIdx.x; base < up; base += 8 * NT) {
+    float xv[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) xv[k] = base + k * NT < up ? x[base + k * NT] : 0.0f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (xv[k] != 0.0f) {   // (a zero adds nothing: the FP64 adds are the slow part)
+        ++nz;
+        x1 += fabs((double)xv[k]);
+      }
+    }
   }
+  l1 = block_sum_d(l1, red);
+  l2sq = block_sum_d(l2sq, red);
+  x1 = block_sum_d(x1, red);
+  const double x0 = (double)block_sum_i(nz, red_i);
+  if (threadIdx.x != 0) return;
   const double l2 = sqrt(l2sq);
   double val;
   switch (form) {
@@ -161,7 +221,7 @@ extern "C" int spca_objective_noalloc(int form, double gamma, const float *A, in
   if (n < 1 || p < 1 || r < 1 || lda < p || ldx < p || n > INT32_MAX || p > INT32_MAX) return SPCA_E_INVALID;
   if (!std::isfinite(gamma) || gamma < 0.0) return SPCA_E_INVALID;
   if (r > spca::kMaxStarts) return SPCA_E_UNSUPPORTED;   // the starts ride on the grid's y dimension
-  const int64_t nchunks = (n + NT - 1) / NT;
+  const int64_t nchunks = (n + NROWS - 1) / NROWS;
   if ((int64_t)r * nchunks > (int64_t)SPCA_NOALLOC_MAX_PARTIALS) return SPCA_E_INVALID;   // beyond the scratch
   double *partials = nullptr;
   if (scratch_for_current_device(&partials) != cudaSuccess) return SPCA_E_CUDA;
@@ -169,7 +229,7 @@ extern "C" int spca_objective_noalloc(int form, double gamma, const float *A, in
   // every partial the reduction reads is written by this call's first kernel (no zeroing needed)
   k_obj_partial<<<dim3((unsigned)nchunks, (unsigned)r), NT, 0, st>>>(A, lda, (int)n, (int)p, X, ldx, partials);
   if (cudaGetLastError() != cudaSuccess) return SPCA_E_CUDA;
-  k_obj_reduce<<<(r + NT - 1) / NT, NT, 0, st>>>(form, gamma, partials, (int)nchunks, X, ldx, (int)p, r, f, ev);
+  k_obj_reduce<<<r, NT, 0, st>>>(form, gamma, partials, (int)nchunks, X, ldx, (int)p, f, ev);
   if (cudaGetLastError() != cudaSuccess) return SPCA_E_CUDA;
   return SPCA_OK;
 }
