@@ -63,9 +63,7 @@ __device__ __forceinline__ unsigned block_max_u(unsigned v, unsigned *red) {
   __syncthreads();
   if (lane == 0) red[w] = v;
   __syncthreads();
-  unsigned t = 0;
-  for (int k = 0; k < nw; ++k) t = max(t, red[k]);
-  return t;
+  return warp_max_u(lane < nw ? red[lane] : 0u);
 }
 
 // Exclusive prefix count of `flag` over the block in thread order; *total gets the count.
@@ -133,6 +131,26 @@ __device__ __forceinline__ F32Pair f32pair_add(const F32Pair &a, const F32Pair &
   r.hi = __fadd_rn(s, lo);
   r.lo = __fsub_rn(lo, __fsub_rn(r.hi, s));
   return r;
+}
+
+// ||w||_2 (as hi + lo) and 1 / ||w||_2 from the FP32 sum of squares, without FP64's square root and
+// division (a block that ran those in every thread spent 3 to 4 us on them): hi = sqrt rounded to
+// FP32, its exact residual from one FMA, and first-order corrections: the norm to about 2^-46
+// relative, the inverse correctly rounded but for ties closer than 2^-20 ulp.  Outside [1e-30, 1e30]:
+// FP64.
+__device__ __forceinline__ void norm_and_inverse(float sumsq, float *hi, float *lo, float *inv) {
+  if (sumsq >= 1e-30f && sumsq <= 1e30f) {
+    const float s = __fsqrt_rn(sumsq), e = __fmaf_rn(-s, s, sumsq), r = __frcp_rn(s);
+    const float d = 0.5f * e * r;   // sqrt(sumsq) = s + d
+    *hi = s;
+    *lo = d;
+    *inv = __fmaf_rn(r, __fmaf_rn(-s, r, 1.0f) - d * r, r);
+  } else {
+    const double n = sqrt((double)sumsq);
+    *hi = (float)n;
+    *lo = n > 0.0 && n < 1e300 ? (float)(n - (double)*hi) : 0.0f;
+    *inv = n > 0.0 ? (float)(1.0 / n) : 0.0f;
+  }
 }
 
 // order-preserving key of |v|: the IEEE bits without the sign (monotone for |v| >= 0)

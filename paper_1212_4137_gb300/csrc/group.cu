@@ -94,11 +94,7 @@ struct spca_group {
   int npool = 0;
   char *pool_mem = nullptr;
   std::vector<int64_t> pool_sig;
-  // the candidate x-step's scratch (per start: kXstepCand values and indices, one int4), grown
-  // with the number of starts; used when some member's v is long enough (kCandMinP)
-  char *cand_mem = nullptr;
-  int cand_cap = 0;
-  bool use_cand = false;
+  bool full_queued = false;        // the full x-step as kernels of its own (some start needed it)
   int *h_active = nullptr;         // pinned: active counts at a segment's end
   int h_active_cap = 0;
   int *h_err = nullptr;            // pinned: the device error word
@@ -276,6 +272,7 @@ int admit_one(spca_group *g, const spca_problem &q, int tag) {
   a.form = m.P.form;
   a.p = m.p;
   a.s = m.P.s;
+  a.sqrt_s = std::sqrt(m.P.s);
   a.thr_fixed = uses_U(m.P.form) ? u_threshold(m.P.gamma) : (float)m.P.gamma;
   a.gamma_fixed = m.P.gamma;
   a.tol = m.P.tol;
@@ -287,6 +284,7 @@ int admit_one(spca_group *g, const spca_problem &q, int tag) {
   a.calib_sweeps = m.target ? m.P.gamma_calib_sweeps : 0;
   a.lowp_sweeps = 0;
   a.stop_enabled = m.P.tol >= 0.0 ? 1 : 0;
+  a.ordered = m.h->resident16 ? 1 : 0;
   d.gamma0 = is_pen(m.P.form) && !m.target ? m.P.gamma : 0.0;
   d.ld0 = m.ldX;
   d.key = seed_key(m.P.seed);
@@ -306,6 +304,7 @@ int admit_one(spca_group *g, const spca_problem &q, int tag) {
   // the starts (seeded, or x0 normalised) and the first active list are set up at the start of the
   // member's first sweep, in one launch each with every other member admitted for that sweep
   m.first_pending = true;
+  if (xstep_may_need_full(m.P.form, m.P.s, m.target)) g->full_queued = true;
   g->members.push_back(m);
   g->tables_ok = false;
   return SPCA_OK;
@@ -377,34 +376,11 @@ int build_tables(spca_group *g) {
     GCK(cudaMemsetAsync(g->pool_mem, 0, std::max<size_t>(PL.off, 256), st));
     g->pool_sig = sig;
   }
-  int R_all = 0;
-  bool use_cand = false;
-  for (const Member &m : g->members) {
-    R_all += m.r;
-    use_cand = use_cand || m.p >= kCandMinPGroup;
-  }
-  const size_t cand_row = sizeof(float) * kXstepCand + sizeof(int) * kXstepCand;
-  if (use_cand && R_all > g->cand_cap) {
-    const int cap = std::max(R_all, g->cand_cap + g->cand_cap / 2);
-    if (g->cand_mem) GCK(cudaFreeAsync(g->cand_mem, st));
-    g->cand_mem = nullptr;
-    g->cand_cap = 0;
-    GCK(cudaMallocFromPoolAsync((void **)&g->cand_mem, (cand_row + sizeof(int4)) * (size_t)cap, g->mempool, st));
-    g->cand_cap = cap;
-  }
-  g->use_cand = use_cand;
-  float *cand_val = use_cand ? reinterpret_cast<float *>(g->cand_mem) : nullptr;
-  int *cand_idx = use_cand ? reinterpret_cast<int *>(g->cand_mem + sizeof(float) * kXstepCand * (size_t)g->cand_cap)
-                           : nullptr;
-  int4 *cand_meta = use_cand ? reinterpret_cast<int4 *>(g->cand_mem + cand_row * (size_t)g->cand_cap) : nullptr;
   int R = 0, max_n = 1, max_p = 1, max_p_small = 0;
   bool any_large_p = false;
   for (int i = 0; i < np; ++i) {
     Member &m = g->members[i];
     const int q = pool_of[i];
-    m.d.cand_val = use_cand ? cand_val + (int64_t)R * kXstepCand : nullptr;
-    m.d.cand_idx = use_cand ? cand_idx + (int64_t)R * kXstepCand : nullptr;
-    m.d.meta = use_cand ? cand_meta + R : nullptr;
     m.d.start0 = R;
     m.d.first = m.first_pending ? 1 : 0;
     m.d.vbase = vbase[i];
@@ -424,7 +400,7 @@ int build_tables(spca_group *g) {
   // column maps, Y row offsets, the pools' Y plane maps
   Layout L;
   const size_t oP = L.take(sizeof(GProb) * np), oS = L.take(sizeof(int) * R),
-               oT = L.take(sizeof(GTask) * (np + 2 * npool)), oA = L.take(sizeof(int) * np);
+               oT = L.take(sizeof(GTask) * (np + 2 * npool)), oA = L.take(2 * sizeof(int) * np);
   std::vector<int2> tl[3];
   const size_t oPool = L.take(sizeof(GPool) * npool), oPM = L.take(sizeof(int) * np),
                oPC = L.take(sizeof(int) * npool), oCM = L.take(sizeof(int) * R), oYO = L.take(sizeof(int) * np),
@@ -543,7 +519,7 @@ int build_tables(spca_group *g) {
     if (g->h_active) cudaFreeHost(g->h_active);
     g->h_active = nullptr;
     g->h_active_cap = 0;
-    GCK(cudaMallocHost((void **)&g->h_active, sizeof(int) * np));
+    GCK(cudaMallocHost((void **)&g->h_active, 2 * sizeof(int) * np));
     g->h_active_cap = np;
   }
   char *tab = g->tab;
@@ -620,10 +596,11 @@ cudaError_t enqueue_sweep(spca_group *g, int64_t k, bool first_of_segment) {
   if (e == cudaSuccess)
     e = launch_gemm_grouped(g->d_tasks + np + cur * g->npool, g->d_tiles[1 + cur], g->total_v, g->bn, g->stages,
                             g->lowp_all, g->sms, g->d_err, wait_ns, st);
-  if (e == cudaSuccess) e = launch_g_ctrl(g->dP, np, nxt, 1, nullptr, st);
+  // the x-step and (unless the full pass follows) each problem's next active list
   if (e == cudaSuccess)
-    e = launch_g_xstep(g->dP, g->d_start_prob, g->R, g->max_p_small, g->any_large_p, g->use_cand, nxt, g->sms, st);
-  if (e == cudaSuccess) e = launch_g_active(g->dP, np, nxt, false, st);
+    e = launch_g_xstep(g->dP, g->d_start_prob, g->R, g->max_p, g->max_p_small, g->any_large_p, g->full_queued, nxt,
+                       g->sms, st);
+  if (e == cudaSuccess && g->full_queued) e = launch_g_active(g->dP, np, nxt, false, st);
   return e;
 }
 
@@ -773,6 +750,7 @@ int run_segment(spca_group *g, int sweeps, bool capture, bool retire, int *finis
     key = fnv(key, &g->bn, sizeof g->bn);
     key = fnv(key, &g->lowp_all, sizeof g->lowp_all);
     key = fnv(key, &g->stages, sizeof g->stages);
+    key = fnv(key, &g->full_queued, sizeof g->full_queued);
     GroupGraph *gg = nullptr;
     for (GroupGraph &q : g->graphs)
       if (q.key == key) gg = &q;
@@ -810,8 +788,8 @@ int run_segment(spca_group *g, int sweeps, bool capture, bool retire, int *finis
     for (Member &m : g->members) m.first_pending = false;
     g->tables_ok = false;
   }
-  GCK(launch_g_ctrl(g->dP, np, (int)(g->k & 1), 0, g->d_active, st));
-  GCK(cudaMemcpyAsync(g->h_active, g->d_active, sizeof(int) * np, cudaMemcpyDeviceToHost, st));
+  GCK(launch_g_ctrl(g->dP, np, (int)(g->k & 1), g->d_active, st));
+  GCK(cudaMemcpyAsync(g->h_active, g->d_active, 2 * sizeof(int) * np, cudaMemcpyDeviceToHost, st));
   GCK(cudaMemcpyAsync(g->h_err, g->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
   GCK(cudaStreamSynchronize(st));
   if (*g->h_err) {
@@ -819,6 +797,8 @@ int run_segment(spca_group *g, int sweeps, bool capture, bool retire, int *finis
     cudaMemsetAsync(g->d_err, 0, sizeof(int), st);
     return gfail(g, code, "a device-side wait timed out");
   }
+  g->full_queued = false;
+  for (int i = 0; i < np; ++i) g->full_queued = g->full_queued || g->h_active[np + i] > 0;
   if (!retire) return SPCA_OK;
   std::vector<Member> keep;
   std::vector<Member *> done;
@@ -884,7 +864,6 @@ void spca_group_destroy(spca_group *g) {
   for (Member &m : g->members) release_member(g, m);
   g->members.clear();
   if (g->pool_mem && g->stream) cudaFreeAsync(g->pool_mem, g->stream);
-  if (g->cand_mem && g->stream) cudaFreeAsync(g->cand_mem, g->stream);
   if (g->stream) cudaStreamSynchronize(g->stream);
   for (GroupGraph &q : g->graphs)
     if (q.exec) cudaGraphExecDestroy(q.exec);

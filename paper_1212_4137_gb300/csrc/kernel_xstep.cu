@@ -1,19 +1,19 @@
 // kernel_xstep.cu -- the x-step of Algorithm 2 for every active start (one CTA per start):
-//   forms 1, 2   S3: T_s(v), the s largest |v_i| (ties: lower index), by radix select
-//   forms 3, 4   S4: V_lambda(v) with lambda = lambda_s(v), by bisection on the sign of
-//                    phi(lambda) = s ||V_lambda||_2^2 - ||V_lambda||_1^2, then the exact
-//                    root of phi on the final piece (fixed active set)
+//   forms 1, 2   S3: T_s(v), the s largest |v_i| (ties: lower index)
+//   forms 3, 4   S4: V_lambda(v) with lambda = lambda_s(v), the root of
+//                    phi(lambda) = s ||V_lambda||_2^2 - ||V_lambda||_1^2
 //   forms 5, 6   S5: U_gamma(v), keep v_i^2 > gamma  (eq. 5)
 //   forms 7, 8   S6: V_gamma(v), soft threshold       (eq. 6)
 // then normalisation (Section 2.2), the Table 3 value F(x^(k+1), y^(k)), the stopping rule,
 // and the support list (ascending indices) used by the sparse u = A x and the FP64 objective.
 // Section 4.1's gamma rule (penalty forms) picks gamma so that exactly s entries survive.
 //
-// Layout: v is staged once in shared memory (p * 4 bytes up to XSTEP_SMEM_MAX, else read from
-// global memory on every pass).  Each warp owns one contiguous index segment, so ordered work
-// (support compaction, ranking of tied magnitudes) needs only warp ballots plus one scan over
-// the 16 warps.  Reductions are in a fixed order: a start's result does not depend on the
-// other starts or on scheduling.
+// Two paths: the threshold x-step (a short list of the entries above a lower bound of the operator's
+// threshold, then the operator on the list), and the full pass for the starts it cannot serve: radix
+// select, or bisection of phi, over all of v, staged in shared memory (p * 4 bytes up to
+// XSTEP_SMEM_MAX, else read from global memory on every pass).  Reductions are in a fixed order that
+// does not depend on the CTA's size: a start's result does not depend on the other starts or on
+// scheduling.
 #include <algorithm>
 #include <cstdint>
 
@@ -24,8 +24,8 @@
 namespace spca {
 
 namespace {
-constexpr int XT = 512;                        // threads per CTA
-constexpr int XW = XT / 32;                    // warps per CTA
+constexpr int XT = 512;                        // threads per CTA of the full-pass kernels
+constexpr int XW = 16;                         // index segments; a CTA's warps share them out
 constexpr int XSTEP_SMEM_MAX = 200 * 1024;     // largest v staged in shared memory (bytes)
 static_assert(kXstepSmemMaxP * 4 == XSTEP_SMEM_MAX, "the grouped x-step's split");
 
@@ -34,44 +34,54 @@ struct XShared {
   double red_d[XW][2];
   float red_f[XW][2];
   int red_i[XW][2];
-  int wcnt[XW];                                // per-warp counts of one pass
-  int woff[XW];                                // their exclusive prefix over warps
+  int wcnt[32];                                // per-segment (or per-warp) counts of one pass
+  int woff[XW];                                // their exclusive prefix over the segments
+  int eoff[XW];                                // the same of the tied keys
   int digit, rem, cnt_bin;
-  unsigned red_u[XW];
+  unsigned red_u[32];
 };
 
 struct Seg {
   int lo, hi;
 };
-// this warp's index segment: 16 contiguous ranges, each a multiple of 32 long (the last shorter)
-__device__ __forceinline__ Seg warp_seg(int p) {
+// index segment w: 16 contiguous ranges, each a multiple of 32 long (the last shorter).  A pass takes
+// them warp by warp (for_segments), and every sum is made per segment and then over the segments in
+// order, so that its bits do not depend on the CTA's size.
+__device__ __forceinline__ Seg index_seg(int p, int w) {
   const int seg = (((p + XW - 1) / XW) + 31) / 32 * 32;
-  const int w = threadIdx.x >> 5;
   Seg s;
   s.lo = min(p, w * seg);
   s.hi = min(p, s.lo + seg);
   return s;
 }
+template <typename Fn>
+__device__ __forceinline__ void for_segments(int p, Fn &&fn) {
+  for (int w = threadIdx.x >> 5; w < XW; w += blockDim.x >> 5) fn(w, index_seg(p, w));
+}
 
-// block sums of (f0, f1, i0, i1) in one round, FP32 in a fixed order; every thread gets them.
-// (GB300's FP64 pipe is ~1/64 of FP32: FP64 stays out of the per-pass reductions.)
-__device__ __forceinline__ void block_sum2f(float &f0, float &f1, int &i0, int &i1, XShared &sh) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+// sums of (f0, f1, i0, i1) over segment w, published by its warp ...
+__device__ __forceinline__ void put_sum2f(int w, float f0, float f1, int i0, int i1, XShared &sh) {
   f0 = warp_sum_f(f0); f1 = warp_sum_f(f1); i0 = warp_sum_i(i0); i1 = warp_sum_i(i1);
-  __syncthreads();
-  if (lane == 0) { sh.red_f[w][0] = f0; sh.red_f[w][1] = f1; sh.red_i[w][0] = i0; sh.red_i[w][1] = i1; }
+  if ((threadIdx.x & 31) == 0) {
+    sh.red_f[w][0] = f0; sh.red_f[w][1] = f1; sh.red_i[w][0] = i0; sh.red_i[w][1] = i1;
+  }
+}
+// ... and added over the segments, FP32 in a fixed order; every thread gets them.
+// (GB300's FP64 pipe is ~1/64 of FP32: FP64 stays out of the per-pass reductions.)
+__device__ __forceinline__ void get_sum2f(float &f0, float &f1, int &i0, int &i1, XShared &sh) {
   __syncthreads();
   f0 = f1 = 0.0f; i0 = i1 = 0;
   for (int k = 0; k < XW; ++k) { f0 += sh.red_f[k][0]; f1 += sh.red_f[k][1]; i0 += sh.red_i[k][0]; i1 += sh.red_i[k][1]; }
+  __syncthreads();
 }
 
-// block sums of two FP64 values (each thread's value already accurate); the warp partials are
+// the same for two FP64 values (each thread's value already accurate); the segments' partials are
 // combined by one thread, so the FP64 work is ~5 adds per thread
-__device__ __forceinline__ void block_sum2d(double &d0, double &d1, XShared &sh) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+__device__ __forceinline__ void put_sum2d(int w, double d0, double d1, XShared &sh) {
   d0 = warp_sum_d(d0); d1 = warp_sum_d(d1);
-  __syncthreads();
-  if (lane == 0) { sh.red_d[w][0] = d0; sh.red_d[w][1] = d1; }
+  if ((threadIdx.x & 31) == 0) { sh.red_d[w][0] = d0; sh.red_d[w][1] = d1; }
+}
+__device__ __forceinline__ void get_sum2d(double &d0, double &d1, XShared &sh) {
   __syncthreads();
   if (threadIdx.x == 0) {
     double a = 0.0, b = 0.0;
@@ -80,6 +90,7 @@ __device__ __forceinline__ void block_sum2d(double &d0, double &d1, XShared &sh)
   }
   __syncthreads();
   d0 = sh.red_d[0][0]; d1 = sh.red_d[0][1];
+  __syncthreads();
 }
 
 // compensated (Neumaier) FP32 accumulation: s + c carries the sum to ~2^-40 relative
@@ -89,11 +100,8 @@ __device__ __forceinline__ void kahan_add(float &s, float &c, float x) {
   s = t;
 }
 
-// per-warp count -> exclusive offsets over warps (sh.woff) and the block total
-__device__ __forceinline__ int warp_offsets(int my_warp_count, XShared &sh) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) sh.wcnt[w] = my_warp_count;
+// the segments' counts (sh.wcnt) -> exclusive offsets over the segments (sh.woff) and the total
+__device__ __forceinline__ int segment_offsets(XShared &sh) {
   __syncthreads();
   if (threadIdx.x == 0) {
     int acc = 0;
@@ -115,7 +123,6 @@ __device__ void radix_select(const float *vv, int p, int j, bool exact, XShared 
   const int shifts[4] = {23, 15, 7, 0};
   const uint32_t wmask[4] = {0xFFu, 0xFFu, 0xFFu, 0x7Fu};
   const int lane = threadIdx.x & 31;
-  const Seg sg = warp_seg(p);
   uint32_t prefix = 0u, mask = 0u;
   int rem = j;
   *whole = false;
@@ -123,14 +130,16 @@ __device__ void radix_select(const float *vv, int p, int j, bool exact, XShared 
     const int sh_ = shifts[t];
     for (int b = threadIdx.x; b < 256; b += blockDim.x) sh.hist[b] = 0u;
     __syncthreads();
-    for (int base = sg.lo; base < sg.hi; base += 32) {
-      const int i = base + lane;
-      const uint32_t key = (i < sg.hi) ? abs_key(vv[i]) : 0xFFFFFFFFu;
-      const bool m = (i < sg.hi) && (key & mask) == prefix;
-      const uint32_t bin = m ? (key >> sh_) & wmask[t] : 0xFFFFFFFFu;
-      const unsigned peers = __match_any_sync(0xffffffffu, bin);
-      if (m && lane == __ffs(peers) - 1) atomicAdd(&sh.hist[bin], (unsigned)__popc(peers));
-    }
+    for_segments(p, [&](int, Seg sg) {
+      for (int base = sg.lo; base < sg.hi; base += 32) {
+        const int i = base + lane;
+        const uint32_t key = (i < sg.hi) ? abs_key(vv[i]) : 0xFFFFFFFFu;
+        const bool m = (i < sg.hi) && (key & mask) == prefix;
+        const uint32_t bin = m ? (key >> sh_) & wmask[t] : 0xFFFFFFFFu;
+        const unsigned peers = __match_any_sync(0xffffffffu, bin);
+        if (m && lane == __ffs(peers) - 1) atomicAdd(&sh.hist[bin], (unsigned)__popc(peers));
+      }
+    });
     __syncthreads();
     if (threadIdx.x < 32) {
       // warp 0 finds the bin holding the rem-th largest: lane l owns the bins
@@ -178,19 +187,16 @@ __device__ void radix_select(const float *vv, int p, int j, bool exact, XShared 
         return;
       }
       unsigned mn = 0xFFFFFFFFu;
-      for (int base = sg.lo; base < sg.hi; base += 32) {
-        const int i = base + lane;
-        if (i < sg.hi) {
-          const uint32_t key = abs_key(vv[i]);
-          if ((key & mask) == prefix) mn = min(mn, key);
-        }
+      for (int i = threadIdx.x; i < p; i += blockDim.x) {
+        const uint32_t key = abs_key(vv[i]);
+        if ((key & mask) == prefix) mn = min(mn, key);
       }
       // block minimum
-      for (int o = 16; o > 0; o >>= 1) mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+      mn = __reduce_min_sync(0xffffffffu, mn);
       if (lane == 0) sh.red_u[threadIdx.x >> 5] = mn;
       __syncthreads();
       unsigned m2 = 0xFFFFFFFFu;
-      for (int k = 0; k < XW; ++k) m2 = min(m2, sh.red_u[k]);
+      for (int k = 0; k < (int)(blockDim.x >> 5); ++k) m2 = min(m2, sh.red_u[k]);
       __syncthreads();
       *K = m2;
       *whole = true;
@@ -207,25 +213,29 @@ __device__ void radix_select(const float *vv, int p, int j, bool exact, XShared 
 __device__ double lambda_s_bisect(const float *vv, int p, double s, uint32_t lo0, uint32_t maxkey, XShared &sh,
                                   uint32_t *lo_out) {
   const int lane = threadIdx.x & 31;
-  const Seg sg = warp_seg(p);
   uint32_t lo = lo0, hi = maxkey;  // phi(key lo) < 0 <= phi(key hi)
   while (hi - lo > 1u) {
     const uint32_t mid = lo + (hi - lo) / 2u;
     const float lam = __uint_as_float(mid);
-    float sw = 0.0f, sw2 = 0.0f;
-    int in_lo = 0, in_hi = 0;  // elements strictly inside (lo, mid) and (mid, hi)
-    for (int i = sg.lo + lane; i < sg.hi; i += 32) {
-      const float a = fabsf(vv[i]);
-      const uint32_t key = __float_as_uint(a);
-      if (a > lam) {
-        const float w = a - lam;
-        sw += w;
-        sw2 = fmaf(w, w, sw2);
+    float sw, sw2;
+    int in_lo, in_hi;          // elements strictly inside (lo, mid) and (mid, hi)
+    for_segments(p, [&](int seg, Seg sg) {
+      sw = sw2 = 0.0f;
+      in_lo = in_hi = 0;
+      for (int i = sg.lo + lane; i < sg.hi; i += 32) {
+        const float a = fabsf(vv[i]);
+        const uint32_t key = __float_as_uint(a);
+        if (a > lam) {
+          const float w = a - lam;
+          sw += w;
+          sw2 = fmaf(w, w, sw2);
+        }
+        in_lo += (key > lo && key < mid);
+        in_hi += (key > mid && key < hi);
       }
-      in_lo += (key > lo && key < mid);
-      in_hi += (key > mid && key < hi);
-    }
-    block_sum2f(sw, sw2, in_lo, in_hi, sh);
+      put_sum2f(seg, sw, sw2, in_lo, in_hi, sh);
+    });
+    get_sum2f(sw, sw2, in_lo, in_hi, sh);
     const float phi = (float)s * sw2 - sw * sw;
     if (phi < 0.0f) {
       lo = mid;
@@ -237,21 +247,27 @@ __device__ double lambda_s_bisect(const float *vv, int p, double s, uint32_t lo0
   }
   // active set {key > lo}: k, S1, S2 (compensated per thread, FP64 across threads), then the
   // root of phi on this piece in FP64
-  float a1 = 0.0f, c1 = 0.0f, a2 = 0.0f, c2 = 0.0f, fz = 0.0f;
-  int kc = 0, unused = 0;
-  for (int i = sg.lo + lane; i < sg.hi; i += 32) {
-    const float a = fabsf(vv[i]);
-    if (__float_as_uint(a) > lo) {
-      ++kc;
-      kahan_add(a1, c1, a);
-      const float aa = a * a;
-      kahan_add(a2, c2, aa);
-      kahan_add(a2, c2, fmaf(a, a, -aa));   // exact square: aa + the FMA residual
+  double s1, s2;
+  float f_unused, f_unused2;
+  int kc, i_unused;
+  for_segments(p, [&](int seg, Seg sg) {
+    float a1 = 0.0f, c1 = 0.0f, a2 = 0.0f, c2 = 0.0f;
+    kc = 0;
+    for (int i = sg.lo + lane; i < sg.hi; i += 32) {
+      const float a = fabsf(vv[i]);
+      if (__float_as_uint(a) > lo) {
+        ++kc;
+        kahan_add(a1, c1, a);
+        const float aa = a * a;
+        kahan_add(a2, c2, aa);
+        kahan_add(a2, c2, fmaf(a, a, -aa));   // exact square: aa + the FMA residual
+      }
     }
-  }
-  double s1 = (double)a1 + (double)c1, s2 = (double)a2 + (double)c2;
-  block_sum2d(s1, s2, sh);
-  block_sum2f(fz, fz, kc, unused, sh);
+    put_sum2d(seg, (double)a1 + (double)c1, (double)a2 + (double)c2, sh);
+    put_sum2f(seg, 0.0f, 0.0f, kc, 0, sh);
+  });
+  get_sum2d(s1, s2, sh);
+  get_sum2f(f_unused, f_unused2, kc, i_unused, sh);
   const double k = (double)kc;
   const double flo = (double)__uint_as_float(lo), fhi = (double)__uint_as_float(hi);
   double lam;
@@ -281,22 +297,24 @@ struct XOp {
 };
 
 // Pass A (||w||_2^2 and nnz of the unnormalised result w), the Table 3 value, pass B (x = w /
-// ||w||_2 and the support list in index order) and the per-start outputs, over vv[0 .. len):
-// element i is entry map[i] of v and x (map == nullptr: entry i).
-__device__ void xstep_finish(const XstepArgs &a, int c, const float *vv, int len, const int *map, const XOp &op,
-                             float *x, StartState st, int *sup_idx, float *sup_val, Ctrl *ctrl, XShared &sh) {
+// ||w||_2 and the support list in index order) and the per-start outputs, over vv[0 .. len).
+__device__ void xstep_finish(const XstepArgs &a, int c, const float *vv, int len, const XOp &op, float *x,
+                             StartState st, int *sup_idx, float *sup_val, Ctrl *ctrl, XShared &sh) {
   const int lane = threadIdx.x & 31;
   const int form = a.form;
-  const Seg sg = warp_seg(len);
 
-  // ---- ties (mode 0): offsets of each warp's equal keys in index order
+  // ---- ties (mode 0): offsets of each segment's equal keys in index order
   if (op.mode == 0) {
-    int eq = 0;
-    for (int i = sg.lo + lane; i < sg.hi; i += 32) eq += abs_key(vv[i]) == op.K;
-    eq = warp_sum_i(eq);
-    warp_offsets(eq, sh);
+    for_segments(len, [&](int seg, Seg sg) {
+      int eq = 0;
+      for (int i = sg.lo + lane; i < sg.hi; i += 32) eq += abs_key(vv[i]) == op.K;
+      eq = warp_sum_i(eq);
+      if (lane == 0) sh.wcnt[seg] = eq;
+    });
+    segment_offsets(sh);
   }
-  const int eq_base = (op.mode == 0) ? sh.woff[threadIdx.x >> 5] : 0;
+  if (threadIdx.x < XW) sh.eoff[threadIdx.x] = op.mode == 0 ? sh.woff[threadIdx.x] : 0;
+  __syncthreads();
   const unsigned lt_mask = (1u << lane) - 1u;
 
   auto wval = [&](float vi, uint32_t key, bool tie_keep) -> float {
@@ -305,10 +323,10 @@ __device__ void xstep_finish(const XstepArgs &a, int c, const float *vv, int len
     if (op.mode == 1) return vi;
     return copysignf(fabsf(vi) - op.tval, vi);
   };
-  float part = 0.0f;
-  int wnnz = 0;
-  {
-    int eq_run = eq_base;
+  for_segments(len, [&](int seg, Seg sg) {
+    float part = 0.0f;
+    int wnnz = 0;
+    int eq_run = sh.eoff[seg];
     for (int base = sg.lo; base < sg.hi; base += 32) {
       const int i = base + lane;
       const float vi = (i < sg.hi) ? vv[i] : 0.0f;
@@ -323,28 +341,31 @@ __device__ void xstep_finish(const XstepArgs &a, int c, const float *vv, int len
       part = fmaf(w, w, part);
       wnnz += __popc(__ballot_sync(0xffffffffu, w != 0.0f));
     }
-  }
-  float fz = 0.0f;
-  int zz = 0, nnz_dummy = 0;
-  block_sum2f(part, fz, zz, nnz_dummy, sh);
-  const double sumsq = (double)part;
-  const int nnz = warp_offsets(wnnz, sh);   // sh.woff: each warp's first slot in the support list
-  const double nrm = sqrt(sumsq);
+    if (lane == 0) sh.wcnt[seg] = wnnz;
+    put_sum2f(seg, part, 0.0f, 0, 0, sh);
+  });
+  float part, fz;
+  int zz, zz2;
+  get_sum2f(part, fz, zz, zz2, sh);
+  const int nnz = segment_offsets(sh);   // sh.woff: each segment's first slot in the support list
+  float nrm_hi, nrm_lo, inv;
+  norm_and_inverse(part, &nrm_hi, &nrm_lo, &inv);
 
   // ---- Table 3 value of the subproblem
-  double F;
-  if (uses_T(form)) F = nrm;                                   // S3: ||T_s(v)||_2
-  else if (uses_lam(form)) F = op.gam * sqrt(a.s) + nrm;       // S4: lambda sqrt(s) + ||V||_2
-  else if (uses_U(form)) F = sumsq - op.gam * (double)nnz;     // S5: ||U||^2 - gamma ||U||_0
-  else F = nrm;                                                // S6: ||V_gamma(v)||_2
+  // (by the thread that uses it, below: FP64 is slow)
+  auto value = [&]() -> double {
+    const double nrm = (double)nrm_hi + (double)nrm_lo;
+    if (uses_lam(form)) return op.gam * a.sqrt_s + nrm;       // S4: lambda sqrt(s) + ||V||_2
+    if (uses_U(form)) return (double)part - op.gam * (double)nnz;     // S5: ||U||^2 - gamma ||U||_0
+    return nrm;                                                // S3: ||T_s(v)||_2, S6: ||V_gamma(v)||_2
+  };
 
   // ---- pass B
-  const float inv = nrm > 0.0 ? (float)(1.0 / nrm) : 0.0f;
   int *gi = sup_idx ? sup_idx + (int64_t)c * a.cap : nullptr;
   float *gv = sup_val ? sup_val + (int64_t)c * a.cap : nullptr;
-  {
-    int eq_run = eq_base;
-    int pos = sh.woff[threadIdx.x >> 5];
+  for_segments(len, [&](int seg, Seg sg) {
+    int eq_run = sh.eoff[seg];
+    int pos = sh.woff[seg];
     for (int base = sg.lo; base < sg.hi; base += 32) {
       const int i = base + lane;
       const float vi = (i < sg.hi) ? vv[i] : 0.0f;
@@ -357,29 +378,29 @@ __device__ void xstep_finish(const XstepArgs &a, int c, const float *vv, int len
       }
       const float w = (i < sg.hi) ? wval(vi, key, tie_keep) : 0.0f;
       const float xi = w * inv;
-      const int j = (i < sg.hi) ? (map ? map[i] : i) : 0;
-      if (i < sg.hi) x[j] = xi;
+      if (i < sg.hi) x[i] = xi;
       const unsigned nzb = __ballot_sync(0xffffffffu, xi != 0.0f);
       if (gi && xi != 0.0f) {
         const int q = pos + __popc(nzb & lt_mask);
         if (q < a.cap) {
-          gi[q] = j;
+          gi[q] = i;
           gv[q] = xi;
         }
       }
       pos += __popc(nzb);
     }
-  }
+  });
 
   // ---- outputs, stopping rule (Section 2.2), control words for the next sweep
   if (threadIdx.x == 0) {
+    const double F = value();
     if (st.F) st.F[c] = F;
     if (st.nnz) st.nnz[c] = nnz;
     if (st.gamma) st.gamma[c] = op.gam;
     if (st.tprev) st.tprev[c] = op.tnext;
     if (st.status) {
       int status = ST_ACTIVE;
-      if (nrm == 0.0) {
+      if (part == 0.0f) {
         status = SPCA_ST_DEGENERATE;
       } else if (a.stop_test && F <= (1.0 + a.tol) * st.F_prev[c]) {
         status = SPCA_ST_CONVERGED;
@@ -401,18 +422,17 @@ __device__ void xstep_full_one(const XstepArgs &a_in, int c, const float *__rest
                                float *__restrict__ X, int64_t ldx, StartState &st, int *__restrict__ sup_idx,
                                float *__restrict__ sup_val, Ctrl *ctrl, float *vsm, XShared &sh) {
   const bool kSmem = vsm != nullptr;
-  const XstepArgs a = xstep_switches(a_in, st.iters, c);
+  const XstepArgs a = xstep_switches(a_in, st.iters ? st.iters[c] : 0);
   const int p = a.p;
   const int lane = threadIdx.x & 31;
   const float *vg = V + (int64_t)c * ldv;
   float *x = X + (int64_t)c * ldx;
   const int form = a.form;
   if (kSmem) {
-    for (int i = threadIdx.x; i < p; i += XT) vsm[i] = vg[i];
+    for (int i = threadIdx.x; i < p; i += blockDim.x) vsm[i] = vg[i];
     __syncthreads();
   }
   const float *vv = kSmem ? vsm : vg;
-  const Seg sg = warp_seg(p);
 
   XOp op;
   const int s_int = (int)a.s;
@@ -433,16 +453,20 @@ __device__ void xstep_full_one(const XstepArgs &a_in, int c, const float *__rest
     }
   } else if (uses_lam(form)) {
     // phi(0) = s ||v||_2^2 - ||v||_1^2 >= 0: the L1 ball is not binding, lambda = 0
-    float f1 = 0.0f, f2 = 0.0f;
+    float f1, f2;
     unsigned mk = 0u;
-    for (int i = sg.lo + lane; i < sg.hi; i += 32) {
-      const float av = fabsf(vv[i]);
-      f1 += av;
-      f2 = fmaf(av, av, f2);
-      mk = max(mk, __float_as_uint(av));
-    }
+    for_segments(p, [&](int seg, Seg sg) {
+      f1 = f2 = 0.0f;
+      for (int i = sg.lo + lane; i < sg.hi; i += 32) {
+        const float av = fabsf(vv[i]);
+        f1 += av;
+        f2 = fmaf(av, av, f2);
+        mk = max(mk, __float_as_uint(av));
+      }
+      put_sum2f(seg, f1, f2, 0, 0, sh);
+    });
     int d0 = 0, d1 = 0;
-    block_sum2f(f1, f2, d0, d1, sh);
+    get_sum2f(f1, f2, d0, d1, sh);
     const uint32_t maxkey = block_max_u(mk, sh.red_u);
     op.mode = 2;
     if ((float)a.s * f2 - f1 * f1 < 0.0f) {
@@ -477,11 +501,11 @@ __device__ void xstep_full_one(const XstepArgs &a_in, int c, const float *__rest
       op.tkey = __float_as_uint(op.tval);
     }
   }
-  xstep_finish(a, c, vv, p, nullptr, op, x, st, sup_idx, sup_val, ctrl, sh);
+  xstep_finish(a, c, vv, p, op, x, st, sup_idx, sup_val, ctrl, sh);
 }
 
 // Every pass over all p entries of v (staged in shared memory when it fits), persistent CTAs over
-// the starts.  Starts that the candidate kernels below already finished in this sweep are skipped.
+// the starts that the threshold x-step below left (xfast = 0, or nnz = -1 without xfast).
 template <bool kSmem>
 __global__ void __launch_bounds__(XT) k_xstep(XstepArgs a_in, const float *__restrict__ V, int64_t ldv, int r,
                                               float *__restrict__ X, int64_t ldx, StartState st,
@@ -491,575 +515,755 @@ __global__ void __launch_bounds__(XT) k_xstep(XstepArgs a_in, const float *__res
   __shared__ XShared sh;
   for (int c = blockIdx.x; c < r; c += gridDim.x) {
     if (st.status && st.status[c] != ST_ACTIVE) continue;
-    if (st.xfast && st.xfast[c]) continue;
+    if (st.xfast ? st.xfast[c] != 0 : st.nnz[c] != -1) continue;
+    __syncthreads();   // (every thread has read the mark; shared memory is reused from start to start)
     xstep_full_one(a_in, c, V, ldv, X, ldx, st, sup_idx, sup_val, ctrl, kSmem ? vsm : nullptr, sh);
-    __syncthreads();   // shared memory is reused by the next start
+    if (threadIdx.x == 0 && st.xfast) st.xfast[c] = 2;
+    __syncthreads();
   }
 }
 
 
-// ---------------------------------------------------------------- one-warp operator
-// After the candidate filter a start's surviving entries are few (at most kCand) and sit in
-// shared memory: one warp finishes the x-step without block barriers.
-
-// the j-th largest key among the |v_i| of vv[0 .. len), 1 <= j <= len, built bit by bit from
-// the top (K = the largest key with at least j keys >= K); *n_gt = #(key > K), *n_eq = #(key == K)
-__device__ uint32_t warp_select(const float *vv, int len, int j, int *n_gt, int *n_eq) {
-  const int lane = threadIdx.x & 31;
-  uint32_t K = 0u;
-  for (int bit = 30; bit >= 0; --bit) {
-    const uint32_t cand = K | (1u << bit);
-    int cnt = 0;
-    for (int i = lane; i < len; i += 32) cnt += abs_key(vv[i]) >= cand;
-    if (warp_sum_i(cnt) >= j) K = cand;
-  }
-  int gt = 0, eq = 0;
-  for (int i = lane; i < len; i += 32) {
-    const uint32_t k = abs_key(vv[i]);
-    gt += k > K;
-    eq += k == K;
-  }
-  *n_gt = warp_sum_i(gt);
-  *n_eq = warp_sum_i(eq);
-  return K;
-}
-
-// lambda_s over vv[0 .. len) when phi(key lo0) < 0 is known: the bisection and exact root of
-// lambda_s_bisect, with warp sums
-__device__ double warp_lambda_s(const float *vv, int len, double s, uint32_t lo0, uint32_t maxkey,
-                                uint32_t *lo_out) {
-  const int lane = threadIdx.x & 31;
-  uint32_t lo = lo0, hi = maxkey;
-  while (hi - lo > 1u) {
-    const uint32_t mid = lo + (hi - lo) / 2u;
-    const float lam = __uint_as_float(mid);
-    float sw = 0.0f, sw2 = 0.0f;
-    int in_lo = 0, in_hi = 0;
-    for (int i = lane; i < len; i += 32) {
-      const float a = fabsf(vv[i]);
-      const uint32_t key = __float_as_uint(a);
-      if (a > lam) {
-        const float w = a - lam;
-        sw += w;
-        sw2 = fmaf(w, w, sw2);
-      }
-      in_lo += (key > lo && key < mid);
-      in_hi += (key > mid && key < hi);
-    }
-    sw = warp_sum_f(sw);
-    sw2 = warp_sum_f(sw2);
-    in_lo = warp_sum_i(in_lo);
-    in_hi = warp_sum_i(in_hi);
-    const float phi = (float)s * sw2 - sw * sw;
-    if (phi < 0.0f) {
-      lo = mid;
-      if (in_hi == 0) break;
-    } else {
-      hi = mid;
-      if (in_lo == 0) break;
-    }
-  }
-  float a1 = 0.0f, c1 = 0.0f, a2 = 0.0f, c2 = 0.0f;
-  int kc = 0;
-  for (int i = lane; i < len; i += 32) {
-    const float a = fabsf(vv[i]);
-    if (__float_as_uint(a) > lo) {
-      ++kc;
-      kahan_add(a1, c1, a);
-      const float aa = a * a;
-      kahan_add(a2, c2, aa);
-      kahan_add(a2, c2, fmaf(a, a, -aa));
-    }
-  }
-  const double s1 = warp_sum_d((double)a1 + (double)c1), s2 = warp_sum_d((double)a2 + (double)c2);
-  const double k = (double)warp_sum_i(kc);
-  const double flo = (double)__uint_as_float(lo), fhi = (double)__uint_as_float(hi);
-  double lam;
-  if (k <= s) {
-    lam = flo;
-  } else {
-    double disc = s * (k * s2 - s1 * s1) / (k - s);
-    if (disc < 0.0) disc = 0.0;
-    lam = (s1 - sqrt(disc)) / k;
-    lam = fmin(fmax(lam, flo), fhi);
-  }
-  *lo_out = lo;
-  return lam;
-}
-
-// xstep_finish for one warp over vv[0 .. len) (element i is entry map[i]): ||w||, nnz, F, x on
-// the candidates, the support list in index order, the per-start outputs and the stopping rule
-__device__ void xstep_finish_warp(const XstepArgs &a, int c, const float *vv, int len, const int *map, const XOp &op,
-                                  float *x, StartState st, int *sup_idx, float *sup_val, Ctrl *ctrl) {
-  const int lane = threadIdx.x & 31;
-  const int form = a.form;
-  const unsigned lt_mask = (1u << lane) - 1u;
-  auto wval = [&](float vi, uint32_t key, bool tie_keep) -> float {
-    if (op.mode == 0) return (key > op.K || (key == op.K && tie_keep)) ? vi : 0.0f;
-    if (key <= op.tkey) return 0.0f;
-    if (op.mode == 1) return vi;
-    return copysignf(fabsf(vi) - op.tval, vi);
-  };
-  float part = 0.0f;
-  int nnz = 0;
-  {
-    int eq_run = 0;
-    for (int base = 0; base < len; base += 32) {
-      const int i = base + lane;
-      const float vi = i < len ? vv[i] : 0.0f;
-      const uint32_t key = abs_key(vi);
-      bool tie_keep = false;
-      if (op.mode == 0) {
-        const unsigned b = __ballot_sync(0xffffffffu, i < len && key == op.K);
-        tie_keep = (eq_run + __popc(b & lt_mask)) < op.need_eq;
-        eq_run += __popc(b);
-      }
-      const float w = i < len ? wval(vi, key, tie_keep) : 0.0f;
-      part = fmaf(w, w, part);
-      nnz += __popc(__ballot_sync(0xffffffffu, w != 0.0f));
-    }
-  }
-  const double sumsq = (double)warp_sum_f(part);
-  const double nrm = sqrt(sumsq);
-  double F;
-  if (uses_T(form)) F = nrm;
-  else if (uses_lam(form)) F = op.gam * sqrt(a.s) + nrm;
-  else if (uses_U(form)) F = sumsq - op.gam * (double)nnz;
-  else F = nrm;
-  const float inv = nrm > 0.0 ? (float)(1.0 / nrm) : 0.0f;
-  int *gi = sup_idx + (int64_t)c * a.cap;
-  float *gv = sup_val + (int64_t)c * a.cap;
-  {
-    int eq_run = 0, pos = 0;
-    for (int base = 0; base < len; base += 32) {
-      const int i = base + lane;
-      const float vi = i < len ? vv[i] : 0.0f;
-      const uint32_t key = abs_key(vi);
-      bool tie_keep = false;
-      if (op.mode == 0) {
-        const unsigned b = __ballot_sync(0xffffffffu, i < len && key == op.K);
-        tie_keep = (eq_run + __popc(b & lt_mask)) < op.need_eq;
-        eq_run += __popc(b);
-      }
-      const float w = i < len ? wval(vi, key, tie_keep) : 0.0f;
-      const float xi = w * inv;
-      if (i < len) x[map[i]] = xi;
-      const unsigned nzb = __ballot_sync(0xffffffffu, xi != 0.0f);
-      if (xi != 0.0f) {
-        const int q = pos + __popc(nzb & lt_mask);
-        if (q < a.cap) {
-          gi[q] = map[i];
-          gv[q] = xi;
-        }
-      }
-      pos += __popc(nzb);
-    }
-  }
-  if (lane == 0) {
-    st.F[c] = F;
-    st.nnz[c] = nnz;
-    st.gamma[c] = op.gam;
-    st.tprev[c] = op.tnext;
-    int status = ST_ACTIVE;
-    if (nrm == 0.0) {
-      status = SPCA_ST_DEGENERATE;
-    } else if (a.stop_test && F <= (1.0 + a.tol) * st.F_prev[c]) {
-      status = SPCA_ST_CONVERGED;
-    } else if (st.iters[c] >= a.max_iter) {
-      status = SPCA_ST_MAXITER;
-    }
-    st.F_prev[c] = F;
-    st.status[c] = status;
-    if (status == ST_ACTIVE && ctrl && nnz > a.sparse_cap) atomicOr(&ctrl->need_dense, 1);
-  }
-}
-
-// ---------------------------------------------------------------- candidate x-step
-// Near convergence v moves little between sweeps, and every operator keeps only entries above a
-// threshold (the s-th or (s+1)-th largest |v_i|, lambda_s, or the penalty's fixed threshold).
-// One coalesced pass keeps the entries above a guess in per-warp lists (index order) and sums
-// |v| and v^2 for the lambda test; the operator then runs on the candidates in shared memory, and
-// x (zero outside the last support list) changes only on the old and the new support.  A guess G
-// is valid when the operator's threshold lies above it: at least s (or s + 1) candidates for the
-// selections, phi(G) < 0 for lambda_s (phi increases through its root); then the candidates hold
-// every surviving entry and the result is the full pass's.
-// Two guesses from last sweep's threshold t: the filter keeps the entries above G_lo = kGuessLo t
-// while every warp's list has room, and above G_hi = kGuess t otherwise (a warp whose list would
-// overflow drops its entries at or below G_hi and goes on with G_hi; then every warp does).  The
-// operator takes G_hi when it is valid (fewer candidates) and G_lo otherwise: early sweeps, where
-// the threshold can fall by more than a few per cent, then still avoid the full pass.  A start
-// whose last sweep took G_hi and moved its threshold by less than kSteady filters with G_hi alone.
-// A penalty with its threshold fixed uses that threshold alone (exact).  When no guess is valid,
-// or a list overflows at G_hi, the start is left to k_xstep (xfast[c] = 0; otherwise 1 for G_hi
-// with a steady threshold, 2 for the rest).
-constexpr int kCandW = 64;               // candidates per warp
-constexpr int kCand = kCandW * XW;       // per start
-static_assert(kCand == kXstepCand, "candidate scratch size");
+// ---------------------------------------------------------------- threshold x-step
+// Every operator keeps only entries above a threshold (the s-th or (s+1)-th largest |v_i|, lambda_s,
+// or the penalty's threshold), so a lower bound G of it turns the x-step into one coalesced pass that
+// lists the entries above G (in index order, a short list) and the operator on that list in shared
+// memory.  The bound comes from
+//   - a fixed threshold itself (exact);
+//   - last sweep's threshold t: G = kGuess t, or kGuessLo t when that is too high and t did not hold
+//     steady;
+//   - the maxima of 2048 disjoint subsets of v (one more pass): at least j entries lie at or above the
+//     j-th largest of them, and for j well below 2048 not many more do;
+//   - 0 for a very short v: the list holds every nonzero entry.
+// A bound is checked before it is used: at least s (or s + 1) listed entries for the selections,
+// phi(G) < 0 for lambda_s (phi increases through its root); then the list holds every surviving
+// entry and the result is that of a pass over all of v.  A start that no bound serves (more than
+// kFastW entries above it in one of the 16 segments, lambda_s = 0, s beyond the list) takes the full
+// pass.
+//
+// One CTA does all of it for a start, in one launch per sweep, and the CTA that finishes last makes
+// the active list of the next sweep.  What bounds it is each start's chain of dependent steps (reads
+// of v from L2 or HBM, then about ten block barriers), so the chain is short: ranks are counted by
+// all threads at once instead of selected bit by bit by one warp, lambda_s takes a few monotone
+// steps instead of a bisection, and FP64 (1/64 of the FP32 rate) is left to single threads.
+// 1024 starts, p = 20011, lambda_s (spca_xstep, the whole call): 109 us, 387 us for the full pass in
+// shared memory.  A solve's x-step and active list per sweep, before (filter, one-warp operator, full
+// pass and list: four launches) and now: p = 20000, T_s, 1024 starts 90 -> 46 us; p = 100000, V_gamma,
+// 16 starts 57 -> 24 us; p = 20000, lambda_s, one start 44 -> 28 us (CUDA events, a few us included).
+constexpr int kFastCand = 1024;                // listed entries per start
+constexpr int kFastBins = 2048, kFastShift = 17;   // bins of 2^-6 octave below the largest |v_i|
+constexpr int kFastAllP = 64;                  // v up to this long: list every nonzero entry
+constexpr int kFastMaxJ = 600;                 // j of the subset maxima: the list stays below kFastCand
 constexpr float kGuess = 0.85f;
 constexpr float kGuessLo = 0.6f;
-constexpr float kSteady = 0.05f;         // |t_new / t - 1| below this: one guess next sweep
-constexpr int kCandMinP = 4096;          // shorter v: the full pass only
-static_assert(kCandMinPGroup <= kCandMinP, "the group's candidate threshold");
-constexpr int kMetaHi = 1, kMetaLo = 2;  // meta[c].w: the list holds the entries above G_hi / G_lo
+constexpr float kHint = 0.98f;
+constexpr float kSteady = 0.05f;               // |t_new / t - 1| below this: t holds steady
+constexpr int kSegOrderP = 4096;               // see xstep_fast_one, "the order of ||w||^2"
+constexpr int kFastSegCap = kFastCand / XW;    // ... and per index segment (a sixteenth of v)
 
-// the candidate x-step's per-start prelude: the guesses (exact: G_hi = G_lo = the threshold
-// itself), the number of candidates the operator needs, and whether the filter applies at all
-struct CandPlan {
-  XstepArgs a;
-  float G, Glo, t;
-  bool exact, usable;
-  int need, s_int;
-};
-__device__ __forceinline__ CandPlan cand_plan(const XstepArgs &a_in, const StartState &st, int c, bool lists) {
-  CandPlan q;
-  q.a = xstep_switches(a_in, st.iters, c);
-  const int p = q.a.p, form = q.a.form;
-  q.s_int = (int)q.a.s;
-  q.exact = false;
-  if (is_pen(form) && !q.a.calibrate) {
-    q.exact = true;
-    q.G = q.a.per_start_thr ? st.thr[c] : q.a.thr_fixed;
-    q.Glo = q.G;
-    q.t = q.G;
-  } else {
-    // one guess while the threshold holds steady (last sweep took G_hi and moved the threshold
-    // by less than kSteady: xfast == 1), two otherwise (the first sweeps, after a G_lo or a full
-    // pass, and while the threshold still moves)
-    const float t = st.tprev[c];
-    q.t = t;
-    q.G = kGuess * t;
-    q.Glo = st.xfast[c] == 1 ? q.G : kGuessLo * t;
-  }
-  q.need = uses_T(form) ? q.s_int : (is_pen(form) && q.a.calibrate ? q.s_int + 1 : 1);
-  // x is zero outside the last x-step's support list, so only that list is cleared; after the
-  // start init (first sweep) x is dense and there is no list: the full pass writes all of x
-  q.usable = !((!q.exact && !(q.Glo > 0.0f)) || q.need > p || (uses_T(form) && q.s_int >= p) || st.iters[c] <= 1 ||
-               !lists || st.nnz[c] > q.a.cap);
-  return q;
-}
-
-// keep the entries of a warp's list (val, idx)[0 .. len) whose key is above Gk, in order, in place;
-// returns the new length (every lane)
-__device__ __forceinline__ int warp_compact_above(float *val, int *idx, int len, uint32_t Gk) {
-  const int lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  int out = 0;
-  __syncwarp();     // the list's entries written by other lanes are visible
-  for (int base = 0; base < len; base += 32) {
-    const int t = base + lane;
-    float v = 0.0f;
-    int ix = 0;
-    bool keep = false;
-    if (t < len) {
-      v = val[t];
-      ix = idx[t];
-      keep = abs_key(v) > Gk;
-    }
-    const unsigned b = __ballot_sync(0xffffffffu, keep);
-    __syncwarp();   // every lane has read its entry before any is overwritten
-    if (keep) {     // slot <= t: entries of later rounds are untouched
-      const int q = out + __popc(b & lt);
-      val[q] = v;
-      idx[q] = ix;
-    }
-    out += __popc(b);
-    __syncwarp();
-  }
-  return out;
-}
-
-// Filter: one coalesced pass keeps the entries above the guess in per-warp lists, concatenated in
-// warp order (the candidates in index order) into cand_val / cand_idx (kCand per start), with the
-// sums of |v| and v^2 (lambda forms) and the count in meta[c]; x is cleared on the last support.
-// A start the filter cannot serve gets xfast[c] = 0 and meta[c].w = 0.
-constexpr int kFilterChunks = 4;      // 128-entry chunks per warp and step, loaded before use
-constexpr int kFilterMinBlocks = 2;   // resident CTAs per SM the register budget is set for
-// shared memory of the filter (one CTA per start)
-struct FilterShared {
+template <int T>
+struct FastShared {
+  static constexpr int W = T / 32;
+  // a warp lists 16 / W segments, or half of one
+  static constexpr int kSegs = W < XW ? XW / W : 1, kWarpCap = kSegs * kFastSegCap;
+  union {
+    struct {
+      float wv[W * kWarpCap];                  // per-warp lists
+      int wi[W * kWarpCap];
+    } w;
+    int rank[kFastCand];
+    struct {
+      float val[kFastCand];                    // the surviving entries, in index order
+      int idx[kFastCand];
+    } s;
+  } a;
+  union {
+    struct {
+      float cv[kFastCand];                     // the list, in index order
+      int ci[kFastCand];
+    } l;
+    float by_index[2 * kFastCand];
+    unsigned hist[kFastBins];
+  } u;
+  float4 red[2][W];                            // (used alternately: one barrier per exchange)
+  int cnt[kFastCand / 32];
+  double lam;                                  // lambda_s, or < 0: the bound is too high
   XShared sh;
-  float wval_s[kCand];
-  int widx_s[kCand];
-  int fail_s, raised_s;
 };
-// start c: its candidates go to gv / gi (kCand each) and its counts to *meta_c
-__device__ __forceinline__ void xstep_filter_one(const XstepArgs &a_in, int c, const float *__restrict__ V,
-                                                 int64_t ldv, float *__restrict__ X, int64_t ldx,
-                                                 const StartState &st, const int *__restrict__ sup_idx,
-                                                 float *__restrict__ gv, int *__restrict__ gi, int4 *meta_c,
-                                                 FilterShared &fs) {
-  XShared &sh = fs.sh;
-  float *wval_s = fs.wval_s;
-  int *widx_s = fs.widx_s;
-  int &fail_s = fs.fail_s, &raised_s = fs.raised_s;
-  if (st.status[c] != ST_ACTIVE) return;
-  const CandPlan q = cand_plan(a_in, st, c, sup_idx != nullptr);
-  if (!q.usable) {
-    if (threadIdx.x == 0) {
-      st.xfast[c] = 0;
-      meta_c->w = 0;
+
+// A row of v read as aligned 16-byte vectors wherever it starts: entry i is at q = i + sh of the aligned
+// base b, and a vector that crosses an end of the row is read entry by entry (0 outside).
+struct Row {
+  const float *b;
+  int sh, end;                                 // valid q: sh .. end - 1
+};
+__device__ __forceinline__ Row row_of(const float *v, int p) {
+  Row r;
+  r.sh = (int)((reinterpret_cast<uintptr_t>(v) >> 2) & 3u);
+  r.b = v - r.sh;
+  r.end = p + r.sh;
+  return r;
+}
+// entries q .. q + 3 (q a multiple of 4), 0 from `hi` on
+__device__ __forceinline__ float4 row_load(const Row &r, int q, int hi) {
+  if (q >= r.sh && q + 4 <= hi) return *reinterpret_cast<const float4 *>(r.b + q);
+  float4 t = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  if (q >= r.sh && q < hi) t.x = r.b[q];
+  if (q + 1 >= r.sh && q + 1 < hi) t.y = r.b[q + 1];
+  if (q + 2 >= r.sh && q + 2 < hi) t.z = r.b[q + 2];
+  if (q + 3 >= r.sh && q + 3 < hi) t.w = r.b[q + 3];
+  return t;
+}
+
+// a lower bound of the j-th largest |v_i| from the maxima of 4 T subsets (four per thread): the lower
+// edge of the histogram bin of the j-th largest maximum.  0 when the bins do not resolve it.
+template <int T>
+__device__ __forceinline__ uint32_t subset_bound(const Row &row, int j, FastShared<T> &fs) {
+  uint32_t m[4] = {0u, 0u, 0u, 0u};
+  constexpr int CH = T > 256 ? 4 : 8;          // loads in flight per thread
+  for (int q0 = 4 * threadIdx.x; q0 < row.end; q0 += 4 * T * CH) {
+    float4 t[CH];
+#pragma unroll
+    for (int k = 0; k < CH; ++k) t[k] = row_load(row, q0 + 4 * T * k, row.end);
+#pragma unroll
+    for (int k = 0; k < CH; ++k) {
+      m[0] = max(m[0], abs_key(t[k].x));
+      m[1] = max(m[1], abs_key(t[k].y));
+      m[2] = max(m[2], abs_key(t[k].z));
+      m[3] = max(m[3], abs_key(t[k].w));
     }
-    return;
   }
-  const int p = q.a.p;
-  const bool sums = uses_lam(q.a.form);   // |v| and v^2 sums: the lambda forms' phi(0) test
+  for (int b = threadIdx.x; b < kFastBins; b += T) fs.u.hist[b] = 0u;
+  const uint32_t top = block_max_u(max(max(m[0], m[1]), max(m[2], m[3])), fs.sh.red_u);   // (a barrier after the zeros)
+#pragma unroll
+  for (int k = 0; k < 4; ++k) atomicAdd(&fs.u.hist[min((top - m[k]) >> kFastShift, (uint32_t)kFastBins - 1u)], 1u);
+  if (threadIdx.x == 0) fs.sh.digit = kFastBins - 1;
+  __syncthreads();
+  // one warp: the first bin, from the largest down, whose running count reaches j (64 bins a step: the
+  // largest maxima lie within a few octaves)
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    int acc = 0;
+    for (int base = 0; base < kFastBins; base += 64) {
+      const int h0 = (int)fs.u.hist[base + 2 * lane], h1 = (int)fs.u.hist[base + 2 * lane + 1];
+      int incl = h0 + h1;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      const int before = acc + incl - h0 - h1;
+      const bool here = before < j && j <= acc + incl;
+      if (here) fs.sh.digit = base + 2 * lane + (before + h0 >= j ? 0 : 1);
+      if (__any_sync(0xffffffffu, here)) break;
+      acc += __shfl_sync(0xffffffffu, incl, 31);
+    }
+  }
+  __syncthreads();
+  const uint32_t bin = (uint32_t)fs.sh.digit;
+  // keys of bins 0 .. bin are above top - (bin + 1) 2^kFastShift
+  const uint32_t down = (bin + 1u) << kFastShift;
+  return bin >= (uint32_t)kFastBins - 1u || down >= top ? 0u : top - down;
+}
+
+// Lists the entries with key > Gk in index order (fs.u.l.cv / ci, *ncand of them) and, for the
+// lambda forms, the block sums of |v| and v^2; false when a segment (a sixteenth of v) holds more than
+// kFastSegCap of them, whatever the number of warps.
+template <int T>
+__device__ __forceinline__ bool list_above(const Row &row, uint32_t Gk, bool sums, FastShared<T> &fs, int &buf,
+                                           int *ncand, float *f1_out, float *f2_out) {
+  using FS = FastShared<T>;
+  constexpr int W = FS::W;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
-  const uint32_t Ghi = __float_as_uint(q.G);
-  uint32_t Gk = __float_as_uint(q.Glo);   // the warp's current guess (warp-uniform)
-  bool raised = Gk == Ghi;
-  // kFilterChunks 128-entry chunks per step, their loads issued before any is used
-  const float *vg = V + (int64_t)c * ldv;
-  float *x = X + (int64_t)c * ldx;
-  const int seg = ((p + XW - 1) / XW + 127) / 128 * 128;
-  const int lo = min(p, w * seg), hi = min(p, lo + seg);
-  float *wv = wval_s + w * kCandW;
-  int *wi = widx_s + w * kCandW;
-  int wc = 0;
+  // this warp's range: its segments (a sixteenth each, a multiple of 128 entries), or half of one; a v
+  // no longer than the list is shared out evenly, and any part of it fits
+  int lo, hi, seg_chunks = 1 << 30;            // 128-entry chunks per segment
+  if (row.end <= kFastCand) {
+    const int per = ((row.end + W - 1) / W + 3) / 4 * 4;
+    lo = min(row.end, w * per);
+    hi = min(row.end, lo + per);
+  } else {
+    const int seg = ((row.end + XW - 1) / XW + 127) / 128 * 128;
+    if (W <= XW) {
+      lo = min(row.end, w * FS::kSegs * seg);
+      hi = min(row.end, lo + FS::kSegs * seg);
+      seg_chunks = seg / 128;
+    } else {
+      lo = min(row.end, (w >> 1) * seg + (w & 1) * (seg / 2));
+      hi = min(row.end, (w >> 1) * seg + (w & 1 ? seg : seg / 2));
+    }
+  }
+  float *wv = fs.a.w.wv + w * FS::kWarpCap;
+  int *wi = fs.a.w.wi + w * FS::kWarpCap;
+  int wc = 0, wc0 = 0, chunk = 0;              // wc0: the list's length where the segment began
   bool over = false;
   float f1 = 0.0f, f2 = 0.0f;
-  for (int base = lo; base < hi && !over; base += 128 * kFilterChunks) {
-    float e[kFilterChunks][4];
-    const bool full = base + 128 * kFilterChunks <= hi;
+  // CH 128-entry chunks per step, the next step's loads in flight while this one is used
+  constexpr int CH = T == 1024 ? 3 : 4;
+  float4 e[CH], nx[CH];
 #pragma unroll
-    for (int h = 0; h < kFilterChunks; ++h) {
-      const int i0 = base + h * 128 + 4 * lane;
-      if (full || i0 + 3 < hi) {
-        const float4 t = *reinterpret_cast<const float4 *>(vg + i0);
-        e[h][0] = t.x; e[h][1] = t.y; e[h][2] = t.z; e[h][3] = t.w;
-      } else {
+  for (int h = 0; h < CH; ++h) e[h] = row_load(row, lo + h * 128 + 4 * lane, hi);
+  for (int base = lo; base < hi && !over; base += 128 * CH) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) e[h][k] = (i0 + k < hi) ? vg[i0 + k] : 0.0f;   // 0 is never kept
+    for (int h = 0; h < CH; ++h) nx[h] = row_load(row, base + (CH + h) * 128 + 4 * lane, hi);
+#pragma unroll
+    for (int h = 0; h < CH; ++h) {
+      if (chunk == seg_chunks) {
+        chunk = 0;
+        wc0 = wc;
       }
-    }
-#pragma unroll
-    for (int h = 0; h < kFilterChunks; ++h) {
-      const int i0 = base + h * 128 + 4 * lane;
+      ++chunk;
+      const float ev[4] = {e[h].x, e[h].y, e[h].z, e[h].w};
       if (sums) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const float av = fabsf(e[h][k]);
+          const float av = fabsf(ev[k]);
           f1 += av;
           f2 = fmaf(av, av, f2);
         }
       }
       int cnt = 0;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) cnt += abs_key(e[h][k]) > Gk ? 1 : 0;
-      if (!__any_sync(0xffffffffu, cnt != 0)) continue;   // the common case: nothing above the guess
+      for (int k = 0; k < 4; ++k) cnt += abs_key(ev[k]) > Gk ? 1 : 0;   // (the 0s past an end are never above)
+      if (!__any_sync(0xffffffffu, cnt != 0)) continue;   // the common case: nothing above the bound
       // the warp's exclusive prefix of cnt (0..4) from the ballots of its three bits
-      unsigned b0 = __ballot_sync(0xffffffffu, cnt & 1), b1 = __ballot_sync(0xffffffffu, cnt & 2),
-               b2 = __ballot_sync(0xffffffffu, cnt & 4);
-      int tot = __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
-      if (wc + tot > kCandW && !raised) {   // no room at G_lo: keep only the entries above G_hi
-        wc = warp_compact_above(wv, wi, wc, Ghi);
-        Gk = Ghi;
-        raised = true;
-        cnt = 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) cnt += abs_key(e[h][k]) > Gk ? 1 : 0;
-        b0 = __ballot_sync(0xffffffffu, cnt & 1);
-        b1 = __ballot_sync(0xffffffffu, cnt & 2);
-        b2 = __ballot_sync(0xffffffffu, cnt & 4);
-        tot = __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
-      }
-      if (wc + tot > kCandW) {
+      const unsigned b0 = __ballot_sync(0xffffffffu, cnt & 1), b1 = __ballot_sync(0xffffffffu, cnt & 2),
+                     b2 = __ballot_sync(0xffffffffu, cnt & 4);
+      const int tot = __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
+      if (wc + tot > FS::kWarpCap || (seg_chunks < (1 << 30) && wc - wc0 + tot > kFastSegCap)) {
         over = true;
         break;
       }
-      int q2 = wc + __popc(b0 & lt) + 2 * __popc(b1 & lt) + 4 * __popc(b2 & lt);
+      int q = wc + __popc(b0 & lt) + 2 * __popc(b1 & lt) + 4 * __popc(b2 & lt);
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        if (abs_key(e[h][k]) > Gk) {
-          wv[q2] = e[h][k];
-          wi[q2] = i0 + k;
-          ++q2;
+        if (abs_key(ev[k]) > Gk) {
+          wv[q] = ev[k];
+          wi[q] = base + h * 128 + 4 * lane + k - row.sh;
+          ++q;
         }
       }
       wc += tot;
     }
+#pragma unroll
+    for (int h = 0; h < CH; ++h) e[h] = nx[h];
   }
-  if (threadIdx.x == 0) {
-    fail_s = 0;
-    raised_s = 0;
+  if (sums) {
+    f1 = warp_sum_f(f1);
+    f2 = warp_sum_f(f2);
+  }
+  if (lane == 0) fs.red[buf][w] = make_float4(f1, f2, __int_as_float(wc), __int_as_float(over ? 1 : 0));
+  __syncthreads();   // (also: the histogram's readers are done before the list overwrites it)
+  // lane q looks at warp q
+  const float4 t = lane < W ? fs.red[buf][lane] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  buf ^= 1;
+  const int n = __float_as_int(t.z);
+  bool too_many = __float_as_int(t.w) != 0;
+  if (W > XW) {      // two warps to a segment
+    const int both = n + __shfl_xor_sync(0xffffffffu, n, 1);
+    too_many = too_many || (row.end > kFastCand && both > kFastSegCap);
+  }
+  int incl = n;
+#pragma unroll
+  for (int o = 1; o < W; o <<= 1) {
+    const int up = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += up;
+  }
+  const int off = __shfl_sync(0xffffffffu, incl - n, w);
+  *ncand = __shfl_sync(0xffffffffu, incl, W - 1);
+  if (sums) {
+    *f1_out = warp_sum_f(t.x);
+    *f2_out = warp_sum_f(t.y);
+  }
+  if (__any_sync(0xffffffffu, too_many)) return false;
+  __syncwarp();
+  for (int t = lane; t < wc; t += 32) {
+    fs.u.l.cv[off + t] = wv[t];
+    fs.u.l.ci[off + t] = wi[t];
   }
   __syncthreads();
-  if (lane == 0 && over) fail_s = 1;
-  if (lane == 0 && Gk != __float_as_uint(q.Glo)) raised_s = 1;   // this warp went on with G_hi
-  int d0 = 0, d1 = 0;
-  block_sum2f(f1, f2, d0, d1, sh);   // (its barriers also publish fail_s and raised_s)
-  if (fail_s) {
-    if (threadIdx.x == 0) {
-      st.xfast[c] = 0;
-      meta_c->w = 0;
-    }
-    return;
-  }
-  const bool at_hi = raised_s || Ghi == __float_as_uint(q.Glo);
-  __syncwarp();
-  if (at_hi && Gk != Ghi) wc = warp_compact_above(wv, wi, wc, Ghi);   // every warp on one guess
-  const int ncand = warp_offsets(lane == 0 ? wc : 0, sh);
-  const int off = sh.woff[w];
-  for (int t = lane; t < wc; t += 32) {
-    gv[off + t] = wv[t];
-    gi[off + t] = wi[t];
-  }
-  const int nnz_old = st.nnz[c];
-  const int *old = sup_idx + (int64_t)c * q.a.cap;
-  for (int t = threadIdx.x; t < nnz_old; t += XT) x[old[t]] = 0.0f;
-  if (threadIdx.x == 0)
-    *meta_c = make_int4(ncand, __float_as_int(f1), __float_as_int(f2), at_hi ? kMetaHi : kMetaLo);
+  return true;
 }
 
-__global__ void __launch_bounds__(XT, kFilterMinBlocks) k_xstep_filter(XstepArgs a_in, const float *__restrict__ V, int64_t ldv,
-                                                     float *__restrict__ X, int64_t ldx, StartState st,
-                                                     const int *__restrict__ sup_idx, float *__restrict__ cand_val,
-                                                     int *__restrict__ cand_idx, int4 *__restrict__ meta) {
-  __shared__ FilterShared fs;
-  const int c = blockIdx.x;
-  xstep_filter_one(a_in, c, V, ldv, X, ldx, st, sup_idx, cand_val + (int64_t)c * kCand, cand_idx + (int64_t)c * kCand,
-                   meta + c, fs);
-}
-
-// Operator: a warp per start on the filter's candidates (staged in the warp's shared memory).
-// A list above G_lo is first cut to the entries above G_hi when G_hi is valid; then the operator,
-// with the check that the guess lies below the operator's threshold, the new x, F and support.
-constexpr int kOpWarps = 4;
-// start c on one warp: its candidates at gv / gi, its counts at *meta_c; cval / cidx: the warp's
-// shared memory (kCand each)
-__device__ __forceinline__ void xstep_op_one(const XstepArgs &a_in, int c, float *__restrict__ X, int64_t ldx,
-                                             const StartState &st, int *__restrict__ sup_idx,
-                                             float *__restrict__ sup_val, const float *__restrict__ gv,
-                                             const int *__restrict__ gi, const int4 *meta_c, Ctrl *ctrl, float *cval,
-                                             int *cidx) {
+// lambda_s over the list, by one warp; < 0 when phi(G) >= 0 (the bound is too high).
+// For the set S of entries above a lower bound of the root, the root of phi restricted to S is a lower
+// bound again (an entry below the root adds to phi), so raising the bound to it and dropping the
+// entries below converges monotonically to the active set.  The steps run in FP32, on w = |v| - lo and
+// lowered by their rounding error, from `hint` when phi(hint) < 0 and from G otherwise; the last ones,
+// on compensated sums, end when no entry lies between the bound and the root: the result is the root
+// of phi on its own active set, by two FP64 Newton steps from its FP32 value (FP64's division and
+// square root took longer than all of the steps).
+__device__ __forceinline__ double list_lambda(const float *cv, int ncand, float s, double s_d, float G, float hint) {
   const int lane = threadIdx.x & 31;
-  if (st.status[c] != ST_ACTIVE) return;
-  const int4 m = *meta_c;
-  if (m.w == 0) return;
-  const CandPlan q = cand_plan(a_in, st, c, true);
-  const XstepArgs &a = q.a;
-  const int form = a.form, s_int = q.s_int;
-  int ncand = m.x;
-  const float f1 = __int_as_float(m.y), f2 = __int_as_float(m.z);
-  for (int t = lane; t < ncand; t += 32) {
-    cval[t] = gv[t];
-    cidx[t] = gi[t];
-  }
-  __syncwarp();
-  // phi(G) < 0 over the candidates above G (all of v's entries above G when the list holds them)
-  auto phi_below = [&](float G, int len) {
-    const uint32_t Gk = __float_as_uint(G);
-    float sw = 0.0f, sw2 = 0.0f;
-    for (int i = lane; i < len; i += 32) {
-      const float av = fabsf(cval[i]);
-      if (__float_as_uint(av) > Gk) {
-        const float wv2 = av - G;
-        sw += wv2;
-        sw2 = fmaf(wv2, wv2, sw2);
+  float lo = hint > G ? hint : G, w1, w2;
+  int k;
+  auto sums = [&]() {                // k, sum w and sum w^2 of w = |v| - lo > 0
+    w1 = w2 = 0.0f;
+    k = 0;
+    for (int t = lane; t < ncand; t += 32) {
+      const float w = fabsf(cv[t]) - lo;
+      if (w > 0.0f) {
+        w1 += w;
+        w2 = fmaf(w, w, w2);
+        ++k;
       }
     }
-    sw = warp_sum_f(sw);
-    sw2 = warp_sum_f(sw2);
-    return (float)a.s * sw2 - sw * sw < 0.0f;
+    w1 = warp_sum_f(w1);
+    w2 = warp_sum_f(w2);
+    k = warp_sum_i(k);
   };
-  float G = q.G;
-  if (m.w == kMetaLo) {   // the list holds the entries above G_lo: cut it to G_hi if G_hi is valid
-    const uint32_t Ghi = __float_as_uint(q.G);
-    bool hi_ok;
-    if (uses_lam(form)) {
-      hi_ok = phi_below(q.G, ncand);
-    } else {
-      int n_hi = 0;
-      for (int i = lane; i < ncand; i += 32) n_hi += abs_key(cval[i]) > Ghi ? 1 : 0;
-      hi_ok = warp_sum_i(n_hi) >= q.need;
-    }
-    if (hi_ok) ncand = warp_compact_above(cval, cidx, ncand, Ghi);
-    else G = q.Glo;
+  sums();
+  if (!(s * w2 - w1 * w1 < 0.0f) && lo > G) {
+    lo = G;
+    sums();
   }
-  const uint32_t Gk = __float_as_uint(G);
+  if (!(s * w2 - w1 * w1 < 0.0f)) return -1.0;
+  for (int it = 0; it < 64 && (float)k > s; ++it) {
+    const float kf = (float)k, mean = w1 / kf;
+    const float var = fmaxf(kf * w2 - w1 * w1, 0.0f) + 2e-6f * kf * w2;
+    const float d = mean - sqrtf(s * var / (kf - s)) / kf - 4e-6f * mean;
+    if (!(lo + d > lo)) break;
+    lo += d;
+    const int kprev = k;
+    sums();
+    if (k == kprev) break;
+  }
+  double bound = (double)lo, lam = bound;
+  float bound_f = lo;                // (for a float v, v > a double b is v > the largest float <= b)
+  for (int it = 0; it < 64; ++it) {
+    float a1 = 0.0f, c1 = 0.0f, a2 = 0.0f, c2 = 0.0f;
+    int kc = 0;
+    for (int i = lane; i < ncand; i += 32) {
+      const float v = fabsf(cv[i]);
+      if (v > bound_f) {
+        ++kc;
+        kahan_add(a1, c1, v);
+        const float vv = v * v;
+        kahan_add(a2, c2, vv);
+        kahan_add(a2, c2, fmaf(v, v, -vv));
+      }
+    }
+    const double s1 = warp_sum_d((double)a1 + (double)c1), s2 = warp_sum_d((double)a2 + (double)c2);
+    const int kn = warp_sum_i(kc);
+    const double kd = (double)kn;
+    if (kd <= s_d) {
+      lam = bound;
+      break;
+    }
+    // sums of w = |v| - bound, and d = lam - bound from them in FP32
+    const double W1 = fma(-kd, bound, s1), W2 = fma(-bound, s1 + W1, s2);
+    const float kf = (float)kn, W1f = (float)W1, gap = (float)(kd - s_d);
+    const float var = fmaxf((float)fma(kd, W2, -W1 * W1), 0.0f);
+    double d = (double)(W1f / kf - sqrtf(s * var / gap) / kf);
+    // phi(d) = s (W2 - 2 d W1 + k d^2) - (W1 - k d)^2, phi'(d) = 2 (k - s) (W1 - k d)
+    float tf = 0.0f;
+#pragma unroll 1
+    for (int q = 0; q < 2; ++q) {
+      const double t = fma(-kd, d, W1);
+      tf = (float)t;
+      if (!(tf > 1e-3f * W1f)) break;
+      const double phi = fma(s_d, fma(-d, W1 + t, W2), -t * t);
+      d -= (double)((float)phi / (2.0f * gap * tf));
+    }
+    if (!(tf > 1e-3f * W1f)) {       // all of the set nearly equal: the root in closed form
+      double disc = s_d * (kd * s2 - s1 * s1) / (kd - s_d);
+      if (disc < 0.0) disc = 0.0;
+      d = (s1 - sqrt(disc)) / kd - bound;
+    }
+    lam = fmax(bound + d, bound);
+    const float lam_f = __double2float_rd(lam);
+    int below = 0;
+    for (int i = lane; i < ncand; i += 32) {
+      const float v = fabsf(cv[i]);
+      below += v > bound_f && v <= lam_f;
+    }
+    if (warp_sum_i(below) == 0) break;
+    bound = lam;
+    bound_f = lam_f;
+  }
+  return lam;
+}
+
+// a start's state as the x-step reads it, all loads in flight at once
+struct XState {
+  int iters = 0, nnz = 0, xfast = 0;
+  float tprev = 0.0f, thr = 0.0f;
+  double gamma = 0.0, F_prev = 0.0;
+};
+__device__ __forceinline__ XState load_state(const StartState &st, int c) {
+  XState q;
+  if (st.iters) q.iters = st.iters[c];
+  if (st.status) {                   // (a solve: every array is there)
+    q.nnz = st.nnz[c];
+    q.xfast = st.xfast[c];
+    q.tprev = st.tprev[c];
+    q.thr = st.thr[c];
+    q.gamma = st.gamma[c];
+    q.F_prev = st.F_prev[c];
+  }
+  return q;
+}
+
+// the x-step of start c (block-wide, T threads); false when it is left to the full pass
+template <int T>
+__device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, const float *__restrict__ V, int64_t ldv,
+                                               float *__restrict__ X, int64_t ldx, const StartState &st,
+                                               const XState &q0, int *__restrict__ sup_idx,
+                                               float *__restrict__ sup_val, Ctrl *ctrl, FastShared<T> &fs) {
+  const XstepArgs a = xstep_switches(a_in, q0.iters);
+  const int p = a.p, form = a.form, s_int = (int)a.s;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const Row row = row_of(V + (int64_t)c * ldv, p);
   float *x = X + (int64_t)c * ldx;
-  XOp op;
-  bool ok = ncand >= q.need;
-  if (ok && uses_T(form)) {
-    int gt, eq;
-    op.K = warp_select(cval, ncand, s_int, &gt, &eq);
-    op.need_eq = s_int - gt;
-    op.tnext = __uint_as_float(op.K);
-    if (op.need_eq >= eq) {   // every key equal to K is kept: keep key >= K
-      op.mode = 1;
-      op.tkey = op.K - 1u;
-    } else {
-      op.mode = 0;            // ties at K: the first need_eq in index order
-    }
-  } else if (ok && uses_lam(form)) {
-    // lambda = 0 (phi(0) >= 0) keeps every entry: left to the full pass
-    ok = (float)a.s * f2 - f1 * f1 < 0.0f;
-    if (ok) ok = phi_below(G, ncand);   // phi(G) < 0: lambda_s > G
-    if (ok) {
-      unsigned mk = 0u;
-      for (int i = lane; i < ncand; i += 32) mk = max(mk, abs_key(cval[i]));
-      mk = warp_max_u(mk);
-      uint32_t lok;
-      op.mode = 2;
-      op.gam = warp_lambda_s(cval, ncand, a.s, Gk, mk, &lok);
-      op.tkey = lok;
-      op.tval = (float)op.gam;
-      op.tnext = op.tval;
-    }
-  } else if (ok) {  // penalties
-    op.mode = uses_U(form) ? 1 : 2;
-    if (a.calibrate) {
-      int gt, eq;
-      const uint32_t tk = warp_select(cval, ncand, s_int + 1, &gt, &eq);   // the (s+1)-th largest
-      op.tkey = tk;
-      op.tval = __uint_as_float(tk);
-      op.gam = uses_U(form) ? (double)op.tval * (double)op.tval : (double)op.tval;
-      op.tnext = op.tval;
-      if (lane == 0) st.thr[c] = op.tval;
-    } else if (a.per_start_thr) {
-      op.tval = st.thr[c];
-      op.gam = st.gamma[c];
-      op.tkey = __float_as_uint(op.tval);
-      op.tnext = st.tprev[c];
-    } else {
-      op.tval = a.thr_fixed;
-      op.gam = a.gamma_fixed;
-      op.tkey = __float_as_uint(op.tval);
-      op.tnext = st.tprev[c];
+  const unsigned lt_mask = (1u << lane) - 1u;
+  const bool lam_form = uses_lam(form), exact = is_pen(form) && !a.calibrate;
+  const bool keep_all = uses_T(form) && s_int >= p;
+  const int need = uses_T(form) ? s_int : (is_pen(form) && a.calibrate ? s_int + 1 : 1);
+  const bool all = p <= kFastAllP || (p <= kFastCand && (need > kFastMaxJ / 2 || keep_all));
+  if (!all && !exact && (need > kFastMaxJ || keep_all)) return false;
+  // j of the subset maxima: the active set of lambda_s has about 2 s entries where |v|'s tail is
+  // exponential, so 3 s lie below its threshold; never so many that subsets hold several of them
+  constexpr int kMaxJ = kFastMaxJ < 2 * T ? kFastMaxJ : 2 * T;
+  int j = lam_form ? (int)fminf(3.0f * (float)a.s + 16.0f, (float)kMaxJ) : need;
+  const float tprev = q0.tprev;
+  const bool steady = q0.xfast == 1;
+  // x is zero outside the last support list, once there is one (before: all of x is written)
+  const bool listed = sup_idx && q0.iters > 1 && q0.nnz <= a.cap;
+  if (listed) {
+    const int nnz_old = q0.nnz;
+    const int *old = sup_idx + (int64_t)c * a.cap;
+    for (int t = threadIdx.x; t < nnz_old; t += T) x[old[t]] = 0.0f;
+  } else {                           // as aligned vectors, whatever the row's alignment
+    const int sh = (int)((reinterpret_cast<uintptr_t>(x) >> 2) & 3u);
+    float *xb = x - sh;
+    for (int q = 4 * threadIdx.x; q < p + sh; q += 4 * T) {
+      if (q >= sh && q + 4 <= p + sh) {
+        *reinterpret_cast<float4 *>(xb + q) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      } else {
+        for (int k = 0; k < 4; ++k)
+          if (q + k >= sh && q + k < p + sh) xb[q + k] = 0.0f;
+      }
     }
   }
-  if (!ok) {   // uniform over the warp: every input of ok is a warp-wide value
-    if (lane == 0) st.xfast[c] = 0;
-    return;
+
+  // ---- a bound, the list above it, and the check (block-uniform throughout)
+  int buf = 0, ncand = 0;
+  double lam = 0.0;
+  bool lam0 = false;                 // lambda_s = 0: the L1 ball does not bind
+  enum { kAll, kExact, kHigh, kLow, kSubsets };
+  int how = exact ? kExact : all ? kAll : listed && tprev > 0.0f ? kHigh : kSubsets;
+  uint32_t Gk;
+  float thr = 0.0f;
+  double gam = 0.0;
+  if (exact) {
+    thr = a.per_start_thr ? q0.thr : a.thr_fixed;
+    gam = a.per_start_thr ? q0.gamma : a.gamma_fixed;
   }
-  xstep_finish_warp(a, c, cval, ncand, cidx, op, x, st, sup_idx, sup_val, ctrl);
-  if (lane == 0) {   // 1: G_hi taken and the threshold steady (a fixed threshold counts as steady)
-    const bool steady = q.exact || (op.tnext >= (1.0f - kSteady) * q.t && op.tnext <= (1.0f + kSteady) * q.t);
-    st.xfast[c] = G == q.G && steady ? 1 : 2;
+  for (;;) {
+    if (how == kExact) Gk = __float_as_uint(thr);
+    else if (how == kAll) Gk = 0u;
+    else if (how == kHigh) Gk = __float_as_uint(kGuess * tprev);
+    else if (how == kLow) Gk = __float_as_uint(kGuessLo * tprev);
+    else Gk = subset_bound<T>(row, j, fs);
+    float f1 = 0.0f, f2 = 0.0f;
+    const bool fits = list_above<T>(row, Gk, lam_form, fs, buf, &ncand, &f1, &f2);
+    if (lam_form && !((float)a.s * f2 - f1 * f1 < 0.0f)) {
+      // phi(0) >= 0: every entry survives
+      if (Gk != 0u || !fits) return false;
+      lam0 = true;
+      break;
+    }
+    bool ok = fits;
+    if (fits && lam_form) {
+      if (w == 0) {                  // (a hint just below the last lambda_s: few steps while it holds steady)
+        const double l = list_lambda(fs.u.l.cv, ncand, (float)a.s, a.s, __uint_as_float(Gk), kHint * tprev);
+        if (lane == 0) fs.lam = l;
+      }
+      __syncthreads();
+      lam = fs.lam;
+      ok = lam >= 0.0;
+    } else if (fits && !exact) ok = ncand >= need || Gk == 0u;
+    if (ok) break;
+    if (how == kHigh) {
+      how = fits && !steady ? kLow : kSubsets;
+    } else if (how == kLow) {
+      how = kSubsets;
+    } else if (how == kSubsets && lam_form && fits && j < kMaxJ) {
+      j = kMaxJ;                     // the root lies lower: a longer list
+    } else {
+      return false;
+    }
+    __syncthreads();                 // the lists are reused
+  }
+
+  // ---- the operator on the list: which entries survive, as
+  //   select: rank < need (T_s; ties at the threshold: the lower indices), or key above the threshold
+  float tval = 0.0f, tnext = tprev;
+  const bool select = (uses_T(form) && !keep_all) || (is_pen(form) && a.calibrate);
+  const bool ranked = select && ncand >= need;
+  uint32_t kmin = 0xFFFFFFFFu;       // the need-th largest key
+  if (ranked) {
+    // rank of each entry = entries with a larger key; the need-th largest key is the smallest one of
+    // rank < need
+    int above = 0;
+    const int n4 = ncand & ~3;
+    for (int t = threadIdx.x; t < ncand; t += T) {
+      const uint32_t mine = abs_key(fs.u.l.cv[t]);
+      int rk = 0;
+#pragma unroll 4
+      for (int i = 0; i < n4; i += 4) {
+        const float4 e = *reinterpret_cast<const float4 *>(fs.u.l.cv + i);
+        rk += (abs_key(e.x) > mine) + (abs_key(e.y) > mine) + (abs_key(e.z) > mine) + (abs_key(e.w) > mine);
+      }
+      for (int i = n4; i < ncand; ++i) rk += abs_key(fs.u.l.cv[i]) > mine;
+      fs.a.rank[t] = rk;             // (read back by this thread)
+      if (rk < need) {
+        kmin = min(kmin, mine);
+        ++above;
+      }
+    }
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    above = warp_sum_i(above);
+    if (lane == 0) fs.red[buf][w] = make_float4(__uint_as_float(kmin), __int_as_float(above), 0.0f, 0.0f);
+    __syncthreads();
+    kmin = __reduce_min_sync(0xffffffffu, lane < T / 32 ? __float_as_uint(fs.red[buf][lane].x) : 0xFFFFFFFFu);
+    above = warp_sum_i(lane < T / 32 ? __float_as_int(fs.red[buf][lane].y) : 0);
+    buf ^= 1;
+    tval = __uint_as_float(kmin);
+    tnext = tval;
+    if (uses_T(form) && above > need) {   // more entries tie at the threshold than fit: by index
+      for (int t = threadIdx.x; t < ncand; t += T) {
+        if (abs_key(fs.u.l.cv[t]) != kmin) continue;
+        int order = 0;
+        for (int i = 0; i < t; ++i) order += abs_key(fs.u.l.cv[i]) == kmin;
+        fs.a.rank[t] += order;
+      }
+      __syncthreads();               // (the list's values are replaced below)
+    }
+  } else if (lam_form) {
+    tval = lam0 ? 0.0f : (float)lam;
+    gam = lam0 ? 0.0 : lam;
+    tnext = tval;
+  } else if (exact) {
+    tval = thr;
+  } else {
+    tnext = 0.0f;                    // at most s (or s + 1) nonzero entries: all of them; gamma = 0
+  }
+  if (is_pen(form) && a.calibrate) gam = uses_U(form) ? (double)tval * (double)tval : (double)tval;
+  const bool soft = lam_form || uses_V(form);
+  // an entry survives when its key is above this one (lambda_s: |v| > lam in FP64)
+  const uint32_t cut = lam_form && !lam0 ? __float_as_uint(__double2float_rd(lam))
+                       : ranked && !uses_T(form) ? kmin : 0u;
+
+  // ---- w, which takes the place of the list's values; the survivors are counted per 32 entries
+  const int rounds = (ncand + T - 1) / T;
+  for (int q = 0; q < rounds; ++q) {
+    const int t = threadIdx.x + q * T;
+    float wq = 0.0f;
+    if (t < ncand) {
+      const float v = fs.u.l.cv[t];
+      const uint32_t mine = abs_key(v);
+      bool keep = mine > cut;
+      if (ranked && uses_T(form)) keep = fs.a.rank[t] < need;
+      if (keep) wq = soft ? copysignf(fabsf(v) - tval, v) : v;
+    }
+    const unsigned ball = __ballot_sync(0xffffffffu, wq != 0.0f);
+    if (lane == 0) fs.cnt[q * (T / 32) + w] = __popc(ball);
+    __syncwarp();
+    if (t < ncand) fs.u.l.cv[t] = wq;
+  }
+  __syncthreads();
+  int incl = lane < rounds * (T / 32) ? fs.cnt[lane] : 0;
+  const int own = incl;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  const int nnz = __shfl_sync(0xffffffffu, incl, 31);
+  for (int q = 0; q < rounds; ++q) {
+    const int t = threadIdx.x + q * T;
+    const float wq = t < ncand ? fs.u.l.cv[t] : 0.0f;
+    const unsigned ball = __ballot_sync(0xffffffffu, wq != 0.0f);
+    const int o = __shfl_sync(0xffffffffu, incl - own, q * (T / 32) + w) + __popc(ball & lt_mask);
+    if (wq != 0.0f) {
+      fs.a.s.val[o] = wq;
+      fs.a.s.idx[o] = fs.u.l.ci[t];
+    }
+  }
+  __syncthreads();
+  // ---- ||w||^2, over the survivors as one warp adds them (lane l entries l, l + 32, ...; every warp
+  // repeats it for itself), so that it does not depend on the list or the number of threads.
+  // On a resident 16-bit matrix (ordered) every sweep rounds y to 11 bits, and a last-bit difference of
+  // ||w|| can end as one of 4e-5 in x (measured after 16 sweeps).  There the sum keeps the order of a warp
+  // over the list when that comes from last sweep's threshold (or is exact), and of the full pass, by
+  // index segment and lane, otherwise.
+  const bool seg_order = a.ordered && (p < kSegOrderP || how == kAll || how == kSubsets || (how == kExact && !listed));
+  float sumsq = 0.0f;
+  if (!a.ordered) {
+    for (int t = lane; t < nnz; t += 32) sumsq = fmaf(fs.a.s.val[t], fs.a.s.val[t], sumsq);
+    sumsq = warp_sum_f(sumsq);
+  } else if (!seg_order) {
+    for (int t = lane; t < ncand; t += 32) sumsq = fmaf(fs.u.l.cv[t], fs.u.l.cv[t], sumsq);
+    sumsq = warp_sum_f(sumsq);
+  } else {
+    const bool by_index = p <= 2 * kFastCand;
+    if (by_index) {                  // w at its index, zeros elsewhere
+      for (int i = threadIdx.x; i < p; i += T) fs.u.by_index[i] = 0.0f;
+      __syncthreads();
+      for (int t = threadIdx.x; t < nnz; t += T) fs.u.by_index[fs.a.s.idx[t]] = fs.a.s.val[t];
+      __syncthreads();
+    }
+    for_segments(p, [&](int sgi, Seg sg) {
+      float part = 0.0f;
+      if (by_index) {
+        for (int i = sg.lo + lane; i < sg.hi; i += 32) part = fmaf(fs.u.by_index[i], fs.u.by_index[i], part);
+      } else {
+        for (int t = 0; t < nnz; ++t) {
+          const int i = fs.a.s.idx[t] - sg.lo;
+          if (i >= 0 && i < sg.hi - sg.lo && (i & 31) == lane) part = fmaf(fs.a.s.val[t], fs.a.s.val[t], part);
+        }
+      }
+      put_sum2f(sgi, part, 0.0f, 0, 0, fs.sh);
+    });
+    float f_unused;
+    int i_unused, i_unused2;
+    get_sum2f(sumsq, f_unused, i_unused, i_unused2, fs.sh);
+  }
+  float inv, nrm_hi, nrm_lo;
+  norm_and_inverse(sumsq, &nrm_hi, &nrm_lo, &inv);
+
+  // ---- x and the support list (the zeros above are ordered before these by the barriers since)
+  int *gi = sup_idx ? sup_idx + (int64_t)c * a.cap : nullptr;
+  float *gv = sup_val ? sup_val + (int64_t)c * a.cap : nullptr;
+  for (int t = threadIdx.x; t < nnz; t += T) {
+    const int i = fs.a.s.idx[t];
+    const float xi = fs.a.s.val[t] * inv;
+    x[i] = xi;
+    if (gi && t < a.cap) {
+      gi[t] = i;
+      gv[t] = xi;
+    }
+  }
+  // ---- outputs, stopping rule (Section 2.2), control word for the next sweep
+  if (threadIdx.x == 0) {
+    const double nrm = (double)nrm_hi + (double)nrm_lo;
+    double F;
+    if (lam_form) F = gam * a.sqrt_s + nrm;                              // S4
+    else if (uses_U(form)) F = (double)sumsq - gam * (double)nnz;        // S5
+    else F = nrm;                                                        // S3, S6
+    if (st.F) st.F[c] = F;
+    if (st.nnz) st.nnz[c] = nnz;
+    if (st.gamma) st.gamma[c] = gam;
+    if (st.thr && is_pen(form) && a.calibrate) st.thr[c] = tval;
+    if (st.tprev) st.tprev[c] = tnext;
+    if (st.xfast) {
+      const bool near = tnext >= (1.0f - kSteady) * tprev && tnext <= (1.0f + kSteady) * tprev;
+      st.xfast[c] = how == kExact || (how == kHigh && near) ? 1 : 2;
+    }
+    if (st.status) {
+      int status = ST_ACTIVE;
+      if (sumsq == 0.0f) {
+        status = SPCA_ST_DEGENERATE;
+      } else if (a.stop_test && F <= (1.0 + a.tol) * q0.F_prev) {
+        status = SPCA_ST_CONVERGED;
+      } else if (q0.iters >= a.max_iter) {
+        status = SPCA_ST_MAXITER;
+      }
+      st.F_prev[c] = F;
+      st.status[c] = status;
+      if (status == ST_ACTIVE && ctrl && nnz > a.sparse_cap) atomicOr(&ctrl->need_dense, 1);
+    }
+  }
+  return true;
+}
+
+// the start's x-step: the threshold x-step, else the full pass from global memory at once (defer
+// false) or a mark for k_xstep / k_g_xstep (xfast = 0; without xfast, nnz = -1).  The starts that
+// needed the full pass are counted in ctrl->n_full: the host queues the full kernel, which stages v in
+// shared memory, only for sweeps after some start needed it.
+__device__ __noinline__ void xstep_full_global(const XstepArgs &a, int c, const float *__restrict__ V, int64_t ldv,
+                                               float *__restrict__ X, int64_t ldx, StartState st,
+                                               int *__restrict__ sup_idx, float *__restrict__ sup_val, Ctrl *ctrl,
+                                               XShared &sh) {
+  xstep_full_one(a, c, V, ldv, X, ldx, st, sup_idx, sup_val, ctrl, nullptr, sh);
+}
+template <int T>
+__device__ __forceinline__ void xstep_start(const XstepArgs &a, int c, const float *__restrict__ V, int64_t ldv,
+                                            float *__restrict__ X, int64_t ldx, const StartState &st,
+                                            const XState &q0, int *__restrict__ sup_idx,
+                                            float *__restrict__ sup_val, Ctrl *ctrl, bool defer, FastShared<T> &fs) {
+  if (xstep_fast_one<T>(a, c, V, ldv, X, ldx, st, q0, sup_idx, sup_val, ctrl, fs)) return;
+  if (ctrl && threadIdx.x == 0) atomicAdd(&ctrl->n_full, 1);
+  __syncthreads();
+  if (!defer) {
+    xstep_full_global(a, c, V, ldv, X, ldx, st, sup_idx, sup_val, ctrl, fs.sh);
+    if (threadIdx.x == 0 && st.xfast) st.xfast[c] = 2;
+  } else if (threadIdx.x == 0) {
+    if (st.xfast) st.xfast[c] = 0;
+    else st.nnz[c] = -1;
   }
 }
 
-__global__ void __launch_bounds__(32 * kOpWarps) k_xstep_op(XstepArgs a_in, int r, float *__restrict__ X,
-                                                            int64_t ldx, StartState st, int *__restrict__ sup_idx,
-                                                            float *__restrict__ sup_val,
-                                                            const float *__restrict__ cand_val,
-                                                            const int *__restrict__ cand_idx,
-                                                            const int4 *__restrict__ meta, Ctrl *ctrl) {
-  __shared__ float cval_s[kOpWarps][kCand];
-  __shared__ int cidx_s[kOpWarps][kCand];
-  const int w = threadIdx.x >> 5;
-  const int c = blockIdx.x * kOpWarps + w;
-  if (c >= r) return;
-  xstep_op_one(a_in, c, X, ldx, st, sup_idx, sup_val, cand_val + (int64_t)c * kCand, cand_idx + (int64_t)c * kCand,
-               meta + c, ctrl, cval_s[w], cidx_s[w]);
+// the last CTA of `total` to get here makes the active list of the next sweep and clears the control
+// word that this sweep read (the next x-step writes it)
+__device__ __forceinline__ void last_makes_active_list(int total, const StartState &st, int r, int *act, int *rank,
+                                                       Ctrl *ctrl, Ctrl *ctrl_read) {
+  __shared__ int last;
+  if (threadIdx.x == 0) {   // (thread 0 wrote the start's status and counts: it releases them)
+    int before;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(&ctrl->done) : "memory");
+    last = before == total - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  active_list_body(st.status, st.nnz, r, act, rank, ctrl);
+  if (threadIdx.x == 0) *ctrl_read = Ctrl{};
+}
+
+// (CTAs per SM for the register budget: 7 x 152 of 128 threads hold 1024 starts at once)
+constexpr int fast_ctas(int t) { return t == 128 ? 7 : t == 256 ? 3 : 1; }
+template <int T>
+__global__ void __launch_bounds__(T, fast_ctas(T)) k_xstep_fast(XstepArgs a, const float *__restrict__ V, int64_t ldv,
+                                                            int r, float *__restrict__ X, int64_t ldx, StartState st,
+                                                            int *__restrict__ sup_idx, float *__restrict__ sup_val,
+                                                            Ctrl *ctrl, Ctrl *ctrl_read, int *act, int *rank, int defer) {
+  __shared__ FastShared<T> fs;
+  const int c = blockIdx.x;
+  const int status = st.status ? st.status[c] : ST_ACTIVE;
+  const XState q0 = load_state(st, c);
+  if (status == ST_ACTIVE) xstep_start<T>(a, c, V, ldv, X, ldx, st, q0, sup_idx, sup_val, ctrl, defer != 0, fs);
+  if (act) last_makes_active_list(r, st, r, act, rank, ctrl, ctrl_read);
+}
+
+// Threads per start, 128 to 1024: reading v shrinks with the threads, barriers and the sums over the
+// warps grow with them, so about 64 entries per thread; and never more than keeps all starts resident
+// at once (fast_ctas).
+int fast_threads(int64_t starts, int p, int sms) {
+  const int by_p = p <= 8192 ? 128 : p <= 16384 ? 256 : p <= 32768 ? 512 : 1024;
+  const int by_r = starts <= sms ? 1024 : starts <= 3 * (int64_t)sms ? 256 : 128;
+  return std::min(by_p, by_r);
+}
+// (function-local static: initialised once, thread-safe)
+int sm_count() {
+  static const int sms = [] {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) !=
+                                                   cudaSuccess)
+      return 0;
+    return v;
+  }();
+  return sms;
 }
 }  // namespace
 
-// groups of problems: the full pass for every active start of every problem, persistent CTAs over
-// the global starts; the kSmem launch takes the problems whose v fits in shared memory (staged
-// there), the other launch the rest
+// groups of problems: the full pass for the starts that k_g_xstep_fast left, persistent CTAs over the
+// global starts; the kSmem launch takes the problems whose v fits in shared memory (staged there),
+// the other launch the rest
 template <bool kSmem>
 __global__ void __launch_bounds__(XT, 2) k_g_xstep(const GProb *__restrict__ P, const int *__restrict__ prob, int R,
-                                                   int parity, int cand) {
+                                                   int parity) {
   extern __shared__ float vsm[];
   __shared__ XShared sh;
   for (int g = blockIdx.x; g < R; g += gridDim.x) {
@@ -1067,60 +1271,41 @@ __global__ void __launch_bounds__(XT, 2) k_g_xstep(const GProb *__restrict__ P, 
     if (kSmem != ((size_t)q.p * sizeof(float) <= (size_t)XSTEP_SMEM_MAX)) continue;
     const int c = g - q.start0;
     StartState st = q.st;
-    if (st.status[c] != ST_ACTIVE) continue;
-    if (cand && st.xfast[c]) continue;   // the candidate kernels finished it this sweep
-    st.xfast = nullptr;
+    if (st.status[c] != ST_ACTIVE || st.xfast[c] != 0) continue;
+    __syncthreads();   // (every thread has read the mark; shared memory is reused from start to start)
     xstep_full_one(q.xa, c, q.V, q.ldX, q.X, q.ldX, st, q.sup_idx, q.sup_val, q.ctrl[parity], kSmem ? vsm : nullptr,
                    sh);
-    __syncthreads();   // shared memory is reused by the next start
+    if (threadIdx.x == 0) st.xfast[c] = 2;
+    __syncthreads();
   }
 }
 
-// groups of problems: the candidate kernels for every active start of every problem, as in
-// launch_xstep (a CTA per global start for the filter, a warp per global start for the operator);
-// a problem whose v is shorter than kCandMinPGroup is left to the full pass (xfast = 0).  The
-// threshold is lower than a single problem's kCandMinP: a group's launches are shared by all its
-// starts, so the filter and operator cost no launches of their own per problem.
-__global__ void __launch_bounds__(XT, kFilterMinBlocks) k_g_xstep_filter(const GProb *__restrict__ P,
-                                                                         const int *__restrict__ prob) {
-  __shared__ FilterShared fs;
+// groups of problems: the threshold x-step, a CTA per global start; each problem's last CTA makes its
+// active list unless the full kernel follows (defer)
+template <int T>
+__global__ void __launch_bounds__(T, fast_ctas(T)) k_g_xstep_fast(const GProb *__restrict__ P,
+                                                              const int *__restrict__ prob, int parity, int defer) {
+  __shared__ FastShared<T> fs;
   const GProb &q = P[prob[blockIdx.x]];
   const int c = (int)blockIdx.x - q.start0;
-  if (q.p < kCandMinPGroup) {
-    if (threadIdx.x == 0 && q.st.status[c] == ST_ACTIVE) {
-      q.st.xfast[c] = 0;
-      q.meta[c].w = 0;
-    }
-    return;
-  }
-  xstep_filter_one(q.xa, c, q.V, q.ldX, q.X, q.ldX, q.st, q.sup_idx, q.cand_val + (int64_t)c * kCand,
-                   q.cand_idx + (int64_t)c * kCand, q.meta + c, fs);
+  const int status = q.st.status[c];
+  const XState q0 = load_state(q.st, c);
+  if (status == ST_ACTIVE)
+    xstep_start<T>(q.xa, c, q.V, q.ldX, q.X, q.ldX, q.st, q0, q.sup_idx, q.sup_val, q.ctrl[parity], defer != 0, fs);
+  if (!defer) last_makes_active_list(q.r, q.st, q.r, q.act, q.rank, q.ctrl[parity], q.ctrl[parity ^ 1]);
 }
 
-__global__ void __launch_bounds__(32 * kOpWarps) k_g_xstep_op(const GProb *__restrict__ P, const int *__restrict__ prob,
-                                                              int R, int parity) {
-  __shared__ float cval_s[kOpWarps][kCand];
-  __shared__ int cidx_s[kOpWarps][kCand];
-  const int w = threadIdx.x >> 5;
-  const int g = blockIdx.x * kOpWarps + w;
-  if (g >= R) return;
-  const GProb &q = P[prob[g]];
-  if (q.p < kCandMinPGroup) return;
-  const int c = g - q.start0;
-  xstep_op_one(q.xa, c, q.X, q.ldX, q.st, q.sup_idx, q.sup_val, q.cand_val + (int64_t)c * kCand,
-               q.cand_idx + (int64_t)c * kCand, q.meta + c, q.ctrl[parity], cval_s[w], cidx_s[w]);
-}
-
-cudaError_t launch_g_xstep(const GProb *P, const int *prob, int R, int max_p_small, bool any_large, bool cand,
-                           int parity, int sms, cudaStream_t st) {
-  if (cand) {
-    k_g_xstep_filter<<<R, XT, 0, st>>>(P, prob);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_g_xstep_op<<<(R + kOpWarps - 1) / kOpWarps, 32 * kOpWarps, 0, st>>>(P, prob, R, parity);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+cudaError_t launch_g_xstep(const GProb *P, const int *prob, int R, int max_p, int max_p_small, bool any_large,
+                           bool defer, int parity, int sms, cudaStream_t st) {
+  const int d = defer ? 1 : 0;
+  switch (fast_threads(R, max_p, sms)) {
+    case 1024: k_g_xstep_fast<1024><<<R, 1024, 0, st>>>(P, prob, parity, d); break;
+    case 512: k_g_xstep_fast<512><<<R, 512, 0, st>>>(P, prob, parity, d); break;
+    case 256: k_g_xstep_fast<256><<<R, 256, 0, st>>>(P, prob, parity, d); break;
+    default: k_g_xstep_fast<128><<<R, 128, 0, st>>>(P, prob, parity, d); break;
   }
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || !defer) return e;
   if (max_p_small > 0) {   // the problems whose v fits in shared memory: staged there
     const size_t bytes = (size_t)max_p_small * sizeof(float);
     if (bytes > (size_t)XSTEP_SMEM_MAX) return cudaErrorInvalidValue;
@@ -1128,12 +1313,12 @@ cudaError_t launch_g_xstep(const GProb *P, const int *prob, int R, int max_p_sma
         cudaFuncSetAttribute(k_g_xstep<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, XSTEP_SMEM_MAX);
     if (configured != cudaSuccess) return configured;
     const int per_sm = bytes <= 100u * 1024u ? 2 : 1;
-    k_g_xstep<true><<<min(R, per_sm * sms), XT, bytes, st>>>(P, prob, R, parity, cand ? 1 : 0);
-    const cudaError_t e = cudaGetLastError();
+    k_g_xstep<true><<<min(R, per_sm * sms), XT, bytes, st>>>(P, prob, R, parity);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   if (any_large) {
-    k_g_xstep<false><<<min(R, 2 * sms), XT, 0, st>>>(P, prob, R, parity, cand ? 1 : 0);
+    k_g_xstep<false><<<min(R, 2 * sms), XT, 0, st>>>(P, prob, R, parity);
     return cudaGetLastError();
   }
   return cudaSuccess;
@@ -1143,9 +1328,9 @@ cudaError_t launch_g_xstep(const GProb *P, const int *prob, int R, int max_p_sma
 // For a small matrix the chain of launches of a sweep, not its work, sets the time.  Here every
 // sweep of a start runs in one CTA, all starts at once (a CTA per start): u = A x as a warp per
 // row of A, v = A^T y as a thread per column of A (both on the CUDA cores, sums in a fixed order;
-// A stays in L2 across the sweeps), then the y-step and the full-pass x-step of the
+// A stays in L2 across the sweeps), then the y-step and the threshold x-step of the
 // single-problem path, until the start stops or `sweeps` sweeps have run.  x and y are staged in
-// shared memory; v too, for the x-step.
+// shared memory (which the x-step then uses for its lists); v too where the full pass is needed.
 __global__ void __launch_bounds__(XT) k_small_sweeps(XstepArgs xa, const float *__restrict__ A, int64_t lda, int n,
                                                      int p, float *__restrict__ X, int64_t ldx, float *__restrict__ U,
                                                      float *__restrict__ Y, int64_t ldu, float *__restrict__ V,
@@ -1153,13 +1338,13 @@ __global__ void __launch_bounds__(XT) k_small_sweeps(XstepArgs xa, const float *
                                                      float *__restrict__ sup_val, int sweeps) {
   extern __shared__ float4 sm4[];
   float *sm = reinterpret_cast<float *>(sm4);
-  __shared__ XShared sh;
+  FastShared<XT> &fs = *reinterpret_cast<FastShared<XT> *>(sm4);   // in the x-step, where x and y are not needed
   __shared__ float redf[32];
   const int c = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int p4 = (p + 3) & ~3, n4 = (n + 3) & ~3;
   float *xs = sm;              // x (p), then y (n) in the same place
-  float *vsm = sm + max(p4, n4);
+  float *vsm = sm + max(max(p4, n4), (int)((sizeof(FastShared<XT>) + 15) / 16 * 4));   // v, for the full pass
   const float *x = X + (int64_t)c * ldx;
   float *u = U + (int64_t)c * ldu;
   const float *y = Y + (int64_t)c * ldu;
@@ -1188,7 +1373,11 @@ __global__ void __launch_bounds__(XT) k_small_sweeps(XstepArgs xa, const float *
       v[j] = acc;
     }
     __syncthreads();
-    xstep_full_one(xa, c, V, ldx, X, ldx, st, sup_idx, sup_val, nullptr, vsm, sh);
+    if (!xstep_fast_one<XT>(xa, c, V, ldx, X, ldx, st, load_state(st, c), sup_idx, sup_val, nullptr, fs)) {
+      __syncthreads();
+      xstep_full_one(xa, c, V, ldx, X, ldx, st, sup_idx, sup_val, nullptr, vsm, fs.sh);
+      if (threadIdx.x == 0) st.xfast[c] = 2;
+    }
   }
 }
 
@@ -1208,55 +1397,44 @@ cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, int n
   static const cudaError_t configured =
       cudaFuncSetAttribute(k_small_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize, XSTEP_SMEM_MAX);
   if (configured != cudaSuccess) return configured;
-  const size_t bytes = 4 * (size_t)((((std::max(n, p) + 3) & ~3)) + ((p + 3) & ~3));
+  const size_t bytes = std::max(4 * (size_t)((std::max(n, p) + 3) & ~3), (sizeof(FastShared<XT>) + 15) / 16 * 16) +
+                       4 * (size_t)((p + 3) & ~3);
   k_small_sweeps<<<r, XT, bytes, st>>>(xa, A, lda, n, p, X, ldx, U, Y, ldu, V, s, sup_idx, sup_val, sweeps);
   return cudaGetLastError();
 }
 
 cudaError_t launch_xstep(XstepArgs a, const float *V, int64_t ldv, int r, float *X, int64_t ldx,
-                         StartState s, int *sup_idx, float *sup_val, Ctrl *ctrl_next, XstepScratch scratch,
-                         cudaStream_t st) {
-  // the candidate kernels need the per-start thresholds of the last sweep, 16-byte rows and their
-  // scratch (candidate lists, per-start counts)
-  // (for short v, p < kCandMinP, the full pass alone is cheaper than three launches)
-  const bool cand = a.p >= kCandMinP && s.status && s.tprev && s.xfast && s.thr && ldv % 4 == 0 && ldx % 4 == 0 &&
-                    (reinterpret_cast<uintptr_t>(V) & 15u) == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0 &&
-                    scratch.cand_val && scratch.cand_idx && scratch.meta;
-  if (cand) {
-    k_xstep_filter<<<r, XT, 0, st>>>(a, V, ldv, X, ldx, s, sup_idx, scratch.cand_val, scratch.cand_idx,
-                                     reinterpret_cast<int4 *>(scratch.meta));
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_xstep_op<<<(r + kOpWarps - 1) / kOpWarps, 32 * kOpWarps, 0, st>>>(
-        a, r, X, ldx, s, sup_idx, sup_val, scratch.cand_val, scratch.cand_idx,
-        reinterpret_cast<const int4 *>(scratch.meta), ctrl_next);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  } else {
-    s.xfast = nullptr;
-  }
-  // the full pass for the starts the candidate kernels left: persistent CTAs (as many as fit),
-  // so that a sweep in which every start took the candidate path costs one short launch
-  // (function-local statics: initialised once, thread-safe)
-  static const int sms = [] {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) !=
-                                                   cudaSuccess)
-      return 0;
-    return v;
-  }();
+                         StartState s, int *sup_idx, float *sup_val, Ctrl *ctrl, Ctrl *ctrl_read, int *act,
+                         int *rank, bool defer, cudaStream_t st) {
+  const int sms = sm_count(), d = defer ? 1 : 0;
   if (sms < 1) return cudaErrorInvalidDevice;
+  int *al = defer ? nullptr : act;
+#define SPCA_FAST(T)                                                                                             \
+  k_xstep_fast<T><<<r, T, 0, st>>>(a, V, ldv, r, X, ldx, s, sup_idx, sup_val, ctrl, ctrl_read, al, rank, d)
+  switch (fast_threads(r, a.p, sms)) {
+    case 1024: SPCA_FAST(1024); break;
+    case 512: SPCA_FAST(512); break;
+    case 256: SPCA_FAST(256); break;
+    default: SPCA_FAST(128); break;
+  }
+#undef SPCA_FAST
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || !defer) return e;
+  // the full pass for the starts left: persistent CTAs (as many as fit), so that a sweep in which no
+  // start needs it costs one short launch
   const size_t bytes = (size_t)a.p * sizeof(float);
   if (bytes <= (size_t)XSTEP_SMEM_MAX) {
     static const cudaError_t configured =
         cudaFuncSetAttribute(k_xstep<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, XSTEP_SMEM_MAX);
     if (configured != cudaSuccess) return configured;
     const int per_sm = bytes <= 100u * 1024u ? 2 : 1;
-    k_xstep<true><<<min(r, per_sm * sms), XT, bytes, st>>>(a, V, ldv, r, X, ldx, s, sup_idx, sup_val, ctrl_next);
+    k_xstep<true><<<min(r, per_sm * sms), XT, bytes, st>>>(a, V, ldv, r, X, ldx, s, sup_idx, sup_val, ctrl);
   } else {
-    k_xstep<false><<<min(r, 2 * sms), XT, 0, st>>>(a, V, ldv, r, X, ldx, s, sup_idx, sup_val, ctrl_next);
+    k_xstep<false><<<min(r, 2 * sms), XT, 0, st>>>(a, V, ldv, r, X, ldx, s, sup_idx, sup_val, ctrl);
   }
-  return cudaGetLastError();
+  e = cudaGetLastError();
+  if (e != cudaSuccess || !act) return e;
+  return launch_active_list(s.status, s.nnz, r, act, rank, ctrl, ctrl_read, st);
 }
 
 }  // namespace spca

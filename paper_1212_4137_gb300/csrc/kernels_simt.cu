@@ -172,8 +172,7 @@ __global__ void __launch_bounds__(256) k_ystep_apply(int form, const float *__re
   }
   float tot = 0.0f;
   for (int q = 0; q < nch; ++q) tot += ysum[(int64_t)c * nch + q];
-  const double nrm = sqrt((double)tot);
-  if (nrm == 0.0) {
+  if (tot == 0.0f) {
     if (b == 0) {
       float *x = X + (int64_t)c * ldX;
       for (int j = threadIdx.x; j < p; j += blockDim.x) x[j] = 0.0f;
@@ -185,7 +184,8 @@ __global__ void __launch_bounds__(256) k_ystep_apply(int form, const float *__re
     }
     return;
   }
-  const float inv = (float)(1.0 / nrm);
+  float hi, lo, inv;
+  norm_and_inverse(tot, &hi, &lo, &inv);
   for (int i = b * kYChunk + threadIdx.x; i < i1; i += blockDim.x) {
     const float yi = u[i] * inv;
     if (y) y[i] = yi;
@@ -219,63 +219,16 @@ cudaError_t launch_ystep(int form, const float *U, int64_t ldu, int n, int r, fl
 }
 
 // ------------------------------------------------------------------ active-start list
-// one CTA: ordered compaction of the flags status[c] == ST_ACTIVE over r starts
-__device__ void active_list_body(const int *__restrict__ status, const int *__restrict__ nnz, int r,
-                                 int *__restrict__ act, int *__restrict__ rank, Ctrl *__restrict__ ctrl) {
-  __shared__ int red[32];
-  __shared__ long long red_l[32];
-  __shared__ int red_m[32];
-  int base_pos = 0;
-  long long nz = 0;
-  int mz = 0;
-  for (int base = 0; base < r; base += blockDim.x) {
-    const int c = base + threadIdx.x;
-    const bool on = c < r && status[c] == ST_ACTIVE;
-    int tot;
-    const int pos = base_pos + block_excl_scan_flag(on, red, &tot);
-    if (on) {
-      act[pos] = c;
-      rank[c] = pos;
-      if (nnz) {
-        nz += nnz[c];
-        mz = max(mz, nnz[c]);
-      }
-    }
-    base_pos += tot;
-  }
-  // sum of the active support sizes (a bound on the size of their union)
-  for (int o = 16; o > 0; o >>= 1) {
-    nz += __shfl_xor_sync(0xffffffffu, nz, o);
-    mz = max(mz, __shfl_xor_sync(0xffffffffu, mz, o));
-  }
-  if ((threadIdx.x & 31) == 0) {
-    red_l[threadIdx.x >> 5] = nz;
-    red_m[threadIdx.x >> 5] = mz;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    long long t = 0;
-    int m = 0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-      t += red_l[k];
-      m = max(m, red_m[k]);
-    }
-    ctrl->max_nnz = m;
-    ctrl->active = base_pos;
-    ctrl->use_gather = (ctrl->need_dense == 0 && base_pos > 0) ? 1 : 0;
-    ctrl->sum_nnz = (int)(t < 0x7fffffffLL ? t : 0x7fffffffLL);
-  }
-}
-
 __global__ void __launch_bounds__(1024) k_active_list(const int *__restrict__ status, const int *__restrict__ nnz,
                                                       int r, int *__restrict__ act, int *__restrict__ rank,
-                                                      Ctrl *__restrict__ ctrl) {
+                                                      Ctrl *__restrict__ ctrl, Ctrl *__restrict__ ctrl_read) {
   active_list_body(status, nnz, r, act, rank, ctrl);
+  if (ctrl_read && threadIdx.x == 0) *ctrl_read = Ctrl{};
 }
 
 cudaError_t launch_active_list(const int *status, const int *nnz, int r, int *act, int *rank, Ctrl *c,
-                               cudaStream_t st) {
-  k_active_list<<<1, 1024, 0, st>>>(status, nnz, r, act, rank, c);
+                               Ctrl *ctrl_read, cudaStream_t st) {
+  k_active_list<<<1, 1024, 0, st>>>(status, nnz, r, act, rank, c, ctrl_read);
   return cudaGetLastError();
 }
 
@@ -643,6 +596,8 @@ __global__ void __launch_bounds__(1024) k_g_active(const GProb *__restrict__ P, 
   const GProb &q = P[blockIdx.x];
   if (only_first && !q.first) return;
   active_list_body(q.st.status, q.st.nnz, q.r, q.act, q.rank, q.ctrl[parity]);
+  // (after an x-step: the control word that the sweep read is cleared for the next one)
+  if (!only_first && threadIdx.x == 0) *q.ctrl[parity ^ 1] = Ctrl{};
 }
 
 cudaError_t launch_g_active(const GProb *P, int np, int parity, bool only_first, cudaStream_t st) {
@@ -672,21 +627,18 @@ cudaError_t launch_copy_list(const CopyDesc *list, int count, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// the control words of one sweep parity: cleared before an x-step, and their active counts gathered
-// for the host (out[i] = problem i's count)
-__global__ void k_g_ctrl(const GProb *__restrict__ P, int np, int parity, int clear, int *__restrict__ out) {
+// the control words of one sweep parity gathered for the host: problem i's active count in out[i], the
+// starts that needed the full x-step in that sweep in out[np + i]
+__global__ void k_g_ctrl(const GProb *__restrict__ P, int np, int parity, int *__restrict__ out) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < np; i += gridDim.x * blockDim.x) {
-    Ctrl *c = P[i].ctrl[parity];
-    if (clear) {
-      *c = Ctrl{};
-    } else {
-      out[i] = c->active;
-    }
+    const Ctrl *c = P[i].ctrl[parity];
+    out[i] = c->active;
+    out[np + i] = c->n_full;
   }
 }
 
-cudaError_t launch_g_ctrl(const GProb *P, int np, int parity, int clear, int *out, cudaStream_t st) {
-  k_g_ctrl<<<(np + 255) / 256, 256, 0, st>>>(P, np, parity, clear, out);
+cudaError_t launch_g_ctrl(const GProb *P, int np, int parity, int *out, cudaStream_t st) {
+  k_g_ctrl<<<(np + 255) / 256, 256, 0, st>>>(P, np, parity, out);
   return cudaGetLastError();
 }
 

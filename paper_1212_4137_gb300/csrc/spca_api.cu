@@ -111,13 +111,12 @@ void free_workspace(spca_handle *h) {
                   h->status, h->iters, h->nnz, h->F, h->F_prev, h->gamma, h->f, h->ev, h->thr, h->tprev, h->xfast,
                   h->partials, h->ctrl, h->best, h->y_out, h->x_out, h->support_out, h->nnz_out,
                   h->mark, h->colpos, h->collist, h->AS, h->XS, h->x_scale, h->x_inv, h->Bt, h->sp_part, h->ysum,
-                  h->xs.cand_val, h->xs.cand_idx, h->xs.meta, h->X8, h->Y8, h->x8_inv};
+                  h->X8, h->Y8, h->x8_inv};
   for (void *q : ptrs)
     if (q) cudaFree(q);
   h->X8 = h->Y8 = nullptr;
   h->x8_inv = nullptr;
   h->Bt = h->sp_part = h->ysum = nullptr;
-  h->xs = XstepScratch{};
   h->ldb = 0;
   h->mark = h->colpos = h->collist = nullptr;
   h->AS = h->XS = nullptr;
@@ -161,9 +160,6 @@ int ensure_workspace(spca_handle *h, int r) {
   CK(dalloc(&h->tprev, r)); CK(dalloc(&h->xfast, r));
   CK(dalloc(&h->partials, (size_t)r * nchunks * 2));
   CK(dalloc(&h->ysum, (size_t)r * ((n + kYChunk - 1) / kYChunk)));
-  CK(dalloc(&h->xs.cand_val, (size_t)r * kXstepCand));
-  CK(dalloc(&h->xs.cand_idx, (size_t)r * kXstepCand));
-  CK(dalloc(&h->xs.meta, (size_t)r * 4));
   CK(dalloc(&h->ctrl, 2)); CK(dalloc(&h->best, 1));
   CK(dalloc(&h->y_out, (size_t)h->ldU)); CK(dalloc(&h->x_out, (size_t)h->ldX));
   CK(dalloc(&h->support_out, (size_t)p)); CK(dalloc(&h->nnz_out, 1));
@@ -984,7 +980,7 @@ int spca_xstep(spca_handle *h, int form, double s, double gamma, int calibrate, 
   if (ldv < h->p || ldx < h->p) return fail(h, SPCA_E_INVALID, "leading dimension < p%s");
   RC(check_form_params(h, form, s, gamma, calibrate ? SPCA_GAMMA_TARGET_NNZ : SPCA_GAMMA_FIXED, h->p));
   XstepArgs a{};
-  a.form = form; a.p = (int)h->p; a.s = s;
+  a.form = form; a.p = (int)h->p; a.s = s; a.sqrt_s = std::sqrt(s);
   a.calibrate = is_pen(form) && calibrate;
   a.per_start_thr = 0;
   a.thr_fixed = uses_U(form) ? u_threshold(gamma) : (float)gamma;
@@ -994,8 +990,9 @@ int spca_xstep(spca_handle *h, int form, double s, double gamma, int calibrate, 
   StartState st{};
   st.nnz = nnz; st.F = F; st.gamma = thr;
   RC(enter(h));
-  CK(timed(h, SPCA_K_XSTEP, 1, [&] {
-    return launch_xstep(a, V, ldv, r, X, ldx, st, nullptr, nullptr, nullptr, XstepScratch{}, h->stream);
+  CK(timed(h, SPCA_K_XSTEP, 2, [&] {
+    return launch_xstep(a, V, ldv, r, X, ldx, st, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, true,
+                        h->stream);
   }));
   CK(cudaStreamSynchronize(h->stream));
   return SPCA_OK;
@@ -1020,7 +1017,7 @@ int spca_products(spca_handle *h, int form, int engine, const float *X, int64_t 
   CK(cudaMemsetAsync(h->status, 0xFF, (size_t)r * sizeof(int), st));   // every row active (-1)
   CK(cudaMemsetAsync(h->iters, 0, (size_t)r * sizeof(int), st));
   CK(cudaMemsetAsync(h->ctrl, 0, sizeof(Ctrl), st));
-  CK(launch_active_list(h->status, nullptr, r, h->act, h->rank, &h->ctrl[0], st));
+  CK(launch_active_list(h->status, nullptr, r, h->act, h->rank, &h->ctrl[0], nullptr, st));
   RC(sweep_u_dense(h, eng, r, nullptr, &h->ctrl[0].active, r, lowp));
   RC(sweep_lowrank_u(h, r, &h->ctrl[0].active, h->act));
   RC(sweep_y_v(h, eng, form, r, state_of(h), &h->ctrl[0].active, r, lowp));
@@ -1116,16 +1113,17 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
   memset(&h->h_ctrl[0], 0, sizeof(Ctrl));
   h->h_ctrl[0].active = r;
   h->h_ctrl[0].need_dense = 1;      // x^(0) is dense: the first sweep's u = A x is the dense one
-  CK(cudaMemcpyAsync(h->ctrl, h->h_ctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, st));
+  memset(&h->h_ctrl[1], 0, sizeof(Ctrl));   // (each sweep clears the word it read for the next one)
+  CK(cudaMemcpyAsync(h->ctrl, h->h_ctrl, 2 * sizeof(Ctrl), cudaMemcpyHostToDevice, st));
   CK(timed(h, SPCA_K_XSTEP, 1,
-           [&] { return launch_active_list(h->status, nullptr, r, h->act, h->rank, &h->ctrl[0], st); }));
+           [&] { return launch_active_list(h->status, nullptr, r, h->act, h->rank, &h->ctrl[0], nullptr, st); }));
   CK(cudaMemcpyAsync(h->h_ctrl + 1, h->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));  // h_ctrl is reused below
   int nhost = h->h_ctrl[1].active;  // active starts as the host knows them (sizes the launches)
 
   // ---- the sweeps (Algorithm 2)
   XstepArgs xa{};
-  xa.form = form; xa.p = p; xa.s = P.s;
+  xa.form = form; xa.p = p; xa.s = P.s; xa.sqrt_s = std::sqrt(P.s);
   xa.thr_fixed = uses_U(form) ? u_threshold(P.gamma) : (float)P.gamma;
   xa.gamma_fixed = P.gamma;
   xa.tol = P.tol; xa.max_iter = max_iter;
@@ -1143,6 +1141,7 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
   // low-precision ones)
   xa.lowp_sweeps = all_lowp ? 0 : F0 + L;
   xa.stop_enabled = P.tol >= 0.0 ? 1 : 0;
+  xa.ordered = all_lowp ? 1 : 0;
   // the host queues this many sweeps before it reads the active count back; every path decision
   // inside a sweep is taken on the device from the control word
   const int check_every = 4;
@@ -1157,13 +1156,17 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
   const int sparse_cap = xa.sparse_cap;
   int64_t max_nnz = uses_T(form) ? std::min<int64_t>((int64_t)P.s, p) : p;
   bool dense_queued = true;   // x^(0) is dense
+  // the full x-step is a kernel of its own (v in shared memory) while some start may need it; else
+  // such a start takes it inside the x-step kernel, and the launch is saved.  Before the first
+  // read-back: when the threshold x-step's short list cannot or may not hold the result
+  bool full_queued = xstep_may_need_full(form, P.s, target);
   // The sweeps are queued in segments that end at a read-back (every check_every sweeps).  A
   // segment's host decisions (the plan: which optional launches, the x-step's switches) are made
   // up front from the last read-back; its kernels are captured into a CUDA graph once per distinct
   // plan and replayed, so that in steady state a segment is one launch.
   struct SweepPlan {
     int k;
-    bool lowp, dense_in, union_in, union_out;
+    bool lowp, dense_in, union_in, union_out, full;
     int sparse_cap;
   };
   auto enqueue = [&](const SweepPlan &pl) -> int {
@@ -1191,11 +1194,13 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
     RC(sweep_lowrank_u(h, r, &cur->active, h->act));
     // y-step, v = A^T y
     RC(sweep_y_v(h, engine, form, r, S, &cur->active, r, pl.lowp));
-    CK(cudaMemsetAsync(nxt, 0, sizeof(Ctrl), st));
     XstepArgs xk = xa;
     xk.sparse_cap = pl.sparse_cap;
-    CK(timed(h, SPCA_K_XSTEP, 3, [&] {   // candidate filter and operator, full x-step
-      return launch_xstep(xk, h->V, h->ldX, r, h->X, h->ldX, S, h->sup_idx, h->sup_val, nxt, h->xs, st);
+    // the x-step, and the active list of the next sweep (on-the-fly replacement makes it below, once
+    // the stopped slots have their next starts)
+    CK(timed(h, SPCA_K_XSTEP, pl.full ? (otf ? 2 : 3) : 1, [&] {
+      return launch_xstep(xk, h->V, h->ldX, r, h->X, h->ldX, S, h->sup_idx, h->sup_val, nxt, cur,
+                          otf ? nullptr : h->act, h->rank, pl.full, st);
     }));
     if (otf) {
       // stopped slots: archive their start, give them the next starts (Section 4.3)
@@ -1206,10 +1211,10 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
         return launch_start_init(x0src, ld0, P.seed, r, p, h->X, h->ldX, S, gamma0, h->new_slot, h->slot_start,
                                  &nxt->n_new, st);
       }));
+      CK(timed(h, SPCA_K_XSTEP, 1, [&] {
+        return launch_active_list(h->status, h->nnz, r, h->act, h->rank, nxt, cur, st);
+      }));
     }
-    CK(timed(h, SPCA_K_XSTEP, 1, [&] {   // the active list of the next sweep
-      return launch_active_list(h->status, h->nnz, r, h->act, h->rank, nxt, st);
-    }));
     if (pl.union_out) {
       CK(timed(h, SPCA_K_U_SPARSE, 2, [&] {
         return launch_union(h->sup_idx, p, S, r, p, h->mark, h->colpos, h->collist, h->kcap, nxt, st);
@@ -1277,13 +1282,14 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
       pl.dense_in = dense_queued;
       pl.union_in = union_built;
       dense_queued = max_nnz > sparse_cap / 2;
+      pl.full = full_queued;
       pl.sparse_cap = dense_queued ? sparse_cap : p;   // p: the gather for every support
       const bool next_lowp = k + 1 > F0 && k + 1 <= F0 + L;
       union_built = engine == SPCA_ENGINE_TC && !otf && !all_lowp && !next_lowp && sum_nnz <= (int64_t)kUnionTry * h->kcap &&
                     h->n * sum_nnz >= kUnionMinReads;
       pl.union_out = union_built;
       plans.push_back(pl);
-      key.insert(key.end(), {pl.lowp, pl.dense_in, pl.union_in, pl.union_out, pl.sparse_cap});
+      key.insert(key.end(), {pl.lowp, pl.dense_in, pl.union_in, pl.union_out, pl.full, pl.sparse_cap});
     }
     SegGraph *g = nullptr;
     for (SegGraph &c : graphs)
@@ -1338,6 +1344,7 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
     nhost = h->h_ctrl->active;   // counts only fall: any earlier value stays an upper bound
     sum_nnz = h->h_ctrl->sum_nnz;
     max_nnz = h->h_ctrl->max_nnz;
+    full_queued = h->h_ctrl->n_full > 0;
     k0 = k1 + 1;
   }
   RC(rc);

@@ -15,7 +15,6 @@ using spca::OtfArchive;
 using spca::PMaps;
 using spca::SpPlan;
 using spca::TcStreamK;
-using spca::XstepScratch;
 
 // one captured segment of sweeps: the plan it was captured for, the executable graph, and the
 // launch counts and timing events of its kernels
@@ -58,7 +57,6 @@ struct spca_handle {
   float *Wd = nullptr, *Zd = nullptr;
   double *lr_coef = nullptr;
   int lr_rows = 0;
-  XstepScratch xs{};                       // the candidate x-step's lists and counts
   bool tc_ok = false;                      // the device has tcgen05 tensor cores (sm_100+)
   // SPCA_FP16_RESIDENT: only the leading FP16 planes of A and A^T (one plane each, A32 and AT32
   // freed after create); every sweep is a low-precision sweep

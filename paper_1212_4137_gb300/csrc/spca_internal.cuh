@@ -54,6 +54,8 @@ struct Ctrl {
   int n_retire;    // on-the-fly replacement: slots whose start stopped in this sweep ...
   int n_new;       // ... and how many of them took a new start (dense x: the next u = A x of
                    // those slots is the dense contraction over them)
+  int n_full;      // starts whose x-step took the full pass in this sweep
+  int done;        // CTAs of the x-step that have finished (the last one makes the active list)
 };
 
 // per-start state of one solve (device arrays, r each)
@@ -67,15 +69,16 @@ struct StartState {
   float *thr;       // the same threshold in |v| units, as a float the kernels compare with
   double *f;        // Table 1 objective (finalise)
   double *ev;       // explained variance (finalise)
-  float *tprev;     // last sweep's x-step threshold in |v| units (0: none); seeds the
-                    // candidate filter of the next x-step
-  int *xfast;       // nonzero when the candidate x-step finished the start in this sweep (its guess)
+  float *tprev;     // last sweep's x-step threshold in |v| units (0: none); the next x-step's bound
+  int *xfast;       // the last x-step: 1 when the threshold held steady, 2 when not, 0 while a start
+                    // is left to the full pass
 };
 
 struct XstepArgs {
   int form;
   int p;
   double s;
+  double sqrt_s;
   int calibrate;       // apply the Section 4.1 gamma rule in this sweep
   int per_start_thr;   // penalty threshold from StartState (frozen after calibration)
   float thr_fixed;     // otherwise: the fixed threshold in |v| units ...
@@ -94,12 +97,13 @@ struct XstepArgs {
   int calib_sweeps;
   int lowp_sweeps;
   int stop_enabled;
+  int ordered;         // ||w||^2 added in an order that does not depend on how the x-step found its
+                       // list (resident 16-bit matrices, whose every sweep rounds y to 11 bits)
 };
 
-// the x-step switches of start c under XstepArgs::schedule (else as given)
-__device__ inline XstepArgs xstep_switches(XstepArgs a, const int *iters, int c) {
+// the x-step switches of a start in its sweep `it` under XstepArgs::schedule (else as given)
+__device__ inline XstepArgs xstep_switches(XstepArgs a, int it) {
   if (!a.schedule) return a;
-  const int it = iters[c];
   a.calibrate = a.target && it <= a.calib_sweeps;
   a.per_start_thr = a.target && it > a.calib_sweeps;
   a.stop_test = a.stop_enabled && it >= 2 && it >= a.calib_sweeps + 1 && it >= a.lowp_sweeps + 2;
@@ -400,11 +404,6 @@ struct GProb {
   int vbase;
   int *yoff;
   int first;                    // its first sweep is the next one (its starts are set up then)
-  // the candidate x-step's scratch of the member's starts (kXstepCand values and indices, one
-  // int4 of counts per start), or null
-  float *cand_val;
-  int *cand_idx;
-  int4 *meta;
   float *X, *V, *U;             // r x ldX, r x ldX, r x ldU
   __half *Xpl, *Ypl;            // two FP16 planes each (x row-scaled, y scaled by kQScale), packed rows
   int64_t xps, yps;             // plane strides (elements)
@@ -443,17 +442,16 @@ struct CopyDesc {
   int64_t bytes;
 };
 cudaError_t launch_copy_list(const CopyDesc *list, int count, cudaStream_t st);
-// clear (clear != 0) the control words of one parity, or gather their active counts into out[np]
-cudaError_t launch_g_ctrl(const GProb *P, int np, int parity, int clear, int *out, cudaStream_t st);
+// one parity's control words: the active counts into out[np], the counts of full x-steps behind them
+cudaError_t launch_g_ctrl(const GProb *P, int np, int parity, int *out, cudaStream_t st);
 cudaError_t launch_g_xplanes(const GProb *P, const int *prob, int R, cudaStream_t st);
 cudaError_t launch_g_gather(const GProb *P, const int *prob, int R, int max_n, cudaStream_t st);
 cudaError_t launch_g_ystep(const GProb *P, const int *prob, int R, cudaStream_t st);
-// (max_p_small: the longest v that fits in shared memory, 0 if none; any_large: some v does not;
-// cand: the candidate kernels first, with the problems' scratch (GProb.cand_val ...))
-cudaError_t launch_g_xstep(const GProb *P, const int *prob, int R, int max_p_small, bool any_large, bool cand,
-                           int parity, int sms, cudaStream_t st);
+// (max_p: the longest v; max_p_small: the longest that fits in shared memory, 0 if none; any_large: some v does not;
+// defer: the full pass in kernels of its own, and no active lists, see launch_xstep)
+cudaError_t launch_g_xstep(const GProb *P, const int *prob, int R, int max_p, int max_p_small, bool any_large,
+                           bool defer, int parity, int sms, cudaStream_t st);
 constexpr int kXstepSmemMaxP = 200 * 1024 / 4;   // the longest v the x-step stages in shared memory
-constexpr int kCandMinPGroup = 512;              // shorter v: the grouped x-step's full pass only
 
 // Grouped contraction: one persistent launch over the tiles of many contractions (one per problem
 // of a group), each described by a task in device memory, its tiles listed in tile_list (task,
@@ -529,18 +527,15 @@ cudaError_t launch_union_operands(const float *AT, int64_t ldat, const float *a_
 // ordered list of the active starts (status == ST_ACTIVE): act[k] = c and rank[c] = k for the
 // k-th active start; c->active = the count, c->use_gather = !c->need_dense (the union step,
 // when it runs afterwards, may take the sweep over)
+// ctrl_read (or null): the control word this sweep read, cleared for the next x-step
 cudaError_t launch_active_list(const int *status, const int *nnz, int r, int *act, int *rank, Ctrl *c,
-                               cudaStream_t st);
+                               Ctrl *ctrl_read, cudaStream_t st);
 
-// x-step (S3..S6), objective F, stopping rule, support lists.  The candidate path needs scratch of
-// kXstepCand candidates (value, index) and one int4 per start; without it every start takes the
-// full pass.
-constexpr int kXstepCand = 1024;
-struct XstepScratch {
-  float *cand_val = nullptr;   // r * kXstepCand
-  int *cand_idx = nullptr;     // r * kXstepCand
-  int *meta = nullptr;         // r * 4 (16-byte aligned)
-};
+// whether the threshold x-step may leave starts to the full pass from the first sweep on: results near
+// or beyond the length of its list (a fixed penalty's first sweep can keep any number of entries)
+inline bool xstep_may_need_full(int form, double s, bool target) {
+  return is_pen(form) && !target ? true : s > (uses_lam(form) ? 150.0 : 500.0);
+}
 // small problems (n p <= kSmallAlwaysEntries, or <= kSmallMaxEntries with at least
 // kSmallMinStarts starts; x, y and v in shared memory): every sweep of every start in one launch,
 // a CTA per start (u = A x and v = A^T y on the CUDA cores from A, the y-step writing Y, the
@@ -552,9 +547,13 @@ bool small_sweeps_fit(int64_t n, int64_t p, int r);
 cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, int n, int p, float *X, int64_t ldx,
                                 float *U, float *Y, int64_t ldu, float *V, StartState s, int *sup_idx, float *sup_val,
                                 int r, int sweeps, cudaStream_t st);
+// x-step (S3..S6), objective F, stopping rule, support lists, and (act given) the next sweep's active
+// list in *ctrl, which must be zero before; ctrl_read is cleared (see launch_active_list).  defer: a
+// second kernel runs the full pass of the starts that need it, with v in shared memory (else the
+// first one does, from global memory)
 cudaError_t launch_xstep(XstepArgs a, const float *V, int64_t ldv, int r, float *X, int64_t ldx,
-                         StartState s, int *sup_idx, float *sup_val, Ctrl *ctrl_next, XstepScratch scratch,
-                         cudaStream_t st);
+                         StartState s, int *sup_idx, float *sup_val, Ctrl *ctrl, Ctrl *ctrl_read, int *act,
+                         int *rank, bool defer, cudaStream_t st);
 
 // a7: Table 1 objective in FP64 for every start; u of each start into U
 // (partials: r * ceil(n / 256) * 2 doubles of scratch)

@@ -1,5 +1,5 @@
 // sweep_bodies.cuh -- the per-start bodies of the start initialisation (Algorithm 2, "select
-// initial point") and of the y-step (Table 3, S1 and S2), shared by the kernels that run them one
+// initial point") and of the y-step (Table 3, S1 and S2), and the active list, shared by the kernels that run them one
 // start per CTA: the single-problem kernels, the grouped kernels and the one-launch solve of small
 // problems.
 #pragma once
@@ -45,13 +45,13 @@ static __device__ void start_init_body(const float *__restrict__ x0, int64_t ld0
     x[j] = gj;
     part = fmaf(gj, gj, part);
   }
-  const double nrm = sqrt((double)block_sum_f(part, redf));
-  const float inv = nrm > 0.0 ? (float)(1.0 / nrm) : 0.0f;
+  float nrm, lo, inv;
+  norm_and_inverse(block_sum_f(part, redf), &nrm, &lo, &inv);
   for (int j = threadIdx.x; j < p; j += blockDim.x) x[j] = x[j] * inv;
   if (threadIdx.x == 0) {
-    s.status[c] = (nrm > 0.0) ? ST_ACTIVE : SPCA_ST_DEGENERATE;
+    s.status[c] = (nrm > 0.0f) ? ST_ACTIVE : SPCA_ST_DEGENERATE;
     s.iters[c] = 0;
-    s.nnz[c] = (nrm > 0.0) ? p : 0;
+    s.nnz[c] = (nrm > 0.0f) ? p : 0;
     s.F[c] = 0.0;
     s.F_prev[c] = 0.0;
     s.gamma[c] = gamma0;
@@ -104,8 +104,8 @@ static __device__ void ystep_body(int form, const float *__restrict__ U, int64_t
     part = fmaf(uv.w, uv.w, part);
   }
   for (int i = n4 + threadIdx.x; i < n; i += blockDim.x) part = fmaf(u[i], u[i], part);
-  const double nrm = sqrt((double)block_sum_f(part, redf));
-  if (nrm == 0.0) {
+  const float sumsq = block_sum_f(part, redf);
+  if (sumsq == 0.0f) {
     float *x = X + (int64_t)c * ldX;
     for (int j = threadIdx.x; j < p; j += blockDim.x) x[j] = 0.0f;
     if (threadIdx.x == 0) {
@@ -115,7 +115,8 @@ static __device__ void ystep_body(int form, const float *__restrict__ U, int64_t
     }
     return;
   }
-  const float inv = (float)(1.0 / nrm);
+  float hi, lo, inv;
+  norm_and_inverse(sumsq, &hi, &lo, &inv);
   // y = u / ||u||_2, and its planes: kQScale y is exact (a power of two), |kQScale y| <= 2^14
   auto planes = [&](float yi, __half &hi, __half &lo) {
     const float ys = yi * kQScale;
@@ -149,6 +150,74 @@ static __device__ void ystep_body(int form, const float *__restrict__ U, int64_t
       yp[i] = hi;
       yp[i + pstride] = lo;
     }
+  }
+}
+
+// ------------------------------------------------------------------ active-start list
+// one CTA: ordered compaction of the flags status[c] == ST_ACTIVE over r starts (read from L2: other
+// CTAs of the same launch may have written them), 4 consecutive starts per thread and round, their
+// loads in flight together
+static __device__ void active_list_body(const int *status, const int *nnz, int r, int *act, int *rank, Ctrl *ctrl) {
+  __shared__ int warp_n[32];
+  __shared__ long long red_l[32];
+  __shared__ int red_m[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+  int base_pos = 0;
+  long long nz = 0;
+  int mz = 0;
+  for (int base = 0; base < r; base += 4 * blockDim.x) {
+    const int c0 = base + 4 * threadIdx.x;
+    int s[4], k[4], mine = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      s[q] = c0 + q < r ? __ldcg(status + c0 + q) : ST_ACTIVE + 1;
+      k[q] = nnz && c0 + q < r ? __ldcg(nnz + c0 + q) : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (s[q] == ST_ACTIVE) {
+        ++mine;
+        nz += k[q];
+        mz = max(mz, k[q]);
+      }
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (base > 0) __syncthreads();   // (the last round's counts are read)
+    if (lane == 31) warp_n[w] = incl;
+    __syncthreads();
+    const int n = lane < nw ? warp_n[lane] : 0;
+    int pos = base_pos + incl - mine + __reduce_add_sync(0xffffffffu, lane < w ? n : 0);
+    base_pos += __reduce_add_sync(0xffffffffu, n);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (s[q] == ST_ACTIVE) {
+        act[pos] = c0 + q;
+        rank[c0 + q] = pos++;
+      }
+  }
+  // sum of the active support sizes (a bound on the size of their union)
+  for (int o = 16; o > 0; o >>= 1) nz += __shfl_xor_sync(0xffffffffu, nz, o);
+  mz = __reduce_max_sync(0xffffffffu, mz);
+  if (lane == 0) {
+    red_l[w] = nz;
+    red_m[w] = mz;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    long long t = 0;
+    int m = 0;
+    for (int k = 0; k < nw; ++k) {
+      t += red_l[k];
+      m = max(m, red_m[k]);
+    }
+    ctrl->max_nnz = m;
+    ctrl->active = base_pos;
+    ctrl->use_gather = (__ldcg(&ctrl->need_dense) == 0 && base_pos > 0) ? 1 : 0;
+    ctrl->sum_nnz = (int)(t < 0x7fffffffLL ? t : 0x7fffffffLL);
   }
 }
 
