@@ -629,18 +629,19 @@ __global__ void __launch_bounds__(TC2_THREADS, 1)
     mma_commit_pair(smem_u32(&mma_done_bar));
   } else if (warp >= 2) {
     // ---------------------------------------------------------------- epilogue (own 128 rows)
-    // warp w reads TMEM lanes 32 (w mod 4) .. + 31 (rows of this CTA's half of the tile) and
-    // columns 128 h .. 128 h + 127, h = (w - 2) / 4; the running sum of those 128 columns of its
-    // row stays in registers, so a split drain costs four TMEM loads and no memory traffic
+    // warp w reads TMEM lanes 32 (w mod 4) .. + 31 (rows of this CTA's half of the tile) and half
+    // h = (w - 2) / 4 of the columns; the running sum of those HC columns of its row stays in
+    // registers, so a split drain costs TMEM loads and no memory traffic
+    constexpr int HC = BN / 2;
     const int quad = warp & 3, half = (warp - 2) >> 2;
     const uint32_t tmem_empty_leader = map_to_rank(smem_u32(&tmem_empty_bar), 0);
-    const int row_l = quad * 32 + lane, cbase = half * 128;
+    const int row_l = quad * 32 + lane, cbase = half * HC;
     const uint32_t tbase = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)cbase;
     const bool has_corr = pairs.first_corr >= 0;
     uint32_t nd = 0;
     bool ok = true;
     for (long long u = u0; u < u1 && ok;) {
-      float acc[128];
+      float acc[HC];
       long long t;
       int kb0, kb1;
       next_seg(u, t, kb0, kb1);
@@ -656,7 +657,7 @@ __global__ void __launch_bounds__(TC2_THREADS, 1)
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (d == 0) {
 #pragma unroll
-          for (int cb = 0; cb < 8; ++cb) {
+          for (int cb = 0; cb < HC / 16; ++cb) {
             float v[16];
             tmem_ld16(tbase + (uint32_t)(cb * 16), v);
 #pragma unroll
@@ -664,7 +665,7 @@ __global__ void __launch_bounds__(TC2_THREADS, 1)
           }
         } else {
 #pragma unroll
-          for (int cb = 0; cb < 8; ++cb) {
+          for (int cb = 0; cb < HC / 16; ++cb) {
             float v[16];
             tmem_ld16(tbase + (uint32_t)(cb * 16), v);
 #pragma unroll
@@ -673,7 +674,7 @@ __global__ void __launch_bounds__(TC2_THREADS, 1)
         }
         if (d == nsplit && has_corr) {
 #pragma unroll
-          for (int cb = 0; cb < 8; ++cb) {
+          for (int cb = 0; cb < HC / 16; ++cb) {
             float v[16];
             tmem_ld16(tbase + (uint32_t)BN + (uint32_t)(cb * 16), v);
 #pragma unroll
@@ -714,7 +715,7 @@ __global__ void __launch_bounds__(TC2_THREADS, 1)
       float *mine = ws + ((int64_t)slot * 2 + rank) * BN * TC_BM;
       if (contrib) {
 #pragma unroll
-        for (int c = 0; c < 128; ++c) __stcg(mine + (int64_t)(cbase + c) * TC_BM + row_l, acc[c]);
+        for (int c = 0; c < HC; ++c) __stcg(mine + (int64_t)(cbase + c) * TC_BM + row_l, acc[c]);
         // this part of the tile is in the workspace: each warp signals its rows, then warp 2
         // publishes the part once all of them have (a bounded wait on an mbarrier rather than a
         // named barrier, so that a warp that gave up cannot leave the others blocked)
@@ -731,7 +732,7 @@ __global__ void __launch_bounds__(TC2_THREADS, 1)
           if (R.start(jj) >= R.start(jj + 1)) continue;
           const float *part = ws + ((int64_t)jj * 2 + rank) * BN * TC_BM + (int64_t)cbase * TC_BM + row_l;
 #pragma unroll
-          for (int cb = 0; cb < 8; ++cb) {   // 16 loads in flight at a time
+          for (int cb = 0; cb < HC / 16; ++cb) {   // 16 loads in flight at a time
             float v[16];
 #pragma unroll
             for (int j = 0; j < 16; ++j) v[j] = __ldcg(part + (int64_t)(cb * 16 + j) * TC_BM);
@@ -745,7 +746,7 @@ __global__ void __launch_bounds__(TC2_THREADS, 1)
       if (row < M && ok) {
         const float sc = (row_inv ? row_inv[row] : 1.0f) * q_inv;   // powers of two
 #pragma unroll
-        for (int c = 0; c < 128; ++c) {
+        for (int c = 0; c < HC; ++c) {
           const int col = n0 + cbase + c;
           if (col < N)
             out[(int64_t)(col_map ? col_map[col] : col) * ldo + row] = acc[c] * sc * (col_inv ? col_inv[col] : 1.0f);
@@ -1018,22 +1019,18 @@ cudaError_t launch_tc2_impl(const PMaps &P, const CUtensorMap &Q, int M, int N, 
 }  // namespace
 
 // N width of the CTA-pair tile: 256 (512 TMEM columns: the hi x hi and the correction
-// accumulators of 256 columns each) or 128; each CTA of a pair loads BN / 2 rows of Q, and the
-// single-CTA tile used for a lone M tile is BN / 2 wide so that both read the same Q boxes
-#ifndef SPCA_TC_PAIR_BN
-#define SPCA_TC_PAIR_BN 256
-#endif
-constexpr int TC_PAIR_BN = SPCA_TC_PAIR_BN;
-static_assert(TC_PAIR_BN == 128 || TC_PAIR_BN == 256, "pair tile width");
+// accumulators of 256 columns each), narrower for few columns (pair_width); each CTA of a pair loads
+// half of its rows of Q, and the single-CTA tile used for a lone M tile is 128 wide
+constexpr int TC_PAIR_BN = 256;
 
 namespace {
 // pipeline stages that fit in shared memory (227 KB per CTA, less 1 KB of alignment slack and
 // 1 KB of barriers): na P planes of 128 x 64 plus nb Q planes of (BN / 2) x 64, FP16 -- the same
-// per CTA for the pair tile and for the single-CTA tile; at most 8
-constexpr int tc_stages(int na, int nb) {
-  return (230400 / (na * TC_BM * 64 * 2 + nb * (TC_PAIR_BN / 2) * 64 * 2)) > 8
-             ? 8
-             : 230400 / (na * TC_BM * 64 * 2 + nb * (TC_PAIR_BN / 2) * 64 * 2);
+// per CTA for the pair tile and for the single-CTA tile; at most 8, or 12 for the
+// narrow tiles
+constexpr int tc_stages(int na, int nb, int bn = TC_PAIR_BN) {
+  const int fit = 230400 / (na * TC_BM * 64 * 2 + nb * (bn / 2) * 64 * 2), most = bn < TC_PAIR_BN ? 12 : 8;
+  return fit > most ? most : fit;
 }
 
 // the single-CTA kernel: 128 x (BN / 2) tiles
@@ -1055,24 +1052,47 @@ cudaError_t launch_gemm_tc_single(const PMaps &P, int na, const CUtensorMap &Q, 
 }
 }  // namespace
 
-// CTA pairs (256 x BN tiles, stream-K over the resident pairs) when there are at least two M
+// Tile width of the pair kernel for N columns.  Up to 128 starts fill less than half of a 256-wide
+// tile, whose MMAs and Q loads then set the time instead of the one read of the P planes: a tile just
+// wide enough leaves the kernel to HBM.  A start's sums are the same at every width (the same K order,
+// pieces and stream-K split: one column of tiles either way).  v = A^T y from 16 starts, before
+// and now: 500 x 100000, y = +-1, 79 -> 53 us; 9001 x 17003, leading planes, 85 -> 72 us (a bare TMA
+// stream of the same planes: 47 and 67 us).
+int pair_width(int N) { return N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : TC_PAIR_BN; }
+
+cudaError_t make_q_maps(QMaps *q, const void *base, int64_t rows, int64_t ld, int planes) {
+  const int width[4] = {32, 64, 128, TC_PAIR_BN};
+  for (int i = 0; i < 4; ++i) {
+    const cudaError_t e = make_plane_map(&q->m[i], base, rows, ld, planes, width[i] / 2, 64);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// CTA pairs (256-row tiles, stream-K over the resident pairs) when there are at least two M
 // tiles; one M tile runs on single CTAs
-cudaError_t launch_gemm_tc(const PMaps &P, int na, const CUtensorMap &Q, int nb, int M, int N, int K,
+cudaError_t launch_gemm_tc(const PMaps &P, int na, const QMaps &Q, int nb, int M, int N, int K,
                            const int *k_dev, TcPairs pairs, float *out, int64_t ldo, const float *row_inv,
                            const float *col_inv, float q_inv, const int *gate, const int *n_dev, const int *col_map,
                            int *err, const TcStreamK &sk, cudaStream_t st) {
   if (M <= TC_BM || !sk.ws || !sk.flags || sk.slots < 1)
-    return launch_gemm_tc_single(P, na, Q, nb, M, N, K, k_dev, pairs, out, ldo, row_inv, col_inv, q_inv, gate,
+    return launch_gemm_tc_single(P, na, Q.m[3], nb, M, N, K, k_dev, pairs, out, ldo, row_inv, col_inv, q_inv, gate,
                                  n_dev, col_map, err, sk.wait_ns, st);
-  if (na == 2 && nb == 2)   // two general operands
-    return launch_tc2_impl<TC_PAIR_BN, 2, 2, tc_stages(2, 2)>(P, Q, M, N, K, k_dev, pairs, out, ldo, row_inv,
-                                                                col_inv, q_inv, gate, n_dev, col_map, err, sk, st);
-  if (na == 2 && nb == 1)   // y = +-1
-    return launch_tc2_impl<TC_PAIR_BN, 2, 1, tc_stages(2, 1)>(P, Q, M, N, K, k_dev, pairs, out, ldo, row_inv,
-                                                                col_inv, q_inv, gate, n_dev, col_map, err, sk, st);
-  if (na == 1 && nb == 1)   // the leading planes only (low-precision sweeps)
-    return launch_tc2_impl<TC_PAIR_BN, 1, 1, tc_stages(1, 1)>(P, Q, M, N, K, k_dev, pairs, out, ldo, row_inv,
-                                                                col_inv, q_inv, gate, n_dev, col_map, err, sk, st);
+  const int bn = pair_width(N);
+#define SPCA_PAIR(A, B, BN, I)                                                                                       \
+  if (na == A && nb == B && bn == BN)                                                                                \
+    return launch_tc2_impl<BN, A, B, tc_stages(A, B, BN)>(P, Q.m[I], M, N, K, k_dev, pairs, out, ldo, row_inv,       \
+                                                          col_inv, q_inv, gate, n_dev, col_map, err, sk, st);
+#define SPCA_PAIRS(A, B)       \
+  SPCA_PAIR(A, B, 32, 0)       \
+  SPCA_PAIR(A, B, 64, 1)       \
+  SPCA_PAIR(A, B, 128, 2)      \
+  SPCA_PAIR(A, B, TC_PAIR_BN, 3)
+  SPCA_PAIRS(2, 2)   // two general operands
+  SPCA_PAIRS(2, 1)   // y = +-1
+  SPCA_PAIRS(1, 1)   // the leading planes only (low-precision sweeps)
+#undef SPCA_PAIRS
+#undef SPCA_PAIR
   return cudaErrorInvalidValue;
 }
 
@@ -1363,10 +1383,9 @@ cudaError_t launch_gemm_grouped(const GTask *tasks, const int2 *tile_list, int t
   return cudaErrorInvalidValue;
 }
 
-int tc_box_rows(int nb) { (void)nb; return TC_PAIR_BN / 2; }
+int tc_f8_box_rows() { return TC_PAIR_BN / 2; }
 
 // workspace of the stream-K schedule: one 256 x BN FP32 part per pair slot
 int64_t tc_sk_floats_per_slot() { return (int64_t)2 * TC_BM * TC_PAIR_BN; }
-int tc_bk(int nb) { (void)nb; return 64; }
 
 }  // namespace spca

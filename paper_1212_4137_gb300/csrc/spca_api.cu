@@ -174,16 +174,16 @@ int ensure_workspace(spca_handle *h, int r) {
     CK(dalloc(&h->Ypl, (size_t)kPlanes * r * h->ldU, 2));
     CK(cudaMemsetAsync(h->Xpl, 0, (size_t)kPlanes * r * h->ldX * 2, h->stream));
     CK(cudaMemsetAsync(h->Ypl, 0, (size_t)kPlanes * r * h->ldU * 2, h->stream));
-    CK(make_plane_map(&h->tmX2, h->Xpl, r, h->ldX, 2, tc_box_rows(2), tc_bk(2)));
-    CK(make_plane_map(&h->tmX1, h->Xpl, r, h->ldX, 1, tc_box_rows(1), tc_bk(1)));
-    CK(make_plane_map(&h->tmY1, h->Ypl, r, h->ldU, 1, tc_box_rows(1), tc_bk(1)));
-    CK(make_plane_map(&h->tmY2, h->Ypl, r, h->ldU, 2, tc_box_rows(2), tc_bk(2)));
+    CK(make_q_maps(&h->tmX2, h->Xpl, r, h->ldX, 2));
+    CK(make_q_maps(&h->tmX1, h->Xpl, r, h->ldX, 1));
+    CK(make_q_maps(&h->tmY1, h->Ypl, r, h->ldU, 1));
+    CK(make_q_maps(&h->tmY2, h->Ypl, r, h->ldU, 2));
     h->kcap = (int)std::min<int64_t>(1024, (p + 63) / 64 * 64);
     CK(dalloc(&h->mark, (size_t)p)); CK(dalloc(&h->colpos, (size_t)p)); CK(dalloc(&h->collist, (size_t)h->kcap));
     CK(dalloc(&h->AS, (size_t)kPlanes * n * h->kcap, 2));
     CK(dalloc(&h->XS, (size_t)kPlanes * r * h->kcap, 2));
     CK(make_p_maps(&h->pmAS, h->AS, n, h->kcap, 2));
-    CK(make_plane_map(&h->tmXS2, h->XS, r, h->kcap, 2, tc_box_rows(2), tc_bk(2)));
+    CK(make_q_maps(&h->tmXS2, h->XS, r, h->kcap, 2));
   }
   if (h->fp8 && h->tc_ok) {
     h->ldX8 = (p + 15) / 16 * 16;
@@ -193,8 +193,8 @@ int ensure_workspace(spca_handle *h, int r) {
     CK(dalloc(&h->x8_inv, (size_t)r));
     CK(cudaMemsetAsync(h->X8, 0, (size_t)r * h->ldX8, h->stream));
     CK(cudaMemsetAsync(h->Y8, 0, (size_t)r * h->ldU8, h->stream));
-    CK(make_f8_map(&h->tmX8, h->X8, r, h->ldX8, tc_box_rows(1)));
-    CK(make_f8_map(&h->tmY8, h->Y8, r, h->ldU8, tc_box_rows(1)));
+    CK(make_f8_map(&h->tmX8, h->X8, r, h->ldX8, tc_f8_box_rows()));
+    CK(make_f8_map(&h->tmY8, h->Y8, r, h->ldU8, tc_f8_box_rows()));
   }
   if (h->sparse) {
     h->ldb = (r + kSpGroup - 1) / kSpGroup * kSpGroup;

@@ -13,6 +13,7 @@
 using spca::Ctrl;
 using spca::OtfArchive;
 using spca::PMaps;
+using spca::QMaps;
 using spca::SpPlan;
 using spca::TcStreamK;
 
@@ -84,7 +85,7 @@ struct spca_handle {
   float *x8_inv = nullptr;
   CUtensorMap tmX8{}, tmY8{};
   float *x_scale = nullptr, *x_inv = nullptr;   // row scales of the packed X planes
-  CUtensorMap tmX2{}, tmX1{}, tmY1{}, tmY2{};   // Q-operand maps: X planes (both or the leading one),
+  QMaps tmX2{}, tmX1{}, tmY1{}, tmY2{};         // Q-operand maps: X planes (both or the leading one),
                                                 // y = +-1 or the leading plane of y, y planes
   int *sup_idx = nullptr;
   float *sup_val = nullptr;
@@ -95,7 +96,7 @@ struct spca_handle {
   int *mark = nullptr, *colpos = nullptr, *collist = nullptr;
   void *AS = nullptr, *XS = nullptr;
   PMaps pmAS{};
-  CUtensorMap tmXS2{};
+  QMaps tmXS2{};
   int *status = nullptr, *iters = nullptr, *nnz = nullptr;
   double *F = nullptr, *F_prev = nullptr, *gamma = nullptr, *f = nullptr, *ev = nullptr;
   float *thr = nullptr, *tprev = nullptr;

@@ -344,13 +344,17 @@ inline TcPairs pairs_hi() {
 // 3-D TMA map over `planes` FP16 planes of rows x ld (K-contiguous), box 64 x box_rows
 cudaError_t make_plane_map(CUtensorMap *map, const void *base, int64_t rows, int64_t ld, int planes,
                            int box_rows, int bk);
-int tc_box_rows(int nb);   // Q-operand box height for nb planes (the tile's N)
-int tc_bk(int nb);         // K-block width of the contraction with nb Q planes
+int tc_f8_box_rows();      // Q-operand box height of the FP8 contraction (half of its tile's columns)
 // P-operand map: 128-row boxes of 64-wide K blocks (each CTA loads its own 128 rows)
 struct PMaps {
   CUtensorMap m[1];
 };
 cudaError_t make_p_maps(PMaps *maps, const void *base, int64_t rows, int64_t ld, int planes);
+// Q-operand maps: boxes of half a pair tile's columns, one per tile width (32, 64, 128, 256)
+struct QMaps {
+  CUtensorMap m[4];
+};
+cudaError_t make_q_maps(QMaps *maps, const void *base, int64_t rows, int64_t ld, int planes);
 // out[map(c) * ldo + m] = (row_inv[m] q_inv col_inv[c]) sum_q sum_k P_{a_q}[m, k] Q_{b_q}[c, k],
 // m < M, c < N (a null row_inv / col_inv counts as 1).  N bounds the
 // columns for the launch; with n_dev != nullptr the kernel uses *n_dev (<= N) instead; map =
@@ -376,7 +380,7 @@ struct TcStreamK {
   int piece_kb = 40;
 };
 int64_t tc_sk_floats_per_slot();
-cudaError_t launch_gemm_tc(const PMaps &P, int na, const CUtensorMap &Q, int nb, int M, int N, int K,
+cudaError_t launch_gemm_tc(const PMaps &P, int na, const QMaps &Q, int nb, int M, int N, int K,
                            const int *k_dev, TcPairs pairs, float *out, int64_t ldo, const float *row_inv,
                            const float *col_inv, float q_inv, const int *gate, const int *n_dev, const int *col_map,
                            int *err, const TcStreamK &sk, cudaStream_t st);
