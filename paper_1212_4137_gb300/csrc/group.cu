@@ -162,15 +162,6 @@ const char *check_problem(const spca_problem &q) {
   return nullptr;
 }
 
-uint64_t seed_key(uint64_t seed) {
-  auto mixh = [](uint64_t z) {
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-  };
-  return mixh(seed ^ mixh(5ull));   // the starts' stream of the single solve
-}
-
 // device bytes of a member's block for r starts on an n x p matrix
 size_t member_layout(Member &m, size_t *o) {
   Layout L;
@@ -181,7 +172,7 @@ size_t member_layout(Member &m, size_t *o) {
   o[3] = L.take(2 * 2 * r * m.ldX);          // X planes
   o[4] = L.take(0);                          // (Y planes: the pool's rows)
   o[5] = L.off;                              // (end of the zeroed part: padded columns)
-  o[6] = L.take(4 * r);                      // x_scale
+  o[6] = L.take(0);
   o[7] = L.take(4 * r);                      // x_inv
   o[8] = L.take(4 * r * m.p);                // sup_idx
   o[9] = L.take(4 * r * m.p);                // sup_val
@@ -235,7 +226,6 @@ int admit_one(spca_group *g, const spca_problem &q, int tag) {
   d.Ypl = nullptr;
   d.xps = (int64_t)m.r * m.ldX;
   d.yps = 0;
-  d.x_scale = reinterpret_cast<float *>(at(6));
   d.x_inv = reinterpret_cast<float *>(at(7));
   d.sup_idx = reinterpret_cast<int *>(at(8));
   d.sup_val = reinterpret_cast<float *>(at(9));
@@ -287,7 +277,7 @@ int admit_one(spca_group *g, const spca_problem &q, int tag) {
   a.ordered = m.h->resident16 ? 1 : 0;
   d.gamma0 = is_pen(m.P.form) && !m.target ? m.P.gamma : 0.0;
   d.ld0 = m.ldX;
-  d.key = seed_key(m.P.seed);
+  d.key = start_key(m.P.seed);
   d.x0 = nullptr;
   if (q.x0) {   // the given starts, copied into X and normalised there (they must be finite)
     d.x0 = d.X;
@@ -447,11 +437,11 @@ int build_tables(spca_group *g) {
       t.qmap = m.maps + 2;
       t.M = m.n;
       t.kblocks = (m.p + 63) / 64;
-      t.nmax = m.r;
+      t.nmax = m.r;                        // (a start that is 0 from the beginning has zero planes)
       t.na = lowp ? 1 : 2;
       t.nb = lowp ? 1 : 2;
-      t.n_dev = &m.d.ctrl[g->k & 1]->active;
-      t.col_map = m.d.act;
+      t.n_dev = nullptr;
+      t.col_map = nullptr;
       t.out = m.d.U;
       t.ldo = m.ldU;
       t.row_inv = m.h->a_inv;
@@ -580,11 +570,9 @@ cudaError_t enqueue_sweep(spca_group *g, int64_t k, bool first_of_segment) {
   const uint64_t wait_ns = 2000000000ull;
   cudaError_t e = cudaSuccess;
   if (first_of_segment && g->n_u > 0) {
-    // the first sweep of the members admitted before this segment: their starts and active lists
-    // (parity cur: the control words this sweep reads), then the dense u = A x
-    e = launch_g_start_init(g->dP, g->d_start_prob, g->R, st);
-    if (e == cudaSuccess) e = launch_g_active(g->dP, np, cur, true, st);
-    if (e == cudaSuccess) e = launch_g_xplanes(g->dP, g->d_start_prob, g->R, st);
+    // the first sweep of the members admitted before this segment: their starts, packed planes and
+    // active lists (parity cur: the control words this sweep reads), then the dense u = A x
+    e = launch_g_start_init(g->dP, g->d_start_prob, g->R, cur, st);
     if (e == cudaSuccess)
       e = launch_gemm_grouped(g->d_tasks, g->d_tiles[0], g->total_u, g->bn, g->stages, g->lowp_all, g->sms, g->d_err,
                               wait_ns, st);
@@ -600,7 +588,7 @@ cudaError_t enqueue_sweep(spca_group *g, int64_t k, bool first_of_segment) {
   if (e == cudaSuccess)
     e = launch_g_xstep(g->dP, g->d_start_prob, g->R, g->max_p, g->max_p_small, g->any_large_p, g->full_queued, nxt,
                        g->sms, st);
-  if (e == cudaSuccess && g->full_queued) e = launch_g_active(g->dP, np, nxt, false, st);
+  if (e == cudaSuccess && g->full_queued) e = launch_g_active(g->dP, np, nxt, st);
   return e;
 }
 

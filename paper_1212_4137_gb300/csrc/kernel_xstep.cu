@@ -1206,22 +1206,6 @@ __device__ __forceinline__ void xstep_start(const XstepArgs &a, int c, const flo
   }
 }
 
-// the last CTA of `total` to get here makes the active list of the next sweep and clears the control
-// word that this sweep read (the next x-step writes it)
-__device__ __forceinline__ void last_makes_active_list(int total, const StartState &st, int r, int *act, int *rank,
-                                                       Ctrl *ctrl, Ctrl *ctrl_read) {
-  __shared__ int last;
-  if (threadIdx.x == 0) {   // (thread 0 wrote the start's status and counts: it releases them)
-    int before;
-    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(&ctrl->done) : "memory");
-    last = before == total - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  active_list_body(st.status, st.nnz, r, act, rank, ctrl);
-  if (threadIdx.x == 0) *ctrl_read = Ctrl{};
-}
-
 // (CTAs per SM for the register budget: 7 x 152 of 128 threads hold 1024 starts at once)
 constexpr int fast_ctas(int t) { return t == 128 ? 7 : t == 256 ? 3 : 1; }
 template <int T>
@@ -1234,7 +1218,7 @@ __global__ void __launch_bounds__(T, fast_ctas(T)) k_xstep_fast(XstepArgs a, con
   const int status = st.status ? st.status[c] : ST_ACTIVE;
   const XState q0 = load_state(st, c);
   if (status == ST_ACTIVE) xstep_start<T>(a, c, V, ldv, X, ldx, st, q0, sup_idx, sup_val, ctrl, defer != 0, fs);
-  if (act) last_makes_active_list(r, st, r, act, rank, ctrl, ctrl_read);
+  if (act) last_makes_active_list(r, st.status, st.nnz, r, act, rank, ctrl, ctrl_read);
 }
 
 // Threads per start, 128 to 1024: reading v shrinks with the threads, barriers and the sums over the
@@ -1292,7 +1276,8 @@ __global__ void __launch_bounds__(T, fast_ctas(T)) k_g_xstep_fast(const GProb *_
   const XState q0 = load_state(q.st, c);
   if (status == ST_ACTIVE)
     xstep_start<T>(q.xa, c, q.V, q.ldX, q.X, q.ldX, q.st, q0, q.sup_idx, q.sup_val, q.ctrl[parity], defer != 0, fs);
-  if (!defer) last_makes_active_list(q.r, q.st, q.r, q.act, q.rank, q.ctrl[parity], q.ctrl[parity ^ 1]);
+  if (!defer)
+    last_makes_active_list(q.r, q.st.status, q.st.nnz, q.r, q.act, q.rank, q.ctrl[parity], q.ctrl[parity ^ 1]);
 }
 
 cudaError_t launch_g_xstep(const GProb *P, const int *prob, int R, int max_p, int max_p_small, bool any_large,

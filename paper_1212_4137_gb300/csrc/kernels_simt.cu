@@ -107,17 +107,44 @@ __global__ void __launch_bounds__(256) k_start_init(const float *__restrict__ x0
   start_init_body(x0, ld0, key, p, X, ldX, s, gamma0, c, start, redf);
 }
 
-cudaError_t launch_start_init(const float *x0, int64_t ld0, uint64_t seed, int r, int p, float *X,
-                              int64_t ldX, StartState s, double gamma0, const int *slot_list,
-                              const int *slot_start, const int *count, cudaStream_t st) {
-  // key = mix(seed ^ mix(stream)), stream 5 = starts (same definition as the host generator)
+// key = mix(seed ^ mix(stream)), stream 5 = starts (same definition as the host generator)
+uint64_t start_key(uint64_t seed) {
   auto mixh = [](uint64_t z) {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
     return z ^ (z >> 31);
   };
-  const uint64_t key = mixh(seed ^ mixh(5ull));
-  k_start_init<<<r, 256, 0, st>>>(x0, ld0, key, p, X, ldX, s, gamma0, slot_list, slot_start, count);
+  return mixh(seed ^ mixh(5ull));
+}
+
+cudaError_t launch_start_init(const float *x0, int64_t ld0, uint64_t seed, int r, int p, float *X,
+                              int64_t ldX, StartState s, double gamma0, const int *slot_list,
+                              const int *slot_start, const int *count, cudaStream_t st) {
+  k_start_init<<<r, 256, 0, st>>>(x0, ld0, start_key(seed), p, X, ldX, s, gamma0, slot_list, slot_start, count);
+  return cudaGetLastError();
+}
+
+// The starts of a solve or of a group's new members (start_pack_body: sweep_bodies.cuh), the CTA that
+// finishes last making the first active list.
+// One kernel reads x0, checks it, normalises it and writes what the first sweep reads; it replaces a
+// copy of x0, a check, an in-place normalisation (three passes), row scales, a plane split and the
+// active list.  Bound by HBM: 4 p bytes read and 4 p written per start (two FP16 planes, or FP32).
+// 1024 starts, p = 20000, tensor cores: 55 us for the kernel (290 us for the launches it replaces and the
+// copy).
+__global__ void __launch_bounds__(256) k_start_pack(const float *x0, int64_t ld0, uint64_t key, int p, float *X,
+                                                    int64_t ldX, XPack pk, StartState s, double gamma0, int *flag,
+                                                    int r, int *act, int *rank, Ctrl *ctrl) {
+  __shared__ float redf[32];
+  __shared__ unsigned redu[32];
+  const int c = (int)blockIdx.x;
+  start_pack_body(x0, ld0, key, p, X, ldX, pk, s, gamma0, flag, c, redf, redu);
+  last_makes_active_list(r, s.status, nullptr, r, act, rank, ctrl, nullptr);
+}
+
+cudaError_t launch_start_pack(const float *x0, int64_t ld0, uint64_t seed, int r, int p, float *X, int64_t ldX,
+                              XPack pk, StartState s, double gamma0, int *flag, int *act, int *rank, Ctrl *ctrl,
+                              cudaStream_t st) {
+  k_start_pack<<<r, 256, 0, st>>>(x0, ld0, start_key(seed), p, X, ldX, pk, s, gamma0, flag, r, act, rank, ctrl);
   return cudaGetLastError();
 }
 
@@ -579,29 +606,37 @@ cudaError_t launch_gemm1_sparse(const float *AT, int64_t ldat, int n, const int 
 // The per-start phases for all problems of a group in one launch each: block g (or blockIdx.x for
 // the per-problem active lists) looks its problem up and runs the single-problem body on that
 // problem's blocks of the workspace.
-__global__ void __launch_bounds__(256) k_g_start_init(const GProb *__restrict__ P, const int *__restrict__ prob) {
+__global__ void __launch_bounds__(256) k_g_start_init(const GProb *__restrict__ P, const int *__restrict__ prob,
+                                                      int parity) {
   __shared__ float redf[32];
+  __shared__ unsigned redu[32];
   const GProb &q = P[prob[blockIdx.x]];
   if (!q.first) return;   // only the members whose first sweep is next
   const int c = (int)blockIdx.x - q.start0;
-  start_init_body(q.x0, q.ld0, q.key, q.p, q.X, q.ldX, q.st, q.gamma0, c, c, redf);
+  XPack pk;               // the two planes of x that the dense u = A x reads, row c
+  pk.planes = q.Xpl;
+  pk.ld = q.ldX;
+  pk.stride = q.xps;
+  pk.n = 2;
+  pk.inv = q.x_inv;
+  start_pack_body(q.x0, q.ld0, q.key, q.p, q.X, q.ldX, pk, q.st, q.gamma0, nullptr, c, redf, redu);
+  last_makes_active_list(q.r, q.st.status, nullptr, q.r, q.act, q.rank, q.ctrl[parity], nullptr);
 }
 
-cudaError_t launch_g_start_init(const GProb *P, const int *prob, int R, cudaStream_t st) {
-  k_g_start_init<<<R, 256, 0, st>>>(P, prob);
+cudaError_t launch_g_start_init(const GProb *P, const int *prob, int R, int parity, cudaStream_t st) {
+  k_g_start_init<<<R, 256, 0, st>>>(P, prob, parity);
   return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(1024) k_g_active(const GProb *__restrict__ P, int parity, int only_first) {
+__global__ void __launch_bounds__(1024) k_g_active(const GProb *__restrict__ P, int parity) {
   const GProb &q = P[blockIdx.x];
-  if (only_first && !q.first) return;
   active_list_body(q.st.status, q.st.nnz, q.r, q.act, q.rank, q.ctrl[parity]);
-  // (after an x-step: the control word that the sweep read is cleared for the next one)
-  if (!only_first && threadIdx.x == 0) *q.ctrl[parity ^ 1] = Ctrl{};
+  // the control word that the sweep read is cleared for the next one
+  if (threadIdx.x == 0) *q.ctrl[parity ^ 1] = Ctrl{};
 }
 
-cudaError_t launch_g_active(const GProb *P, int np, int parity, bool only_first, cudaStream_t st) {
-  k_g_active<<<np, 1024, 0, st>>>(P, parity, only_first ? 1 : 0);
+cudaError_t launch_g_active(const GProb *P, int np, int parity, cudaStream_t st) {
+  k_g_active<<<np, 1024, 0, st>>>(P, parity);
   return cudaGetLastError();
 }
 
@@ -639,41 +674,6 @@ __global__ void k_g_ctrl(const GProb *__restrict__ P, int np, int parity, int *_
 
 cudaError_t launch_g_ctrl(const GProb *P, int np, int parity, int *out, cudaStream_t st) {
   k_g_ctrl<<<(np + 255) / 256, 256, 0, st>>>(P, np, parity, out);
-  return cudaGetLastError();
-}
-
-// FP16 planes of x for the dense u = A x (the first sweep): per active start, the power-of-two
-// scale putting max |x_j| in [2^13, 2^14), then hi = fp16(s x), lo = fp16(s x - hi) at the start's
-// packed row (its rank), and 1 / s at the same index
-__global__ void __launch_bounds__(256) k_g_xplanes(const GProb *__restrict__ P, const int *__restrict__ prob) {
-  __shared__ unsigned red[32];
-  const GProb &q = P[prob[blockIdx.x]];
-  const int c = (int)blockIdx.x - q.start0;
-  // only starts not swept yet (a problem's first sweep; the others take the support gather)
-  if (q.st.status[c] != ST_ACTIVE || q.st.iters[c] != 0) return;
-  const float *x = q.X + (int64_t)c * q.ldX;
-  unsigned mk = 0u;
-  for (int j = threadIdx.x; j < q.p; j += blockDim.x) mk = max(mk, __float_as_uint(fabsf(x[j])));
-  const unsigned m = block_max_u(mk, red);
-  int e = 0;
-  if (m != 0u) e = max(-120, min(120, 13 - ilogbf(__uint_as_float(m))));
-  const float sc = ldexpf(1.0f, e);
-  const int row = q.rank[c];
-  __half *hi = q.Xpl + (int64_t)row * q.ldX;
-  for (int j = threadIdx.x; j < q.p; j += blockDim.x) {
-    const float a = x[j] * sc;
-    const __half h = __float2half_rn(a);
-    hi[j] = h;
-    hi[j + q.xps] = __float2half_rn(a - __half2float(h));
-  }
-  if (threadIdx.x == 0) {
-    q.x_scale[row] = sc;
-    q.x_inv[row] = ldexpf(1.0f, -e);
-  }
-}
-
-cudaError_t launch_g_xplanes(const GProb *P, const int *prob, int R, cudaStream_t st) {
-  k_g_xplanes<<<R, 256, 0, st>>>(P, prob);
   return cudaGetLastError();
 }
 

@@ -351,13 +351,20 @@ int sweep_u_rows(spca_handle *h, int r, const int *gate, const int *count, const
 
 // u = A x for every active row of h->X: dense contraction (gated: runs only if *gate != 0).  The
 // tensor-core engine packs the active starts (h->act, count *nact) into consecutive plane rows.
+// packed: the first sweep, whose planes the start initialisation wrote (row c = start c).
 int sweep_u_dense(spca_handle *h, int engine, int r, const int *gate, const int *nact, int nhost, bool lowp,
-                  const int *list = nullptr) {
+                  const int *list = nullptr, bool packed = false) {
   if (!list) list = h->act;
   if (h->sparse) return sweep_u_rows(h, r, gate, nact, list);
   const int n = (int)h->n, p = (int)h->p;
   cudaStream_t st = h->stream;
-  if (engine == SPCA_ENGINE_TC && lowp && f8_sweeps(h)) {
+  if (packed) {
+    CK(timed(h, SPCA_K_U_DENSE, 1, [&] {
+      return launch_gemm_tc(h->pmA, lowp ? 1 : 2, lowp ? h->tmX1 : h->tmX2, lowp ? 1 : 2, n, nhost, p, nullptr,
+                            lowp ? pairs_hi() : pairs_general(), h->U, h->ldU, h->a_inv, h->x_inv, 1.0f, gate, nullptr,
+                            nullptr, h->dev_err, h->sk, st);
+    }));
+  } else if (engine == SPCA_ENGINE_TC && lowp && f8_sweeps(h)) {
     // FP8 low-precision sweep: x in E4M3 with the planes' row scales times 2^-6
     CK(timed(h, SPCA_K_U_DENSE, 4, [&] {
       cudaError_t e = launch_row_scales(h->X, nhost, p, h->ldX, h->x_scale, h->x_inv, gate, nact, list, st);
@@ -1073,53 +1080,65 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
 
   // ---- a1: starting points
   const double gamma0 = is_pen(form) && !target ? P.gamma : 0.0;
-  // the starts' source: x0 rows (copied into X for a plain solve, kept whole for on-the-fly
-  // replacement, where slots take later rows), or the seeded stream
+  // the starts' source: x0 rows (on-the-fly replacement keeps them whole: slots take later rows), or
+  // the seeded stream
   const float *x0src = nullptr;
   int64_t ld0 = 0;
   if (x0) {
-    if (otf) {
-      if (P.x0_is_device) {
-        x0src = x0;
-      } else {
-        CK(cudaMemcpyAsync(h->otf_x0, x0, (size_t)l * p * sizeof(float), cudaMemcpyHostToDevice, st));
-        x0src = h->otf_x0;
-      }
-      ld0 = p;
-    } else {
-      CK(cudaMemcpy2DAsync(h->X, h->ldX * sizeof(float), x0, (size_t)p * sizeof(float), (size_t)p * sizeof(float),
-                           r, P.x0_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
-      x0src = h->X;
-      ld0 = h->ldX;
+    x0src = x0;
+    ld0 = p;
+    if (!P.x0_is_device) {
+      float *dst = otf ? h->otf_x0 : h->X;
+      ld0 = otf ? p : h->ldX;
+      CK(cudaMemcpy2DAsync(dst, ld0 * sizeof(float), x0, (size_t)p * sizeof(float), (size_t)p * sizeof(float), l,
+                           cudaMemcpyHostToDevice, st));
+      x0src = dst;
     }
     CK(cudaMemsetAsync(h->flag, 0, sizeof(int), st));
-    CK(timed(h, SPCA_K_PREP, 1,
-             [&] { return launch_check_finite(x0src, otf ? l : r, p, ld0, h->flag, st); }));
-    CK(cudaMemcpyAsync(h->h_flag, h->flag, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    if (*h->h_flag) return fail(h, SPCA_E_INVALID, "x0 has a non-finite entry%s");
   }
-  CK(timed(h, SPCA_K_INIT, 1, [&] {
-    return launch_start_init(x0src, ld0, P.seed, r, p, h->X, h->ldX, S, gamma0, nullptr, nullptr, nullptr, st);
-  }));
+  CK(cudaMemsetAsync(h->ctrl, 0, 2 * sizeof(Ctrl), st));   // (each sweep clears the word it read for the next one)
+  // the first sweep reads x^(0) as FP16 planes (tensor cores, but for an FP8 copy of A) or as FP32
+  const bool packed = engine == SPCA_ENGINE_TC && !otf && !(F0 == 0 && L > 0 && f8_sweeps(h));
   std::vector<int> iota;
   if (otf) {   // slot c holds start c; the next start is r
+    if (x0) CK(timed(h, SPCA_K_PREP, 1, [&] { return launch_check_finite(x0src, l, p, ld0, h->flag, st); }));
+    CK(timed(h, SPCA_K_INIT, 1, [&] {
+      return launch_start_init(x0src, ld0, P.seed, r, p, h->X, h->ldX, S, gamma0, nullptr, nullptr, nullptr, st);
+    }));
     iota.resize(r + 1);
     for (int c = 0; c < r; ++c) iota[c] = c;
     iota[r] = r;
     CK(cudaMemcpyAsync(h->slot_start, iota.data(), r * sizeof(int), cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(h->next_start, iota.data() + r, sizeof(int), cudaMemcpyHostToDevice, st));
+    h->h_ctrl[0] = Ctrl{};
+    h->h_ctrl[0].need_dense = 1;      // x^(0) is dense: the first sweep's u = A x is the dense one
+    CK(cudaMemcpyAsync(h->ctrl, h->h_ctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, st));
+    CK(timed(h, SPCA_K_XSTEP, 1, [&] {
+      return launch_active_list(h->status, nullptr, r, h->act, h->rank, &h->ctrl[0], nullptr, st);
+    }));
+  } else {
+    XPack pk;
+    pk.x32 = !packed;
+    if (packed) {
+      pk.planes = static_cast<__half *>(h->Xpl);
+      pk.ld = h->ldX;
+      pk.stride = (int64_t)h->r_cap * h->ldX;
+      pk.n = F0 == 0 && L > 0 ? 1 : 2;
+      pk.inv = h->x_inv;
+    }
+    CK(timed(h, SPCA_K_INIT, 1, [&] {
+      return launch_start_pack(x0src, ld0, P.seed, r, p, h->X, h->ldX, pk, S, gamma0, h->flag, h->act, h->rank,
+                               &h->ctrl[0], st);
+    }));
   }
-  memset(&h->h_ctrl[0], 0, sizeof(Ctrl));
-  h->h_ctrl[0].active = r;
-  h->h_ctrl[0].need_dense = 1;      // x^(0) is dense: the first sweep's u = A x is the dense one
-  memset(&h->h_ctrl[1], 0, sizeof(Ctrl));   // (each sweep clears the word it read for the next one)
-  CK(cudaMemcpyAsync(h->ctrl, h->h_ctrl, 2 * sizeof(Ctrl), cudaMemcpyHostToDevice, st));
-  CK(timed(h, SPCA_K_XSTEP, 1,
-           [&] { return launch_active_list(h->status, nullptr, r, h->act, h->rank, &h->ctrl[0], nullptr, st); }));
-  CK(cudaMemcpyAsync(h->h_ctrl + 1, h->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));  // h_ctrl is reused below
-  int nhost = h->h_ctrl[1].active;  // active starts as the host knows them (sizes the launches)
+  if (x0) {
+    CK(cudaMemcpyAsync(h->h_flag, h->flag, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    if (*h->h_flag) return fail(h, SPCA_E_INVALID, "x0 has a non-finite entry%s");
+  } else if (otf) {
+    CK(cudaStreamSynchronize(st));   // iota and h_ctrl are reused
+  }
+  int nhost = r;   // active starts as the host knows them (an upper bound)
 
   // ---- the sweeps (Algorithm 2)
   XstepArgs xa{};
@@ -1166,14 +1185,14 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
   // plan and replayed, so that in steady state a segment is one launch.
   struct SweepPlan {
     int k;
-    bool lowp, dense_in, union_in, union_out, full;
+    bool lowp, dense_in, packed, union_in, union_out, full;
     int sparse_cap;
   };
   auto enqueue = [&](const SweepPlan &pl) -> int {
     Ctrl *cur = h->ctrl + ((pl.k - 1) & 1), *nxt = h->ctrl + (pl.k & 1);
     // u = A x: over the union of the supports when it is small (tensor cores), else the dense
     // contraction, or the per-start support gather when every support is small
-    if (pl.dense_in) RC(sweep_u_dense(h, engine, r, &cur->need_dense, &cur->active, r, pl.lowp));
+    if (pl.dense_in) RC(sweep_u_dense(h, engine, r, &cur->need_dense, &cur->active, r, pl.lowp, nullptr, pl.packed));
     // slots that took a new start in the last sweep have a dense x (the gather skips them)
     if (otf) RC(sweep_u_dense(h, engine, r, &cur->n_new, &cur->n_new, r, false, h->new_slot));
     if (pl.union_in) RC(sweep_u_union(h, S, cur, r));
@@ -1280,6 +1299,7 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
       // sweeps F0 + 1 .. F0 + L read the low-precision copy of A (the leading FP16 plane or E4M3)
       pl.lowp = k > F0 && k <= F0 + L;
       pl.dense_in = dense_queued;
+      pl.packed = packed && k == 1;
       pl.union_in = union_built;
       dense_queued = max_nnz > sparse_cap / 2;
       pl.full = full_queued;
@@ -1289,7 +1309,7 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
                     h->n * sum_nnz >= kUnionMinReads;
       pl.union_out = union_built;
       plans.push_back(pl);
-      key.insert(key.end(), {pl.lowp, pl.dense_in, pl.union_in, pl.union_out, pl.full, pl.sparse_cap});
+      key.insert(key.end(), {pl.lowp, pl.dense_in, pl.packed, pl.union_in, pl.union_out, pl.full, pl.sparse_cap});
     }
     SegGraph *g = nullptr;
     for (SegGraph &c : graphs)

@@ -129,6 +129,22 @@ cudaError_t launch_start_init(const float *x0, int64_t ld0, uint64_t seed, int r
                               float *X, int64_t ldX, StartState s, double gamma0, const int *slot_list,
                               const int *slot_start, const int *count, cudaStream_t st);
 
+// what a solve's first sweep reads: x^(0) as FP32 (x32) or as n FP16 planes of the row-scaled x
+// (`stride` elements apart, row c at c * ld, 1 / scale in inv[c])
+struct XPack {
+  bool x32 = false;
+  __half *planes = nullptr;
+  int64_t ld = 0, stride = 0;
+  int n = 0;
+  float *inv = nullptr;
+};
+uint64_t start_key(uint64_t seed);
+// a1 for a whole solve: checks x0 (*flag |= 1 on a non-finite entry), the starting points packed for the
+// first sweep, the per-start state, and the first active list in *ctrl (zeroed before; need_dense set)
+cudaError_t launch_start_pack(const float *x0, int64_t ld0, uint64_t seed, int r, int p, float *X, int64_t ldX,
+                              XPack pk, StartState s, double gamma0, int *flag, int *act, int *rank, Ctrl *ctrl,
+                              cudaStream_t st);
+
 // on-the-fly replacement (Section 4.3): the archive of the l starts' results
 struct OtfArchive {
   float *x;        // l x ldX final iterates
@@ -409,9 +425,9 @@ struct GProb {
   int *yoff;
   int first;                    // its first sweep is the next one (its starts are set up then)
   float *X, *V, *U;             // r x ldX, r x ldX, r x ldU
-  __half *Xpl, *Ypl;            // two FP16 planes each (x row-scaled, y scaled by kQScale), packed rows
+  __half *Xpl, *Ypl;            // two FP16 planes each (x row-scaled; y scaled by kQScale, packed rows)
   int64_t xps, yps;             // plane strides (elements)
-  float *x_scale, *x_inv;       // per packed row of Xpl
+  float *x_inv;                 // per row of Xpl
   int *sup_idx;                 // r x p support lists (index, value)
   float *sup_val;
   int *act, *rank;              // active list (r)
@@ -436,9 +452,11 @@ cudaError_t launch_g_pools(const GPool *pools, int npool, const GProb *P, const 
                            cudaStream_t st);
 // the phases of a sweep for every problem of a group, one launch each (prob[g] = the problem of
 // global start g, R starts in all)
-// (the start initialisation runs for the members whose first sweep is next, GProb.first)
-cudaError_t launch_g_start_init(const GProb *P, const int *prob, int R, cudaStream_t st);
-cudaError_t launch_g_active(const GProb *P, int np, int parity, bool only_first, cudaStream_t st);
+// (the start initialisation, with the planes of x that the dense u = A x reads (row c of a member's
+// planes is its start c) and the first active list in the control word of `parity`, runs for the
+// members whose first sweep is next, GProb.first)
+cudaError_t launch_g_start_init(const GProb *P, const int *prob, int R, int parity, cudaStream_t st);
+cudaError_t launch_g_active(const GProb *P, int np, int parity, cudaStream_t st);
 // many small device-to-device copies in one launch
 struct CopyDesc {
   const void *src;
@@ -448,7 +466,6 @@ struct CopyDesc {
 cudaError_t launch_copy_list(const CopyDesc *list, int count, cudaStream_t st);
 // one parity's control words: the active counts into out[np], the counts of full x-steps behind them
 cudaError_t launch_g_ctrl(const GProb *P, int np, int parity, int *out, cudaStream_t st);
-cudaError_t launch_g_xplanes(const GProb *P, const int *prob, int R, cudaStream_t st);
 cudaError_t launch_g_gather(const GProb *P, const int *prob, int R, int max_n, cudaStream_t st);
 cudaError_t launch_g_ystep(const GProb *P, const int *prob, int R, cudaStream_t st);
 // (max_p: the longest v; max_p_small: the longest that fits in shared memory, 0 if none; any_large: some v does not;

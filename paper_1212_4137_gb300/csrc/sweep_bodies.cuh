@@ -60,6 +60,100 @@ static __device__ void start_init_body(const float *__restrict__ x0, int64_t ld0
   }
 }
 
+// The same for a solve's first sweep, which reads x^(0) as FP32 (pk.x32) or as FP16 planes of the
+// row-scaled x (pk.planes, row c, with 1 / scale in pk.inv[c]) and never as both.  x0 (checked: a
+// non-finite entry sets *flag and ends the start) is read twice, the second time mostly from L2; a
+// seeded start's raw normals are kept in X between the passes.  ||g||^2 is added as in start_init_body.
+static __device__ void start_pack_body(const float *x0, int64_t ld0, uint64_t key, int p, float *X, int64_t ldX,
+                                       const XPack &pk, StartState s, double gamma0, int *flag, int c, float *redf,
+                                       unsigned *redu) {
+  float *x = X + (int64_t)c * ldX;
+  const float *g = x0 ? x0 + (int64_t)c * ld0 : nullptr;
+  float part = 0.0f;
+  unsigned mk = 0u;
+  const int nt = (int)blockDim.x;
+  constexpr int U = 8;                         // loads in flight per thread
+  if (g) {
+    for (int j0 = threadIdx.x; j0 < p; j0 += U * nt) {
+      float v[U];
+#pragma unroll
+      for (int k = 0; k < U; ++k) v[k] = j0 + k * nt < p ? g[j0 + k * nt] : 0.0f;
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        part = fmaf(v[k], v[k], part);
+        mk = max(mk, abs_key(v[k]));
+      }
+    }
+  } else {
+    for (int j = threadIdx.x; j < p; j += nt) {
+      const float v = (float)bm_normal(key, (uint64_t)c * (uint64_t)p + (uint64_t)j);
+      x[j] = v;
+      part = fmaf(v, v, part);
+      mk = max(mk, abs_key(v));
+    }
+    g = x;
+  }
+  float nrm, lo, inv;
+  norm_and_inverse(block_sum_f(part, redf), &nrm, &lo, &inv);
+  const unsigned top = block_max_u(mk, redu);  // (its barriers also order a seeded start's x)
+  const bool bad = top >= 0x7f800000u;         // a non-finite entry
+  if (bad) inv = 0.0f;
+  const bool alive = nrm > 0.0f && !bad;
+  // the planes' scale puts max |x_j| = max |g_j| / ||g|| in [2^13, 2^14) (rounding is monotone)
+  const float mx = __uint_as_float(bad ? 0u : top) * inv;
+  int e = 0;
+  if (mx > 0.0f) e = max(-120, min(120, 13 - ilogbf(mx)));
+  const float sc = ldexpf(1.0f, e);
+  auto norm = [&](int j) { return alive ? g[j] * inv : 0.0f; };
+  if (pk.x32 || !alive) {                      // (a start that never sweeps keeps x = 0)
+    for (int j0 = threadIdx.x; j0 < p; j0 += U * nt) {
+      float v[U];
+#pragma unroll
+      for (int k = 0; k < U; ++k) v[k] = j0 + k * nt < p ? norm(j0 + k * nt) : 0.0f;
+#pragma unroll
+      for (int k = 0; k < U; ++k)
+        if (j0 + k * nt < p) x[j0 + k * nt] = v[k];
+    }
+  }
+  if (pk.planes) {
+    __half *hi = pk.planes + (int64_t)c * pk.ld;
+    constexpr int W = 4;                       // pairs of entries in flight per thread
+    for (int j0 = 2 * threadIdx.x; j0 < p; j0 += 2 * W * nt) {
+      float v[W][2];
+#pragma unroll
+      for (int k = 0; k < W; ++k) {
+        const int j = j0 + 2 * k * nt;
+        v[k][0] = j < p ? norm(j) * sc : 0.0f;
+        v[k][1] = j + 1 < p ? norm(j + 1) * sc : 0.0f;
+      }
+#pragma unroll
+      for (int k = 0; k < W; ++k) {
+        const int j = j0 + 2 * k * nt;
+        if (j >= p) break;
+        // (the entry past an odd p is a zero of the row's padding)
+        const __half2 h = __floats2half2_rn(v[k][0], v[k][1]);
+        *reinterpret_cast<__half2 *>(hi + j) = h;
+        if (pk.n > 1) {
+          const float2 f = __half22float2(h);
+          *reinterpret_cast<__half2 *>(hi + pk.stride + j) = __floats2half2_rn(v[k][0] - f.x, v[k][1] - f.y);
+        }
+      }
+    }
+    if (threadIdx.x == 0) pk.inv[c] = ldexpf(1.0f, -e);
+  }
+  if (threadIdx.x == 0) {
+    if (bad && flag) atomicOr(flag, 1);
+    s.status[c] = alive ? ST_ACTIVE : SPCA_ST_DEGENERATE;
+    s.iters[c] = 0;
+    s.nnz[c] = alive ? p : 0;
+    s.F[c] = 0.0;
+    s.F_prev[c] = 0.0;
+    s.gamma[c] = gamma0;
+    s.thr[c] = 0.0f;
+    if (s.tprev) s.tprev[c] = 0.0f;
+  }
+}
+
 // ------------------------------------------------------------------ y-step (Table 3 S1, S2)
 // Counts the sweep for every active start; L1 variance: y = sgn(u) with sgn(0) = +1;
 // L2 variance: y = u / ||u||_2, and ||u||_2 = 0 ends the start as degenerate (x = 0).
@@ -216,8 +310,29 @@ static __device__ void active_list_body(const int *status, const int *nnz, int r
     }
     ctrl->max_nnz = m;
     ctrl->active = base_pos;
-    ctrl->use_gather = (__ldcg(&ctrl->need_dense) == 0 && base_pos > 0) ? 1 : 0;
+    ctrl->use_gather = (nnz && __ldcg(&ctrl->need_dense) == 0 && base_pos > 0) ? 1 : 0;
     ctrl->sum_nnz = (int)(t < 0x7fffffffLL ? t : 0x7fffffffLL);
+  }
+}
+
+// the last CTA of `total` to get here makes the active list of the next sweep (every CTA's thread 0 has
+// written its start's status and counts: it releases them) and clears the control word that this sweep
+// read (the next x-step writes it); a null nnz: the first list of a solve, whose x are dense
+static __device__ __forceinline__ void last_makes_active_list(int total, const int *status, const int *nnz, int r,
+                                                              int *act, int *rank, Ctrl *ctrl, Ctrl *ctrl_read) {
+  __shared__ int last;
+  if (threadIdx.x == 0) {
+    int before;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(&ctrl->done) : "memory");
+    last = before == total - 1;
+    if (last && !nnz) ctrl->need_dense = 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  active_list_body(status, nnz, r, act, rank, ctrl);
+  if (threadIdx.x == 0) {
+    if (ctrl_read) *ctrl_read = Ctrl{};
+    if (!nnz) ctrl->done = 0;
   }
 }
 
