@@ -51,10 +51,6 @@ struct Member {
   char *mem = nullptr;            // the member's device block
   GProb d{};                      // its table entry (start0 set when the table is built)
   CUtensorMap *maps = nullptr;    // device: A planes, A^T planes, X planes
-  double *partials = nullptr;
-  float *y_out = nullptr, *x_out = nullptr;
-  int64_t *support_out = nullptr, *nnz_out = nullptr;
-  int *best = nullptr;
   bool first_pending = true;      // its first sweep (the dense u = A x) is still to run
 };
 
@@ -171,8 +167,8 @@ size_t member_layout(Member &m, size_t *o) {
   o[2] = L.take(4 * r * m.ldU);              // U
   o[3] = L.take(2 * 2 * r * m.ldX);          // X planes
   o[4] = L.take(0);                          // (Y planes: the pool's rows)
-  o[5] = L.off;                              // (end of the zeroed part: padded columns)
-  o[6] = L.take(0);
+  o[5] = L.off;
+  o[6] = L.take(4 * (r + 1));                // finalise counters
   o[7] = L.take(4 * r);                      // x_inv
   o[8] = L.take(4 * r * m.p);                // sup_idx
   o[9] = L.take(4 * r * m.p);                // sup_val
@@ -207,7 +203,7 @@ int admit_one(spca_group *g, const spca_problem &q, int tag) {
   const size_t bytes = member_layout(m, o);
   GCK(cudaMallocFromPoolAsync((void **)&m.mem, bytes, g->mempool, st));
   auto at = [&](int i) { return m.mem + o[i]; };
-  GCK(cudaMemsetAsync(m.mem, 0, o[5], st));
+  GCK(cudaMemsetAsync(m.mem, 0, o[7], st));   // (the padded columns and the finalise counters)
   GProb &d = m.d;
   d.n = m.n;
   d.p = m.p;
@@ -229,10 +225,12 @@ int admit_one(spca_group *g, const spca_problem &q, int tag) {
   d.x_inv = reinterpret_cast<float *>(at(7));
   d.sup_idx = reinterpret_cast<int *>(at(8));
   d.sup_val = reinterpret_cast<float *>(at(9));
-  m.partials = reinterpret_cast<double *>(at(10));
-  m.y_out = reinterpret_cast<float *>(at(11));
-  m.x_out = reinterpret_cast<float *>(at(12));
-  m.support_out = reinterpret_cast<int64_t *>(at(13));
+  d.partials = reinterpret_cast<double *>(at(10));
+  d.y_out = reinterpret_cast<float *>(at(11));
+  d.x_out = reinterpret_cast<float *>(at(12));
+  d.support_out = reinterpret_cast<int64_t *>(at(13));
+  d.fin_cnt = reinterpret_cast<int *>(at(6));
+  d.use_ev = m.target;
   int *ip = reinterpret_cast<int *>(at(14));
   double *dp = reinterpret_cast<double *>(at(15));
   float *fp = reinterpret_cast<float *>(at(16));
@@ -253,8 +251,8 @@ int admit_one(spca_group *g, const spca_problem &q, int tag) {
   Ctrl *ctrl = reinterpret_cast<Ctrl *>(at(17));
   d.ctrl[0] = ctrl;
   d.ctrl[1] = ctrl + 1;
-  m.best = reinterpret_cast<int *>(at(18));
-  m.nnz_out = reinterpret_cast<int64_t *>(at(18) + 8);
+  d.best = reinterpret_cast<int *>(at(18));
+  d.nnz_out = reinterpret_cast<int64_t *>(at(18) + 8);
   m.maps = reinterpret_cast<CUtensorMap *>(at(19));
   GCK(cudaMemsetAsync(ctrl, 0, sizeof(Ctrl) * 2, st));
   XstepArgs &a = d.xa;
@@ -610,18 +608,20 @@ int finish_members(spca_group *g, const std::vector<Member *> &list) {
     pieces[k].push_back(Piece{off, bytes});
     off += (bytes + 15) / 16 * 16;
   };
+  // the finishing members' starts and outputs, one launch each over the tables of the last sweeps
+  const int np = (int)g->members.size();
+  const int *done = nullptr;
+  std::vector<int> flags;
+  if ((int)list.size() < np) {
+    flags.assign(np, 0);
+    for (const Member *m : list) flags[m - g->members.data()] = 1;
+    GCK(cudaMemcpyAsync(g->d_active, flags.data(), sizeof(int) * np, cudaMemcpyHostToDevice, st));
+    done = g->d_active;   // (the counts it held have been read)
+  }
+  GCK(launch_g_finish(g->dP, g->d_start_prob, g->R, np, g->max_n, g->max_p, done, st));
   for (size_t k = 0; k < list.size(); ++k) {
-    Member &m = *list[k];
+    const Member &m = *list[k];
     const GProb &d = m.d;
-    if (m.h->resident16)
-      GCK(launch_finalise_h(m.P.form, d.AT16, d.at_inv, m.h->ldAT, m.n, d.st, m.r, d.U, m.ldU, d.sup_idx, d.sup_val,
-                            m.p, m.partials, st));
-    else
-      GCK(launch_finalise(m.P.form, m.h->AT32, m.h->ldAT, m.n, m.p, d.X, m.ldX, d.st, m.r, d.U, m.ldU, d.sup_idx,
-                          d.sup_val, m.p, m.partials, st));
-    GCK(launch_best(m.P.form, m.target, d.st, m.r, m.best, st));
-    GCK(launch_best_outputs(m.P.form, m.best, d.U, m.ldU, m.n, d.X, m.ldX, m.p, m.y_out, m.x_out, m.support_out,
-                            m.nnz_out, st));
     const int64_t r = m.r;
     add(k, d.st.status, 4 * r);
     add(k, d.st.iters, 4 * r);
@@ -629,11 +629,11 @@ int finish_members(spca_group *g, const std::vector<Member *> &list) {
     add(k, d.st.ev, 8 * r);
     add(k, d.st.gamma, 8 * r);
     add(k, d.st.F, 8 * r);
-    add(k, m.best, 4);
-    add(k, m.nnz_out, 8);
-    add(k, m.x_out, 4 * (int64_t)m.p);
-    add(k, m.y_out, 4 * (int64_t)m.n);
-    add(k, m.support_out, 8 * (int64_t)m.p);
+    add(k, d.best, 4);
+    add(k, d.nnz_out, 8);
+    add(k, d.x_out, 4 * (int64_t)m.p);
+    add(k, d.y_out, 4 * (int64_t)m.n);
+    add(k, d.support_out, 8 * (int64_t)m.p);
   }
   if (off > g->stage_bytes) {
     GCK(cudaStreamSynchronize(st));

@@ -2,6 +2,7 @@
 // u = A x accumulated as a compensated FP32-pair dot product (about twice FP32's precision) and
 // the norms of u summed in FP64, the explained variance (Section 4.1), the best start (ties:
 // lower index), and y(x) and the support of the best x.
+#include <algorithm>
 #include <cstdint>
 
 #include "block_util.cuh"
@@ -10,125 +11,21 @@
 namespace spca {
 
 namespace {
-constexpr int FT = 256;
-}
+constexpr int FT = 128;            // threads per CTA, four rows of A each
+constexpr int FR = 4 * FT;         // rows per chunk
+}  // namespace
+int finalise_chunks(int64_t n) { return (int)((n + FR - 1) / FR); }
 
-// grid (r, ceil(n / FT)): u_i = sum_t x_{j_t} A[i, j_t] over the support (compensated FP32
-// pairs); per-CTA FP64 partial sums of |u_i| and u_i^2 go to partials (fixed order later).
-// Starts on x, row chunks on y: the CTAs in flight share row chunks, so a column slice used by
-// several starts' supports is read from DRAM about once.  The columns of A are the rows of A^T:
-// FP32 (row_inv null), or FP16 entries times their row's power-of-two inverse scale (the 16-bit
-// copy of a resident handle; the scaled entry is exact in FP32).
-template <typename T>
-__global__ void __launch_bounds__(FT) k_fin_partial(const T *__restrict__ AT, const float *__restrict__ row_inv,
-                                                    int64_t ldat, int n, const int *__restrict__ sup_idx,
-                                                    const float *__restrict__ sup_val, int cap,
-                                                    StartState st, float *__restrict__ U,
-                                                    int64_t ldu, double *__restrict__ partials) {
-  __shared__ int sidx[FT];
-  __shared__ float sval[FT];
-  __shared__ float sinv[FT];
-  __shared__ double red[32];
-  const int c = blockIdx.x;
-  const int i = blockIdx.y * FT + threadIdx.x;
-  const int nnz = st.nnz[c];
-  const int *gi = sup_idx + (int64_t)c * cap;
-  const float *gv = sup_val + (int64_t)c * cap;
-  F32Pair acc2;
-  for (int t0 = 0; t0 < nnz; t0 += FT) {
-    __syncthreads();
-    if (t0 + (int)threadIdx.x < nnz) {
-      const int j = gi[t0 + threadIdx.x];
-      sidx[threadIdx.x] = j;
-      sval[threadIdx.x] = gv[t0 + threadIdx.x];
-      sinv[threadIdx.x] = row_inv ? row_inv[j] : 1.0f;
-    }
-    __syncthreads();
-    const int m = min(FT, nnz - t0);
-    if (i < n)
-      for (int t = 0; t < m; ++t) {
-        const float a = static_cast<float>(AT[(int64_t)sidx[t] * ldat + i]) * sinv[t];
-        f32pair_fma(acc2, sval[t], a);
-      }
-  }
-  const double acc = f32pair_value(acc2);
-  if (i < n) U[(int64_t)c * ldu + i] = (float)acc;
-  const double l1 = block_sum_d(i < n ? fabs(acc) : 0.0, red);
-  const double l2 = block_sum_d(i < n ? acc * acc : 0.0, red);
-  if (threadIdx.x == 0) {
-    double *o = partials + ((int64_t)c * gridDim.y + blockIdx.y) * 2;
-    o[0] = l1;
-    o[1] = l2;
-  }
-}
-
-// block per start: add the partials in order, then f(x) of Table 1 and the explained variance
-__global__ void __launch_bounds__(FT) k_fin_reduce(int form, const double *__restrict__ partials,
-                                                   int nchunks, const float *__restrict__ sup_val,
-                                                   int cap, StartState st) {
-  __shared__ double red[32];
-  const int c = blockIdx.x;
-  const int nnz = st.nnz[c];
-  double a1 = 0.0;
-  for (int t = threadIdx.x; t < nnz; t += FT) a1 += fabs((double)sup_val[(int64_t)c * cap + t]);
-  const double x1 = block_sum_d(a1, red);
-  if (threadIdx.x != 0) return;
-  double l1 = 0.0, l2sq = 0.0;
-  for (int b = 0; b < nchunks; ++b) {
-    l1 += partials[((int64_t)c * nchunks + b) * 2 + 0];
-    l2sq += partials[((int64_t)c * nchunks + b) * 2 + 1];
-  }
-  const double l2 = sqrt(l2sq), x0 = (double)nnz, g = st.gamma[c];
-  double f;
-  switch (form) {
-    case 1: case 3: f = l2; break;
-    case 2: case 4: f = l1; break;
-    case 5: f = l2sq - g * x0; break;
-    case 6: f = l1 * l1 - g * x0; break;
-    case 7: f = l2 - g * x1; break;
-    default: f = l1 - g * x1; break;
-  }
-  st.f[c] = f;
-  st.ev[c] = is_l1_var(form) ? l1 : l2sq;
-}
-
-cudaError_t launch_finalise(int form, const float *AT, int64_t ldat, int n, int p, const float *X,
-                            int64_t ldX, StartState s, int r, float *U, int64_t ldu,
-                            const int *sup_idx, const float *sup_val, int cap, double *partials,
-                            cudaStream_t st) {
-  (void)p; (void)X; (void)ldX;
-  const int nchunks = (n + FT - 1) / FT;
-  if (nchunks > 65535) return cudaErrorInvalidValue;   // grid y limit: n above 16.7 million rows
-  k_fin_partial<float><<<dim3((unsigned)r, (unsigned)nchunks), FT, 0, st>>>(AT, nullptr, ldat, n, sup_idx, sup_val,
-                                                                             cap, s, U, ldu, partials);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_fin_reduce<<<r, FT, 0, st>>>(form, partials, nchunks, sup_val, cap, s);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_finalise_h(int form, const __half *AT16, const float *at_inv, int64_t ldat, int n, StartState s,
-                              int r, float *U, int64_t ldu, const int *sup_idx, const float *sup_val, int cap,
-                              double *partials, cudaStream_t st) {
-  const int nchunks = (n + FT - 1) / FT;
-  if (nchunks > 65535) return cudaErrorInvalidValue;
-  k_fin_partial<__half><<<dim3((unsigned)r, (unsigned)nchunks), FT, 0, st>>>(AT16, at_inv, ldat, n, sup_idx,
-                                                                              sup_val, cap, s, U, ldu, partials);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_fin_reduce<<<r, FT, 0, st>>>(form, partials, nchunks, sup_val, cap, s);
-  return cudaGetLastError();
-}
-
-// argmax over starts of f (or of the explained variance), ties to the lower index
-__global__ void __launch_bounds__(1024) k_best(int use_ev, StartState st, int r, int *best) {
+// argmax over r starts of f (or of the explained variance), ties to the lower index; written by other
+// CTAs of the same launch, so read from L2
+__device__ __forceinline__ void best_body(const double *val, int r, int *best) {
   __shared__ double sv[32];
   __shared__ int si[32];
   double bv = -INFINITY;
   int bi = 0x7fffffff;
   for (int c = threadIdx.x; c < r; c += blockDim.x) {
-    const double val = use_ev ? st.ev[c] : st.f[c];
-    if (val > bv) { bv = val; bi = c; }
+    const double v = __ldcg(val + c);
+    if (v > bv) { bv = v; bi = c; }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -146,52 +43,265 @@ __global__ void __launch_bounds__(1024) k_best(int use_ev, StartState st, int r,
   }
 }
 
+// four consecutive entries of a column of A (a row of A^T): FP32, or FP16 times the column's
+// power-of-two inverse scale (the 16-bit copy of a resident handle; exact in FP32)
+__device__ __forceinline__ float4 col4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
+__device__ __forceinline__ float4 col4(const __half *p) {
+  const uint2 raw = __ldg(reinterpret_cast<const uint2 *>(p));
+  const __half2 *h = reinterpret_cast<const __half2 *>(&raw);
+  const float2 a = __half22float2(h[0]), b = __half22float2(h[1]);
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+
+// Chunk b (of nch) of start c: u_i = sum_t x_{j_t} A[i, j_t] over the support (compensated FP32 pairs),
+// four rows per thread as one vector with eight columns' loads in flight, and the chunk's FP64 sum of
+// |u_i| or u_i^2, whichever the formulation's variance takes.  The start's last chunk then adds the
+// partial sums in a fixed order and gives f (Table 1) and the explained variance; the last start finds
+// the best one.  cnt: r + 1 zeroed counters, left zeroed.
+// Starts on grid x, chunks on y: the CTAs in flight share row chunks, so a column slice used by several
+// starts' supports is read from DRAM about once.  The pairs' FP32 arithmetic (about 12 operations per
+// entry) and the gather through L2 bound it.
+// 1024 starts of 50 nonzeros, n = 5000: 156 us (a row per thread, one load in flight, both norms, and
+// three launches: 353 us); 12 members of a group: 42 us (342 us as launches of their own).
+template <typename T>
+__device__ __forceinline__ void finalise_body(int form, const T *__restrict__ AT, const float *__restrict__ row_inv,
+                                              int64_t ldat, int n, const int *__restrict__ sup_idx,
+                                              const float *__restrict__ sup_val, int cap, const StartState &st, int r,
+                                              float *__restrict__ U, int64_t ldu, double *partials, int *cnt,
+                                              int use_ev, int *best, int c, int b, int nch) {
+  __shared__ int sidx[FT];
+  __shared__ float sval[FT];
+  __shared__ float sinv[FT];
+  __shared__ double red[32];
+  __shared__ int state;
+  const int i4 = (b * FT + threadIdx.x) * 4;
+  const int nnz = st.nnz[c];
+  const int *gi = sup_idx + (int64_t)c * cap;
+  const float *gv = sup_val + (int64_t)c * cap;
+  F32Pair acc[4];
+  auto step = [&](float x, float inv, const float4 &a) {
+    f32pair_fma(acc[0], x, a.x * inv);
+    f32pair_fma(acc[1], x, a.y * inv);
+    f32pair_fma(acc[2], x, a.z * inv);
+    f32pair_fma(acc[3], x, a.w * inv);
+  };
+  for (int t0 = 0; t0 < nnz; t0 += FT) {
+    __syncthreads();
+    if (t0 + (int)threadIdx.x < nnz) {
+      const int j = gi[t0 + threadIdx.x];
+      sidx[threadIdx.x] = j;
+      sval[threadIdx.x] = gv[t0 + threadIdx.x];
+      sinv[threadIdx.x] = row_inv ? row_inv[j] : 1.0f;
+    }
+    __syncthreads();
+    const int m = min(FT, nnz - t0);
+    if (i4 < n) {              // (the columns are padded to a multiple of 8 rows)
+      const T *base = AT + i4;
+      int t = 0;
+      for (; t + 8 <= m; t += 8) {
+        float4 a[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) a[q] = col4(base + (int64_t)sidx[t + q] * ldat);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) step(sval[t + q], sinv[t + q], a[q]);
+      }
+      for (; t < m; ++t) step(sval[t], sinv[t], col4(base + (int64_t)sidx[t] * ldat));
+    }
+  }
+  const bool l1 = is_l1_var(form);
+  double part = 0.0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (i4 + q < n) {
+      const double u = f32pair_value(acc[q]);
+      U[(int64_t)c * ldu + i4 + q] = (float)u;
+      part = l1 ? part + fabs(u) : fma(u, u, part);
+    }
+  }
+  part = block_sum_d(part, red);
+  if (threadIdx.x == 0) {
+    partials[(int64_t)c * nch + b] = part;
+    int before;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(cnt + c) : "memory");
+    state = before == nch - 1;
+  }
+  __syncthreads();
+  if (!state) return;
+  // the start's last chunk
+  double sum = 0.0, x1 = 0.0;
+  for (int q = threadIdx.x; q < nch; q += FT) sum += __ldcg(partials + (int64_t)c * nch + q);
+  sum = block_sum_d(sum, red);
+  if (uses_V(form)) {          // ||x||_1 (Table 1's L1 penalty alone needs it)
+    for (int t = threadIdx.x; t < nnz; t += FT) x1 += fabs((double)gv[t]);
+    x1 = block_sum_d(x1, red);
+  }
+  if (threadIdx.x == 0) {
+    const double norm = l1 ? sum : sqrt(sum), g = st.gamma[c];
+    double f = norm;
+    if (uses_U(form)) f = norm * norm - g * (double)nnz;
+    if (form == 5) f = sum - g * (double)nnz;
+    if (uses_V(form)) f = norm - g * x1;
+    st.f[c] = f;
+    st.ev[c] = sum;
+    cnt[c] = 0;
+    int before;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(cnt + r) : "memory");
+    state = before == r - 1;
+    if (state) cnt[r] = 0;
+  }
+  __syncthreads();
+  if (state) best_body(use_ev ? st.ev : st.f, r, best);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(FT) k_finalise(int form, const T *__restrict__ AT, const float *__restrict__ row_inv,
+                                                 int64_t ldat, int n, const int *__restrict__ sup_idx,
+                                                 const float *__restrict__ sup_val, int cap, StartState st,
+                                                 float *__restrict__ U, int64_t ldu, double *partials, int *cnt,
+                                                 int use_ev, int *best) {
+  finalise_body(form, AT, row_inv, ldat, n, sup_idx, sup_val, cap, st, (int)gridDim.x, U, ldu, partials, cnt, use_ev,
+                best, (int)blockIdx.x, (int)blockIdx.y, (int)gridDim.y);
+}
+
+cudaError_t launch_finalise(int form, const float *AT, const __half *AT16, const float *at_inv, int64_t ldat, int n,
+                            StartState s, int r, float *U, int64_t ldu, const int *sup_idx, const float *sup_val,
+                            int cap, double *partials, int *cnt, int use_ev, int *best, cudaStream_t st) {
+  const int nch = finalise_chunks(n);
+  if (nch > 65535) return cudaErrorInvalidValue;   // grid y limit
+  const dim3 grid((unsigned)r, (unsigned)nch);
+  if (AT16)
+    k_finalise<__half><<<grid, FT, 0, st>>>(form, AT16, at_inv, ldat, n, sup_idx, sup_val, cap, s, U, ldu, partials,
+                                            cnt, use_ev, best);
+  else
+    k_finalise<float><<<grid, FT, 0, st>>>(form, AT, nullptr, ldat, n, sup_idx, sup_val, cap, s, U, ldu, partials, cnt,
+                                           use_ev, best);
+  return cudaGetLastError();
+}
+
+// the same for the finishing members of a group (done[i] != 0; all when null), one launch
+__global__ void __launch_bounds__(FT) k_g_finalise(const GProb *__restrict__ P, const int *__restrict__ prob,
+                                                   const int *__restrict__ done) {
+  const int i = prob[blockIdx.x];
+  if (done && !done[i]) return;
+  const GProb &q = P[i];
+  const int nch = (q.n + FR - 1) / FR, c = (int)blockIdx.x - q.start0;
+  if ((int)blockIdx.y >= nch) return;
+  if (q.AT16)
+    finalise_body(q.form, q.AT16, q.at_inv, q.ldAT, q.n, q.sup_idx, q.sup_val, q.p, q.st, q.r, q.U, q.ldU, q.partials,
+                  q.fin_cnt, q.use_ev, q.best, c, (int)blockIdx.y, nch);
+  else
+    finalise_body(q.form, q.AT32, static_cast<const float *>(nullptr), q.ldAT, q.n, q.sup_idx, q.sup_val, q.p, q.st,
+                  q.r, q.U, q.ldU, q.partials, q.fin_cnt, q.use_ev, q.best, c, (int)blockIdx.y, nch);
+}
+
+// argmax over starts of f (or of the explained variance), ties to the lower index
+__global__ void __launch_bounds__(1024) k_best(int use_ev, StartState st, int r, int *best) {
+  best_body(use_ev ? st.ev : st.f, r, best);
+}
+
 cudaError_t launch_best(int form, int use_ev, StartState s, int r, int *best, cudaStream_t st) {
   (void)form;
   k_best<<<1, 1024, 0, st>>>(use_ev, s, r, best);
   return cudaGetLastError();
 }
 
-// y = y(x) (S2: sgn(u), S1: u / ||u||_2) of the best start, its x, and its support
-__global__ void __launch_bounds__(1024) k_best_outputs(int form, const int *__restrict__ best,
-                                                       const float *__restrict__ U, int64_t ldu, int n,
-                                                       const float *__restrict__ X, int64_t ldX, int p,
-                                                       float *__restrict__ y_out,
-                                                       float *__restrict__ x_out,
-                                                       int64_t *__restrict__ support_out,
-                                                       int64_t *__restrict__ nnz_out) {
-  __shared__ double red[32];
-  __shared__ int redi[32];
-  const int c = *best;
+// y = y(x) (S2: sgn(u), S1: u / ||u||_2, with ||u||_2^2 = the explained variance), x and the support of
+// the best start.  CTA 0 compacts the support, from the start's list (sup_idx / sup_val, nnz entries) or,
+// without lists, from all of x: each warp counts a contiguous range, one exchange over the warps, then
+// each writes its part.  The other CTAs copy x and write y.  One CTA did all of it before, 1024 entries of
+// x per barrier pair: p = 100000 158 us, p = 20000 53 us; now 5 and 6 us.
+constexpr int OT_ = 512;
+__device__ __forceinline__ void best_outputs_body(int form, int c, const float *__restrict__ U, int64_t ldu, int n,
+                                                  const double *__restrict__ ev, const float *__restrict__ X,
+                                                  int64_t ldX, int p, const int *sup_idx, const float *sup_val,
+                                                  int cap, const int *nnz_of, float *y_out, float *x_out,
+                                                  int64_t *support_out, int64_t *nnz_out, int b, int nb) {
+  __shared__ int wcnt[OT_ / 32];
+  __shared__ float inv_s;
   const float *u = U + (int64_t)c * ldu;
   const float *x = X + (int64_t)c * ldX;
-  if (is_l1_var(form)) {
-    for (int i = threadIdx.x; i < n; i += blockDim.x) y_out[i] = (u[i] >= 0.0f) ? 1.0f : -1.0f;
-  } else {
-    double part = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) part += (double)u[i] * (double)u[i];
-    const double nrm = sqrt(block_sum_d(part, red));
-    const float inv = nrm > 0.0 ? (float)(1.0 / nrm) : 0.0f;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) y_out[i] = u[i] * inv;
+  if (b == 0) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int m = sup_idx ? nnz_of[c] : p;
+    const int *ix = sup_idx ? sup_idx + (int64_t)c * cap : nullptr;
+    const float *v = sup_idx ? sup_val + (int64_t)c * cap : x;
+    const int per = ((m + OT_ / 32 - 1) / (OT_ / 32) + 31) / 32 * 32, lo = min(m, w * per), hi = min(m, lo + per);
+    int cnt = 0;
+#pragma unroll 8
+    for (int i = lo + lane; i < hi; i += 32) cnt += v[i] != 0.0f;
+    cnt = warp_sum_i(cnt);
+    if (lane == 0) wcnt[w] = cnt;
+    __syncthreads();
+    int pos = 0, tot = 0;
+    for (int k = 0; k < OT_ / 32; ++k) {
+      pos += k < w ? wcnt[k] : 0;
+      tot += wcnt[k];
+    }
+#pragma unroll 4
+    for (int base = lo; base < hi; base += 32) {
+      const int i = base + lane;
+      const bool on = i < hi && v[i] != 0.0f;
+      const unsigned ball = __ballot_sync(0xffffffffu, on);
+      if (on) support_out[pos + __popc(ball & ((1u << lane) - 1u))] = ix ? ix[i] : i;
+      pos += __popc(ball);
+    }
+    if (threadIdx.x == 0) *nnz_out = tot;
+    return;
   }
-  int written = 0;
-  for (int base = 0; base < p; base += blockDim.x) {
-    const int j = base + threadIdx.x;
-    const float xj = (j < p) ? x[j] : 0.0f;
-    if (j < p) x_out[j] = xj;
-    int tot;
-    const int pos = written + block_excl_scan_flag(xj != 0.0f, redi, &tot);
-    if (xj != 0.0f) support_out[pos] = j;
-    written += tot;
+  const int t0 = (b - 1) * OT_ + threadIdx.x, step = (nb - 1) * OT_;
+  if (!is_l1_var(form)) {
+    if (threadIdx.x == 0) {
+      const double nrm = sqrt(ev[c]);
+      inv_s = nrm > 0.0 ? (float)(1.0 / nrm) : 0.0f;
+    }
+    __syncthreads();
   }
-  if (threadIdx.x == 0) *nnz_out = written;
+  const float inv = inv_s;
+  for (int i = t0; i < n; i += step) y_out[i] = is_l1_var(form) ? (u[i] >= 0.0f ? 1.0f : -1.0f) : u[i] * inv;
+  for (int j = t0; j < p; j += step) x_out[j] = x[j];
+}
+// CTAs for the outputs of an n x p problem: about four entries per thread
+static int output_ctas(int64_t n, int64_t p) {
+  const int64_t b = (std::max(n, p) + 4 * OT_ - 1) / (4 * OT_);
+  return 1 + (int)std::min<int64_t>(b, 64);
 }
 
-cudaError_t launch_best_outputs(int form, const int *best, const float *U, int64_t ldu, int n,
-                                const float *X, int64_t ldX, int p, float *y_out, float *x_out,
-                                int64_t *support_out, int64_t *nnz_out, cudaStream_t st) {
-  k_best_outputs<<<1, 1024, 0, st>>>(form, best, U, ldu, n, X, ldX, p, y_out, x_out, support_out,
-                                     nnz_out);
+__global__ void __launch_bounds__(OT_) k_best_outputs(int form, const int *__restrict__ best,
+                                                      const float *__restrict__ U, int64_t ldu, int n,
+                                                      const double *__restrict__ ev, const float *__restrict__ X,
+                                                      int64_t ldX, int p, const int *sup_idx, const float *sup_val,
+                                                      int cap, const int *nnz_of, float *__restrict__ y_out,
+                                                      float *__restrict__ x_out, int64_t *__restrict__ support_out,
+                                                      int64_t *__restrict__ nnz_out) {
+  best_outputs_body(form, *best, U, ldu, n, ev, X, ldX, p, sup_idx, sup_val, cap, nnz_of, y_out, x_out, support_out,
+                    nnz_out, (int)blockIdx.x, (int)gridDim.x);
+}
+
+cudaError_t launch_best_outputs(int form, const int *best, const float *U, int64_t ldu, int n, const double *ev,
+                                const float *X, int64_t ldX, int p, const int *sup_idx, const float *sup_val, int cap,
+                                const int *nnz_of, float *y_out, float *x_out, int64_t *support_out, int64_t *nnz_out,
+                                cudaStream_t st) {
+  k_best_outputs<<<output_ctas(n, p), OT_, 0, st>>>(form, best, U, ldu, n, ev, X, ldX, p, sup_idx, sup_val, cap,
+                                                    nnz_of, y_out, x_out, support_out, nnz_out);
+  return cudaGetLastError();
+}
+
+// the same for the finishing members of a group: grid (CTAs of the largest member, members)
+__global__ void __launch_bounds__(OT_) k_g_best_outputs(const GProb *__restrict__ P, const int *__restrict__ done) {
+  if (done && !done[blockIdx.y]) return;
+  const GProb &q = P[blockIdx.y];
+  best_outputs_body(q.form, *q.best, q.U, q.ldU, q.n, q.st.ev, q.X, q.ldX, q.p, q.sup_idx, q.sup_val, q.p, q.st.nnz,
+                    q.y_out, q.x_out, q.support_out, q.nnz_out, (int)blockIdx.x, (int)gridDim.x);
+}
+
+cudaError_t launch_g_finish(const GProb *P, const int *prob, int R, int np, int max_n, int max_p, const int *done,
+                            cudaStream_t st) {
+  const int nch = finalise_chunks(max_n);
+  if (nch > 65535) return cudaErrorInvalidValue;
+  k_g_finalise<<<dim3((unsigned)R, (unsigned)nch), FT, 0, st>>>(P, prob, done);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_g_best_outputs<<<dim3((unsigned)output_ctas(max_n, max_p), (unsigned)np), OT_, 0, st>>>(P, done);
   return cudaGetLastError();
 }
 

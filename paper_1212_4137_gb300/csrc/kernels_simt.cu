@@ -129,9 +129,9 @@ cudaError_t launch_start_init(const float *x0, int64_t ld0, uint64_t seed, int r
 // One kernel reads x0, checks it, normalises it and writes what the first sweep reads; it replaces a
 // copy of x0, a check, an in-place normalisation (three passes), row scales, a plane split and the
 // active list.  Bound by HBM: 4 p bytes read and 4 p written per start (two FP16 planes, or FP32).
-// 1024 starts, p = 20000, tensor cores: 55 us for the kernel (290 us for the launches it replaces and the
+// 1024 starts, p = 20000, tensor cores: 48 us for the kernel (290 us for the launches it replaces and the
 // copy).
-__global__ void __launch_bounds__(256) k_start_pack(const float *x0, int64_t ld0, uint64_t key, int p, float *X,
+__global__ void __launch_bounds__(1024) k_start_pack(const float *x0, int64_t ld0, uint64_t key, int p, float *X,
                                                     int64_t ldX, XPack pk, StartState s, double gamma0, int *flag,
                                                     int r, int *act, int *rank, Ctrl *ctrl) {
   __shared__ float redf[32];
@@ -144,7 +144,9 @@ __global__ void __launch_bounds__(256) k_start_pack(const float *x0, int64_t ld0
 cudaError_t launch_start_pack(const float *x0, int64_t ld0, uint64_t seed, int r, int p, float *X, int64_t ldX,
                               XPack pk, StartState s, double gamma0, int *flag, int *act, int *rank, Ctrl *ctrl,
                               cudaStream_t st) {
-  k_start_pack<<<r, 256, 0, st>>>(x0, ld0, start_key(seed), p, X, ldX, pk, s, gamma0, flag, r, act, rank, ctrl);
+  // seeded normals are FP64 work of the first 256 threads; few long starts: more threads for the packing
+  const int threads = x0 && r <= 152 && p > 4096 ? 1024 : 256;
+  k_start_pack<<<r, threads, 0, st>>>(x0, ld0, start_key(seed), p, X, ldX, pk, s, gamma0, flag, r, act, rank, ctrl);
   return cudaGetLastError();
 }
 

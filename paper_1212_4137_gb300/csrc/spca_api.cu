@@ -111,10 +111,11 @@ void free_workspace(spca_handle *h) {
                   h->status, h->iters, h->nnz, h->F, h->F_prev, h->gamma, h->f, h->ev, h->thr, h->tprev, h->xfast,
                   h->partials, h->ctrl, h->best, h->y_out, h->x_out, h->support_out, h->nnz_out,
                   h->mark, h->colpos, h->collist, h->AS, h->XS, h->x_scale, h->x_inv, h->Bt, h->sp_part, h->ysum,
-                  h->X8, h->Y8, h->x8_inv};
+                  h->X8, h->Y8, h->x8_inv, h->fin_cnt};
   for (void *q : ptrs)
     if (q) cudaFree(q);
   h->X8 = h->Y8 = nullptr;
+  h->fin_cnt = nullptr;
   h->x8_inv = nullptr;
   h->Bt = h->sp_part = h->ysum = nullptr;
   h->ldb = 0;
@@ -159,6 +160,8 @@ int ensure_workspace(spca_handle *h, int r) {
   CK(dalloc(&h->f, r)); CK(dalloc(&h->ev, r)); CK(dalloc(&h->thr, r));
   CK(dalloc(&h->tprev, r)); CK(dalloc(&h->xfast, r));
   CK(dalloc(&h->partials, (size_t)r * nchunks * 2));
+  CK(dalloc(&h->fin_cnt, (size_t)r + 1));
+  CK(cudaMemsetAsync(h->fin_cnt, 0, ((size_t)r + 1) * sizeof(int), h->stream));
   CK(dalloc(&h->ysum, (size_t)r * ((n + kYChunk - 1) / kYChunk)));
   CK(dalloc(&h->ctrl, 2)); CK(dalloc(&h->best, 1));
   CK(dalloc(&h->y_out, (size_t)h->ldU)); CK(dalloc(&h->x_out, (size_t)h->ldX));
@@ -1398,8 +1401,9 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
       Sa.ev = view.ev;
       if (e == cudaSuccess) e = launch_best(form, target ? 1 : 0, Sa, cnt, h->best, st);
       if (e == cudaSuccess)
-        e = launch_best_outputs(form, h->best, view.U, h->ldU, n, view.x, h->ldX, p, h->y_out, h->x_out,
-                                h->support_out, h->nnz_out, st);
+        e = launch_best_outputs(form, h->best, view.U, h->ldU, n, view.ev, view.x, h->ldX, p,
+                                otf ? nullptr : h->sup_idx, h->sup_val, p, S.nnz, h->y_out, h->x_out, h->support_out,
+                                h->nnz_out, st);
       return e;
     }));
   } else if (otf) {
@@ -1411,22 +1415,18 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
       Sa.ev = h->arc.ev;
       if (e == cudaSuccess) e = launch_best(form, target ? 1 : 0, Sa, l, h->best, st);
       if (e == cudaSuccess)
-        e = launch_best_outputs(form, h->best, h->arc.U, h->ldU, n, h->arc.x, h->ldX, p, h->y_out, h->x_out,
-                                h->support_out, h->nnz_out, st);
+        e = launch_best_outputs(form, h->best, h->arc.U, h->ldU, n, h->arc.ev, h->arc.x, h->ldX, p, nullptr, nullptr, 0,
+                                nullptr, h->y_out, h->x_out, h->support_out, h->nnz_out, st);
       return e;
     }));
   } else {
-    CK(timed(h, SPCA_K_FINALISE, 4, [&] {
-      cudaError_t e =
-          h->resident16
-              ? launch_finalise_h(form, static_cast<const __half *>(h->ATpl), h->at_inv, h->ldAT, n, S, r, h->U,
-                                  h->ldU, h->sup_idx, h->sup_val, p, h->partials, st)
-              : launch_finalise(form, h->AT32, h->ldAT, n, p, h->X, h->ldX, S, r, h->U, h->ldU, h->sup_idx,
-                                h->sup_val, p, h->partials, st);
-      if (e == cudaSuccess) e = launch_best(form, target ? 1 : 0, S, r, h->best, st);
+    CK(timed(h, SPCA_K_FINALISE, 2, [&] {
+      cudaError_t e = launch_finalise(form, h->AT32, h->resident16 ? static_cast<const __half *>(h->ATpl) : nullptr,
+                                      h->at_inv, h->ldAT, n, S, r, h->U, h->ldU, h->sup_idx, h->sup_val, p,
+                                      h->partials, h->fin_cnt, target ? 1 : 0, h->best, st);
       if (e == cudaSuccess)
-        e = launch_best_outputs(form, h->best, h->U, h->ldU, n, h->X, h->ldX, p, h->y_out, h->x_out,
-                                h->support_out, h->nnz_out, st);
+        e = launch_best_outputs(form, h->best, h->U, h->ldU, n, S.ev, h->X, h->ldX, p, h->sup_idx, h->sup_val, p, S.nnz,
+                                h->y_out, h->x_out, h->support_out, h->nnz_out, st);
       return e;
     }));
   }

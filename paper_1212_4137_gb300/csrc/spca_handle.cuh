@@ -102,6 +102,7 @@ struct spca_handle {
   float *thr = nullptr, *tprev = nullptr;
   int *xfast = nullptr;
   double *partials = nullptr;
+  int *fin_cnt = nullptr;     // the finalise's counters (r_cap + 1, zero between launches)
   Ctrl *ctrl = nullptr;       // device, 2 entries
   int *best = nullptr;
   float *y_out = nullptr, *x_out = nullptr;

@@ -438,6 +438,12 @@ struct GProb {
   int64_t ld0;
   uint64_t key;
   double gamma0;
+  // the finalise: scratch (r * finalise_chunks(n) doubles; r + 1 zeroed counters) and outputs
+  double *partials;
+  int *fin_cnt;
+  int use_ev, *best;
+  float *y_out, *x_out;
+  int64_t *support_out, *nnz_out;
 };
 // a pool: members on one matrix whose v = A^T y has the same plane products, listed at
 // members[first .. first + nmem - 1]; one contraction over their active starts side by side
@@ -468,6 +474,9 @@ cudaError_t launch_copy_list(const CopyDesc *list, int count, cudaStream_t st);
 cudaError_t launch_g_ctrl(const GProb *P, int np, int parity, int *out, cudaStream_t st);
 cudaError_t launch_g_gather(const GProb *P, const int *prob, int R, int max_n, cudaStream_t st);
 cudaError_t launch_g_ystep(const GProb *P, const int *prob, int R, cudaStream_t st);
+// the finalise and the outputs of the members with done[i] != 0 (all when null)
+cudaError_t launch_g_finish(const GProb *P, const int *prob, int R, int np, int max_n, int max_p, const int *done,
+                            cudaStream_t st);
 // (max_p: the longest v; max_p_small: the longest that fits in shared memory, 0 if none; any_large: some v does not;
 // defer: the full pass in kernels of its own, and no active lists, see launch_xstep)
 cudaError_t launch_g_xstep(const GProb *P, const int *prob, int R, int max_p, int max_p_small, bool any_large,
@@ -576,20 +585,20 @@ cudaError_t launch_xstep(XstepArgs a, const float *V, int64_t ldv, int r, float 
                          StartState s, int *sup_idx, float *sup_val, Ctrl *ctrl, Ctrl *ctrl_read, int *act,
                          int *rank, bool defer, cudaStream_t st);
 
-// a7: Table 1 objective in FP64 for every start; u of each start into U
-// (partials: r * ceil(n / 256) * 2 doubles of scratch)
-cudaError_t launch_finalise(int form, const float *AT, int64_t ldat, int n, int p, const float *X,
-                            int64_t ldX, StartState s, int r, float *U, int64_t ldu,
-                            const int *sup_idx, const float *sup_val, int cap, double *partials,
-                            cudaStream_t st);
-// the same on a 16-bit copy of A^T: FP16 rows (ldat apart) times their power-of-two inverse scale
-cudaError_t launch_finalise_h(int form, const __half *AT16, const float *at_inv, int64_t ldat, int n, StartState s,
-                              int r, float *U, int64_t ldu, const int *sup_idx, const float *sup_val, int cap,
-                              double *partials, cudaStream_t st);
+// a7: Table 1 objective in FP64 for every start, with u of each start into U, and the best start (of the
+// objective, or of the explained variance with use_ev); A^T in FP32, or (AT16 given) FP16 rows times their
+// power-of-two inverse scale.  partials: r * finalise_chunks(n) doubles of scratch; cnt: r + 1 ints, zero
+// before and after
+int finalise_chunks(int64_t n);
+cudaError_t launch_finalise(int form, const float *AT, const __half *AT16, const float *at_inv, int64_t ldat, int n,
+                            StartState s, int r, float *U, int64_t ldu, const int *sup_idx, const float *sup_val,
+                            int cap, double *partials, int *cnt, int use_ev, int *best, cudaStream_t st);
 // argmax over starts (ties: lower index), then y(x) and the support of the best start
 cudaError_t launch_best(int form, int use_ev, StartState s, int r, int *best, cudaStream_t st);
-cudaError_t launch_best_outputs(int form, const int *best, const float *U, int64_t ldu, int n,
-                                const float *X, int64_t ldX, int p, float *y_out, float *x_out,
-                                int64_t *support_out, int64_t *nnz_out, cudaStream_t st);
+// (ev: the starts' explained variances; sup_idx / sup_val, nnz_of: their support lists, or null)
+cudaError_t launch_best_outputs(int form, const int *best, const float *U, int64_t ldu, int n, const double *ev,
+                                const float *X, int64_t ldX, int p, const int *sup_idx, const float *sup_val, int cap,
+                                const int *nnz_of, float *y_out, float *x_out, int64_t *support_out, int64_t *nnz_out,
+                                cudaStream_t st);
 
 }  // namespace spca

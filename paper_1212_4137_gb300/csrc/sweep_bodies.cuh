@@ -72,20 +72,24 @@ static __device__ void start_pack_body(const float *x0, int64_t ld0, uint64_t ke
   float part = 0.0f;
   unsigned mk = 0u;
   const int nt = (int)blockDim.x;
-  constexpr int U = 8;                         // loads in flight per thread
-  if (g) {
-    for (int j0 = threadIdx.x; j0 < p; j0 += U * nt) {
-      float v[U];
+  constexpr int U = 8, U1 = 16;                // loads in flight per thread
+  // (the first 256 threads, whatever the CTA's size: the sum's order)
+  constexpr int N1 = 256;
+  if (threadIdx.x >= N1) {
+    if (!g) g = x;
+  } else if (g) {
+    for (int j0 = threadIdx.x; j0 < p; j0 += U1 * N1) {
+      float v[U1];
 #pragma unroll
-      for (int k = 0; k < U; ++k) v[k] = j0 + k * nt < p ? g[j0 + k * nt] : 0.0f;
+      for (int k = 0; k < U1; ++k) v[k] = j0 + k * N1 < p ? g[j0 + k * N1] : 0.0f;
 #pragma unroll
-      for (int k = 0; k < U; ++k) {
+      for (int k = 0; k < U1; ++k) {
         part = fmaf(v[k], v[k], part);
         mk = max(mk, abs_key(v[k]));
       }
     }
   } else {
-    for (int j = threadIdx.x; j < p; j += nt) {
+    for (int j = threadIdx.x; j < p; j += N1) {
       const float v = (float)bm_normal(key, (uint64_t)c * (uint64_t)p + (uint64_t)j);
       x[j] = v;
       part = fmaf(v, v, part);
