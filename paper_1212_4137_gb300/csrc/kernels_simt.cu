@@ -329,9 +329,121 @@ __global__ void __launch_bounds__(256) k_gemm_nt_f32(const float *__restrict__ P
   }
 }
 
+// The same for products too small to fill the chip with 128 x 128 tiles (few starts, or one short
+// side): 16 x 32 tiles, each with its K range split over `split` CTAs so that the launch has about two
+// CTAs per SM.  128 threads; slices of 64 K entries of both operands in shared memory (the next one
+// prefetched into registers); a thread adds 4 starts of one column, one 16-byte broadcast and one
+// 4-byte read per 4 FMAs.  The CTA that finishes a tile last adds its parts in K order, so the result
+// does not depend on the timing.  Bound by latency (a few L2 round trips and barriers).
+// 16 starts, ncu, against 128 x 128 tiles: u, 400 x 4000, 595 -> 12 us; v, 4000 x 400, 67 -> 7 us.
+namespace {
+constexpr int FM = 16, FN = 32, FK = 64, FTH = 128;
+}
+__global__ void __launch_bounds__(FTH) k_gemm_few(const float *__restrict__ P, int64_t ldp,
+                                                  const float *__restrict__ Q, int64_t ldq, float *__restrict__ C,
+                                                  int64_t ldc, int M, int N, int K, int kslices,
+                                                  const int *__restrict__ gate, float *parts, int *cnt) {
+  if (gate && *gate == 0) return;
+  __shared__ __align__(16) float Ps[FK][FM];
+  __shared__ float Qs[FK][FN + 1];
+  __shared__ int last;
+  const int tid = threadIdx.x, n0 = blockIdx.x * FN, m0 = blockIdx.y * FM;
+  const int split = gridDim.z, z = blockIdx.z;
+  const int k0 = z * kslices * FK, k1 = min(K, k0 + kslices * FK);   // (K and the slices: multiples of 8)
+  const int mq = (tid >> 5) * 4, nj = tid & 31;   // this thread's starts mq .. mq + 3, column nj
+  float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  // loads of one slice: 16 entries of Q (4 vectors: row q, 16-byte column v) and 8 of P per thread
+  float4 rq[4], rp[2];
+  auto load = [&](int k) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = tid + u * FTH, row = e >> 4, kk = k + (e & 15) * 4;
+      rq[u] = n0 + row < N && kk < k1 ? __ldg(reinterpret_cast<const float4 *>(Q + (int64_t)(n0 + row) * ldq + kk))
+                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {   // (rows fastest: the stores below meet few bank conflicts)
+      const int e = tid + u * FTH, row = e & 15, kk = k + (e >> 4) * 4;
+      rp[u] = m0 + row < M && kk < k1 ? __ldg(reinterpret_cast<const float4 *>(P + (int64_t)(m0 + row) * ldp + kk))
+                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  load(k0);
+  for (int k = k0; k < k1; k += FK) {
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = tid + u * FTH, row = e >> 4, kk = (e & 15) * 4;
+      Qs[kk][row] = rq[u].x; Qs[kk + 1][row] = rq[u].y; Qs[kk + 2][row] = rq[u].z; Qs[kk + 3][row] = rq[u].w;
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int e = tid + u * FTH, row = e & 15, kk = (e >> 4) * 4;
+      Ps[kk][row] = rp[u].x; Ps[kk + 1][row] = rp[u].y; Ps[kk + 2][row] = rp[u].z; Ps[kk + 3][row] = rp[u].w;
+    }
+    __syncthreads();
+    if (k + FK < k1) load(k + FK);
+#pragma unroll 16
+    for (int kk = 0; kk < FK; ++kk) {
+      const float4 p4 = *reinterpret_cast<const float4 *>(&Ps[kk][mq]);
+      const float q = Qs[kk][nj];
+      acc[0] = fmaf(p4.x, q, acc[0]);
+      acc[1] = fmaf(p4.y, q, acc[1]);
+      acc[2] = fmaf(p4.z, q, acc[2]);
+      acc[3] = fmaf(p4.w, q, acc[3]);
+    }
+  }
+  if (split > 1) {
+    const int tile = blockIdx.y * gridDim.x + blockIdx.x;
+    float *mine = parts + ((int64_t)tile * split + z) * (FM * FN);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) __stcg(mine + (mq + q) * FN + nj, acc[q]);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+      int before;
+      asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(cnt + tile) : "memory");
+      last = before == split - 1;
+      if (last) cnt[tile] = 0;
+    }
+    __syncthreads();
+    if (!last) return;
+    const float *all = parts + (int64_t)tile * split * (FM * FN) + mq * FN + nj;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[q] = 0.0f;
+    for (int s = 0; s < split; ++s)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[q] += __ldcg(all + (int64_t)s * (FM * FN) + q * FN);
+  }
+  if (n0 + nj < N)
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (m0 + mq + q < M) C[(int64_t)(m0 + mq + q) * ldc + n0 + nj] = acc[q];
+}
+
+// scratch of k_gemm_few: parts only of launches with fewer than 2 CTAs per SM before the split
+int64_t gemm_few_floats(int sms) { return (int64_t)4 * sms * FM * FN; }
+int gemm_few_tiles(int sms) { return 2 * sms; }
+
+// The 128 x 128 tiles run near the FP32 peak once there are enough of them; the small ones do half as
+// many FMAs per shared-memory read.  So they take products below 2^27 multiply-adds (AUTO's CUDA-core
+// range ends at 2^26), and larger ones while the large tiles would leave SMs idle.
 cudaError_t launch_gemm_nt_f32(const float *P, int64_t ldp, const float *Q, int64_t ldq, float *C,
-                               int64_t ldc, int M, int N, int K, const int *gate, cudaStream_t st) {
+                               int64_t ldc, int M, int N, int K, const int *gate, float *parts, int *cnt, int sms,
+                               cudaStream_t st) {
   dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM));
+  const int64_t work = (int64_t)M * N * K;
+  const int64_t fm = (M + FM - 1) / FM, fn = (N + FN - 1) / FN, slices = (K + FK - 1) / FK;
+  if (parts && fm <= 65535 && (work < (int64_t(1) << 27) || (int64_t)grid.x * grid.y < sms)) {
+    // about two CTAs per SM, at least two slices each
+    int64_t split = 1;
+    if (fm * fn < 2 * (int64_t)sms) split = std::max<int64_t>(1, std::min(4 * (int64_t)sms / (fm * fn), (slices + 1) / 2));
+    const int64_t per = (slices + split - 1) / split;
+    split = (slices + per - 1) / per;
+    k_gemm_few<<<dim3((unsigned)fn, (unsigned)fm, (unsigned)split), FTH, 0, st>>>(P, ldp, Q, ldq, C, ldc, M, N, K,
+                                                                                 (int)per, gate, parts, cnt);
+    return cudaGetLastError();
+  }
   k_gemm_nt_f32<<<grid, 256, 0, st>>>(P, ldp, Q, ldq, C, ldc, M, N, K, gate);
   return cudaGetLastError();
 }

@@ -111,11 +111,12 @@ void free_workspace(spca_handle *h) {
                   h->status, h->iters, h->nnz, h->F, h->F_prev, h->gamma, h->f, h->ev, h->thr, h->tprev, h->xfast,
                   h->partials, h->ctrl, h->best, h->y_out, h->x_out, h->support_out, h->nnz_out,
                   h->mark, h->colpos, h->collist, h->AS, h->XS, h->x_scale, h->x_inv, h->Bt, h->sp_part, h->ysum,
-                  h->X8, h->Y8, h->x8_inv, h->fin_cnt};
+                  h->X8, h->Y8, h->x8_inv, h->fin_cnt, h->few_parts, h->few_cnt};
   for (void *q : ptrs)
     if (q) cudaFree(q);
   h->X8 = h->Y8 = nullptr;
-  h->fin_cnt = nullptr;
+  h->fin_cnt = h->few_cnt = nullptr;
+  h->few_parts = nullptr;
   h->x8_inv = nullptr;
   h->Bt = h->sp_part = h->ysum = nullptr;
   h->ldb = 0;
@@ -166,6 +167,11 @@ int ensure_workspace(spca_handle *h, int r) {
   CK(dalloc(&h->ctrl, 2)); CK(dalloc(&h->best, 1));
   CK(dalloc(&h->y_out, (size_t)h->ldU)); CK(dalloc(&h->x_out, (size_t)h->ldX));
   CK(dalloc(&h->support_out, (size_t)p)); CK(dalloc(&h->nnz_out, 1));
+  if (!h->sparse) {
+    CK(dalloc(&h->few_parts, (size_t)gemm_few_floats(h->sms)));
+    CK(dalloc(&h->few_cnt, (size_t)gemm_few_tiles(h->sms)));
+    CK(cudaMemsetAsync(h->few_cnt, 0, (size_t)gemm_few_tiles(h->sms) * sizeof(int), h->stream));
+  }
   // zero pads: the contractions read the padded K range
   CK(cudaMemsetAsync(h->X, 0, (size_t)r * h->ldX * sizeof(float), h->stream));
   CK(cudaMemsetAsync(h->V, 0, (size_t)r * h->ldX * sizeof(float), h->stream));
@@ -398,7 +404,8 @@ int sweep_u_dense(spca_handle *h, int engine, int r, const int *gate, const int 
     }));
   } else {
     CK(timed(h, SPCA_K_U_DENSE, 1, [&] {
-      return launch_gemm_nt_f32(h->X, h->ldX, h->A32, h->ldA, h->U, h->ldU, r, n, (int)h->ldX, gate, st);
+      return launch_gemm_nt_f32(h->X, h->ldX, h->A32, h->ldA, h->U, h->ldU, r, n, (int)h->ldX, gate, h->few_parts,
+                                h->few_cnt, h->sms, st);
     }));
   }
   return SPCA_OK;
@@ -492,7 +499,8 @@ int sweep_y_v(spca_handle *h, int engine, int form, int r, StartState S, const i
     }));
   } else {
     CK(timed(h, SPCA_K_V, 1, [&] {
-      return launch_gemm_nt_f32(h->Y, h->ldU, h->AT32, h->ldAT, h->V, h->ldX, r, p, (int)h->ldU, nullptr, st);
+      return launch_gemm_nt_f32(h->Y, h->ldU, h->AT32, h->ldAT, h->V, h->ldX, r, p, (int)h->ldU, nullptr,
+                                h->few_parts, h->few_cnt, h->sms, st);
     }));
   }
   return SPCA_OK;

@@ -102,6 +102,8 @@ struct spca_handle {
   float *thr = nullptr, *tprev = nullptr;
   int *xfast = nullptr;
   double *partials = nullptr;
+  float *few_parts = nullptr; // the CUDA-core product's split parts and tile counters
+  int *few_cnt = nullptr;
   int *fin_cnt = nullptr;     // the finalise's counters (r_cap + 1, zero between launches)
   Ctrl *ctrl = nullptr;       // device, 2 entries
   int *best = nullptr;

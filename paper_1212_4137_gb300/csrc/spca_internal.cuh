@@ -273,7 +273,11 @@ cudaError_t launch_gemv(const float *P, int64_t ldp, int M, int K, const float *
 // launch does nothing unless *gate != 0 (the dense u = A x is needed this sweep)
 cudaError_t launch_gemm_nt_f32(const float *P, int64_t ldp, const float *Q, int64_t ldq,
                                float *C, int64_t ldc, int M, int N, int K, const int *gate,
-                               cudaStream_t st);
+                               float *parts, int *cnt, int sms, cudaStream_t st);
+// (parts, cnt: scratch of the split products, gemm_few_floats and gemm_few_tiles ints, the latter zero
+// before and after; null: never split)
+int64_t gemm_few_floats(int sms);
+int gemm_few_tiles(int sms);
 
 // U[c, i] = sum_t val[c, t] AT[idx[c, t], i] for every active start; runs only when
 // *gate != 0 (the control word chose the per-start gather)
