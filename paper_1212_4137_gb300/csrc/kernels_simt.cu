@@ -860,34 +860,61 @@ cudaError_t launch_g_ystep(const GProb *P, const int *prob, int R, cudaStream_t 
 // sums in a fixed butterfly.  Q rows longer than the shared memory holds are taken in chunks of
 // Kc columns (the row sums carried in registers across the chunks, in K order).
 // P's rows and Q's rows are zero past K up to the next multiple of 4 (padded layouts).
+// The rows are walked in steps of NR per warp over the whole grid; the last, partial step gives each
+// row to as many warps of a CTA (2, 4, 8 or 16) as there are to spare, which split its columns, so that
+// the chip stays busy to the end (2.06 steps took the time of three).  Bound by HBM: v = A^T y,
+// 5000 x 20000 (400 MB), before and now, CUDA events (about 5 us more than the kernel): one start 74 -> 64 us,
+// two 102 -> 65, eight 106 -> 86; u = A x: 92 -> 67, 109 -> 77, 405 -> 131 us (its Q rows in chunks).
 template <int R, int NR>
-__global__ void __launch_bounds__(512, 1) k_gemv(const float *__restrict__ P, int64_t ldp, int M, int K, int Kc,
+__global__ void __launch_bounds__(512, R <= 2 ? 2 : 1) k_gemv(const float *__restrict__ P, int64_t ldp, int M, int K, int Kc,
                                                  const float *__restrict__ Q, int64_t ldq,
                                                  const int *__restrict__ rows, const int *__restrict__ count,
                                                  float *__restrict__ out, int64_t ldo, const int *__restrict__ gate) {
   extern __shared__ __align__(16) float qs[];
+  __shared__ float part[R][16];
+  constexpr int U = NR == 1 ? 6 : 4;   // vectors of each row in flight per lane
   if (gate && *gate == 0) return;
   const int cnt = count ? min(*count, R) : R;
   if (cnt <= 0) return;
   const int K4 = (K + 3) / 4, Kp = 4 * K4;
   const int nchunks = (Kp + Kc - 1) / Kc;
-  // columns [k0, k0 + Kc) of the Q rows into shared memory (zero past K)
+  // columns [k0, k0 + Kc) of the Q rows into shared memory (zero past K: the rows' padding), as vectors,
+  // 4 in flight per thread
   auto load_q = [&](int k0) {
+    const int c4 = Kc / 4, have = min(Kp - k0, Kc) / 4;
+#pragma unroll 1
     for (int c = 0; c < R; ++c) {
-      const float *q = Q + (int64_t)(c < cnt ? (rows ? rows[c] : c) : 0) * ldq;
-      for (int k = threadIdx.x; k < Kc; k += blockDim.x)
-        qs[c * Kc + k] = c < cnt && k0 + k < K ? q[k0 + k] : 0.0f;
+      const float4 *q = reinterpret_cast<const float4 *>(Q + (int64_t)(c < cnt ? (rows ? rows[c] : c) : 0) * ldq + k0);
+      float4 *s = reinterpret_cast<float4 *>(qs + c * Kc);
+      const int n = c < cnt ? have : 0;
+      for (int e = threadIdx.x; e < c4; e += 4 * blockDim.x) {
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          v[u] = e + u * (int)blockDim.x < n ? __ldg(q + e + u * blockDim.x) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (e + u * (int)blockDim.x < c4) s[e + u * blockDim.x] = v[u];
+      }
     }
   };
   if (nchunks == 1) {
     load_q(0);
     __syncthreads();
   }
-  const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const int all = gridDim.x * warps;   // warps of the grid
   // NR rows per warp and step: every shared-memory read of Q serves all of them.  The loop count
   // is the same for every warp of the CTA (the chunked path synchronises inside it).
-  for (int base = NR * blockIdx.x * warps; base < M; base += NR * gridDim.x * warps) {
-    const int m0 = base + NR * (threadIdx.x >> 5);
+  for (int base = 0; base < M;) {
+    int g = 1;                         // warps per row (uniform over the grid)
+    const int left = M - base;
+    if (left < NR * all)
+      while (g < 16 && left * 2 * g <= all) g *= 2;
+    const int per = g > 1 ? 1 : NR;    // rows of this warp's step
+    const int m0 = base + per * ((blockIdx.x * warps + warp) / g), sub = warp & (g - 1);
+    base += g > 1 ? left : NR * all;
+    if (nchunks == 1 && g == 1 && m0 >= M) continue;
     const float4 *pr[NR];
 #pragma unroll
     for (int t = 0; t < NR; ++t) pr[t] = reinterpret_cast<const float4 *>(P + (int64_t)min(m0 + t, M - 1) * ldp);
@@ -904,30 +931,51 @@ __global__ void __launch_bounds__(512, 1) k_gemv(const float *__restrict__ P, in
         __syncthreads();
       }
       const int c4 = min(Kc, Kp - k0) / 4;   // float4 columns of this chunk
-#pragma unroll 4
-      for (int k4 = lane; k4 < c4; k4 += 32) {
-        float4 a[NR];
+      // (the last batch of a row is predicated: a rolled remainder would wait for its loads one by one)
+      for (int k4 = sub * 32 + lane; k4 < c4 && m0 < M; k4 += 32 * U * g) {
+        float4 a[U][NR];
 #pragma unroll
-        for (int t = 0; t < NR; ++t) a[t] = m0 < M ? __ldg(pr[t] + k0 / 4 + k4) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int u = 0; u < U; ++u)
 #pragma unroll
-        for (int c = 0; c < R; ++c) {
-          const float4 q = reinterpret_cast<const float4 *>(qs + c * Kc)[k4];
+          for (int t = 0; t < NR; ++t)
+            if (k4 + 32 * u * g < c4 && t < per) a[u][t] = __ldg(pr[t] + k0 / 4 + k4 + 32 * u * g);
 #pragma unroll
-          for (int t = 0; t < NR; ++t) {
-            acc[t][c] = fmaf(a[t].x, q.x, acc[t][c]);
-            acc[t][c] = fmaf(a[t].y, q.y, acc[t][c]);
-            acc[t][c] = fmaf(a[t].z, q.z, acc[t][c]);
-            acc[t][c] = fmaf(a[t].w, q.w, acc[t][c]);
+        for (int u = 0; u < U; ++u) {
+          if (k4 + 32 * u * g < c4) {
+#pragma unroll
+            for (int c = 0; c < R; ++c) {
+              const float4 q = reinterpret_cast<const float4 *>(qs + c * Kc)[k4 + 32 * u * g];
+#pragma unroll
+              for (int t = 0; t < NR; ++t) {
+                if (t < per) {
+                  acc[t][c] = fmaf(a[u][t].x, q.x, acc[t][c]);
+                  acc[t][c] = fmaf(a[u][t].y, q.y, acc[t][c]);
+                  acc[t][c] = fmaf(a[u][t].z, q.z, acc[t][c]);
+                  acc[t][c] = fmaf(a[u][t].w, q.w, acc[t][c]);
+                }
+              }
+            }
           }
         }
       }
     }
-    if (m0 >= M) continue;   // uniform over the warp
 #pragma unroll
     for (int t = 0; t < NR; ++t)
 #pragma unroll
       for (int c = 0; c < R; ++c) acc[t][c] = warp_sum_f(acc[t][c]);
-    if (lane < cnt) {
+    if (g > 1) {                       // the row's warps, added in order
+      __syncthreads();
+#pragma unroll
+      for (int c = 0; c < R; ++c)
+        if (lane == 0) part[c][warp] = acc[0][c];
+      __syncthreads();
+      if (sub == 0) {
+#pragma unroll
+        for (int c = 0; c < R; ++c)
+          for (int q = 1; q < g; ++q) acc[0][c] += part[c][warp + q];
+      }
+    }
+    if (lane < cnt && sub == 0) {
       float *o = out + (int64_t)(rows ? rows[lane] : lane) * ldo;
 #pragma unroll
       for (int t = 0; t < NR; ++t) {
@@ -935,7 +983,7 @@ __global__ void __launch_bounds__(512, 1) k_gemv(const float *__restrict__ P, in
 #pragma unroll
         for (int c = 1; c < R; ++c)
           if (lane == c) v = acc[t][c];
-        if (m0 + t < M) o[m0 + t] = v;
+        if (t < per && m0 + t < M) o[m0 + t] = v;
       }
     }
   }
@@ -964,10 +1012,10 @@ cudaError_t launch_gemv(const float *P, int64_t ldp, int M, int K, const float *
   int64_t Kc = Kp;
   if ((int64_t)w * Kp * 4 > kGemvSmemMax) Kc = (int64_t)kGemvSmemMax / (4 * w) / 128 * 128;
   const size_t smem = (size_t)w * Kc * sizeof(float);
-  // CTAs resident per SM by shared memory (two at least for the streaming), a grid of that many
-  // per SM, each CTA loading the Q rows once (per row batch when they are chunked)
-  const int per_sm = smem <= 48 * 1024 ? 4 : (smem <= 100 * 1024 ? 2 : 1);
-  const int blocks = std::min((M + 15) / 16, per_sm * sms);
+  // CTAs resident per SM (registers: two for one or two starts, else one; shared memory), a grid of
+  // that many per SM, each CTA loading the Q rows once (per row batch when they are chunked)
+  const int per_sm = w <= 2 && smem <= 100 * 1024 ? 2 : 1;
+  const int blocks = std::min(M, per_sm * sms);
   auto go = [&](auto kern, cudaError_t configured) -> cudaError_t {
     if (configured != cudaSuccess) return configured;
     kern<<<blocks, 512, smem, st>>>(P, ldp, M, K, (int)Kc, Q, ldq, rows, count, out, ldo, gate);
