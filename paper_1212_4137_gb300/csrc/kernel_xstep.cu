@@ -530,15 +530,14 @@ __global__ void __launch_bounds__(XT) k_xstep(XstepArgs a_in, const float *__res
 // lists the entries above G (in index order, a short list) and the operator on that list in shared
 // memory.  The bound comes from
 //   - a fixed threshold itself (exact);
-//   - last sweep's threshold t: G = kGuess t, or kGuessLo t when that is too high and t did not hold
-//     steady;
+//   - last sweep's threshold t: G = kGuess t (kGuessSteady t while t holds steady);
 //   - the maxima of 2048 disjoint subsets of v (one more pass): at least j entries lie at or above the
 //     j-th largest of them, and for j well below 2048 not many more do;
 //   - 0 for a very short v: the list holds every nonzero entry.
 // A bound is checked before it is used: at least s (or s + 1) listed entries for the selections,
 // phi(G) < 0 for lambda_s (phi increases through its root); then the list holds every surviving
 // entry and the result is that of a pass over all of v.  A start that no bound serves (more than
-// kFastW entries above it in one of the 16 segments, lambda_s = 0, s beyond the list) takes the full
+// kFastSegCap entries above it in one of the 16 segments, lambda_s = 0, s beyond the list) takes the full
 // pass.
 //
 // One CTA does all of it for a start, in one launch per sweep, and the CTA that finishes last makes
@@ -555,6 +554,7 @@ constexpr int kFastBins = 2048, kFastShift = 17;   // bins of 2^-6 octave below 
 constexpr int kFastAllP = 64;                  // v up to this long: list every nonzero entry
 constexpr int kFastMaxJ = 600;                 // j of the subset maxima: the list stays below kFastCand
 constexpr float kGuess = 0.85f;
+constexpr float kGuessSteady = 0.95f;          // while t holds steady
 constexpr float kGuessLo = 0.6f;
 constexpr float kHint = 0.98f;
 constexpr float kSteady = 0.05f;               // |t_new / t - 1| below this: t holds steady
@@ -963,7 +963,7 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
   for (;;) {
     if (how == kExact) Gk = __float_as_uint(thr);
     else if (how == kAll) Gk = 0u;
-    else if (how == kHigh) Gk = __float_as_uint(kGuess * tprev);
+    else if (how == kHigh) Gk = __float_as_uint((steady && !a.ordered ? kGuessSteady : kGuess) * tprev);
     else if (how == kLow) Gk = __float_as_uint(kGuessLo * tprev);
     else Gk = subset_bound<T>(row, j, fs);
     float f1 = 0.0f, f2 = 0.0f;
@@ -986,7 +986,9 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
     } else if (fits && !exact) ok = ncand >= need || Gk == 0u;
     if (ok) break;
     if (how == kHigh) {
-      how = fits && !steady ? kLow : kSubsets;
+      how = a.ordered && fits && !steady ? kLow : kSubsets;
+      // lambda_s lies below this bound: its active set is larger than the list
+      if (lam_form && fits) j = min(kMaxJ, max(j, ncand + ncand / 2 + 32));
     } else if (how == kLow) {
       how = kSubsets;
     } else if (how == kSubsets && lam_form && fits && j < kMaxJ) {
