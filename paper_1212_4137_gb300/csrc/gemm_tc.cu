@@ -1051,10 +1051,13 @@ cudaError_t launch_tc2_impl(const PMaps &P, const CUtensorMap &Q, int M, int N, 
   int S = max_pairs < sk.slots ? max_pairs : sk.slots;
   if (units < S) S = (int)(units > 0 ? units : 1);
   cfg.gridDim = dim3((unsigned)(2 * S), 1);
-  // the flags of the parts start at 0 for every launch (a memset, so that a launch replayed from a
-  // CUDA graph does not see the parts of the previous replay); a published part sets its flag to 1
-  cudaError_t e = cudaMemsetAsync(sk.flags, 0, (size_t)2 * S * sizeof(int), st);
-  if (e != cudaSuccess) return e;
+  // the flags of the parts start at 0 for every launch (a memset, or a kernel before it in the same
+  // stream, so that a launch replayed from a CUDA graph does not see the parts of the previous replay);
+  // a published part sets its flag to 1
+  if (!sk.zeroed) {
+    const cudaError_t e = cudaMemsetAsync(sk.flags, 0, (size_t)2 * S * sizeof(int), st);
+    if (e != cudaSuccess) return e;
+  }
   // the main product's K pieces: as even as possible, at most sk.piece_kb K-blocks each (with
   // correction products only: the leading-plane products need no FP32-class accuracy)
   int piece = 0;

@@ -1214,9 +1214,12 @@ template <int T>
 __global__ void __launch_bounds__(T, fast_ctas(T)) k_xstep_fast(XstepArgs a, const float *__restrict__ V, int64_t ldv,
                                                             int r, float *__restrict__ X, int64_t ldx, StartState st,
                                                             int *__restrict__ sup_idx, float *__restrict__ sup_val,
-                                                            Ctrl *ctrl, Ctrl *ctrl_read, int *act, int *rank, int defer) {
+                                                            Ctrl *ctrl, Ctrl *ctrl_read, int *act, int *rank,
+                                                            int defer, int *flags, int nflags) {
   __shared__ FastShared<T> fs;
   const int c = blockIdx.x;
+  if (flags && c == 0)
+    for (int i = threadIdx.x; i < nflags; i += T) flags[i] = 0;
   const int status = st.status ? st.status[c] : ST_ACTIVE;
   const XState q0 = load_state(st, c);
   if (status == ST_ACTIVE) xstep_start<T>(a, c, V, ldv, X, ldx, st, q0, sup_idx, sup_val, ctrl, defer != 0, fs);
@@ -1392,12 +1395,12 @@ cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, int n
 
 cudaError_t launch_xstep(XstepArgs a, const float *V, int64_t ldv, int r, float *X, int64_t ldx,
                          StartState s, int *sup_idx, float *sup_val, Ctrl *ctrl, Ctrl *ctrl_read, int *act,
-                         int *rank, bool defer, cudaStream_t st) {
+                         int *rank, bool defer, int *flags, int nflags, cudaStream_t st) {
   const int sms = sm_count(), d = defer ? 1 : 0;
   if (sms < 1) return cudaErrorInvalidDevice;
   int *al = defer ? nullptr : act;
 #define SPCA_FAST(T)                                                                                             \
-  k_xstep_fast<T><<<r, T, 0, st>>>(a, V, ldv, r, X, ldx, s, sup_idx, sup_val, ctrl, ctrl_read, al, rank, d)
+  k_xstep_fast<T><<<r, T, 0, st>>>(a, V, ldv, r, X, ldx, s, sup_idx, sup_val, ctrl, ctrl_read, al, rank, d, flags, nflags)
   switch (fast_threads(r, a.p, sms)) {
     case 1024: SPCA_FAST(1024); break;
     case 512: SPCA_FAST(512); break;

@@ -152,12 +152,21 @@ cudaError_t launch_start_pack(const float *x0, int64_t ld0, uint64_t seed, int r
 
 // ------------------------------------------------------------------ y-step (Table 3 S1, S2)
 // (ystep_body: sweep_bodies.cuh)
+// skip: the sweep's y is written by the gather kernel when *skip != 0; flags: the stream-K flags that
+// the next contraction needs zeroed (null: none)
+__device__ __forceinline__ void zero_flags(int *flags, int nflags) {
+  if (flags && blockIdx.x == 0 && blockIdx.y == 0)
+    for (int i = threadIdx.x; i < nflags; i += blockDim.x) flags[i] = 0;
+}
 __global__ void __launch_bounds__(256) k_ystep(int form, const float *__restrict__ U, int64_t ldu,
                                                int n, float *__restrict__ Y,
                                                __half *__restrict__ Ypl, int64_t pstride,
                                                const int *__restrict__ rank, StartState s,
-                                               float *__restrict__ X, int64_t ldX, int p) {
+                                               float *__restrict__ X, int64_t ldX, int p,
+                                               const int *__restrict__ skip, int *flags, int nflags) {
   __shared__ float redf[32];
+  zero_flags(flags, nflags);
+  if (skip && *skip != 0) return;   // (the gather kernel has done it)
   ystep_body(form, U, ldu, n, Y, Ypl, pstride, rank, s, X, ldX, p, (int)blockIdx.x, redf);
 }
 
@@ -181,8 +190,9 @@ __global__ void __launch_bounds__(256) k_ystep_apply(int form, const float *__re
                                                      float *__restrict__ Y, __half *__restrict__ Ypl,
                                                      int64_t pstride, const int *__restrict__ rank, StartState s,
                                                      float *__restrict__ X, int64_t ldX, int p,
-                                                     const float *__restrict__ ysum) {
+                                                     const float *__restrict__ ysum, int *flags, int nflags) {
   const int b = blockIdx.x, c = blockIdx.y, nch = gridDim.x;
+  zero_flags(flags, nflags);
   // (the chunk-0 CTA alone may change the status below, and only when every CTA of the start
   // returns without writing: ||u||_2 = 0)
   if (s.status[c] != ST_ACTIVE) return;
@@ -229,9 +239,9 @@ __global__ void __launch_bounds__(256) k_ystep_apply(int form, const float *__re
 
 cudaError_t launch_ystep(int form, const float *U, int64_t ldu, int n, int r, float *Y, void *Ypl,
                          int64_t plane_stride, const int *rank, StartState s, float *X, int64_t ldX,
-                         int p, float *ysum, cudaStream_t st) {
+                         int p, float *ysum, const int *skip, int *flags, int nflags, cudaStream_t st) {
   const int nch = (n + kYChunk - 1) / kYChunk;
-  if (ysum && nch > 2) {
+  if (ysum && nch > 2) {   // (skip: not for such u, see ystep_with_gather)
     const dim3 grid((unsigned)nch, (unsigned)r);
     if (!is_l1_var(form)) {
       k_ystep_norm<<<grid, 256, 0, st>>>(U, ldu, n, s, ysum);
@@ -239,11 +249,11 @@ cudaError_t launch_ystep(int form, const float *U, int64_t ldu, int n, int r, fl
       if (e != cudaSuccess) return e;
     }
     k_ystep_apply<<<grid, 256, 0, st>>>(form, U, ldu, n, Y, static_cast<__half *>(Ypl), plane_stride, rank, s, X,
-                                        ldX, p, ysum);
+                                        ldX, p, ysum, flags, nflags);
     return cudaGetLastError();
   }
   k_ystep<<<r, 256, 0, st>>>(form, U, ldu, n, Y, static_cast<__half *>(Ypl), plane_stride, rank,
-                             s, X, ldX, p);
+                             s, X, ldX, p, skip, flags, nflags);
   return cudaGetLastError();
 }
 
@@ -555,64 +565,6 @@ __device__ void gather_lowp_body(const __half *__restrict__ AT0, const float *__
     if (i4 + q < n) u[i4 + q] = acc[q];
 }
 
-// The same gather over the leading FP16 plane of A^T (the low-precision sweeps): row j of the
-// plane is A[:, j] times at_scale[j]; the inverse scale is folded into x_j.  8 rows per thread as
-// one 16-byte load, products and sums in FP32 in support order.
-__global__ void __launch_bounds__(256) k_gemm1_sparse_lowp(const __half *__restrict__ AT0, int64_t ldat,
-                                                           const float *__restrict__ at_inv, int n,
-                                                           const int *__restrict__ sup_idx,
-                                                           const float *__restrict__ sup_val, int cap,
-                                                           StartState s, float *__restrict__ U, int64_t ldu,
-                                                           const int *__restrict__ gate) {
-  if (*gate == 0) return;
-  const int c = blockIdx.x;
-  if (s.status[c] != ST_ACTIVE) return;
-  __shared__ int sidx[256];
-  __shared__ float sval[256];
-  const int nnz = s.nnz[c];
-  const int i8 = (blockIdx.y * blockDim.x + threadIdx.x) * 8;
-  const int *gi = sup_idx + (int64_t)c * cap;
-  const float *gv = sup_val + (int64_t)c * cap;
-  float acc[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) acc[q] = 0.0f;
-  auto step = [&](float xv, uint4 raw) {
-    const __half2 *h2 = reinterpret_cast<const __half2 *>(&raw);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float2 f = __half22float2(h2[q]);
-      acc[2 * q] = fmaf(xv, f.x, acc[2 * q]);
-      acc[2 * q + 1] = fmaf(xv, f.y, acc[2 * q + 1]);
-    }
-  };
-  for (int t0 = 0; t0 < nnz; t0 += 256) {
-    __syncthreads();
-    if (t0 + (int)threadIdx.x < nnz) {
-      const int j = gi[t0 + threadIdx.x];
-      sidx[threadIdx.x] = j;
-      sval[threadIdx.x] = gv[t0 + threadIdx.x] * at_inv[j];
-    }
-    __syncthreads();
-    const int m = min(256, nnz - t0);
-    if (i8 < n) {
-      const __half *base = AT0 + i8;
-      int t = 0;
-      for (; t + 8 <= m; t += 8) {
-        uint4 a[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) a[q] = __ldg(reinterpret_cast<const uint4 *>(base + (int64_t)sidx[t + q] * ldat));
-#pragma unroll
-        for (int q = 0; q < 8; ++q) step(sval[t + q], a[q]);
-      }
-      for (; t < m; ++t) step(sval[t], __ldg(reinterpret_cast<const uint4 *>(base + (int64_t)sidx[t] * ldat)));
-    }
-  }
-  float *u = U + (int64_t)c * ldu;
-#pragma unroll
-  for (int q = 0; q < 8; ++q)
-    if (i8 + q < n) u[i8 + q] = acc[q];
-}
-
 // The same gather over the FP8 E4M3 copy of A^T (the low-precision sweeps of an FP8 handle): row j
 // is A[:, j] times its scale, undone with at8_inv[j] folded into x_j; 16 rows per thread as one
 // 16-byte load, products and sums in FP32 in support order.
@@ -684,36 +636,173 @@ cudaError_t launch_gemm1_sparse_f8(const uint8_t *AT8, int64_t ldat, const float
   return cudaGetLastError();
 }
 
-cudaError_t launch_gemm1_sparse_lowp(const void *AT0, int64_t ldat, const float *at_inv, int n, const int *sup_idx,
-                                     const float *sup_val, int cap, StartState s, int r, float *U, int64_t ldu,
-                                     const int *gate, cudaStream_t st) {
-  if (ldat % 8 != 0 || (reinterpret_cast<uintptr_t>(AT0) & 15u) != 0) return cudaErrorInvalidValue;
-  dim3 grid((unsigned)r, (unsigned)((n + 2047) / 2048));
-  k_gemm1_sparse_lowp<<<grid, 256, 0, st>>>(static_cast<const __half *>(AT0), ldat, at_inv, n, sup_idx, sup_val,
-                                            cap, s, U, ldu, gate);
-  return cudaGetLastError();
-}
+// u = A x over the support.  T = float: A^T in FP32; __half: its leading FP16 plane, the inverse scale
+// at_inv[j] folded into x_j (exact).  V rows per thread as one vector, L columns' loads in flight.
+// Many starts (S = 1): a CTA per start and row block, FMAs in support order; DRAM (the distinct columns
+// of all supports) and L2 bound it.
+// Few starts: the round trips of a start's columns bound it, so the support is staged at once, V is small
+// (more CTAs), L large, and S slices of a CTA's threads take every S-th column each (FP32 only: the FP16
+// plane keeps the support order); the start's last CTA then runs the y-step on the whole of u (from L2)
+// instead of a launch of its own.  cnt: r zeroed counters, left zeroed (y and ypl null: u alone).
+// Gather and y-step of a sweep before and now (ncu, cold caches): one start of 5000 rows and ~500 columns
+// 36 -> 10 us (one row per thread, 4-column batches, y-step of its own before); 16 starts of 9001 rows in
+// FP16 24 -> 16 us; 16 of 500 rows 11 -> 9 us; 1024 of 5000 rows (S = 1, y-step of its own) 72 + 11 us, as
+// before: with the y-step fused 95 us (its tail runs at the gather's occupancy).
+template <typename T, int V>
+struct RowVec;
+template <>
+struct RowVec<float, 4> {
+  float4 v;
+  __device__ void load(const float *p) { v = __ldg(reinterpret_cast<const float4 *>(p)); }
+  __device__ void fma_into(float x, float (&a)[4]) const {
+    a[0] = fmaf(x, v.x, a[0]); a[1] = fmaf(x, v.y, a[1]); a[2] = fmaf(x, v.z, a[2]); a[3] = fmaf(x, v.w, a[3]);
+  }
+};
+template <>
+struct RowVec<float, 1> {
+  float v;
+  __device__ void load(const float *p) { v = __ldg(p); }
+  __device__ void fma_into(float x, float (&a)[1]) const { a[0] = fmaf(x, v, a[0]); }
+};
+template <int V>
+struct RowVec<__half, V> {
+  uint32_t v[V / 2];
+  __device__ void load(const __half *p) {
+    if constexpr (V == 8) {
+      const uint4 t = __ldg(reinterpret_cast<const uint4 *>(p));
+      v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+    } else {
+      v[0] = __ldg(reinterpret_cast<const uint32_t *>(p));
+    }
+  }
+  __device__ void fma_into(float x, float (&a)[V]) const {
+#pragma unroll
+    for (int q = 0; q < V / 2; ++q) {
+      const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&v[q]));
+      a[2 * q] = fmaf(x, f.x, a[2 * q]);
+      a[2 * q + 1] = fmaf(x, f.y, a[2 * q + 1]);
+    }
+  }
+};
 
-__global__ void __launch_bounds__(kGatherThreads) k_gemm1_sparse(const float *__restrict__ AT, int64_t ldat,
-                                                      int n, const int *__restrict__ sup_idx,
-                                                      const float *__restrict__ sup_val, int cap,
-                                                      StartState s, float *__restrict__ U,
-                                                      int64_t ldu, const int *__restrict__ gate) {
-  __shared__ int sidx[kGatherThreads];
-  __shared__ float sval[kGatherThreads];
+template <typename T, int V, int L, int NT, int S>
+__global__ void __launch_bounds__(NT) k_gather_y(int form, const T *__restrict__ AT, const float *__restrict__ at_inv,
+                                                 int64_t ldat, int n, const int *__restrict__ sup_idx,
+                                                 const float *__restrict__ sup_val, int cap, StartState s,
+                                                 float *__restrict__ U, int64_t ldu, const int *__restrict__ gate,
+                                                 float *Y, __half *Ypl, int64_t pstride, const int *__restrict__ rank,
+                                                 float *X, int64_t ldX, int p, int *cnt) {
+  constexpr int R = NT / S, kTile = V < 4 ? 1024 : NT;   // threads of a slice, columns staged at once
+  static_assert(S == 1 || V == 1, "the slices' sums are added for one row per thread");
+  __shared__ int sidx[kTile];
+  __shared__ float sval[kTile];
+  __shared__ float redf[32];
+  __shared__ int last;
   if (*gate == 0) return;
-  gather_body(AT, ldat, n, sup_idx, sup_val, cap, s, U, ldu, (int)blockIdx.x, (int)blockIdx.y, sidx, sval);
+  const int c = blockIdx.x;
+  if (s.status[c] != ST_ACTIVE || s.iters[c] == 0) return;   // a start not swept yet has a dense x
+  const int nnz = s.nnz[c], slice = threadIdx.x / R;
+  const int i0 = (blockIdx.y * R + threadIdx.x % R) * V;
+  const int *gi = sup_idx + (int64_t)c * cap;
+  const float *gv = sup_val + (int64_t)c * cap;
+  float acc[V];
+#pragma unroll
+  for (int q = 0; q < V; ++q) acc[q] = 0.0f;
+  for (int t0 = 0; t0 < nnz; t0 += kTile) {
+    __syncthreads();
+    const int m = min(kTile, nnz - t0);
+    for (int t = threadIdx.x; t < m; t += NT) {
+      const int j = gi[t0 + t];
+      sidx[t] = j;
+      sval[t] = at_inv ? gv[t0 + t] * at_inv[j] : gv[t0 + t];
+    }
+    __syncthreads();
+    if (i0 < n) {              // (the columns are padded to a multiple of 8 rows)
+      const T *base = AT + i0;
+      RowVec<T, V> a[L];
+      int t = slice;
+      for (; t + (L - 1) * S < m; t += L * S) {
+#pragma unroll
+        for (int q = 0; q < L; ++q) a[q].load(base + (int64_t)sidx[t + q * S] * ldat);
+#pragma unroll
+        for (int q = 0; q < L; ++q) a[q].fma_into(sval[t + q * S], acc);
+      }
+      if (t < m) {
+#pragma unroll
+        for (int q = 0; q < L; ++q)
+          if (t + q * S < m) a[q].load(base + (int64_t)sidx[t + q * S] * ldat);
+#pragma unroll
+        for (int q = 0; q < L; ++q)
+          if (t + q * S < m) a[q].fma_into(sval[t + q * S], acc);
+      }
+    }
+  }
+  float *u = U + (int64_t)c * ldu;
+  if constexpr (S > 1) {
+    __shared__ float part[S][R];
+    part[slice][threadIdx.x % R] = acc[0];
+    __syncthreads();
+    if (slice == 0 && i0 < n) {
+      float t = part[0][threadIdx.x];
+#pragma unroll
+      for (int q = 1; q < S; ++q) t += part[q][threadIdx.x];
+      u[i0] = t;
+    }
+  } else if constexpr (V >= 4) {
+#pragma unroll
+    for (int h = 0; h < V; h += 4) {
+      if (i0 + h + 4 <= n) {
+        *reinterpret_cast<float4 *>(u + i0 + h) = make_float4(acc[h], acc[h + 1], acc[h + 2], acc[h + 3]);
+      } else {
+        for (int q = h; q < h + 4; ++q)
+          if (i0 + q < n) u[i0 + q] = acc[q];
+      }
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < V; ++q)
+      if (i0 + q < n) u[i0 + q] = acc[q];
+  }
+  if (!Y && !Ypl) return;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int before = 0;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(cnt + c) : "memory");
+    last = before == (int)gridDim.y - 1;
+    if (last) cnt[c] = 0;
+  }
+  __syncthreads();
+  if (last) ystep_body<true>(form, U, ldu, n, Y, Ypl, pstride, rank, s, X, ldX, p, c, redf);
 }
 
-cudaError_t launch_gemm1_sparse(const float *AT, int64_t ldat, int n, const int *sup_idx,
-                                const float *sup_val, int cap, StartState s, int r, float *U,
-                                int64_t ldu, const int *gate, cudaStream_t st) {
-  if (ldat % 4 != 0 || (reinterpret_cast<uintptr_t>(AT) & 15u) != 0) return cudaErrorInvalidValue;
-  const int blocks = (n + 4 * kGatherThreads - 1) / (4 * kGatherThreads);
-  if (blocks > 65535) return cudaErrorInvalidValue;   // grid y limit: n above 33.5 million rows
-  dim3 grid((unsigned)r, (unsigned)blocks);
-  k_gemm1_sparse<<<grid, kGatherThreads, 0, st>>>(AT, ldat, n, sup_idx, sup_val, cap, s, U, ldu, gate);
-  return cudaGetLastError();
+// The variants for few starts serve where the wide vectors' CTAs are fewer than two per SM (below that the
+// chip is idle between round trips), while the narrow ones' row blocks fit the grid: measured above on
+// both sides
+bool gather_few(bool half, int r, int64_t n, int sms) {
+  return half ? r * ((n + 2047) / 2048) < 2 * sms && n <= (int64_t)65535 * 512
+              : r * ((n + 511) / 512) < 2 * sms && n <= (int64_t)65535 * 64;
+}
+
+cudaError_t launch_gather_y(int form, const float *AT, const void *AT16, const float *at_inv, int64_t ldat, int n,
+                            const int *sup_idx, const float *sup_val, int cap, StartState s, int r, float *U,
+                            int64_t ldu, const int *gate, float *Y, void *Ypl, int64_t pstride, const int *rank,
+                            float *X, int64_t ldX, int p, int *cnt, int sms, cudaStream_t st) {
+  const void *base = AT16 ? AT16 : AT;
+  if (ldat % 8 != 0 || ldu % 8 != 0 || (reinterpret_cast<uintptr_t>(base) & 15u) != 0) return cudaErrorInvalidValue;
+  __half *yp = static_cast<__half *>(Ypl);
+  auto go = [&](auto kern, const auto *at, int rows, int nt) -> cudaError_t {
+    const int64_t blocks = (n + (int64_t)rows - 1) / rows;
+    if (blocks > 65535) return cudaErrorInvalidValue;   // grid y limit
+    kern<<<dim3((unsigned)r, (unsigned)blocks), nt, 0, st>>>(form, at, at_inv, ldat, n, sup_idx, sup_val, cap, s, U, ldu,
+                                                             gate, Y, yp, pstride, rank, X, ldX, p, cnt);
+    return cudaGetLastError();
+  };
+  const bool few = gather_few(AT16 != nullptr, r, n, sms);
+  if (AT16) {   // (256 threads: the order in which the y-step kernel adds ||u||^2)
+    const __half *a = static_cast<const __half *>(AT16);
+    return few ? go(k_gather_y<__half, 2, 32, 256, 1>, a, 512, 256) : go(k_gather_y<__half, 8, 8, 256, 1>, a, 2048, 256);
+  }
+  return few ? go(k_gather_y<float, 1, 32, 512, 8>, AT, 64, 512) : go(k_gather_y<float, 4, 8, 128, 1>, AT, 512, 128);
 }
 
 // ------------------------------------------------------------------ groups of problems

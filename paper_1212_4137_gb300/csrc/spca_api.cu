@@ -362,7 +362,7 @@ int sweep_u_rows(spca_handle *h, int r, const int *gate, const int *count, const
 // tensor-core engine packs the active starts (h->act, count *nact) into consecutive plane rows.
 // packed: the first sweep, whose planes the start initialisation wrote (row c = start c).
 int sweep_u_dense(spca_handle *h, int engine, int r, const int *gate, const int *nact, int nhost, bool lowp,
-                  const int *list = nullptr, bool packed = false) {
+                  const TcStreamK &sk, const int *list = nullptr, bool packed = false) {
   if (!list) list = h->act;
   if (h->sparse) return sweep_u_rows(h, r, gate, nact, list);
   const int n = (int)h->n, p = (int)h->p;
@@ -371,7 +371,7 @@ int sweep_u_dense(spca_handle *h, int engine, int r, const int *gate, const int 
     CK(timed(h, SPCA_K_U_DENSE, 1, [&] {
       return launch_gemm_tc(h->pmA, lowp ? 1 : 2, lowp ? h->tmX1 : h->tmX2, lowp ? 1 : 2, n, nhost, p, nullptr,
                             lowp ? pairs_hi() : pairs_general(), h->U, h->ldU, h->a_inv, h->x_inv, 1.0f, gate, nullptr,
-                            nullptr, h->dev_err, h->sk, st);
+                            nullptr, h->dev_err, sk, st);
     }));
   } else if (engine == SPCA_ENGINE_TC && lowp && f8_sweeps(h)) {
     // FP8 low-precision sweep: x in E4M3 with the planes' row scales times 2^-6
@@ -383,7 +383,7 @@ int sweep_u_dense(spca_handle *h, int engine, int r, const int *gate, const int 
       e = launch_scale_copy(h->x_inv, r, 1.0f / kF8Mul, h->x8_inv, gate, st);
       if (e != cudaSuccess) return e;
       return launch_gemm_tc_f8(h->pmA8, h->tmX8, n, nhost, p, nullptr, h->U, h->ldU, h->a8_inv, h->x8_inv, 1.0f,
-                               gate, nact, list, h->dev_err, h->sk, st);
+                               gate, nact, list, h->dev_err, sk, st);
     }));
   } else if (engine == SPCA_ENGINE_TC) {
     CK(timed(h, SPCA_K_U_DENSE, 3, [&] {
@@ -394,9 +394,9 @@ int sweep_u_dense(spca_handle *h, int engine, int r, const int *gate, const int 
       if (e != cudaSuccess) return e;
       if (lowp)
         return launch_gemm_tc(h->pmA, 1, h->tmX1, 1, n, nhost, p, nullptr, pairs_hi(), h->U, h->ldU, h->a_inv,
-                              h->x_inv, 1.0f, gate, nact, list, h->dev_err, h->sk, st);
+                              h->x_inv, 1.0f, gate, nact, list, h->dev_err, sk, st);
       return launch_gemm_tc(h->pmA, 2, h->tmX2, 2, n, nhost, p, nullptr, pairs_general(), h->U, h->ldU, h->a_inv,
-                            h->x_inv, 1.0f, gate, nact, list, h->dev_err, h->sk, st);
+                            h->x_inv, 1.0f, gate, nact, list, h->dev_err, sk, st);
     }));
   } else if (gemv_fits(r, p)) {
     CK(timed(h, SPCA_K_U_DENSE, 1, [&] {
@@ -413,7 +413,7 @@ int sweep_u_dense(spca_handle *h, int engine, int r, const int *gate, const int 
 
 // u = A x for every active row over the union S of the active supports, when the control word
 // c chose it (|S| <= h->kcap): compact FP16 operands, then the tensor-core contraction over |S|
-int sweep_u_union(spca_handle *h, StartState S, const Ctrl *c, int nhost) {
+int sweep_u_union(spca_handle *h, StartState S, const Ctrl *c, int nhost, const TcStreamK &sk) {
   const int n = (int)h->n, p = (int)h->p;
   CK(timed(h, SPCA_K_U_SPARSE, 3, [&] {
     cudaError_t e = launch_union_operands(h->AT32, h->ldAT, h->a_scale, n, h->collist, h->kcap, h->AS,
@@ -421,15 +421,16 @@ int sweep_u_union(spca_handle *h, StartState S, const Ctrl *c, int nhost) {
                                           h->colpos, h->XS, (int64_t)h->r_cap * h->kcap, c, h->stream);
     if (e != cudaSuccess) return e;
     return launch_gemm_tc(h->pmAS, 2, h->tmXS2, 2, n, nhost, h->kcap, &c->kunion, pairs_general(), h->U, h->ldU,
-                          h->a_inv, nullptr, kQInv, &c->use_union, &c->active, h->act, h->dev_err, h->sk,
+                          h->a_inv, nullptr, kQInv, &c->use_union, &c->active, h->act, h->dev_err, sk,
                           h->stream);
   }));
   return SPCA_OK;
 }
 
 // y-step and v = A^T y for every active row (tensor-core engine: packed active rows, see above)
-int sweep_y_v(spca_handle *h, int engine, int form, int r, StartState S, const int *nact, int nhost,
-              bool lowp = false) {
+// y_skip: the gather kernel writes the sweep's y when *y_skip != 0 (no_ystep: always, no launch here)
+int sweep_y_v(spca_handle *h, int engine, int form, int r, StartState S, const int *nact, int nhost, bool lowp,
+              const int *y_skip, bool no_ystep, const TcStreamK &sk) {
   const int n = (int)h->n, p = (int)h->p;
   cudaStream_t st = h->stream;
   const bool tc = engine == SPCA_ENGINE_TC;
@@ -440,7 +441,7 @@ int sweep_y_v(spca_handle *h, int engine, int form, int r, StartState S, const i
     const bool half = is_l1_var(form);
     CK(timed(h, SPCA_K_YSTEP, half ? 1 : 2, [&] {
       cudaError_t e = launch_ystep(form, h->U, h->ldU, n, r, h->Y, nullptr, 0, nullptr, S, h->X, h->ldX, p, h->ysum,
-                                   st);
+                                   nullptr, nullptr, 0, st);
       if (e != cudaSuccess || half) return e;
       return launch_pack_t(h->Y, h->ldU, n, h->act, nact, nullptr, r, h->Bt, h->ldb, st);
     }));
@@ -468,10 +469,12 @@ int sweep_y_v(spca_handle *h, int engine, int form, int r, StartState S, const i
   }
   // the FP8 low-precision sweep reads y as FP32 (converted to E4M3 below); the others read the planes
   const bool f8 = tc && lowp && f8_sweeps(h);
-  CK(timed(h, SPCA_K_YSTEP, 1, [&] {
-    return launch_ystep(form, h->U, h->ldU, n, r, tc && !f8 ? nullptr : h->Y, tc && !f8 ? h->Ypl : nullptr,
-                        ypstride, tc ? h->rank : nullptr, S, h->X, h->ldX, p, h->ysum, st);
-  }));
+  if (!no_ystep)
+    CK(timed(h, SPCA_K_YSTEP, 1, [&] {
+      return launch_ystep(form, h->U, h->ldU, n, r, tc && !f8 ? nullptr : h->Y, tc && !f8 ? h->Ypl : nullptr,
+                          ypstride, tc ? h->rank : nullptr, S, h->X, h->ldX, p, h->ysum, y_skip,
+                          sk.zeroed ? sk.flags : nullptr, 2 * sk.slots, st);
+    }));
   if (f8) {
     // FP8 low-precision sweep: y (written as FP32 by the y-step) in E4M3 at scale 2^7
     CK(timed(h, SPCA_K_V, 2, [&] {
@@ -479,19 +482,19 @@ int sweep_y_v(spca_handle *h, int engine, int form, int r, StartState S, const i
                                       st);
       if (e != cudaSuccess) return e;
       return launch_gemm_tc_f8(h->pmAT8, h->tmY8, p, nhost, n, nullptr, h->V, h->ldX, h->at8_inv, nullptr,
-                               1.0f / kF8QScale, nullptr, nact, h->act, h->dev_err, h->sk, st);
+                               1.0f / kF8QScale, nullptr, nact, h->act, h->dev_err, sk, st);
     }));
   } else if (tc && lowp) {
     CK(timed(h, SPCA_K_V, 1, [&] {
       return launch_gemm_tc(h->pmAT, 1, h->tmY1, 1, p, nhost, n, nullptr, pairs_hi(), h->V, h->ldX, h->at_inv,
-                            nullptr, kQInv, nullptr, nact, h->act, h->dev_err, h->sk, st);
+                            nullptr, kQInv, nullptr, nact, h->act, h->dev_err, sk, st);
     }));
   } else if (tc) {
     const bool l1 = is_l1_var(form);
     CK(timed(h, SPCA_K_V, 1, [&] {
       return launch_gemm_tc(h->pmAT, 2, l1 ? h->tmY1 : h->tmY2, l1 ? 1 : 2, p, nhost, n, nullptr,
                             l1 ? pairs_sign() : pairs_general(), h->V, h->ldX, h->at_inv, nullptr, kQInv, nullptr,
-                            nact, h->act, h->dev_err, h->sk, st);
+                            nact, h->act, h->dev_err, sk, st);
     }));
   } else if (gemv_fits(r, n)) {
     CK(timed(h, SPCA_K_V, 1, [&] {
@@ -1010,7 +1013,7 @@ int spca_xstep(spca_handle *h, int form, double s, double gamma, int calibrate, 
   RC(enter(h));
   CK(timed(h, SPCA_K_XSTEP, 2, [&] {
     return launch_xstep(a, V, ldv, r, X, ldx, st, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, true,
-                        h->stream);
+                        nullptr, 0, h->stream);
   }));
   CK(cudaStreamSynchronize(h->stream));
   return SPCA_OK;
@@ -1036,9 +1039,9 @@ int spca_products(spca_handle *h, int form, int engine, const float *X, int64_t 
   CK(cudaMemsetAsync(h->iters, 0, (size_t)r * sizeof(int), st));
   CK(cudaMemsetAsync(h->ctrl, 0, sizeof(Ctrl), st));
   CK(launch_active_list(h->status, nullptr, r, h->act, h->rank, &h->ctrl[0], nullptr, st));
-  RC(sweep_u_dense(h, eng, r, nullptr, &h->ctrl[0].active, r, lowp));
+  RC(sweep_u_dense(h, eng, r, nullptr, &h->ctrl[0].active, r, lowp, h->sk));
   RC(sweep_lowrank_u(h, r, &h->ctrl[0].active, h->act));
-  RC(sweep_y_v(h, eng, form, r, state_of(h), &h->ctrl[0].active, r, lowp));
+  RC(sweep_y_v(h, eng, form, r, state_of(h), &h->ctrl[0].active, r, lowp, nullptr, false, h->sk));
   CK(cudaMemcpy2DAsync(U, ldu * sizeof(float), h->U, h->ldU * sizeof(float), (size_t)n * sizeof(float), r,
                        cudaMemcpyDeviceToDevice, st));
   CK(cudaMemcpy2DAsync(V, ldv * sizeof(float), h->V, h->ldX * sizeof(float), (size_t)p * sizeof(float), r,
@@ -1108,6 +1111,11 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
     CK(cudaMemsetAsync(h->flag, 0, sizeof(int), st));
   }
   CK(cudaMemsetAsync(h->ctrl, 0, 2 * sizeof(Ctrl), st));   // (each sweep clears the word it read for the next one)
+  // the stream-K flags: zero here, and again after every contraction that may have used them (the y-step
+  // kernel clears them between a dense u = A x and v = A^T y, the x-step after v)
+  if (h->sk.flags) CK(cudaMemsetAsync(h->sk.flags, 0, (size_t)2 * h->sk.slots * sizeof(int), st));
+  TcStreamK sk = h->sk;
+  sk.zeroed = true;
   // the first sweep reads x^(0) as FP16 planes (tensor cores, but for an FP8 copy of A) or as FP32
   const bool packed = engine == SPCA_ENGINE_TC && !otf && !(F0 == 0 && L > 0 && f8_sweeps(h));
   std::vector<int> iota;
@@ -1203,34 +1211,41 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
     Ctrl *cur = h->ctrl + ((pl.k - 1) & 1), *nxt = h->ctrl + (pl.k & 1);
     // u = A x: over the union of the supports when it is small (tensor cores), else the dense
     // contraction, or the per-start support gather when every support is small
-    if (pl.dense_in) RC(sweep_u_dense(h, engine, r, &cur->need_dense, &cur->active, r, pl.lowp, nullptr, pl.packed));
+    if (pl.dense_in)
+      RC(sweep_u_dense(h, engine, r, &cur->need_dense, &cur->active, r, pl.lowp, sk, nullptr, pl.packed));
     // slots that took a new start in the last sweep have a dense x (the gather skips them)
-    if (otf) RC(sweep_u_dense(h, engine, r, &cur->n_new, &cur->n_new, r, false, h->new_slot));
-    if (pl.union_in) RC(sweep_u_union(h, S, cur, r));
+    // (this contraction clears its flags itself: the one above may have used them)
+    if (otf) RC(sweep_u_dense(h, engine, r, &cur->n_new, &cur->n_new, r, false, h->sk, h->new_slot));
+    if (pl.union_in) RC(sweep_u_union(h, S, cur, r, sk));
+    // the gather, with the y-step of the starts it serves (all active ones when it runs at all, but for
+    // on-the-fly replacement)
+    const bool f8 = pl.lowp && f8_sweeps(h), y_fused = !h->sparse && !otf && !f8 && ystep_with_gather(n) && gather_few(pl.lowp, r, n, h->sms);
     CK(timed(h, SPCA_K_U_SPARSE, 1, [&] {
       if (h->sparse)
         return launch_spmv_support(sp_cols(h), n, h->sup_idx, h->sup_val, p, S, r, h->U, h->ldU, &cur->use_gather,
                                    st);
-      if (pl.lowp && f8_sweeps(h))
+      if (f8)
         return launch_gemm1_sparse_f8(h->AT8, h->ldAT8, h->at8_inv, n, h->sup_idx, h->sup_val, p, S, r, h->U, h->ldU,
                                       &cur->use_gather, st);
-      if (pl.lowp)
-        return launch_gemm1_sparse_lowp(h->ATpl, h->ldAT, h->at_inv, n, h->sup_idx, h->sup_val, p, S, r, h->U, h->ldU,
-                                        &cur->use_gather, st);
-      return launch_gemm1_sparse(h->AT32, h->ldAT, n, h->sup_idx, h->sup_val, p, S, r, h->U, h->ldU,
-                                 &cur->use_gather, st);
+      const bool tc = engine == SPCA_ENGINE_TC;
+      return launch_gather_y(form, h->AT32, pl.lowp ? h->ATpl : nullptr, pl.lowp ? h->at_inv : nullptr, h->ldAT, n,
+                             h->sup_idx, h->sup_val, p, S, r, h->U, h->ldU, &cur->use_gather,
+                             y_fused && !tc ? h->Y : nullptr, y_fused && tc ? h->Ypl : nullptr,
+                             (int64_t)h->r_cap * h->ldU, tc ? h->rank : nullptr, h->X, h->ldX, p, h->fin_cnt, h->sms,
+                             st);
     }));
     // deflated sparse A: u -= W (Z^T x)
     RC(sweep_lowrank_u(h, r, &cur->active, h->act));
-    // y-step, v = A^T y
-    RC(sweep_y_v(h, engine, form, r, S, &cur->active, r, pl.lowp));
+    // y-step (where the gather did not do it), v = A^T y
+    RC(sweep_y_v(h, engine, form, r, S, &cur->active, r, pl.lowp, y_fused ? &cur->use_gather : nullptr,
+                 y_fused && !pl.dense_in && !pl.union_in, sk));
     XstepArgs xk = xa;
     xk.sparse_cap = pl.sparse_cap;
     // the x-step, and the active list of the next sweep (on-the-fly replacement makes it below, once
     // the stopped slots have their next starts)
     CK(timed(h, SPCA_K_XSTEP, pl.full ? (otf ? 2 : 3) : 1, [&] {
       return launch_xstep(xk, h->V, h->ldX, r, h->X, h->ldX, S, h->sup_idx, h->sup_val, nxt, cur,
-                          otf ? nullptr : h->act, h->rank, pl.full, st);
+                          otf ? nullptr : h->act, h->rank, pl.full, sk.flags, sk.flags ? 2 * sk.slots : 0, st);
     }));
     if (otf) {
       // stopped slots: archive their start, give them the next starts (Section 4.3)

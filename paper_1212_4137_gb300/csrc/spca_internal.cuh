@@ -279,28 +279,32 @@ cudaError_t launch_gemm_nt_f32(const float *P, int64_t ldp, const float *Q, int6
 int64_t gemm_few_floats(int sms);
 int gemm_few_tiles(int sms);
 
-// U[c, i] = sum_t val[c, t] AT[idx[c, t], i] for every active start; runs only when
-// *gate != 0 (the control word chose the per-start gather)
-cudaError_t launch_gemm1_sparse(const float *AT, int64_t ldat, int n, const int *sup_idx,
-                                const float *sup_val, int cap, StartState s, int r, float *U,
-                                int64_t ldu, const int *gate, cudaStream_t st);
-
-// the same over the leading FP16 plane of A^T (low-precision sweeps): row j of that plane holds
-// A[:, j] times at_scale[j], undone here with at_inv[j]
-cudaError_t launch_gemm1_sparse_lowp(const void *AT0, int64_t ldat, const float *at_inv, int n, const int *sup_idx,
-                                     const float *sup_val, int cap, StartState s, int r, float *U, int64_t ldu,
-                                     const int *gate, cudaStream_t st);
+// U[c, i] = sum_t val[c, t] AT[idx[c, t], i] for every active start that has been swept, and (Y or Ypl
+// given, as for launch_ystep) its y-step; runs only when *gate != 0 (the control word chose the
+// per-start gather).  AT16 (with at_inv): the leading FP16 plane of A^T instead, whose row j holds A[:, j]
+// times at_scale[j].  cnt: r ints, zero before and after.  gather_few: the variant for few starts is used,
+// in which the y-step belongs
+bool gather_few(bool half, int r, int64_t n, int sms);
+cudaError_t launch_gather_y(int form, const float *AT, const void *AT16, const float *at_inv, int64_t ldat, int n,
+                            const int *sup_idx, const float *sup_val, int cap, StartState s, int r, float *U,
+                            int64_t ldu, const int *gate, float *Y, void *Ypl, int64_t pstride, const int *rank,
+                            float *X, int64_t ldX, int p, int *cnt, int sms, cudaStream_t st);
 
 // y-step (S1 / S2 of Table 3) for active starts.  Writes Y as FP32 (Y != nullptr, row c) and/or
 // as tensor-core planes (Ypl != nullptr, row rank[c] when rank is given, else c; plane t at
 // Ypl + t * plane_stride): 1 plane of +-kQScale for L1 variance, the 2 planes of kQScale y for
 // L2 variance)
+// skip: nothing is written when *skip != 0 (the gather kernel has done the y-step); flags: nflags ints
+// set to 0 (the stream-K flags of the next contraction).
 // With ysum (r * ceil(n / kYChunk) floats of scratch) and n > 2 kYChunk, a CTA per chunk of
 // kYChunk entries and start (L2 variance: the chunks' sums of u_i^2 added in chunk order).
 constexpr int kYChunk = 8192;
+// long u, cut into chunks over several CTAs, keep their own y-step kernels
+inline bool ystep_with_gather(int64_t n) { return n <= 2 * kYChunk; }
 cudaError_t launch_ystep(int form, const float *U, int64_t ldu, int n, int r, float *Y,
                          void *Ypl, int64_t plane_stride, const int *rank, StartState s, float *X,
-                         int64_t ldX, int p, float *ysum, cudaStream_t st);
+                         int64_t ldX, int p, float *ysum, const int *skip, int *flags, int nflags,
+                         cudaStream_t st);
 
 // projection deflation A <- A (I - z z^T), z = x / ||x||_2, in place on the FP32 A (n x p, lda):
 // *inv = 1 / ||x||_2 (0 when x = 0: A is then left as is), w (n doubles) = A z
@@ -382,7 +386,7 @@ cudaError_t make_q_maps(QMaps *maps, const void *base, int64_t rows, int64_t ld,
 // a timed-out wait sets *err = SPCA_E_TIMEOUT
 // (K from *k_dev when k_dev != nullptr, K being then only an upper bound)
 // Stream-K scratch of the CTA-pair contraction: `slots` parts of tc_sk_floats_per_slot() floats
-// and 2 flags per slot (zeroed by every launch).  Without it (ws == nullptr) the single-CTA kernel
+// and 2 flags per slot (zeroed by every launch unless `zeroed`).  Without it (ws == nullptr) the single-CTA kernel
 // runs.
 // Every wait inside the contraction kernels gives up after wait_ns nanoseconds (SPCA_E_TIMEOUT in
 // *err); the owners of split tiles wait for parts flagged wait_epoch (parts are published as 1, so
@@ -395,6 +399,7 @@ struct TcStreamK {
   float *ws = nullptr;
   int *flags = nullptr;
   int slots = 0;
+  bool zeroed = false;          // the flags are zero already (a kernel before the launch clears them)
   uint64_t wait_ns = 2000000000ull;
   int wait_epoch = 1;
   int piece_kb = 40;
@@ -582,12 +587,13 @@ cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, int n
                                 float *U, float *Y, int64_t ldu, float *V, StartState s, int *sup_idx, float *sup_val,
                                 int r, int sweeps, cudaStream_t st);
 // x-step (S3..S6), objective F, stopping rule, support lists, and (act given) the next sweep's active
-// list in *ctrl, which must be zero before; ctrl_read is cleared (see launch_active_list).  defer: a
+// list in *ctrl, which must be zero before; ctrl_read is cleared (see launch_active_list), and so are the
+// nflags ints at flags (the stream-K flags of the next contraction; null: none).  defer: a
 // second kernel runs the full pass of the starts that need it, with v in shared memory (else the
 // first one does, from global memory)
 cudaError_t launch_xstep(XstepArgs a, const float *V, int64_t ldv, int r, float *X, int64_t ldx,
                          StartState s, int *sup_idx, float *sup_val, Ctrl *ctrl, Ctrl *ctrl_read, int *act,
-                         int *rank, bool defer, cudaStream_t st);
+                         int *rank, bool defer, int *flags, int nflags, cudaStream_t st);
 
 // a7: Table 1 objective in FP64 for every start, with u of each start into U, and the best start (of the
 // objective, or of the explained variance with use_ev); A^T in FP32, or (AT16 given) FP16 rows times their

@@ -162,6 +162,8 @@ static __device__ void start_pack_body(const float *x0, int64_t ld0, uint64_t ke
 // Counts the sweep for every active start; L1 variance: y = sgn(u) with sgn(0) = +1;
 // L2 variance: y = u / ||u||_2, and ||u||_2 = 0 ends the start as degenerate (x = 0).
 // y goes to Y (FP32) and/or to the FP16 planes of kQScale y (hi, lo; one exact plane for +-1).
+// (kCg: u was written by other CTAs of the same launch, and is read from L2)
+template <bool kCg = false>
 static __device__ void ystep_body(int form, const float *__restrict__ U, int64_t ldu, int n,
                                   float *__restrict__ Y, __half *__restrict__ Ypl, int64_t pstride,
                                   const int *__restrict__ rank, StartState s, float *__restrict__ X, int64_t ldX,
@@ -175,7 +177,7 @@ static __device__ void ystep_body(int form, const float *__restrict__ U, int64_t
   const int n4 = n & ~3;
   if (is_l1_var(form)) {
     for (int i = 4 * threadIdx.x; i < n4; i += 4 * blockDim.x) {
-      const float4 uv = *reinterpret_cast<const float4 *>(u + i);
+      const float4 uv = kCg ? __ldcg(reinterpret_cast<const float4 *>(u + i)) : *reinterpret_cast<const float4 *>(u + i);
       const float4 yv = make_float4(uv.x >= 0.0f ? 1.0f : -1.0f, uv.y >= 0.0f ? 1.0f : -1.0f,
                                     uv.z >= 0.0f ? 1.0f : -1.0f, uv.w >= 0.0f ? 1.0f : -1.0f);
       if (y) *reinterpret_cast<float4 *>(y + i) = yv;
@@ -187,7 +189,7 @@ static __device__ void ystep_body(int form, const float *__restrict__ U, int64_t
       }
     }
     for (int i = n4 + threadIdx.x; i < n; i += blockDim.x) {
-      const float yi = (u[i] >= 0.0f) ? 1.0f : -1.0f;
+      const float yi = ((kCg ? __ldcg(u + i) : u[i]) >= 0.0f) ? 1.0f : -1.0f;
       if (y) y[i] = yi;
       if (yp) yp[i] = __float2half_rn(yi * kQScale);
     }
@@ -195,13 +197,16 @@ static __device__ void ystep_body(int form, const float *__restrict__ U, int64_t
   }
   float part = 0.0f;
   for (int i = 4 * threadIdx.x; i < n4; i += 4 * blockDim.x) {
-    const float4 uv = *reinterpret_cast<const float4 *>(u + i);
+    const float4 uv = kCg ? __ldcg(reinterpret_cast<const float4 *>(u + i)) : *reinterpret_cast<const float4 *>(u + i);
     part = fmaf(uv.x, uv.x, part);
     part = fmaf(uv.y, uv.y, part);
     part = fmaf(uv.z, uv.z, part);
     part = fmaf(uv.w, uv.w, part);
   }
-  for (int i = n4 + threadIdx.x; i < n; i += blockDim.x) part = fmaf(u[i], u[i], part);
+  for (int i = n4 + threadIdx.x; i < n; i += blockDim.x) {
+    const float ui = kCg ? __ldcg(u + i) : u[i];
+    part = fmaf(ui, ui, part);
+  }
   const float sumsq = block_sum_f(part, redf);
   if (sumsq == 0.0f) {
     float *x = X + (int64_t)c * ldX;
@@ -222,7 +227,7 @@ static __device__ void ystep_body(int form, const float *__restrict__ U, int64_t
     lo = __float2half_rn(ys - __half2float(hi));
   };
   for (int i = 4 * threadIdx.x; i < n4; i += 4 * blockDim.x) {
-    const float4 uv = *reinterpret_cast<const float4 *>(u + i);
+    const float4 uv = kCg ? __ldcg(reinterpret_cast<const float4 *>(u + i)) : *reinterpret_cast<const float4 *>(u + i);
     const float4 yv = make_float4(uv.x * inv, uv.y * inv, uv.z * inv, uv.w * inv);
     if (y) *reinterpret_cast<float4 *>(y + i) = yv;
     if (yp) {
@@ -240,7 +245,7 @@ static __device__ void ystep_body(int form, const float *__restrict__ U, int64_t
     }
   }
   for (int i = n4 + threadIdx.x; i < n; i += blockDim.x) {
-    const float yi = u[i] * inv;
+    const float yi = (kCg ? __ldcg(u + i) : u[i]) * inv;
     if (y) y[i] = yi;
     if (yp) {
       __half hi, lo;
