@@ -108,12 +108,12 @@ cudaError_t dalloc(T **p, size_t count, size_t elem = sizeof(T)) {
 
 void free_workspace(spca_handle *h) {
   void *ptrs[] = {h->X, h->V, h->U, h->Y, h->Xpl, h->Ypl, h->sup_idx, h->sup_val, h->act, h->rank,
-                  h->status, h->iters, h->nnz, h->F, h->F_prev, h->gamma, h->f, h->ev, h->thr, h->tprev, h->xfast,
-                  h->partials, h->ctrl, h->best, h->y_out, h->x_out, h->support_out, h->nnz_out,
-                  h->mark, h->colpos, h->collist, h->AS, h->XS, h->x_scale, h->x_inv, h->Bt, h->sp_part, h->ysum,
+                  h->nnz, h->F_prev, h->thr, h->tprev, h->xfast, h->partials, h->ctrl, h->res_block, h->mark, h->colpos, h->collist, h->AS, h->XS, h->x_scale, h->x_inv, h->Bt, h->sp_part, h->ysum,
                   h->X8, h->Y8, h->x8_inv, h->fin_cnt, h->few_parts, h->few_cnt};
   for (void *q : ptrs)
     if (q) cudaFree(q);
+  if (h->h_res) cudaFreeHost(h->h_res);
+  h->res_block = h->h_res = nullptr;
   h->X8 = h->Y8 = nullptr;
   h->fin_cnt = h->few_cnt = nullptr;
   h->few_parts = nullptr;
@@ -140,6 +140,38 @@ void free_workspace(spca_handle *h) {
 constexpr int kUnionTry = 16;
 constexpr int64_t kUnionMinReads = int64_t(1) << 22;
 
+// the support's entries that come with a solve's one copy of results (more need a second one), and the
+// longest x and y together that do (longer ones are copied straight to the caller's arrays)
+constexpr int64_t kSupportFirst = 2048, kResStaged = int64_t(1) << 20;
+
+int ensure_results(spca_handle *h, int r) {
+  size_t o = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at = o;
+    o += (bytes + 15) / 16 * 16;
+    return at;
+  };
+  const size_t f = take(8 * (size_t)r), ev = take(8 * (size_t)r), gam = take(8 * (size_t)r), F = take(8 * (size_t)r);
+  const size_t nz = take(8), best = take(4), status = take(4 * (size_t)r), iters = take(4 * (size_t)r);
+  h->res_small = o;
+  const size_t y = take(4 * (size_t)h->ldU), x = take(4 * (size_t)h->ldX), sup = take(8 * (size_t)h->p);
+  h->res_copy = h->ldU + h->ldX <= kResStaged ? sup + 8 * (size_t)std::min(h->p, kSupportFirst) : h->res_small;
+  CK(dalloc(&h->res_block, o));
+  CK(cudaMallocHost((void **)&h->h_res, h->res_copy));
+  h->f = reinterpret_cast<double *>(h->res_block + f);
+  h->ev = reinterpret_cast<double *>(h->res_block + ev);
+  h->gamma = reinterpret_cast<double *>(h->res_block + gam);
+  h->F = reinterpret_cast<double *>(h->res_block + F);
+  h->nnz_out = reinterpret_cast<int64_t *>(h->res_block + nz);
+  h->best = reinterpret_cast<int *>(h->res_block + best);
+  h->status = reinterpret_cast<int *>(h->res_block + status);
+  h->iters = reinterpret_cast<int *>(h->res_block + iters);
+  h->y_out = reinterpret_cast<float *>(h->res_block + y);
+  h->x_out = reinterpret_cast<float *>(h->res_block + x);
+  h->support_out = reinterpret_cast<int64_t *>(h->res_block + sup);
+  return SPCA_OK;
+}
+
 int ensure_workspace(spca_handle *h, int r) {
   if (r <= h->r_cap) return SPCA_OK;
   release_graphs(h);   // they hold pointers into the workspace
@@ -156,17 +188,14 @@ int ensure_workspace(spca_handle *h, int r) {
   CK(dalloc(&h->sup_idx, (size_t)r * p));
   CK(dalloc(&h->sup_val, (size_t)r * p));
   CK(dalloc(&h->act, r)); CK(dalloc(&h->rank, r));
-  CK(dalloc(&h->status, r)); CK(dalloc(&h->iters, r)); CK(dalloc(&h->nnz, r));
-  CK(dalloc(&h->F, r)); CK(dalloc(&h->F_prev, r)); CK(dalloc(&h->gamma, r));
-  CK(dalloc(&h->f, r)); CK(dalloc(&h->ev, r)); CK(dalloc(&h->thr, r));
-  CK(dalloc(&h->tprev, r)); CK(dalloc(&h->xfast, r));
+  RC(ensure_results(h, r));
+  CK(dalloc(&h->nnz, r)); CK(dalloc(&h->F_prev, r));
+  CK(dalloc(&h->thr, r)); CK(dalloc(&h->tprev, r)); CK(dalloc(&h->xfast, r));
   CK(dalloc(&h->partials, (size_t)r * nchunks * 2));
   CK(dalloc(&h->fin_cnt, (size_t)r + 1));
   CK(cudaMemsetAsync(h->fin_cnt, 0, ((size_t)r + 1) * sizeof(int), h->stream));
   CK(dalloc(&h->ysum, (size_t)r * ((n + kYChunk - 1) / kYChunk)));
-  CK(dalloc(&h->ctrl, 2)); CK(dalloc(&h->best, 1));
-  CK(dalloc(&h->y_out, (size_t)h->ldU)); CK(dalloc(&h->x_out, (size_t)h->ldX));
-  CK(dalloc(&h->support_out, (size_t)p)); CK(dalloc(&h->nnz_out, 1));
+  CK(dalloc(&h->ctrl, 2));
   if (!h->sparse) {
     CK(dalloc(&h->few_parts, (size_t)gemm_few_floats(h->sms)));
     CK(dalloc(&h->few_cnt, (size_t)gemm_few_tiles(h->sms)));
@@ -509,9 +538,8 @@ int sweep_y_v(spca_handle *h, int engine, int form, int r, StartState S, const i
   return SPCA_OK;
 }
 
-int read_dev_err(spca_handle *h) {
-  CK(cudaMemcpyAsync(h->h_flag + 1, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
+// the error word, once its copy (to h_flag[1]) is known to have arrived
+int check_dev_err(spca_handle *h) {
   if (h->h_flag[1] != 0) {
     const int code = h->h_flag[1];
     h->h_flag[1] = 0;
@@ -519,6 +547,12 @@ int read_dev_err(spca_handle *h) {
     return fail(h, code, "a device-side wait timed out%s");
   }
   return SPCA_OK;
+}
+
+int read_dev_err(spca_handle *h) {
+  CK(cudaMemcpyAsync(h->h_flag + 1, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  CK(cudaStreamSynchronize(h->stream));
+  return check_dev_err(h);
 }
 
 // Projection deflation of a sparse A: A_k = A_{k-1} (I - z z^T) = A_{k-1} - w z^T with
@@ -719,7 +753,7 @@ void spca_destroy(spca_handle *h) {
   free_workspace(h);
   free_otf(h);
   // this handle's own buffers
-  void *own[] = {h->flag, h->dev_err, h->sk.ws, h->sk.flags, h->defl_x, h->defl_w, h->lr_coef};
+  void *own[] = {h->flag, h->sk.ws, h->sk.flags, h->defl_x, h->defl_w, h->lr_coef};
   for (void *q : own)
     if (q) cudaFree(q);
   // the matrix, with the last handle that holds it
@@ -781,8 +815,8 @@ int spca_create(spca_handle **out, const void *A, int64_t n, int64_t p, int64_t 
     CK(cudaMallocHost((void **)&h->h_ctrl, 2 * sizeof(Ctrl)));
     CK(cudaMallocHost((void **)&h->h_flag, 2 * sizeof(int)));
     h->h_flag[0] = h->h_flag[1] = 0;
-    CK(dalloc(&h->flag, 1));
-    CK(dalloc(&h->dev_err, 1));
+    CK(dalloc(&h->flag, 2));
+    h->dev_err = h->flag + 1;
     CK(cudaMemsetAsync(h->dev_err, 0, sizeof(int), h->stream));
     CK(dalloc(&h->A32, (size_t)n * h->ldA));
     CK(dalloc(&h->AT32, (size_t)p * h->ldAT));
@@ -875,8 +909,8 @@ int spca_create_csr(spca_handle **out, int64_t n, int64_t p, int64_t nnz, const 
     CK(cudaMallocHost((void **)&h->h_ctrl, 2 * sizeof(Ctrl)));
     CK(cudaMallocHost((void **)&h->h_flag, 2 * sizeof(int)));
     h->h_flag[0] = h->h_flag[1] = 0;
-    CK(dalloc(&h->flag, 1));
-    CK(dalloc(&h->dev_err, 1));
+    CK(dalloc(&h->flag, 2));
+    h->dev_err = h->flag + 1;
     CK(cudaMemsetAsync(h->dev_err, 0, sizeof(int), h->stream));
     // the input on the host (the canonical layouts are built there)
     std::vector<int64_t> hp;
@@ -978,8 +1012,8 @@ int spca_clone(spca_handle **out, spca_handle *src, void *cuda_stream) {
     CK(cudaMallocHost((void **)&h->h_ctrl, 2 * sizeof(Ctrl)));
     CK(cudaMallocHost((void **)&h->h_flag, 2 * sizeof(int)));
     h->h_flag[0] = h->h_flag[1] = 0;
-    CK(dalloc(&h->flag, 1));
-    CK(dalloc(&h->dev_err, 1));
+    CK(dalloc(&h->flag, 2));
+    h->dev_err = h->flag + 1;
     CK(cudaMemsetAsync(h->dev_err, 0, sizeof(int), h->stream));
     // no stream-K scratch: its schedule needs every CTA of a launch resident at once, which
     // launches of other handles running at the same time cannot guarantee; the contractions take
@@ -1154,13 +1188,13 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
                                &h->ctrl[0], st);
     }));
   }
-  if (x0) {
-    CK(cudaMemcpyAsync(h->h_flag, h->flag, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    if (*h->h_flag) return fail(h, SPCA_E_INVALID, "x0 has a non-finite entry%s");
-  } else if (otf) {
-    CK(cudaStreamSynchronize(st));   // iota and h_ctrl are reused
-  }
+  // x0's check comes back with the first read-back (a start that fails it never sweeps)
+  if (otf) CK(cudaStreamSynchronize(st));   // iota and h_ctrl are reused
+  auto read_flags = [&] { return cudaMemcpyAsync(h->h_flag, h->flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, st); };
+  auto check_flags = [&]() -> int {
+    if (x0 && h->h_flag[0]) return fail(h, SPCA_E_INVALID, "x0 has a non-finite entry%s");
+    return check_dev_err(h);
+  };
   int nhost = r;   // active starts as the host knows them (an upper bound)
 
   // ---- the sweeps (Algorithm 2)
@@ -1187,6 +1221,10 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
   // the host queues this many sweeps before it reads the active count back; every path decision
   // inside a sweep is taken on the device from the control word
   const int check_every = 4;
+  // with nothing to stop early for (no tolerance, no timeout), and no optional launch left to drop, a
+  // read-back has nothing to tell, so there are fewer (a read-back idles the GPU for 15-20 us)
+  const int check_rarely = 16;
+  const bool no_stop = P.tol < 0.0 && P.timeout_us == 0 && !otf;
   // the union of the active supports is built only while the sum of their sizes (read back
   // with the active count; dense before the first read) could let it fit the union operands
   int64_t sum_nnz = (int64_t)nhost * p;
@@ -1196,7 +1234,7 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
   // sparse_cap (T_s keeps at most s entries; otherwise read back with the active count), and the
   // x-step of the sweep before requests it only then
   const int sparse_cap = xa.sparse_cap;
-  int64_t max_nnz = uses_T(form) ? std::min<int64_t>((int64_t)P.s, p) : p;
+  int64_t max_nnz = uses_T(form) || target ? std::min<int64_t>((int64_t)P.s, p) : p;
   bool dense_queued = true;   // x^(0) is dense
   // the full x-step is a kernel of its own (v in shared memory) while some start may need it; else
   // such a start takes it inside the x-step kernel, and the launch is saved.  Before the first
@@ -1319,7 +1357,9 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
     }
   }
   for (int k0 = 1; k0 <= max_total && rc == SPCA_OK && !small;) {
-    const int k1 = std::min(max_total, (k0 + check_every - 1) / check_every * check_every);
+    // the first read-back comes early: after it the launches that dense x^(0) needed are dropped
+    const int seg = k0 == 1 ? 2 : no_stop && !dense_queued && !full_queued ? check_rarely : check_every;
+    const int k1 = std::min(max_total, k0 - 1 + seg);
     plans.clear();
     key = solve_key;
     key.insert(key.end(), {k0 & 1, k1 - k0});
@@ -1374,11 +1414,13 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
     }
     for (int q = 0; q < SPCA_K_COUNT; ++q) h->launches[q] += g->counts[q];
     Ctrl *last = h->ctrl + (k1 & 1);
+    if (k1 == max_total && g->timings.empty() && P.timeout_us == 0) break;   // the results' copy waits for them
     if (cudaMemcpyAsync(h->h_ctrl, last, sizeof(Ctrl), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess) {
+        read_flags() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) {
       rc = fail(h, SPCA_E_CUDA, "CUDA error: %s", cudaGetErrorString(cudaGetLastError()));
       break;
     }
+    if ((rc = check_flags()) != SPCA_OK) break;
     for (auto &t : g->timings) {
       float ms = 0.0f;
       cudaEventElapsedTime(&ms, std::get<1>(t), std::get<2>(t));
@@ -1398,7 +1440,6 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
     k0 = k1 + 1;
   }
   RC(rc);
-  RC(read_dev_err(h));
 
   // ---- a7: FP64-class objective, best start, y(x) and support of the best x
   if (h->sparse) {
@@ -1460,31 +1501,49 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
 
   // ---- results to the host (the archive of all l starts with on-the-fly replacement)
   const int nres = l;
-  const int *d_status = otf ? h->arc.status : h->status, *d_iters = otf ? h->arc.iters : h->iters;
-  const double *d_f = otf ? h->arc.f : h->f, *d_ev = otf ? h->arc.ev : h->ev;
-  const double *d_gam = otf ? h->arc.gamma : h->gamma, *d_F = otf ? h->arc.F : h->F;
   const float *d_x = otf ? h->arc.x : h->X;
-  std::vector<int> status(nres), iters(nres);
-  std::vector<double> f(nres), ev(nres), gam(nres), F(nres);
-  int best = 0;
-  int64_t nnz = 0;
-  CK(cudaMemcpyAsync(status.data(), d_status, nres * sizeof(int), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(iters.data(), d_iters, nres * sizeof(int), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(f.data(), d_f, nres * sizeof(double), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(ev.data(), d_ev, nres * sizeof(double), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(gam.data(), d_gam, nres * sizeof(double), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(F.data(), d_F, nres * sizeof(double), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(&best, h->best, sizeof(int), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(&nnz, h->nnz_out, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+  CK(read_flags());
+  CK(cudaMemcpyAsync(h->h_res, h->res_block, h->res_copy, cudaMemcpyDeviceToHost, st));
+  std::vector<int> otf_int(otf ? 2 * (size_t)nres : 0);
+  std::vector<double> otf_dbl(otf ? 4 * (size_t)nres : 0);
+  if (otf) {
+    const int *src_i[] = {h->arc.status, h->arc.iters};
+    const double *src_d[] = {h->arc.f, h->arc.ev, h->arc.gamma, h->arc.F};
+    for (int q = 0; q < 2; ++q)
+      CK(cudaMemcpyAsync(&otf_int[(size_t)q * nres], src_i[q], nres * sizeof(int), cudaMemcpyDeviceToHost, st));
+    for (int q = 0; q < 4; ++q)
+      CK(cudaMemcpyAsync(&otf_dbl[(size_t)q * nres], src_d[q], nres * sizeof(double), cudaMemcpyDeviceToHost, st));
+  }
   CK(cudaStreamSynchronize(st));
-  if (res->x) CK(cudaMemcpyAsync(res->x, h->x_out, (size_t)p * sizeof(float), cudaMemcpyDeviceToHost, st));
-  if (res->y) CK(cudaMemcpyAsync(res->y, h->y_out, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost, st));
-  if (res->support && nnz > 0)
-    CK(cudaMemcpyAsync(res->support, h->support_out, (size_t)nnz * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+  RC(check_flags());
+  auto host = [&](const auto *dev) {   // where the copy put *dev
+    return reinterpret_cast<decltype(dev)>(h->h_res + (reinterpret_cast<const char *>(dev) - h->res_block));
+  };
+  const int *status = otf ? otf_int.data() : host(h->status), *iters = otf ? &otf_int[nres] : host(h->iters);
+  const double *f = otf ? &otf_dbl[0] : host(h->f), *ev = otf ? &otf_dbl[nres] : host(h->ev);
+  const double *gam = otf ? &otf_dbl[2 * (size_t)nres] : host(h->gamma), *F = otf ? &otf_dbl[3 * (size_t)nres] : host(h->F);
+  const int best = *host(h->best);
+  const int64_t nnz = *host(h->nnz_out);
+  if (h->res_copy > h->res_small) {
+    const int64_t first = std::min(nnz, kSupportFirst);
+    if (res->x) memcpy(res->x, host(h->x_out), (size_t)p * sizeof(float));
+    if (res->y) memcpy(res->y, host(h->y_out), (size_t)n * sizeof(float));
+    if (res->support) {
+      memcpy(res->support, host(h->support_out), (size_t)first * sizeof(int64_t));
+      if (nnz > first)
+        CK(cudaMemcpyAsync(res->support + first, h->support_out + first, (size_t)(nnz - first) * sizeof(int64_t),
+                           cudaMemcpyDeviceToHost, st));
+    }
+  } else {
+    if (res->x) CK(cudaMemcpyAsync(res->x, h->x_out, (size_t)p * sizeof(float), cudaMemcpyDeviceToHost, st));
+    if (res->y) CK(cudaMemcpyAsync(res->y, h->y_out, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost, st));
+    if (res->support && nnz > 0)
+      CK(cudaMemcpyAsync(res->support, h->support_out, (size_t)nnz * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+  }
   if (res->start_x)
     CK(cudaMemcpy2DAsync(res->start_x, (size_t)p * sizeof(float), d_x, h->ldX * sizeof(float),
                          (size_t)p * sizeof(float), nres, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
+  if (res->start_x || h->res_copy == h->res_small || nnz > kSupportFirst) CK(cudaStreamSynchronize(st));
 
   int64_t sweeps = 0;
   int nconv = 0, ndeg = 0;
@@ -1503,11 +1562,11 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
   res->degenerate = ndeg;
   res->sweeps_total = sweeps;
   res->nnz = nnz;
-  if (res->start_objective) memcpy(res->start_objective, f.data(), nres * sizeof(double));
-  if (res->start_explained) memcpy(res->start_explained, ev.data(), nres * sizeof(double));
-  if (res->start_F) memcpy(res->start_F, F.data(), nres * sizeof(double));
-  if (res->start_iters) memcpy(res->start_iters, iters.data(), nres * sizeof(int));
-  if (res->start_status) memcpy(res->start_status, status.data(), nres * sizeof(int));
+  if (res->start_objective) memcpy(res->start_objective, f, nres * sizeof(double));
+  if (res->start_explained) memcpy(res->start_explained, ev, nres * sizeof(double));
+  if (res->start_F) memcpy(res->start_F, F, nres * sizeof(double));
+  if (res->start_iters) memcpy(res->start_iters, iters, nres * sizeof(int));
+  if (res->start_status) memcpy(res->start_status, status, nres * sizeof(int));
   if (res->start_gamma) {
     for (int c = 0; c < nres; ++c) res->start_gamma[c] = is_pen(form) ? gam[c] : 0.0;
   }

@@ -109,8 +109,13 @@ struct spca_handle {
   int *best = nullptr;
   float *y_out = nullptr, *x_out = nullptr;
   int64_t *support_out = nullptr, *nnz_out = nullptr;
-  int *flag = nullptr;        // device scratch flag
-  int *dev_err = nullptr;     // device error word written by kernels (SPCA_E_TIMEOUT)
+  int *flag = nullptr;        // device scratch flag, and behind it
+  int *dev_err = nullptr;     // the error word written by kernels (SPCA_E_TIMEOUT)
+  // what a solve returns, in one block so that one copy brings it to the host: f, ev, gamma, F, nnz_out, best,
+  // status, iters (the first res_small bytes), y_out, x_out and the support (res_copy: with its first
+  // kSupportFirst entries); h_res: its pinned mirror
+  char *res_block = nullptr, *h_res = nullptr;
+  size_t res_small = 0, res_copy = 0;
   // on-the-fly replacement (grown on demand): the archive of the starts' results, the slots'
   // starts, the next start, the stopped / refilled slot lists, and a device copy of host x0
   int otf_l = 0, otf_r = 0;
@@ -124,7 +129,7 @@ struct spca_handle {
   // stream-K scratch of the CTA-pair contraction (one part per resident pair, flags)
   TcStreamK sk;
   Ctrl *h_ctrl = nullptr;     // pinned host mirror
-  int *h_flag = nullptr;      // pinned host mirror (2 ints)
+  int *h_flag = nullptr;      // pinned host mirror of flag and dev_err
 
   // measurement hooks: launch counts, and event pairs per kernel id while profiling is on
   unsigned prof_mask = 0u;   // bit k: kernel id k is timed
