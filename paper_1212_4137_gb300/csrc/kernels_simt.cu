@@ -775,12 +775,12 @@ __global__ void __launch_bounds__(NT) k_gather_y(int form, const T *__restrict__
   if (last) ystep_body<true>(form, U, ldu, n, Y, Ypl, pstride, rank, s, X, ldX, p, c, redf);
 }
 
-// The variants for few starts serve where the wide vectors' CTAs are fewer than two per SM (below that the
-// chip is idle between round trips), while the narrow ones' row blocks fit the grid: measured above on
-// both sides
+// The few-start variants serve while their CTAs are at most 8 per SM (256 threads of one row; FP16: 3, two
+// rows): gather and y-step of n = 2000, 10 columns, in event times: 8 starts 12.7 us (wide vectors and the
+// y-step of its own 16.5), 40 starts (1280 CTAs) 15.8 (17.4), 100 starts 24 (18); FP16: 100 starts (400 CTAs)
+// 14.6 (16.3), 200 starts 18.6 (16.9).
 bool gather_few(bool half, int r, int64_t n, int sms) {
-  return half ? r * ((n + 2047) / 2048) < 2 * sms && n <= (int64_t)65535 * 512
-              : r * ((n + 511) / 512) < 2 * sms && n <= (int64_t)65535 * 64;
+  return half ? r * ((n + 511) / 512) <= 3 * sms : r * ((n + 63) / 64) <= 8 * sms;
 }
 
 cudaError_t launch_gather_y(int form, const float *AT, const void *AT16, const float *at_inv, int64_t ldat, int n,
@@ -802,7 +802,7 @@ cudaError_t launch_gather_y(int form, const float *AT, const void *AT16, const f
     const __half *a = static_cast<const __half *>(AT16);
     return few ? go(k_gather_y<__half, 2, 32, 256, 1>, a, 512, 256) : go(k_gather_y<__half, 8, 8, 256, 1>, a, 2048, 256);
   }
-  return few ? go(k_gather_y<float, 1, 32, 512, 8>, AT, 64, 512) : go(k_gather_y<float, 4, 8, 128, 1>, AT, 512, 128);
+  return few ? go(k_gather_y<float, 1, 16, 256, 4>, AT, 64, 256) : go(k_gather_y<float, 4, 8, 128, 1>, AT, 512, 128);
 }
 
 // ------------------------------------------------------------------ groups of problems
