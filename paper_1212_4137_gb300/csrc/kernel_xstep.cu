@@ -378,7 +378,7 @@ __device__ void xstep_finish(const XstepArgs &a, int c, const float *vv, int len
       }
       const float w = (i < sg.hi) ? wval(vi, key, tie_keep) : 0.0f;
       const float xi = w * inv;
-      if (i < sg.hi) x[i] = xi;
+      if (x && i < sg.hi) x[i] = xi;
       const unsigned nzb = __ballot_sync(0xffffffffu, xi != 0.0f);
       if (gi && xi != 0.0f) {
         const int q = pos + __popc(nzb & lt_mask);
@@ -426,7 +426,7 @@ __device__ void xstep_full_one(const XstepArgs &a_in, int c, const float *__rest
   const int p = a.p;
   const int lane = threadIdx.x & 31;
   const float *vg = V + (int64_t)c * ldv;
-  float *x = X + (int64_t)c * ldx;
+  float *x = X ? X + (int64_t)c * ldx : nullptr;   // (null: the support list is all that is wanted)
   const int form = a.form;
   if (kSmem) {
     for (int i = threadIdx.x; i < p; i += blockDim.x) vsm[i] = vg[i];
@@ -915,7 +915,7 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
   const int p = a.p, form = a.form, s_int = (int)a.s;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const Row row = row_of(V + (int64_t)c * ldv, p);
-  float *x = X + (int64_t)c * ldx;
+  float *x = X ? X + (int64_t)c * ldx : nullptr;   // (null: the support list is all that is wanted)
   const unsigned lt_mask = (1u << lane) - 1u;
   const bool lam_form = uses_lam(form), exact = is_pen(form) && !a.calibrate;
   const bool keep_all = uses_T(form) && s_int >= p;
@@ -930,7 +930,8 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
   const bool steady = q0.xfast == 1;
   // x is zero outside the last support list, once there is one (before: all of x is written)
   const bool listed = sup_idx && q0.iters > 1 && q0.nnz <= a.cap;
-  if (listed) {
+  if (!x) {
+  } else if (listed) {
     const int nnz_old = q0.nnz;
     const int *old = sup_idx + (int64_t)c * a.cap;
     for (int t = threadIdx.x; t < nnz_old; t += T) x[old[t]] = 0.0f;
@@ -1142,7 +1143,7 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
   for (int t = threadIdx.x; t < nnz; t += T) {
     const int i = fs.a.s.idx[t];
     const float xi = fs.a.s.val[t] * inv;
-    x[i] = xi;
+    if (x) x[i] = xi;
     if (gi && t < a.cap) {
       gi[t] = i;
       gv[t] = xi;
@@ -1315,82 +1316,246 @@ cudaError_t launch_g_xstep(const GProb *P, const int *prob, int R, int max_p, in
 }
 
 // ---------------------------------------------------------------- small problems in one launch
-// For a small matrix the chain of launches of a sweep, not its work, sets the time.  Here every
-// sweep of a start runs in one CTA, all starts at once (a CTA per start): u = A x as a warp per
-// row of A, v = A^T y as a thread per column of A (both on the CUDA cores, sums in a fixed order;
-// A stays in L2 across the sweeps), then the y-step and the threshold x-step of the
-// single-problem path, until the start stops or `sweeps` sweeps have run.  x and y are staged in
-// shared memory (which the x-step then uses for its lists); v too where the full pass is needed.
-__global__ void __launch_bounds__(XT) k_small_sweeps(XstepArgs xa, const float *__restrict__ A, int64_t lda, int n,
-                                                     int p, float *__restrict__ X, int64_t ldx, float *__restrict__ U,
-                                                     float *__restrict__ Y, int64_t ldu, float *__restrict__ V,
-                                                     StartState st, int *__restrict__ sup_idx,
-                                                     float *__restrict__ sup_val, int sweeps) {
+// For a small matrix the chain of launches of a sweep, not its work, sets the time.  Here every sweep of
+// every start runs in one launch, a cluster of C CTAs per start, until the start stops or `sweeps` sweeps
+// have run: u = A x over the support's rows of A^T, the y-step, v = A^T y over the CTA's share of A's
+// columns (in its shared memory where they fit), v's pieces to every CTA of the cluster, the threshold
+// x-step.  u, y, v, the support list and the start's state live in shared memory, in every CTA alike: the
+// CTAs of a cluster repeat the same steps on the same v and so decide alike, and meet once a sweep.
+// What bounds a sweep is its chain of dependent steps (a round trip to L2 for u, then about 15 barriers).
+// 16 starts, n = 100, p = 500, 40 sweeps: 535 -> 235 us; n = 250, p = 1000, 20 sweeps 1250 -> 240 us
+// (one CTA per start, u by whole rows of A, u, y and v through memory before).
+
+// for every o < out: put(o, sum over k of w[k] M[row(k) ld + o]), row(k) = idx[k] or k: a thread per four
+// outputs and slice of the k (part: 4 T floats for the slices' sums)
+template <int T, typename Put>
+__device__ __forceinline__ void small_product(const float *M, int64_t ld, const int *idx, const float *w, int K,
+                                              int out, float *part, const Put &put) {
+  constexpr int L = 8;
+  const int quads = (out + 3) / 4, width = (quads + 7) / 8 * 8;
+  const int S = width >= T ? 1 : min(min(32, K), T / width);   // (K >= 1)
+  const int slice = S == 1 ? 0 : (int)threadIdx.x / width, q0 = S == 1 ? (int)threadIdx.x : (int)threadIdx.x % width;
+  for (int q = q0; q < quads && slice < S; q += T) {
+    const float *m = M + 4 * q;
+    float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    auto load = [&](int k) { return *reinterpret_cast<const float4 *>(m + (int64_t)(idx ? idx[k] : k) * ld); };
+    auto add = [&](float x, float4 a) {
+      acc.x = fmaf(x, a.x, acc.x); acc.y = fmaf(x, a.y, acc.y);
+      acc.z = fmaf(x, a.z, acc.z); acc.w = fmaf(x, a.w, acc.w);
+    };
+    float4 a[L];
+    int k = slice;
+    for (; k + (L - 1) * S < K; k += L * S) {
+#pragma unroll
+      for (int h = 0; h < L; ++h) a[h] = load(k + h * S);
+#pragma unroll
+      for (int h = 0; h < L; ++h) add(w[k + h * S], a[h]);
+    }
+    if (k < K) {
+#pragma unroll
+      for (int h = 0; h < L; ++h)
+        if (k + h * S < K) a[h] = load(k + h * S);
+#pragma unroll
+      for (int h = 0; h < L; ++h)
+        if (k + h * S < K) add(w[k + h * S], a[h]);
+    }
+    if (S == 1) {
+      put(4 * q, acc.x);
+      if (4 * q + 1 < out) put(4 * q + 1, acc.y);
+      if (4 * q + 2 < out) put(4 * q + 2, acc.z);
+      if (4 * q + 3 < out) put(4 * q + 3, acc.w);
+    } else {
+      reinterpret_cast<float4 *>(part)[slice * width + q] = acc;
+    }
+  }
+  if (S == 1) return;
+  __syncthreads();
+  for (int o = threadIdx.x; o < out; o += T) {
+    float t = part[o];
+#pragma unroll 4
+    for (int h = 1; h < S; ++h) t += part[h * 4 * width + o];
+    put(o, t);
+  }
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// a float to shared-memory address `addr` of the cluster's CTA `rank`
+__device__ __forceinline__ void store_cluster(uint32_t addr, int rank, float v) {
+  asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, %1;\n\tst.shared::cluster.f32 [a], %2;\n\t}"
+               ::"r"(addr), "r"(rank), "f"(v) : "memory");
+}
+
+// a start's state in shared memory, addressed as StartState with c = 0
+struct SmallState {
+  double F, F_prev, gamma;
+  float thr, tprev;
+  int status, iters, nnz, xfast;
+};
+__device__ __forceinline__ StartState small_state(SmallState &s) {
+  StartState t{};
+  t.status = &s.status; t.iters = &s.iters; t.nnz = &s.nnz; t.xfast = &s.xfast;
+  t.F = &s.F; t.F_prev = &s.F_prev; t.gamma = &s.gamma;
+  t.thr = &s.thr; t.tprev = &s.tprev;
+  return t;
+}
+
+// the CTA's columns of v = A^T y (all but the last CTAs the same number, a multiple of 4)
+__host__ __device__ inline int small_cols(int p, int ctas) { return ((p + ctas - 1) / ctas + 3) / 4 * 4; }
+// shared memory in floats: v (two buffers when the pieces come from several CTAs), the support's indices
+// and values, and u (n) with the slices' sums, or the x-step's lists in their place; then A's columns
+template <int T>
+__host__ __device__ inline int64_t small_words(int64_t n, int64_t p, int ctas) {
+  const int64_t p4 = (p + 3) & ~int64_t(3), n4 = (n + 3) & ~int64_t(3);
+  const int64_t a = n4 + 4 * T, b = (sizeof(FastShared<T>) + 15) / 16 * 4;
+  return (ctas > 1 ? 4 : 3) * p4 + (a > b ? a : b);
+}
+
+template <int T>
+__global__ void __launch_bounds__(T) k_small_sweeps(XstepArgs xa, const float *__restrict__ A, int64_t lda,
+                                                    const float *__restrict__ AT, int64_t ldat, int n, int p,
+                                                    int ctas, int a_smem, float *__restrict__ X, int64_t ldx,
+                                                    StartState st, int *__restrict__ sup_idx,
+                                                    float *__restrict__ sup_val, int sweeps) {
   extern __shared__ float4 sm4[];
-  float *sm = reinterpret_cast<float *>(sm4);
-  FastShared<XT> &fs = *reinterpret_cast<FastShared<XT> *>(sm4);   // in the x-step, where x and y are not needed
   __shared__ float redf[32];
-  const int c = blockIdx.x;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __shared__ SmallState ss;
+  const int c = blockIdx.x / ctas, rank = blockIdx.x % ctas;
   const int p4 = (p + 3) & ~3, n4 = (n + 3) & ~3;
-  float *xs = sm;              // x (p), then y (n) in the same place
-  float *vsm = sm + max(max(p4, n4), (int)((sizeof(FastShared<XT>) + 15) / 16 * 4));   // v, for the full pass
-  const float *x = X + (int64_t)c * ldx;
-  float *u = U + (int64_t)c * ldu;
-  const float *y = Y + (int64_t)c * ldu;
-  float *v = V + (int64_t)c * ldx;
+  float *vb = reinterpret_cast<float *>(sm4);
+  float *lv = vb + (ctas > 1 ? 2 : 1) * p4;
+  int *li = reinterpret_cast<int *>(lv + p4);
+  float *u = lv + 2 * p4, *part = u + n4;
+  FastShared<T> &fs = *reinterpret_cast<FastShared<T> *>(u);
+  float *as = vb + small_words<T>(n, p, ctas);
+  const int pc = small_cols(p, ctas), j0 = rank * pc, mine = max(0, min(pc, p - j0));
+  float *x = X + (int64_t)c * ldx;
+  // x^(0), the start's state, this CTA's columns of A
+  for (int j = threadIdx.x; j < p; j += T) {
+    lv[j] = x[j];
+    li[j] = j;
+  }
+  if (a_smem) {
+    for (int q = threadIdx.x; q < n * (pc / 4); q += T) {
+      const int i = q / (pc / 4), h = 4 * (q % (pc / 4));
+      if (h < mine) *reinterpret_cast<float4 *>(as + (int64_t)i * pc + h) =
+          *reinterpret_cast<const float4 *>(A + (int64_t)i * lda + j0 + h);   // (rows are padded to a multiple of 8)
+    }
+  }
+  if (threadIdx.x == 0) {
+    ss.status = st.status[c]; ss.iters = st.iters[c]; ss.nnz = p; ss.xfast = st.xfast[c];
+    ss.F = st.F[c]; ss.F_prev = st.F_prev[c]; ss.gamma = st.gamma[c];
+    ss.thr = st.thr[c]; ss.tprev = st.tprev[c];
+  }
+  StartState sl = small_state(ss);
+  const uint32_t vaddr = (uint32_t)__cvta_generic_to_shared(vb);
+  if (ctas > 1) cluster_barrier();   // (every CTA has started and read its state)
+  else __syncthreads();
+  if (ss.status != ST_ACTIVE) return;   // (the same in every CTA of the cluster)
   for (int k = 0; k < sweeps; ++k) {
-    __syncthreads();   // (the status and x written by the last x-step)
-    if (st.status[c] != ST_ACTIVE) break;
-    for (int j = threadIdx.x; j < p; j += XT) xs[j] = x[j];
+    float *v = vb + (ctas > 1 && (k & 1) ? p4 : 0);
+    small_product<T>(AT, ldat, k == 0 ? nullptr : li, lv, ss.nnz, n, part, [&](int i, float t) { u[i] = t; });
     __syncthreads();
-    for (int i = warp; i < n; i += XW) {   // u = A x
-      const float *a = A + (int64_t)i * lda;
-      float acc = 0.0f;
-      for (int j = lane; j < p; j += 32) acc = fmaf(a[j], xs[j], acc);
-      acc = warp_sum_f(acc);
-      if (lane == 0) u[i] = acc;
+    // y-step
+    if (threadIdx.x == 0) ss.iters += 1;
+    if (is_l1_var(xa.form)) {
+      for (int i = threadIdx.x; i < n; i += T) u[i] = u[i] >= 0.0f ? 1.0f : -1.0f;
+    } else {
+      float sq = 0.0f;
+      for (int i = threadIdx.x; i < n; i += T) sq = fmaf(u[i], u[i], sq);
+      const float sumsq = block_sum_f(sq, redf);
+      if (sumsq == 0.0f) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+          ss.status = SPCA_ST_DEGENERATE;
+          ss.nnz = 0;
+          ss.F = 0.0;
+        }
+        __syncthreads();
+        break;
+      }
+      float hi, lo, inv;
+      norm_and_inverse(sumsq, &hi, &lo, &inv);
+      for (int i = threadIdx.x; i < n; i += T) u[i] *= inv;
     }
     __syncthreads();
-    ystep_body(xa.form, U, ldu, n, Y, nullptr, 0, nullptr, st, X, ldx, p, c, redf);
-    __syncthreads();
-    if (st.status[c] != ST_ACTIVE) break;   // u = 0 under L2 variance: degenerate
-    for (int i = threadIdx.x; i < n; i += XT) xs[i] = y[i];
-    __syncthreads();
-    for (int j = threadIdx.x; j < p; j += XT) {   // v = A^T y, a column of A per thread
-      float acc = 0.0f;
-      for (int i = 0; i < n; ++i) acc = fmaf(A[(int64_t)i * lda + j], xs[i], acc);
-      v[j] = acc;
+    // v = A^T y, to every CTA
+    if (mine > 0) {
+      const int at = (int)(v - vb) + j0;
+      small_product<T>(a_smem ? as : A + j0, a_smem ? pc : lda, nullptr, u, n, mine, part, [&](int o, float t) {
+        if (ctas == 1) v[o] = t;
+        else
+          for (int h = 0; h < ctas; ++h) store_cluster(vaddr + 4u * (uint32_t)(at + o), h, t);
+      });
     }
-    __syncthreads();
-    if (!xstep_fast_one<XT>(xa, c, V, ldx, X, ldx, st, load_state(st, c), sup_idx, sup_val, nullptr, fs)) {
+    if (ctas > 1) cluster_barrier();
+    else __syncthreads();
+    if (!xstep_fast_one<T>(xa, 0, v, 0, nullptr, 0, sl, load_state(sl, 0), li, lv, nullptr, fs)) {
       __syncthreads();
-      xstep_full_one(xa, c, V, ldx, X, ldx, st, sup_idx, sup_val, nullptr, vsm, fs.sh);
-      if (threadIdx.x == 0) st.xfast[c] = 2;
+      xstep_full_one(xa, 0, v, 0, nullptr, 0, sl, li, lv, nullptr, nullptr, fs.sh);
+      if (threadIdx.x == 0) ss.xfast = 2;
     }
+    __syncthreads();
+    if (ss.status != ST_ACTIVE) break;
+  }
+  if (rank != 0) return;
+  // the results: x, its support list, the state
+  const int nnz = ss.nnz;
+  for (int j = threadIdx.x; j < p; j += T) x[j] = 0.0f;
+  __syncthreads();
+  for (int t = threadIdx.x; t < nnz; t += T) {
+    x[li[t]] = lv[t];
+    sup_idx[(int64_t)c * p + t] = li[t];
+    sup_val[(int64_t)c * p + t] = lv[t];
+  }
+  if (threadIdx.x == 0) {
+    st.status[c] = ss.status; st.iters[c] = ss.iters; st.nnz[c] = nnz; st.xfast[c] = ss.xfast;
+    st.F[c] = ss.F; st.F_prev[c] = ss.F_prev; st.gamma[c] = ss.gamma;
+    st.thr[c] = ss.thr; st.tprev[c] = ss.tprev;
   }
 }
 
 // (measured on GB300: with one CTA per start, a start's sweep costs about as much as the launch
 // chain it replaces at n p ~ 4e5, so mid-sized matrices take this path only with enough starts
 // to fill the device)
+constexpr int kSmallT = 256, kSmallCtas = 8;
 bool small_sweeps_fit(int64_t n, int64_t p, int r) {
-  const int64_t words = ((std::max(n, p) + 3) & ~int64_t(3)) + ((p + 3) & ~int64_t(3));
-  if (words * 4 > (int64_t)XSTEP_SMEM_MAX) return false;
+  if (small_words<kSmallT>(n, p, kSmallCtas) * 4 > (int64_t)XSTEP_SMEM_MAX) return false;
   return n * p <= kSmallAlwaysEntries || (n * p <= kSmallMaxEntries && r >= kSmallMinStarts);
 }
 
-cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, int n, int p, float *X, int64_t ldx,
-                                float *U, float *Y, int64_t ldu, float *V, StartState s, int *sup_idx, float *sup_val,
-                                int r, int sweeps, cudaStream_t st) {
-  if (!small_sweeps_fit(n, p, r)) return cudaErrorInvalidValue;
+cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, const float *AT, int64_t ldat, int n, int p,
+                                float *X, int64_t ldx, StartState s, int *sup_idx, float *sup_val, int r, int sweeps,
+                                cudaStream_t st) {
+  if (!small_sweeps_fit(n, p, r) || lda % 8 != 0 || ldat % 8 != 0) return cudaErrorInvalidValue;
   static const cudaError_t configured =
-      cudaFuncSetAttribute(k_small_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize, XSTEP_SMEM_MAX);
+      cudaFuncSetAttribute(k_small_sweeps<kSmallT>, cudaFuncAttributeMaxDynamicSharedMemorySize, XSTEP_SMEM_MAX);
   if (configured != cudaSuccess) return configured;
-  const size_t bytes = std::max(4 * (size_t)((std::max(n, p) + 3) & ~3), (sizeof(FastShared<XT>) + 15) / 16 * 16) +
-                       4 * (size_t)((p + 3) & ~3);
-  k_small_sweeps<<<r, XT, bytes, st>>>(xa, A, lda, n, p, X, ldx, U, Y, ldu, V, s, sup_idx, sup_val, sweeps);
-  return cudaGetLastError();
+  // CTAs per start, of at least 32 columns each: as many as are resident at once (a cluster lies in one GPC,
+  // so of 152 SMs clusters of 8 reach 120 and clusters of 4 reach 144, at a CTA per SM; a second wave doubled
+  // the time: 16 starts of p = 500 in clusters of 8 565 us, of 4 320)
+  const int sms = sm_count();
+  if (sms < 1) return cudaErrorInvalidDevice;
+  int ctas = kSmallCtas;
+  while (ctas > 1 && ((int64_t)r * ctas > sms * (ctas == 8 ? 6 : 7) / 8 || p < 32 * ctas)) ctas /= 2;
+  size_t bytes = 4 * (size_t)small_words<kSmallT>(n, p, ctas);
+  const size_t a_bytes = 4 * (size_t)n * (size_t)small_cols(p, ctas);
+  const int a_smem = bytes + a_bytes <= (size_t)XSTEP_SMEM_MAX ? 1 : 0;
+  if (a_smem) bytes += a_bytes;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(r * ctas));
+  cfg.blockDim = dim3(kSmallT);
+  cfg.dynamicSmemBytes = bytes;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)ctas;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_small_sweeps<kSmallT>, xa, A, lda, AT, ldat, n, p, ctas, a_smem, X, ldx, s, sup_idx,
+                            sup_val, sweeps);
 }
 
 cudaError_t launch_xstep(XstepArgs a, const float *V, int64_t ldv, int r, float *X, int64_t ldx,

@@ -1345,8 +1345,8 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
                      h->defl_k == 0 && h->A32 && small_sweeps_fit(h->n, h->p, r);
   if (small) {
     CK(timed(h, SPCA_K_XSTEP, 1, [&] {
-      return launch_small_sweeps(xa, h->A32, h->ldA, n, p, h->X, h->ldX, h->U, h->Y, h->ldU, h->V, S, h->sup_idx,
-                                 h->sup_val, r, max_iter, st);
+      return launch_small_sweeps(xa, h->A32, h->ldA, h->AT32, h->ldAT, n, p, h->X, h->ldX, S, h->sup_idx, h->sup_val, r,
+                                 max_iter, st);
     }));
     if (P.timeout_us > 0 && std::chrono::duration_cast<std::chrono::microseconds>(
                                 std::chrono::steady_clock::now() - t_start).count() > P.timeout_us) {

@@ -576,16 +576,15 @@ inline bool xstep_may_need_full(int form, double s, bool target) {
   return is_pen(form) && !target ? true : s > (uses_lam(form) ? 150.0 : 500.0);
 }
 // small problems (n p <= kSmallAlwaysEntries, or <= kSmallMaxEntries with at least
-// kSmallMinStarts starts; x, y and v in shared memory): every sweep of every start in one launch,
-// a CTA per start (u = A x and v = A^T y on the CUDA cores from A, the y-step writing Y, the
-// full-pass x-step); sweeps = the most sweeps a start may run
+// kSmallMinStarts starts; x, u, y and v in shared memory): every sweep of every start in one launch, a CTA
+// per start; sweeps = the most sweeps a start may run
 constexpr int64_t kSmallAlwaysEntries = int64_t(1) << 17;
 constexpr int64_t kSmallMaxEntries = int64_t(1) << 19;
 constexpr int kSmallMinStarts = 16;
 bool small_sweeps_fit(int64_t n, int64_t p, int r);
-cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, int n, int p, float *X, int64_t ldx,
-                                float *U, float *Y, int64_t ldu, float *V, StartState s, int *sup_idx, float *sup_val,
-                                int r, int sweeps, cudaStream_t st);
+cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, const float *AT, int64_t ldat, int n, int p,
+                                float *X, int64_t ldx, StartState s, int *sup_idx, float *sup_val, int r, int sweeps,
+                                cudaStream_t st);
 // x-step (S3..S6), objective F, stopping rule, support lists, and (act given) the next sweep's active
 // list in *ctrl, which must be zero before; ctrl_read is cleared (see launch_active_list), and so are the
 // nflags ints at flags (the stream-K flags of the next contraction; null: none).  defer: a
