@@ -1516,13 +1516,10 @@ __global__ void __launch_bounds__(T) k_small_sweeps(XstepArgs xa, const float *_
   }
 }
 
-// (measured on GB300: with one CTA per start, a start's sweep costs about as much as the launch
-// chain it replaces at n p ~ 4e5, so mid-sized matrices take this path only with enough starts
-// to fill the device)
 constexpr int kSmallT = 256, kSmallCtas = 8;
 bool small_sweeps_fit(int64_t n, int64_t p, int r) {
   if (small_words<kSmallT>(n, p, kSmallCtas) * 4 > (int64_t)XSTEP_SMEM_MAX) return false;
-  return n * p <= kSmallAlwaysEntries || (n * p <= kSmallMaxEntries && r >= kSmallMinStarts);
+  return n * p <= kSmallEntries && r <= 2 * sm_count();
 }
 
 cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, const float *AT, int64_t ldat, int n, int p,

@@ -575,12 +575,11 @@ cudaError_t launch_active_list(const int *status, const int *nnz, int r, int *ac
 inline bool xstep_may_need_full(int form, double s, bool target) {
   return is_pen(form) && !target ? true : s > (uses_lam(form) ? 150.0 : 500.0);
 }
-// small problems (n p <= kSmallAlwaysEntries, or <= kSmallMaxEntries with at least
-// kSmallMinStarts starts; x, u, y and v in shared memory): every sweep of every start in one launch, a CTA
-// per start; sweeps = the most sweeps a start may run
-constexpr int64_t kSmallAlwaysEntries = int64_t(1) << 17;
-constexpr int64_t kSmallMaxEntries = int64_t(1) << 19;
-constexpr int kSmallMinStarts = 16;
+// small problems (n p <= kSmallEntries, at most two starts per SM; x, u, y and v in shared memory): every
+// sweep of every start in one launch, a cluster of CTAs per start; sweeps = the most sweeps a start may run.
+// The lines: 20 sweeps of 1, 16 and 60 starts at n p = 1e6 321, 418 and 595 us (by sweeps 463, 544, 789), of
+// 16 and 40 at 1.4e6 517 and 756 (564, 713); 300 starts at n p = 5e4 371 us (553), 1000 starts 1105 (730)
+constexpr int64_t kSmallEntries = int64_t(1) << 20;
 bool small_sweeps_fit(int64_t n, int64_t p, int r);
 cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, const float *AT, int64_t ldat, int n, int p,
                                 float *X, int64_t ldx, StartState s, int *sup_idx, float *sup_val, int r, int sweeps,
