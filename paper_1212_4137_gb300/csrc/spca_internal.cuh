@@ -188,8 +188,11 @@ struct SpPlan {       // device arrays of items and long rows
   SpLong *longs = nullptr;
   int nitems = 0, nlong = 0, nseg = 0;
 };
-constexpr int kSpItemNnz = 2048;
-constexpr int kSpItemRows = 32;
+// (a warp walks an item's rows one after another, each a chain of dependent loads, so items are small:
+// v = A^T y of a 40000 x 20000 corpus and 20 starts 104 us with 2048 entries and 32 rows, 82 with 2048 and 8,
+// 79 with 512 and 8; 64 starts 192, 230 and 154 us)
+constexpr int kSpItemNnz = 512;
+constexpr int kSpItemRows = 8;
 constexpr int kSpGroup = 8;     // starts per pass of the SpMM (one 32-byte sector of Bt)
 constexpr int kSpSupportCap = 256;   // largest support the column scatter serves
 // host side (sparse_host.cu): a CSR matrix in host memory
