@@ -237,6 +237,82 @@ __global__ void __launch_bounds__(256) k_ystep_apply(int form, const float *__re
   }
 }
 
+// The y-step of long u under L2 variance straight into the packed operand of the sparse product (see
+// k_pack_t), y itself not being wanted: a CTA per 128 rows and 32 listed starts, y's bits those of
+// k_ystep_apply.  Bound by the launch and two round trips; with the chunk norms before it 11 us for 20 starts
+// of 40000 rows, where y-step and packing were three launches of 18 us.
+__global__ void __launch_bounds__(256) k_ystep_pack(const float *__restrict__ U, int64_t ldu, int n,
+                                                    const int *__restrict__ list, const int *__restrict__ count,
+                                                    StartState s, float *__restrict__ X, int64_t ldX, int p,
+                                                    const float *__restrict__ ysum, int nch, float *__restrict__ Bt,
+                                                    int ldb) {
+  constexpr int SUB = 4;
+  __shared__ float tile[SUB][32][33], inv[32];
+  __shared__ int start[32], zero[32];
+  const int cnt = *count, k0 = blockIdx.y * 32;
+  const int kpad = (cnt + kSpGroup - 1) / kSpGroup * kSpGroup;
+  if (k0 >= kpad) return;
+  const int tx = threadIdx.x, j00 = blockIdx.x * 32 * SUB;
+  if (threadIdx.y == 0) {
+    const int c = k0 + tx < cnt ? list[k0 + tx] : -1;
+    float tot = 0.0f, hi, lo, iv = 0.0f;
+    if (c >= 0) {
+      for (int q = 0; q < nch; ++q) tot += ysum[(int64_t)c * nch + q];
+      if (tot != 0.0f) norm_and_inverse(tot, &hi, &lo, &iv);
+    }
+    start[tx] = c;
+    inv[tx] = iv;
+    zero[tx] = c >= 0 && tot == 0.0f;
+    if (c >= 0 && blockIdx.x == 0) {
+      s.iters[c] += 1;
+      if (tot == 0.0f) {
+        s.status[c] = SPCA_ST_DEGENERATE;
+        s.nnz[c] = 0;
+        s.F[c] = 0.0;
+      }
+    }
+  }
+  __syncthreads();
+  if (blockIdx.x == 0) {
+    for (int q = 0; q < 32; ++q) {
+      if (!zero[q]) continue;
+      for (int j = threadIdx.y * 32 + tx; j < p; j += 256) X[(int64_t)start[q] * ldX + j] = 0.0f;
+    }
+  }
+  float v[SUB][4];
+#pragma unroll
+  for (int b = 0; b < SUB; ++b)
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int c = start[threadIdx.y + 8 * h], j = j00 + 32 * b + tx;
+      v[b][h] = c >= 0 && j < n ? U[(int64_t)c * ldu + j] : 0.0f;
+    }
+#pragma unroll
+  for (int b = 0; b < SUB; ++b)
+#pragma unroll
+    for (int h = 0; h < 4; ++h) tile[b][threadIdx.y + 8 * h][tx] = v[b][h] * inv[threadIdx.y + 8 * h];
+  __syncthreads();
+#pragma unroll
+  for (int b = 0; b < SUB; ++b)
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int j = j00 + 32 * b + threadIdx.y + 8 * h, k = k0 + tx;
+      if (j < n && k < kpad) Bt[(int64_t)j * ldb + k] = tile[b][tx][threadIdx.y + 8 * h];
+    }
+}
+
+cudaError_t launch_ystep_pack(const float *U, int64_t ldu, int n, int r, const int *list, const int *count,
+                              StartState s, float *X, int64_t ldX, int p, float *ysum, float *Bt, int ldb,
+                              cudaStream_t st) {
+  const int nch = (n + kYChunk - 1) / kYChunk;
+  k_ystep_norm<<<dim3((unsigned)nch, (unsigned)r), 256, 0, st>>>(U, ldu, n, s, ysum);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_ystep_pack<<<dim3((unsigned)((n + 127) / 128), (unsigned)((r + 31) / 32)), dim3(32, 8), 0, st>>>(
+      U, ldu, n, list, count, s, X, ldX, p, ysum, nch, Bt, ldb);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_ystep(int form, const float *U, int64_t ldu, int n, int r, float *Y, void *Ypl,
                          int64_t plane_stride, const int *rank, StartState s, float *X, int64_t ldX,
                          int p, float *ysum, const int *skip, int *flags, int nflags, cudaStream_t st) {

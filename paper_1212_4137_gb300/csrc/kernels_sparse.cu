@@ -125,6 +125,23 @@ __device__ __forceinline__ int64_t lower_bound_col(const int *__restrict__ col, 
 }
 }  // namespace
 
+// the same by the 16 lanes of a half-warp together, 16 probes a step; every lane gets the result
+__device__ __forceinline__ int64_t lower_bound_16(const int *__restrict__ col, int64_t b, int64_t e, int v) {
+  const int lane = threadIdx.x & 15, sh = threadIdx.x & 16;
+  const unsigned half = 0xffffu << sh;
+  while (b < e) {
+    const int64_t step = (e - b + 15) / 16, at = b + lane * step;   // probes b, b + step, ...
+    const bool less = at < e && col[at] < v;
+    const int cnt = __popc((__ballot_sync(half, less) >> sh) & 0xffffu);   // a prefix of the probes: ascending
+    if (cnt == 0) return b;
+    const int64_t nb = b + (cnt - 1) * step + 1;
+    e = min(e, b + cnt * step);
+    b = nb;
+  }
+  return b;
+}
+constexpr int kSpHalfWarps = 32;   // columns up to which the support's columns are searched this way
+
 // grid (ceil(len / 32), ceil(rmax / 32)), block (32, 8): a 32 x 32 tile through shared memory
 __global__ void k_pack_t(const float *__restrict__ src, int64_t ld, int len, const int *__restrict__ list,
                          const int *__restrict__ count, int rmax, const int *__restrict__ gate,
@@ -568,7 +585,18 @@ __global__ void __launch_bounds__(256) k_spmv_support(SpMat AT, int n, const int
   const float *gv = sup_val + (int64_t)c * cap;
   for (int t0 = 0; t0 < nnz; t0 += 256) {
     __syncthreads();
-    if (t0 + (int)threadIdx.x < nnz) {
+    const int m = min(256, nnz - t0);
+    if (m <= kSpHalfWarps) {
+      // few columns: a half-warp finds each end of the chunk in a column, 16 probes a round trip
+      for (int e = threadIdx.x >> 4; e < 2 * m; e += 16) {
+        const int q = e >> 1, j = gi[t0 + q];
+        const int64_t k = lower_bound_16(AT.col, AT.ptr[j], AT.ptr[j + 1], e & 1 ? base + rows : base);
+        if ((threadIdx.x & 15) == 0) {
+          (e & 1 ? hi : lo)[q] = k;
+          if (!(e & 1)) xv[q] = gv[t0 + q];
+        }
+      }
+    } else if ((int)threadIdx.x < m) {
       const int j = gi[t0 + threadIdx.x];
       xv[threadIdx.x] = gv[t0 + threadIdx.x];
       const int64_t b = lower_bound_col(AT.col, AT.ptr[j], AT.ptr[j + 1], base);
@@ -576,11 +604,25 @@ __global__ void __launch_bounds__(256) k_spmv_support(SpMat AT, int n, const int
       hi[threadIdx.x] = lower_bound_col(AT.col, b, AT.ptr[j + 1], base + rows);
     }
     __syncthreads();
-    const int m = min(256, nnz - t0);
+    // a thread's first entries of the next column load while this column is added
+    int ni = 0;
+    float nv = 0.0f;
+    auto first = [&](int q) {
+      if (q < m && lo[q] + threadIdx.x < hi[q]) {
+        ni = __ldg(AT.col + lo[q] + threadIdx.x) - base;
+        nv = __ldg(AT.val + lo[q] + threadIdx.x);
+      }
+    };
+    first(0);
     for (int q = 0; q < m; ++q) {
       // the rows of one column are distinct: no two threads update the same u_i
       const float x = xv[q];
-      for (int64_t k = lo[q] + threadIdx.x; k < hi[q]; k += 256) {
+      const int64_t b = lo[q] + threadIdx.x, e = hi[q];
+      const int ci = ni;
+      const float cv = nv;
+      first(q + 1);
+      if (b < e) us[ci] = fmaf(x, cv, us[ci]);
+      for (int64_t k = b + 256; k < e; k += 256) {
         const int i = __ldg(AT.col + k) - base;
         us[i] = fmaf(x, __ldg(AT.val + k), us[i]);
       }

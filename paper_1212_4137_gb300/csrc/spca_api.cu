@@ -471,6 +471,8 @@ int sweep_y_v(spca_handle *h, int engine, int form, int r, StartState S, const i
     // variance) is packed in FP16, exactly, 16 starts to a 32-byte sector
     const bool half = is_l1_var(form);
     CK(timed(h, SPCA_K_YSTEP, half ? 1 : 2, [&] {
+      if (!half && h->defl_k == 0 && !ystep_with_gather(n))   // (the low-rank update reads y)
+        return launch_ystep_pack(h->U, h->ldU, n, r, h->act, nact, S, h->X, h->ldX, p, h->ysum, h->Bt, h->ldb, st);
       cudaError_t e = launch_ystep(form, h->U, h->ldU, n, r, h->Y, nullptr, 0, nullptr, S, h->X, h->ldX, p, h->ysum,
                                    nullptr, nullptr, 0, st);
       if (e != cudaSuccess || half) return e;

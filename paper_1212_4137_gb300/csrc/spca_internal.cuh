@@ -302,6 +302,11 @@ cudaError_t launch_gather_y(int form, const float *AT, const void *AT16, const f
 // With ysum (r * ceil(n / kYChunk) floats of scratch) and n > 2 kYChunk, a CTA per chunk of
 // kYChunk entries and start (L2 variance: the chunks' sums of u_i^2 added in chunk order).
 constexpr int kYChunk = 8192;
+// the same under L2 variance for long u (n > 2 kYChunk) of a sparse A, y written only as the packed operand Bt
+// of the listed starts (see launch_pack_t)
+cudaError_t launch_ystep_pack(const float *U, int64_t ldu, int n, int r, const int *list, const int *count,
+                              StartState s, float *X, int64_t ldX, int p, float *ysum, float *Bt, int ldb,
+                              cudaStream_t st);
 // long u, cut into chunks over several CTAs, keep their own y-step kernels
 inline bool ystep_with_gather(int64_t n) { return n <= 2 * kYChunk; }
 cudaError_t launch_ystep(int form, const float *U, int64_t ldu, int n, int r, float *Y,
