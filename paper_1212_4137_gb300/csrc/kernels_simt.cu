@@ -179,9 +179,13 @@ __global__ void __launch_bounds__(256) k_ystep_norm(const float *__restrict__ U,
   const int b = blockIdx.x, c = blockIdx.y;
   if (s.status[c] != ST_ACTIVE) return;
   const float *u = U + (int64_t)c * ldu;
-  const int i1 = min(n, (b + 1) * kYChunk);
-  float part = 0.0f;
-  for (int i = b * kYChunk + threadIdx.x; i < i1; i += blockDim.x) part = fmaf(u[i], u[i], part);
+  const int i0 = b * kYChunk + threadIdx.x, i1 = min(n, (b + 1) * kYChunk);
+  constexpr int E = kYChunk / 256;   // a thread's entries, all loads in flight
+  float v[E], part = 0.0f;
+#pragma unroll
+  for (int k = 0; k < E; ++k) v[k] = i0 + 256 * k < i1 ? u[i0 + 256 * k] : 0.0f;
+#pragma unroll
+  for (int k = 0; k < E; ++k) part = fmaf(v[k], v[k], part);
   const float t = block_sum_f(part, redf);
   if (threadIdx.x == 0) ysum[(int64_t)c * gridDim.x + b] = t;
 }
