@@ -51,7 +51,7 @@ __device__ __forceinline__ double group_reduce(const double (&acc)[RPL], int lan
   return v + __shfl_xor_sync(0xffffffffu, v, 1);
 }
 
-// grid (nchunks, r): u_i = sum_j x_j A[i, j] over the nonzeros of x, products and sums in FP64,
+// grid nchunks x r, the starts fastest: u_i = sum_j x_j A[i, j] over the nonzeros of x, products and sums in FP64,
 // for the 256 rows of chunk b; this CTA's sums of |u_i| and u_i^2 go to
 // partials[(c * nchunks + b) * 2].
 // Bound by finding the nonzeros (each CTA scans the p entries of its x from L2) and by the FP64 pipe.
@@ -60,18 +60,21 @@ __device__ __forceinline__ double group_reduce(const double (&acc)[RPL], int lan
 // at a time, 4 times: with few nonzeros most lanes have work, a lane has 4 rows' loads in flight,
 // and the lane sums end in the reduce-scatter above.  The staged columns ascend, so 8 lanes read one
 // 32-byte sector of a row when x is dense.
-// 64 starts with 50 nonzeros each, n = 5000, p = 20000: 252 us (659 us before).
+// All starts of a row chunk run side by side, so that a 32-byte sector of A that several starts need comes
+// from memory once (A is larger than L2).
+// 64 starts with 50 nonzeros each, n = 5000, p = 20000: 168 us (659 with a scan of 256 entries per barrier
+// pair, 252 with the row chunks of a start side by side).
 __global__ void __launch_bounds__(NT) k_obj_partial(const float *__restrict__ A, int64_t lda, int n, int p,
-                                                    const float *__restrict__ X, int64_t ldx,
+                                                    const float *__restrict__ X, int64_t ldx, int r, int nchunks,
                                                     double *__restrict__ partials) {
   __shared__ int sj[XSTAGE];
   __shared__ float sx[XSTAGE];
   __shared__ int wcnt[NW];
   __shared__ double red[32];
-  const int c = blockIdx.y;
+  const int c = blockIdx.x % r, chunk = blockIdx.x / r;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int sub = lane / LPR, l8 = lane % LPR;
-  const int row0 = blockIdx.x * NROWS + w * RPW + sub;   // this lane's rows: row0 + k (32 / LPR)
+  const int row0 = chunk * NROWS + w * RPW + sub;   // this lane's rows: row0 + k (32 / LPR)
   const float *x = X + (int64_t)c * ldx;
   const float *arow[RPL];
 #pragma unroll
@@ -136,7 +139,7 @@ __global__ void __launch_bounds__(NT) k_obj_partial(const float *__restrict__ A,
   const double l1 = block_sum_d(mine ? fabs(u) : 0.0, red);
   const double l2 = block_sum_d(mine ? u * u : 0.0, red);
   if (threadIdx.x == 0) {
-    double *o = partials + ((int64_t)c * gridDim.x + blockIdx.x) * 2;
+    double *o = partials + ((int64_t)c * nchunks + chunk) * 2;
     o[0] = l1;
     o[1] = l2;
   }
@@ -227,7 +230,7 @@ extern "C" int spca_objective_noalloc(int form, double gamma, const float *A, in
   if (scratch_for_current_device(&partials) != cudaSuccess) return SPCA_E_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   // every partial the reduction reads is written by this call's first kernel (no zeroing needed)
-  k_obj_partial<<<dim3((unsigned)nchunks, (unsigned)r), NT, 0, st>>>(A, lda, (int)n, (int)p, X, ldx, partials);
+  k_obj_partial<<<(unsigned)(nchunks * r), NT, 0, st>>>(A, lda, (int)n, (int)p, X, ldx, r, (int)nchunks, partials);
   if (cudaGetLastError() != cudaSuccess) return SPCA_E_CUDA;
   k_obj_reduce<<<r, NT, 0, st>>>(form, gamma, partials, (int)nchunks, X, ldx, (int)p, f, ev);
   if (cudaGetLastError() != cudaSuccess) return SPCA_E_CUDA;
