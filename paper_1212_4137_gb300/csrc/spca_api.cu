@@ -1075,8 +1075,7 @@ int spca_products(spca_handle *h, int form, int engine, const float *X, int64_t 
   RC(ensure_lr_coef(h, r));
   const int n = (int)h->n, p = (int)h->p;
   cudaStream_t st = h->stream;
-  CK(cudaMemcpy2DAsync(h->X, h->ldX * sizeof(float), X, ldx * sizeof(float), (size_t)p * sizeof(float), r,
-                       cudaMemcpyDeviceToDevice, st));
+  CK(launch_copy_rows(X, ldx, h->X, h->ldX, p, r, st));
   CK(cudaMemsetAsync(h->status, 0xFF, (size_t)r * sizeof(int), st));   // every row active (-1)
   CK(cudaMemsetAsync(h->iters, 0, (size_t)r * sizeof(int), st));
   CK(cudaMemsetAsync(h->ctrl, 0, sizeof(Ctrl), st));
@@ -1084,10 +1083,8 @@ int spca_products(spca_handle *h, int form, int engine, const float *X, int64_t 
   RC(sweep_u_dense(h, eng, r, nullptr, &h->ctrl[0].active, r, lowp, h->sk));
   RC(sweep_lowrank_u(h, r, &h->ctrl[0].active, h->act));
   RC(sweep_y_v(h, eng, form, r, state_of(h), &h->ctrl[0].active, r, lowp, nullptr, false, h->sk));
-  CK(cudaMemcpy2DAsync(U, ldu * sizeof(float), h->U, h->ldU * sizeof(float), (size_t)n * sizeof(float), r,
-                       cudaMemcpyDeviceToDevice, st));
-  CK(cudaMemcpy2DAsync(V, ldv * sizeof(float), h->V, h->ldX * sizeof(float), (size_t)p * sizeof(float), r,
-                       cudaMemcpyDeviceToDevice, st));
+  CK(launch_copy_rows(h->U, h->ldU, U, ldu, n, r, st));
+  CK(launch_copy_rows(h->V, h->ldX, V, ldv, p, r, st));
   RC(read_dev_err(h));
   return SPCA_OK;
 }

@@ -293,6 +293,10 @@ cudaError_t launch_gather_y(int form, const float *AT, const void *AT16, const f
                             int64_t ldu, const int *gate, float *Y, void *Ypl, int64_t pstride, const int *rank,
                             float *X, int64_t ldX, int p, int *cnt, int sms, cudaStream_t st);
 
+// cols floats of each of `rows` rows (at most 65535), src rows lds apart, dst rows ldd apart, any alignment
+cudaError_t launch_copy_rows(const float *src, int64_t lds, float *dst, int64_t ldd, int64_t cols, int rows,
+                             cudaStream_t st);
+
 // y-step (S1 / S2 of Table 3) for active starts.  Writes Y as FP32 (Y != nullptr, row c) and/or
 // as tensor-core planes (Ypl != nullptr, row rank[c] when rank is given, else c; plane t at
 // Ypl + t * plane_stride): 1 plane of +-kQScale for L1 variance, the 2 planes of kQScale y for
