@@ -438,8 +438,8 @@ int spca_set_waits(spca_handle *h, int64_t wait_limit_us, int unpublished_parts)
  * matrix (a handle), formulation, s or gamma and starts (the batching of Section 4 carried across
  * problems).  Every phase of a sweep is one launch over all the group's problems: the dense
  * u = A x of a problem's first sweep and v = A^T y of every sweep as one persistent tensor-core
- * launch over the tiles of all problems; the start set-up, support gather, y-step, x-step (the
- * candidate filter and operator, then the full pass for the starts they leave) and active lists
+ * launch over the tiles of all problems; the start set-up, support gather, y-step and x-step (with
+ * the active lists; then the full pass for the starts it leaves, while some start may need it)
  * as one launch each over all starts or problems.  Each problem's results do not depend on the
  * other problems of the group (the same bits alone and in any mix) and agree with spca_solve's
  * for it up to the order of rounding in the contractions and the x-step's sums.  The problems on one
