@@ -885,6 +885,22 @@ __device__ __forceinline__ double list_lambda(const float *cv, int ncand, float 
   return lam;
 }
 
+// An entry within a quarter of its last bit of lambda_s survives or not by the rounding of phi alone.  The
+// x-step of given v leaves a start that has one to the full pass (one start in 25000 of p = 40000, s = 50),
+// so that the number of survivors is the full pass's in every case.
+constexpr double kLamTie = -2.0;
+__device__ __forceinline__ bool lambda_tie(const float *cv, int ncand, double lam) {
+  const int lane = threadIdx.x & 31, near = __float_as_int(__double2float_rd(lam));
+  bool tie = false;
+  for (int i = lane; i < ncand; i += 32) {
+    const int key = (int)abs_key(cv[i]);
+    if (key < near || key > near + 1) continue;
+    const double v = (double)__int_as_float(key), ulp = (double)__int_as_float(key + 1) - v;
+    tie = tie || fabs(v - lam) < 0.25 * ulp;
+  }
+  return __any_sync(0xffffffffu, tie);
+}
+
 // a start's state as the x-step reads it, all loads in flight at once
 struct XState {
   int iters = 0, nnz = 0, xfast = 0;
@@ -978,11 +994,14 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
     bool ok = fits;
     if (fits && lam_form) {
       if (w == 0) {                  // (a hint just below the last lambda_s: few steps while it holds steady)
-        const double l = list_lambda(fs.u.l.cv, ncand, (float)a.s, a.s, __uint_as_float(Gk), kHint * tprev);
+        double l = list_lambda(fs.u.l.cv, ncand, (float)a.s, a.s, __uint_as_float(Gk), kHint * tprev);
+        // (given v: see kLamTie)
+        if (!st.status && l >= 0.0 && lambda_tie(fs.u.l.cv, ncand, l)) l = kLamTie;
         if (lane == 0) fs.lam = l;
       }
       __syncthreads();
       lam = fs.lam;
+      if (lam == kLamTie) return false;
       ok = lam >= 0.0;
     } else if (fits && !exact) ok = ncand >= need || Gk == 0u;
     if (ok) break;
