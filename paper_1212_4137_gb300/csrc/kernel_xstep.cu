@@ -1247,12 +1247,13 @@ __global__ void __launch_bounds__(T, fast_ctas(T)) k_xstep_fast(XstepArgs a, con
 }
 
 // Threads per start, 128 to 1024: reading v shrinks with the threads, barriers and the sums over the
-// warps grow with them, so 16 to 64 entries per thread (a sweep's x-step of 16 starts, forms 1 and 3, event
+// warps grow with them, so 16 to 256 entries per thread (a sweep's x-step of 16 starts, forms 1 and 3, event
 // times: p = 4000 with 128 threads 15.3 and 20.0 us, 256 14.2 and 18.5; p = 12000 with 256 15.4 and 20.4, 512
-// 15.4 and 18.7; p = 25000 with 512 17.3 and 21.4, 1024 21.0 and 24.9); and never more than keeps all starts
+// 15.4 and 18.7; p = 40000 with 512 18.3 and 23.1, 1024 20.0 and 25.7; p = 200000 with 512 37.6 and 38.7, 1024
+// 35.0 and 38.6); and never more than keeps all starts
 // resident at once (fast_ctas).
 int fast_threads(int64_t starts, int p, int sms) {
-  const int by_p = p <= 2048 ? 128 : p <= 8192 ? 256 : p <= 32768 ? 512 : 1024;
+  const int by_p = p <= 2048 ? 128 : p <= 8192 ? 256 : p <= 131072 ? 512 : 1024;
   const int by_r = starts <= sms ? 1024 : starts <= 3 * (int64_t)sms ? 256 : 128;
   return std::min(by_p, by_r);
 }
