@@ -206,3 +206,31 @@ def test_sparse_sweeps(lib, oracle, n, r, s):
     M.data = rng.integers(1, 9, M.nnz).astype(np.float32)
     M = (sps.csr_matrix(M) + sps.csr_matrix(np.outer(rng.random(n) < 0.05, np.arange(400) < 40) * 3.0)).astype(np.float32).tocsr()
     _solve_matches(lib, oracle, M, 1, r, s, 3, lib.SPCA_ENGINE_AUTO)
+
+
+# an entry exactly at lambda_s (s = 4.5 and 10, 9, 9, 9, 9 above 8: s sum w^2 = (sum w)^2 at 8) does not survive,
+# whether the full pass it is left to runs in the first kernel or in its own
+@pytest.mark.parametrize("p", [70, 1025, 8192, 8193, 20011])
+@pytest.mark.parametrize("form", [3, 4])
+def test_entry_at_lambda(lib, p, form):
+    import torch
+    rng = np.random.default_rng(p)
+    V = np.zeros((3, p), np.float32)
+    V[:, 7:] = rng.uniform(-6, 6, (3, p - 7))
+    V[:, 1:7] = [10, -9, 9, 8, -9, 9]
+    V[2, 4] = 7                                              # the same without the entry
+    V = np.roll(V, p // 3, axis=1)
+    h = lib.Handle(np.zeros((2, p), np.float32))
+    Vd = torch.from_numpy(V).cuda()
+    Xd = torch.full((3, p), np.nan, dtype=torch.float32, device="cuda")
+    F, T = (torch.zeros(3, dtype=torch.float64, device="cuda") for _ in range(2))
+    N = torch.zeros(3, dtype=torch.int32, device="cuda")
+    st = lib.spca_xstep(h.h, form, 4.5, 0.0, False, Vd.data_ptr(), p, 3, Xd.data_ptr(), p, F.data_ptr(), N.data_ptr(),
+                        T.data_ptr())
+    assert st == 0, lib.spca_last_error(h.h)
+    h.close()
+    w = np.sign(V) * np.maximum(np.abs(V) - 8.0, 0.0)
+    assert N.tolist() == [5, 5, 5]
+    assert np.abs(Xd.cpu().numpy() - w / np.sqrt(8.0)).max() <= 1e-6
+    assert np.abs(T.cpu().numpy() - 8.0).max() <= 1e-6 * 8.0
+    assert np.abs(F.cpu().numpy() - (8.0 * np.sqrt(4.5) + np.sqrt(8.0))).max() <= 1e-6 * 20.0
