@@ -531,14 +531,16 @@ __global__ void __launch_bounds__(XT) k_xstep(XstepArgs a_in, const float *__res
 // memory.  The bound comes from
 //   - a fixed threshold itself (exact);
 //   - last sweep's threshold t: G = kGuess t (kGuessSteady t while t holds steady);
-//   - the maxima of 2048 disjoint subsets of v (one more pass): at least j entries lie at or above the
-//     j-th largest of them, and for j well below 2048 not many more do;
+//   - the maxima of 2048 disjoint subsets of v (one more pass), the same ones whatever the CTA's size: at
+//     least j entries lie at or above the j-th largest of them, and for j well below 2048 not many more do;
 //   - 0 for a very short v: the list holds every nonzero entry.
 // A bound is checked before it is used: at least s (or s + 1) listed entries for the selections,
 // phi(G) < 0 for lambda_s (phi increases through its root); then the list holds every surviving
 // entry and the result is that of a pass over all of v.  A start that no bound serves (more than
 // kFastSegCap entries above it in one of the 16 segments, lambda_s = 0, s beyond the list) takes the full
-// pass.
+// pass.  Bound, list and these choices do not depend on the CTA's size, so neither does the path that a
+// start takes nor any bit of its result: in a group, whose starts and longest v choose the size, a member
+// has the same bits alone and in any mix.
 //
 // One CTA does all of it for a start, in one launch per sweep, and the CTA that finishes last makes
 // the active list of the next sweep.  What bounds it is each start's chain of dependent steps (reads
@@ -551,6 +553,7 @@ __global__ void __launch_bounds__(XT) k_xstep(XstepArgs a_in, const float *__res
 // 16 starts 57 -> 24 us; p = 20000, lambda_s, one start 44 -> 28 us (CUDA events, a few us included).
 constexpr int kFastCand = 1024;                // listed entries per start
 constexpr int kFastBins = 2048, kFastShift = 17;   // bins of 2^-6 octave below the largest |v_i|
+constexpr int kFastSubsets = 2048;             // disjoint subsets of v whose maxima bound the threshold
 constexpr int kFastAllP = 64;                  // v up to this long: list every nonzero entry
 constexpr int kFastMaxJ = 600;                 // j of the subset maxima: the list stays below kFastCand
 constexpr float kGuess = 0.85f;
@@ -572,6 +575,7 @@ struct FastShared {
       int wi[W * kWarpCap];
     } w;
     int rank[kFastCand];
+    uint4 maxima[kFastSubsets / 4];            // of the upper half of 1024 threads, see subset_bound
     struct {
       float val[kFastCand];                    // the surviving entries, in index order
       int idx[kFastCand];
@@ -615,28 +619,50 @@ __device__ __forceinline__ float4 row_load(const Row &r, int q, int hi) {
   return t;
 }
 
-// a lower bound of the j-th largest |v_i| from the maxima of 4 T subsets (four per thread): the lower
-// edge of the histogram bin of the j-th largest maximum.  0 when the bins do not resolve it.
+// a lower bound of the j-th largest |v_i| from the maxima of 2048 subsets (the entries at q, q + 2048, ...
+// of the row): the lower edge of the histogram bin of the j-th largest maximum.  0 when the bins do not
+// resolve it.
 template <int T>
 __device__ __forceinline__ uint32_t subset_bound(const Row &row, int j, FastShared<T> &fs) {
-  uint32_t m[4] = {0u, 0u, 0u, 0u};
   constexpr int CH = T > 256 ? 4 : 8;          // loads in flight per thread
+  // the subsets of a thread: G groups of four, load k of it being group k mod G; with 1024 threads two
+  // threads share four
+  constexpr int G = kFastSubsets > 4 * T ? kFastSubsets / (4 * T) : 1;
+  static_assert(CH % G == 0, "a step covers whole rounds of the subsets");
+  uint32_t m[G][4];
+#pragma unroll
+  for (int k = 0; k < G; ++k) m[k][0] = m[k][1] = m[k][2] = m[k][3] = 0u;
   for (int q0 = 4 * threadIdx.x; q0 < row.end; q0 += 4 * T * CH) {
     float4 t[CH];
 #pragma unroll
     for (int k = 0; k < CH; ++k) t[k] = row_load(row, q0 + 4 * T * k, row.end);
 #pragma unroll
     for (int k = 0; k < CH; ++k) {
-      m[0] = max(m[0], abs_key(t[k].x));
-      m[1] = max(m[1], abs_key(t[k].y));
-      m[2] = max(m[2], abs_key(t[k].z));
-      m[3] = max(m[3], abs_key(t[k].w));
+      m[k % G][0] = max(m[k % G][0], abs_key(t[k].x));
+      m[k % G][1] = max(m[k % G][1], abs_key(t[k].y));
+      m[k % G][2] = max(m[k % G][2], abs_key(t[k].z));
+      m[k % G][3] = max(m[k % G][3], abs_key(t[k].w));
     }
   }
   for (int b = threadIdx.x; b < kFastBins; b += T) fs.u.hist[b] = 0u;
-  const uint32_t top = block_max_u(max(max(m[0], m[1]), max(m[2], m[3])), fs.sh.red_u);   // (a barrier after the zeros)
+  if (4 * T > kFastSubsets && threadIdx.x >= kFastSubsets / 4)
+    fs.a.maxima[threadIdx.x - kFastSubsets / 4] = make_uint4(m[0][0], m[0][1], m[0][2], m[0][3]);
+  uint32_t all = 0u;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) atomicAdd(&fs.u.hist[min((top - m[k]) >> kFastShift, (uint32_t)kFastBins - 1u)], 1u);
+  for (int k = 0; k < G; ++k) all = max(all, max(max(m[k][0], m[k][1]), max(m[k][2], m[k][3])));
+  const uint32_t top = block_max_u(all, fs.sh.red_u);   // (barriers after the zeros and the shared maxima)
+  if (4 * T > kFastSubsets && threadIdx.x < kFastSubsets / 4) {
+    const uint4 o = fs.a.maxima[threadIdx.x];
+    m[0][0] = max(m[0][0], o.x); m[0][1] = max(m[0][1], o.y);
+    m[0][2] = max(m[0][2], o.z); m[0][3] = max(m[0][3], o.w);
+  }
+  if (threadIdx.x < kFastSubsets / 4) {
+#pragma unroll
+    for (int k = 0; k < G; ++k)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        atomicAdd(&fs.u.hist[min((top - m[k][e]) >> kFastShift, (uint32_t)kFastBins - 1u)], 1u);
+  }
   if (threadIdx.x == 0) fs.sh.digit = kFastBins - 1;
   __syncthreads();
   // one warp: the first bin, from the largest down, whose running count reaches j (64 bins a step: the
@@ -940,8 +966,7 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
   if (!all && !exact && (need > kFastMaxJ || keep_all)) return false;
   // j of the subset maxima: the active set of lambda_s has about 2 s entries where |v|'s tail is
   // exponential, so 3 s lie below its threshold; never so many that subsets hold several of them
-  constexpr int kMaxJ = kFastMaxJ < 2 * T ? kFastMaxJ : 2 * T;
-  int j = lam_form ? (int)fminf(3.0f * (float)a.s + 16.0f, (float)kMaxJ) : need;
+  int j = lam_form ? (int)fminf(3.0f * (float)a.s + 16.0f, (float)kFastMaxJ) : need;
   const float tprev = q0.tprev;
   const bool steady = q0.xfast == 1;
   // x is zero outside the last support list, once there is one (before: all of x is written)
@@ -985,12 +1010,10 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
     else Gk = subset_bound<T>(row, j, fs);
     float f1 = 0.0f, f2 = 0.0f;
     const bool fits = list_above<T>(row, Gk, lam_form, fs, buf, &ncand, &f1, &f2);
-    if (lam_form && !((float)a.s * f2 - f1 * f1 < 0.0f)) {
-      // phi(0) >= 0: every entry survives
-      if (Gk != 0u || !fits) return false;
-      lam0 = true;
-      break;
-    }
+    // phi(0) >= 0, every entry survives: no bound above 0 can serve.  (The sums' last bits depend on T: with
+    // this margin the start would fail the check of phi(G) below all the same, for sqrt(s) ||V||_2 / ||V||_1
+    // grows with the threshold.)
+    if (lam_form && Gk != 0u && (float)a.s * f2 > 1.001f * (f1 * f1)) return false;
     bool ok = fits;
     if (fits && lam_form) {
       if (w == 0) {                  // (a hint just below the last lambda_s: few steps while it holds steady)
@@ -1003,16 +1026,17 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
       lam = fs.lam;
       if (lam == kLamTie) return false;
       ok = lam >= 0.0;
+      if (!ok && Gk == 0u) ok = lam0 = true;   // phi(0) >= 0 over all of v's nonzero entries
     } else if (fits && !exact) ok = ncand >= need || Gk == 0u;
     if (ok) break;
     if (how == kHigh) {
       how = a.ordered && fits && !steady ? kLow : kSubsets;
       // lambda_s lies below this bound: its active set is larger than the list
-      if (lam_form && fits) j = min(kMaxJ, max(j, ncand + ncand / 2 + 32));
+      if (lam_form && fits) j = min(kFastMaxJ, max(j, ncand + ncand / 2 + 32));
     } else if (how == kLow) {
       how = kSubsets;
-    } else if (how == kSubsets && lam_form && fits && j < kMaxJ) {
-      j = kMaxJ;                     // the root lies lower: a longer list
+    } else if (how == kSubsets && lam_form && fits && j < kFastMaxJ) {
+      j = kFastMaxJ;                     // the root lies lower: a longer list
     } else {
       return false;
     }
