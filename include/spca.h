@@ -307,7 +307,8 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
  *   form, s, gamma   as in spca_params; calibrate != 0 applies the Section 4.1 rule
  *                    (penalty forms) before thresholding.
  *   V     device, r x p float, leading dimension ldv >= p.
- *   X     device, r x p float output (ldx >= p): the normalised x-step result, or 0.
+ *   X     device, r x p float output (ldx >= p): the normalised x-step result, or 0.  X = V with
+ *         ldx = ldv replaces each v by its result.
  *   F     device, r doubles: the Table 3 value of the subproblem.
  *   nnz   device, r ints: nonzeros of each result.
  *   thr   device, r doubles: the threshold used (gamma for U/V, lambda_s for S4, 0 for T_s).

@@ -971,12 +971,14 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
   const bool steady = q0.xfast == 1;
   // x is zero outside the last support list, once there is one (before: all of x is written)
   const bool listed = sup_idx && q0.iters > 1 && q0.nnz <= a.cap;
-  if (!x) {
-  } else if (listed) {
-    const int nnz_old = q0.nnz;
-    const int *old = sup_idx + (int64_t)c * a.cap;
-    for (int t = threadIdx.x; t < nnz_old; t += T) x[old[t]] = 0.0f;
-  } else {                           // as aligned vectors, whatever the row's alignment
+  auto clear_x = [&] {
+    if (listed) {
+      const int nnz_old = q0.nnz;
+      const int *old = sup_idx + (int64_t)c * a.cap;
+      for (int t = threadIdx.x; t < nnz_old; t += T) x[old[t]] = 0.0f;
+      return;
+    }
+    // as aligned vectors, whatever the row's alignment
     const int sh = (int)((reinterpret_cast<uintptr_t>(x) >> 2) & 3u);
     float *xb = x - sh;
     for (int q = 4 * threadIdx.x; q < p + sh; q += 4 * T) {
@@ -987,7 +989,12 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
           if (q + k >= sh && q + k < p + sh) xb[q + k] = 0.0f;
       }
     }
-  }
+  };
+  // the zeros are stored while v is read, but for an x over v itself (the x-step of given v, in place):
+  // there once the list is made, which v is read for
+  const float *vrow = V + (int64_t)c * ldv;
+  const bool over_v = x && x < vrow + p && vrow < x + p;
+  if (x && !over_v) clear_x();
 
   // ---- a bound, the list above it, and the check (block-uniform throughout)
   int buf = 0, ncand = 0;
@@ -1042,6 +1049,7 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
     }
     __syncthreads();                 // the lists are reused
   }
+  if (over_v) clear_x();             // (every thread has read its part of v: the list's barrier)
 
   // ---- the operator on the list: which entries survive, as
   //   select: rank < need (T_s; ties at the threshold: the lower indices), or key above the threshold

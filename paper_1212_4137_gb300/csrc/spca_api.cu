@@ -1051,7 +1051,10 @@ int spca_xstep(spca_handle *h, int form, double s, double gamma, int calibrate, 
   // starts that need the full pass are left to a kernel of their own (v in shared memory), but for short
   // rows, whose full pass costs less inside the first kernel than a second launch (one start of p = 600:
   // 46 -> 42 us a call; p = 3000: 51 -> 48 us)
-  const bool defer = h->p > 8192 || xstep_may_need_full(form, s, a.calibrate != 0);
+  // (and for an x over v but not in place, whose full pass needs v staged)
+  const float *v_end = V + (int64_t)(r - 1) * ldv + h->p, *x_end = X + (int64_t)(r - 1) * ldx + h->p;
+  const bool overlap = X < v_end && V < x_end && !(X == V && ldx == ldv);
+  const bool defer = overlap || h->p > 8192 || xstep_may_need_full(form, s, a.calibrate != 0);
   RC(enter(h));
   CK(timed(h, SPCA_K_XSTEP, defer ? 2 : 1, [&] {
     return launch_xstep(a, V, ldv, r, X, ldx, st, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, defer,
