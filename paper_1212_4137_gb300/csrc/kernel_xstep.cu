@@ -54,9 +54,16 @@ __device__ __forceinline__ Seg index_seg(int p, int w) {
   s.hi = min(p, s.lo + seg);
   return s;
 }
-template <typename Fn>
+// (kOne: the CTA has XT threads, a warp per segment, and writes x.  Loops over segments and a test of x inside
+// the passes keep them from being unrolled: 1024 starts of p = 20011, T_s, whole call 268 us for 212.)
+template <bool kOne, typename Fn>
 __device__ __forceinline__ void for_segments(int p, Fn &&fn) {
-  for (int w = threadIdx.x >> 5; w < XW; w += blockDim.x >> 5) fn(w, index_seg(p, w));
+  if constexpr (kOne) {
+    const int w = threadIdx.x >> 5;
+    fn(w, index_seg(p, w));
+  } else {
+    for (int w = threadIdx.x >> 5; w < XW; w += blockDim.x >> 5) fn(w, index_seg(p, w));
+  }
 }
 
 // sums of (f0, f1, i0, i1) over segment w, published by its warp ...
@@ -118,6 +125,7 @@ __device__ __forceinline__ int segment_offsets(XShared &sh) {
 // stops: every element of the bin is in the top j.  Then, with exact == false, *K is the bin's
 // lower bound and *whole = true; with exact == true one more pass finds the bin's minimum,
 // which is the j-th largest key.  Otherwise *need_eq / *eq_total describe ties at *K.
+template <bool kOne>
 __device__ void radix_select(const float *vv, int p, int j, bool exact, XShared &sh, uint32_t *K,
                              bool *whole, int *need_eq, int *eq_total) {
   const int shifts[4] = {23, 15, 7, 0};
@@ -130,7 +138,7 @@ __device__ void radix_select(const float *vv, int p, int j, bool exact, XShared 
     const int sh_ = shifts[t];
     for (int b = threadIdx.x; b < 256; b += blockDim.x) sh.hist[b] = 0u;
     __syncthreads();
-    for_segments(p, [&](int, Seg sg) {
+    for_segments<kOne>(p, [&](int, Seg sg) {
       for (int base = sg.lo; base < sg.hi; base += 32) {
         const int i = base + lane;
         const uint32_t key = (i < sg.hi) ? abs_key(vv[i]) : 0xFFFFFFFFu;
@@ -210,6 +218,7 @@ __device__ void radix_select(const float *vv, int p, int j, bool exact, XShared 
 // the sign of phi, stopping as soon as no |v_i| lies strictly inside the bracket (the active
 // set is then fixed); then the root of phi on that piece in FP64.
 // *lo_out: the active set is {key_i > *lo_out}.
+template <bool kOne>
 __device__ double lambda_s_bisect(const float *vv, int p, double s, uint32_t lo0, uint32_t maxkey, XShared &sh,
                                   uint32_t *lo_out) {
   const int lane = threadIdx.x & 31;
@@ -219,7 +228,7 @@ __device__ double lambda_s_bisect(const float *vv, int p, double s, uint32_t lo0
     const float lam = __uint_as_float(mid);
     float sw, sw2;
     int in_lo, in_hi;          // elements strictly inside (lo, mid) and (mid, hi)
-    for_segments(p, [&](int seg, Seg sg) {
+    for_segments<kOne>(p, [&](int seg, Seg sg) {
       sw = sw2 = 0.0f;
       in_lo = in_hi = 0;
       for (int i = sg.lo + lane; i < sg.hi; i += 32) {
@@ -250,7 +259,7 @@ __device__ double lambda_s_bisect(const float *vv, int p, double s, uint32_t lo0
   double s1, s2;
   float f_unused, f_unused2;
   int kc, i_unused;
-  for_segments(p, [&](int seg, Seg sg) {
+  for_segments<kOne>(p, [&](int seg, Seg sg) {
     float a1 = 0.0f, c1 = 0.0f, a2 = 0.0f, c2 = 0.0f;
     kc = 0;
     for (int i = sg.lo + lane; i < sg.hi; i += 32) {
@@ -298,6 +307,7 @@ struct XOp {
 
 // Pass A (||w||_2^2 and nnz of the unnormalised result w), the Table 3 value, pass B (x = w /
 // ||w||_2 and the support list in index order) and the per-start outputs, over vv[0 .. len).
+template <bool kOne>
 __device__ void xstep_finish(const XstepArgs &a, int c, const float *vv, int len, const XOp &op, float *x,
                              StartState st, int *sup_idx, float *sup_val, Ctrl *ctrl, XShared &sh) {
   const int lane = threadIdx.x & 31;
@@ -305,7 +315,7 @@ __device__ void xstep_finish(const XstepArgs &a, int c, const float *vv, int len
 
   // ---- ties (mode 0): offsets of each segment's equal keys in index order
   if (op.mode == 0) {
-    for_segments(len, [&](int seg, Seg sg) {
+    for_segments<kOne>(len, [&](int seg, Seg sg) {
       int eq = 0;
       for (int i = sg.lo + lane; i < sg.hi; i += 32) eq += abs_key(vv[i]) == op.K;
       eq = warp_sum_i(eq);
@@ -323,7 +333,7 @@ __device__ void xstep_finish(const XstepArgs &a, int c, const float *vv, int len
     if (op.mode == 1) return vi;
     return copysignf(fabsf(vi) - op.tval, vi);
   };
-  for_segments(len, [&](int seg, Seg sg) {
+  for_segments<kOne>(len, [&](int seg, Seg sg) {
     float part = 0.0f;
     int wnnz = 0;
     int eq_run = sh.eoff[seg];
@@ -363,7 +373,7 @@ __device__ void xstep_finish(const XstepArgs &a, int c, const float *vv, int len
   // ---- pass B
   int *gi = sup_idx ? sup_idx + (int64_t)c * a.cap : nullptr;
   float *gv = sup_val ? sup_val + (int64_t)c * a.cap : nullptr;
-  for_segments(len, [&](int seg, Seg sg) {
+  for_segments<kOne>(len, [&](int seg, Seg sg) {
     int eq_run = sh.eoff[seg];
     int pos = sh.woff[seg];
     for (int base = sg.lo; base < sg.hi; base += 32) {
@@ -378,7 +388,7 @@ __device__ void xstep_finish(const XstepArgs &a, int c, const float *vv, int len
       }
       const float w = (i < sg.hi) ? wval(vi, key, tie_keep) : 0.0f;
       const float xi = w * inv;
-      if (x && i < sg.hi) x[i] = xi;
+      if ((kOne || x) && i < sg.hi) x[i] = xi;
       const unsigned nzb = __ballot_sync(0xffffffffu, xi != 0.0f);
       if (gi && xi != 0.0f) {
         const int q = pos + __popc(nzb & lt_mask);
@@ -416,12 +426,12 @@ __device__ void xstep_finish(const XstepArgs &a, int c, const float *vv, int len
 }
 
 // ---------------------------------------------------------------- full x-step
-// the full x-step of start c (block-wide; vsm: p floats of shared memory, or null to read v from
-// global memory)
+// the full x-step of start c (block-wide; kSmem: by XT threads, with v staged in vsm, p floats of shared
+// memory; kOne: see for_segments)
+template <bool kSmem, bool kOne>
 __device__ void xstep_full_one(const XstepArgs &a_in, int c, const float *__restrict__ V, int64_t ldv,
                                float *__restrict__ X, int64_t ldx, StartState &st, int *__restrict__ sup_idx,
                                float *__restrict__ sup_val, Ctrl *ctrl, float *vsm, XShared &sh) {
-  const bool kSmem = vsm != nullptr;
   const XstepArgs a = xstep_switches(a_in, st.iters ? st.iters[c] : 0);
   const int p = a.p;
   const int lane = threadIdx.x & 31;
@@ -429,7 +439,7 @@ __device__ void xstep_full_one(const XstepArgs &a_in, int c, const float *__rest
   float *x = X ? X + (int64_t)c * ldx : nullptr;   // (null: the support list is all that is wanted)
   const int form = a.form;
   if (kSmem) {
-    for (int i = threadIdx.x; i < p; i += blockDim.x) vsm[i] = vg[i];
+    for (int i = threadIdx.x; i < p; i += XT) vsm[i] = vg[i];
     __syncthreads();
   }
   const float *vv = kSmem ? vsm : vg;
@@ -441,7 +451,7 @@ __device__ void xstep_full_one(const XstepArgs &a_in, int c, const float *__rest
     if (s_int < p) {
       bool whole;
       int eq_total;
-      radix_select(vv, p, s_int, false, sh, &op.K, &whole, &op.need_eq, &eq_total);
+      radix_select<kOne>(vv, p, s_int, false, sh, &op.K, &whole, &op.need_eq, &eq_total);
       op.tnext = __uint_as_float(op.K);
       if (whole) {
         op.tkey = op.K == 0u ? 0u : op.K - 1u;   // keep every key >= the bin's lower bound
@@ -455,7 +465,7 @@ __device__ void xstep_full_one(const XstepArgs &a_in, int c, const float *__rest
     // phi(0) = s ||v||_2^2 - ||v||_1^2 >= 0: the L1 ball is not binding, lambda = 0
     float f1, f2;
     unsigned mk = 0u;
-    for_segments(p, [&](int seg, Seg sg) {
+    for_segments<kOne>(p, [&](int seg, Seg sg) {
       f1 = f2 = 0.0f;
       for (int i = sg.lo + lane; i < sg.hi; i += 32) {
         const float av = fabsf(vv[i]);
@@ -471,7 +481,7 @@ __device__ void xstep_full_one(const XstepArgs &a_in, int c, const float *__rest
     op.mode = 2;
     if ((float)a.s * f2 - f1 * f1 < 0.0f) {
       uint32_t lo;
-      op.gam = lambda_s_bisect(vv, p, a.s, 0u, maxkey, sh, &lo);
+      op.gam = lambda_s_bisect<kOne>(vv, p, a.s, 0u, maxkey, sh, &lo);
       op.tkey = lo;
       op.tval = (float)op.gam;
       op.tnext = op.tval;
@@ -484,7 +494,7 @@ __device__ void xstep_full_one(const XstepArgs &a_in, int c, const float *__rest
       if (j <= p) {
         int ne, et;
         bool whole;
-        radix_select(vv, p, j, true, sh, &tk, &whole, &ne, &et);
+        radix_select<kOne>(vv, p, j, true, sh, &tk, &whole, &ne, &et);
       }
       op.tkey = tk;
       op.tval = __uint_as_float(tk);
@@ -501,23 +511,24 @@ __device__ void xstep_full_one(const XstepArgs &a_in, int c, const float *__rest
       op.tkey = __float_as_uint(op.tval);
     }
   }
-  xstep_finish(a, c, vv, p, op, x, st, sup_idx, sup_val, ctrl, sh);
+  xstep_finish<kOne>(a, c, vv, p, op, x, st, sup_idx, sup_val, ctrl, sh);
 }
 
 // Every pass over all p entries of v (staged in shared memory when it fits), persistent CTAs over
-// the starts that the threshold x-step below left (xfast = 0, or nnz = -1 without xfast).
+// the starts that the threshold x-step below left (xfast = 0, or nnz = -1 without xfast), or over every
+// active start.
 template <bool kSmem>
 __global__ void __launch_bounds__(XT) k_xstep(XstepArgs a_in, const float *__restrict__ V, int64_t ldv, int r,
                                               float *__restrict__ X, int64_t ldx, StartState st,
                                               int *__restrict__ sup_idx, float *__restrict__ sup_val,
-                                              Ctrl *ctrl) {
+                                              Ctrl *ctrl, int every) {
   extern __shared__ float vsm[];
   __shared__ XShared sh;
   for (int c = blockIdx.x; c < r; c += gridDim.x) {
     if (st.status && st.status[c] != ST_ACTIVE) continue;
-    if (st.xfast ? st.xfast[c] != 0 : st.nnz[c] != -1) continue;
+    if (!every && (st.xfast ? st.xfast[c] != 0 : st.nnz[c] != -1)) continue;
     __syncthreads();   // (every thread has read the mark; shared memory is reused from start to start)
-    xstep_full_one(a_in, c, V, ldv, X, ldx, st, sup_idx, sup_val, ctrl, kSmem ? vsm : nullptr, sh);
+    xstep_full_one<kSmem, true>(a_in, c, V, ldv, X, ldx, st, sup_idx, sup_val, ctrl, vsm, sh);
     if (threadIdx.x == 0 && st.xfast) st.xfast[c] = 2;
     __syncthreads();
   }
@@ -555,7 +566,15 @@ constexpr int kFastCand = 1024;                // listed entries per start
 constexpr int kFastBins = 2048, kFastShift = 17;   // bins of 2^-6 octave below the largest |v_i|
 constexpr int kFastSubsets = 2048;             // disjoint subsets of v whose maxima bound the threshold
 constexpr int kFastAllP = 64;                  // v up to this long: list every nonzero entry
-constexpr int kFastMaxJ = 600;                 // j of the subset maxima: the list stays below kFastCand
+// j of the subset maxima: some 570 entries lie above the bound for 500, 36 in a segment, and rarely more than
+// the 64 that a segment may list (for 600 more than that in every other start)
+constexpr int kFastMaxJ = 500;
+constexpr int kFastMaxNeed = 600;              // selected entries, above last sweep's bound
+// Entries of v per selected one below which the full pass is the faster one: ranks are counted against the
+// whole list, so their cost grows with its square (20 sweeps of 16 starts by T_s, list and full pass:
+// p = 1000, s = 333 1.7 times the time, s = 166 as long; p = 1500, s = 300 1.08, s = 187 0.97; p = 3000,
+// s = 600 1.24, s = 500 1.14, s = 375 0.99)
+constexpr int kFastPerNeed = 6;
 constexpr float kGuess = 0.85f;
 constexpr float kGuessSteady = 0.95f;          // while t holds steady
 constexpr float kGuessLo = 0.6f;
@@ -622,8 +641,60 @@ __device__ __forceinline__ float4 row_load(const Row &r, int q, int hi) {
 // a lower bound of the j-th largest |v_i| from the maxima of 2048 subsets (the entries at q, q + 2048, ...
 // of the row): the lower edge of the histogram bin of the j-th largest maximum.  0 when the bins do not
 // resolve it.
+// lam_s > 0, for lambda_s: the maxima are a sample of v's largest entries, so phi over them tells, but for a
+// few percent, whether lambda_s lies above the bound.  If not for j, a larger one is taken (j becomes it), half as
+// much again each time; if not for kFastMaxJ either, kNoBound: the start's active set is longer than the list, as one
+// pass has shown.  (Sums over whole counts in a fixed order: not a matter of T.)
+constexpr uint32_t kNoBound = 0xFFFFFFFFu;
+__device__ __forceinline__ int bin_of_rank(const unsigned *hist, int j) {
+  // one warp: the first bin, from the largest down, whose running count reaches j (64 bins a step: the
+  // largest maxima lie within a few octaves)
+  const int lane = threadIdx.x & 31;
+  int acc = 0;
+  for (int base = 0; base < kFastBins; base += 64) {
+    const int h0 = (int)hist[base + 2 * lane], h1 = (int)hist[base + 2 * lane + 1];
+    int incl = h0 + h1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    const int before = acc + incl - h0 - h1;
+    const unsigned here = __ballot_sync(0xffffffffu, before < j && j <= acc + incl);
+    if (here) return __shfl_sync(0xffffffffu, base + 2 * lane + (before + h0 >= j ? 0 : 1), __ffs(here) - 1);
+    acc += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  return kFastBins - 1;
+}
+// keys of bins 0 .. bin are above this one; 0 for the last bin (it holds all smaller keys)
+__device__ __forceinline__ uint32_t bin_edge(uint32_t top, int bin) {
+  const uint32_t down = (uint32_t)(bin + 1) << kFastShift;
+  return bin >= kFastBins - 1 || down >= top ? 0u : top - down;
+}
+__device__ __forceinline__ bool root_above(const unsigned *hist, uint32_t top, int bin, float s, int p) {
+  const uint32_t Gk = bin_edge(top, bin);
+  if (Gk == 0u) return true;
+  const int lane = threadIdx.x & 31;
+  const float G = __uint_as_float(Gk);
+  float w1 = 0.0f, w2 = 0.0f;
+  int n = 0;
+  for (int b = lane; b <= bin; b += 32) {
+    const int h = (int)hist[b];
+    const float w = __uint_as_float(top - ((uint32_t)b << kFastShift) - (1u << (kFastShift - 1))) - G;
+    w1 = fmaf((float)h, w, w1);
+    w2 = fmaf((float)h * w, w, w2);
+    n += h;
+  }
+  w1 = warp_sum_f(w1);
+  w2 = warp_sum_f(w2);
+  n = warp_sum_i(n);
+  // of m entries above G, spread over subsets of q entries each, n are their subset's maximum
+  const float q = fmaxf(1.0f, (float)p / kFastSubsets), sub = (float)kFastSubsets;
+  const float m = sub * q * (1.0f - powf(1.0f - (float)n / sub, 1.0f / q));
+  return s * w2 < 1.02f * (m / (float)n) * (w1 * w1);
+}
 template <int T>
-__device__ __forceinline__ uint32_t subset_bound(const Row &row, int j, FastShared<T> &fs) {
+__device__ __forceinline__ uint32_t subset_bound(const Row &row, int &j, float lam_s, FastShared<T> &fs) {
   constexpr int CH = T > 256 ? 4 : 8;          // loads in flight per thread
   // the subsets of a thread: G groups of four, load k of it being group k mod G; with 1024 threads two
   // threads share four
@@ -663,33 +734,40 @@ __device__ __forceinline__ uint32_t subset_bound(const Row &row, int j, FastShar
       for (int e = 0; e < 4; ++e)
         atomicAdd(&fs.u.hist[min((top - m[k][e]) >> kFastShift, (uint32_t)kFastBins - 1u)], 1u);
   }
-  if (threadIdx.x == 0) fs.sh.digit = kFastBins - 1;
   __syncthreads();
-  // one warp: the first bin, from the largest down, whose running count reaches j (64 bins a step: the
-  // largest maxima lie within a few octaves)
   if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    int acc = 0;
-    for (int base = 0; base < kFastBins; base += 64) {
-      const int h0 = (int)fs.u.hist[base + 2 * lane], h1 = (int)fs.u.hist[base + 2 * lane + 1];
-      int incl = h0 + h1;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      const int before = acc + incl - h0 - h1;
-      const bool here = before < j && j <= acc + incl;
-      if (here) fs.sh.digit = base + 2 * lane + (before + h0 >= j ? 0 : 1);
-      if (__any_sync(0xffffffffu, here)) break;
-      acc += __shfl_sync(0xffffffffu, incl, 31);
+    int jn = j, bin = bin_of_rank(fs.u.hist, jn);
+    while (lam_s > 0.0f && bin >= 0 && !root_above(fs.u.hist, top, bin, lam_s, row.end - row.sh)) {
+      const bool longer = jn < kFastMaxJ;
+      jn = min(kFastMaxJ, jn + jn / 2);
+      bin = longer ? bin_of_rank(fs.u.hist, jn) : -1;
+    }
+    if (threadIdx.x == 0) {
+      fs.sh.digit = bin;
+      fs.sh.rem = jn;
     }
   }
   __syncthreads();
-  const uint32_t bin = (uint32_t)fs.sh.digit;
-  // keys of bins 0 .. bin are above top - (bin + 1) 2^kFastShift
-  const uint32_t down = (bin + 1u) << kFastShift;
-  return bin >= (uint32_t)kFastBins - 1u || down >= top ? 0u : top - down;
+  j = fs.sh.rem;
+  return fs.sh.digit < 0 ? kNoBound : bin_edge(top, fs.sh.digit);
+}
+
+// An index segment of more than 1024 entries of v (a sixteenth, as list_above cuts it)
+__device__ __forceinline__ int list_seg(const Row &row) { return ((row.end + XW - 1) / XW + 127) / 128 * 128; }
+
+// Whether the first segment alone holds more entries above a fixed threshold than the list takes: any number
+// of entries may survive one, and a start with too many should go to the full pass without a pass over v
+// (1024 starts of p = 20011, half of v above: 172 us for a whole call of 109 us before).
+template <int T>
+__device__ __forceinline__ bool first_segment_full(const Row &row, uint32_t Gk, FastShared<T> &fs) {
+  if (row.end <= kFastCand) return false;
+  const int hi = min(row.end, list_seg(row));
+  int n = 0;
+  for (int q = 4 * threadIdx.x; q < hi; q += 4 * T) {
+    const float4 e = row_load(row, q, hi);
+    n += (abs_key(e.x) > Gk) + (abs_key(e.y) > Gk) + (abs_key(e.z) > Gk) + (abs_key(e.w) > Gk);
+  }
+  return block_sum_i(n, reinterpret_cast<int *>(fs.sh.red_u)) > kFastSegCap;
 }
 
 // Lists the entries with key > Gk in index order (fs.u.l.cv / ci, *ncand of them) and, for the
@@ -710,7 +788,7 @@ __device__ __forceinline__ bool list_above(const Row &row, uint32_t Gk, bool sum
     lo = min(row.end, w * per);
     hi = min(row.end, lo + per);
   } else {
-    const int seg = ((row.end + XW - 1) / XW + 127) / 128 * 128;
+    const int seg = list_seg(row);
     if (W <= XW) {
       lo = min(row.end, w * FS::kSegs * seg);
       hi = min(row.end, lo + FS::kSegs * seg);
@@ -962,8 +1040,8 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
   const bool lam_form = uses_lam(form), exact = is_pen(form) && !a.calibrate;
   const bool keep_all = uses_T(form) && s_int >= p;
   const int need = uses_T(form) ? s_int : (is_pen(form) && a.calibrate ? s_int + 1 : 1);
-  const bool all = p <= kFastAllP || (p <= kFastCand && (need > kFastMaxJ / 2 || keep_all));
-  if (!all && !exact && (need > kFastMaxJ || keep_all)) return false;
+  const bool all = p <= kFastAllP || (p <= kFastCand && keep_all);
+  if (!all && !exact && (need > kFastMaxNeed || keep_all || need * kFastPerNeed > p)) return false;
   // j of the subset maxima: the active set of lambda_s has about 2 s entries where |v|'s tail is
   // exponential, so 3 s lie below its threshold; never so many that subsets hold several of them
   int j = lam_form ? (int)fminf(3.0f * (float)a.s + 16.0f, (float)kFastMaxJ) : need;
@@ -990,11 +1068,12 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
       }
     }
   };
-  // the zeros are stored while v is read, but for an x over v itself (the x-step of given v, in place):
-  // there once the list is made, which v is read for
+  // the zeros are stored while v is read, but for an x over v itself (the x-step of given v, in place), and
+  // for a fixed threshold, above which there may be any number of entries (and the full pass writes all of
+  // x): there once the list is made, which v is read for
   const float *vrow = V + (int64_t)c * ldv;
-  const bool over_v = x && x < vrow + p && vrow < x + p;
-  if (x && !over_v) clear_x();
+  const bool late = (x < vrow + p && vrow < x + p) || (exact && !listed);
+  if (x && !late) clear_x();
 
   // ---- a bound, the list above it, and the check (block-uniform throughout)
   int buf = 0, ncand = 0;
@@ -1010,11 +1089,14 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
     gam = a.per_start_thr ? q0.gamma : a.gamma_fixed;
   }
   for (;;) {
-    if (how == kExact) Gk = __float_as_uint(thr);
-    else if (how == kAll) Gk = 0u;
+    if (how == kExact) {
+      Gk = __float_as_uint(thr);
+      if (!listed && first_segment_full<T>(row, Gk, fs)) return false;
+    } else if (how == kAll) Gk = 0u;
     else if (how == kHigh) Gk = __float_as_uint((steady && !a.ordered ? kGuessSteady : kGuess) * tprev);
     else if (how == kLow) Gk = __float_as_uint(kGuessLo * tprev);
-    else Gk = subset_bound<T>(row, j, fs);
+    else Gk = j <= kFastMaxJ ? subset_bound<T>(row, j, lam_form ? (float)a.s : 0.0f, fs) : kNoBound;
+    if (Gk == kNoBound) return false;
     float f1 = 0.0f, f2 = 0.0f;
     const bool fits = list_above<T>(row, Gk, lam_form, fs, buf, &ncand, &f1, &f2);
     // phi(0) >= 0, every entry survives: no bound above 0 can serve.  (The sums' last bits depend on T: with
@@ -1049,7 +1131,7 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
     }
     __syncthreads();                 // the lists are reused
   }
-  if (over_v) clear_x();             // (every thread has read its part of v: the list's barrier)
+  if (x && late) clear_x();          // (every thread has read its part of v: the list's barrier)
 
   // ---- the operator on the list: which entries survive, as
   //   select: rank < need (T_s; ties at the threshold: the lower indices), or key above the threshold
@@ -1169,7 +1251,7 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
       for (int t = threadIdx.x; t < nnz; t += T) fs.u.by_index[fs.a.s.idx[t]] = fs.a.s.val[t];
       __syncthreads();
     }
-    for_segments(p, [&](int sgi, Seg sg) {
+    for_segments<false>(p, [&](int sgi, Seg sg) {
       float part = 0.0f;
       if (by_index) {
         for (int i = sg.lo + lane; i < sg.hi; i += 32) part = fmaf(fs.u.by_index[i], fs.u.by_index[i], part);
@@ -1237,11 +1319,12 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
 // false) or a mark for k_xstep / k_g_xstep (xfast = 0; without xfast, nnz = -1).  The starts that
 // needed the full pass are counted in ctrl->n_full: the host queues the full kernel, which stages v in
 // shared memory, only for sweeps after some start needed it.
+template <bool kOne>
 __device__ __noinline__ void xstep_full_global(const XstepArgs &a, int c, const float *__restrict__ V, int64_t ldv,
                                                float *__restrict__ X, int64_t ldx, StartState st,
                                                int *__restrict__ sup_idx, float *__restrict__ sup_val, Ctrl *ctrl,
                                                XShared &sh) {
-  xstep_full_one(a, c, V, ldv, X, ldx, st, sup_idx, sup_val, ctrl, nullptr, sh);
+  xstep_full_one<false, kOne>(a, c, V, ldv, X, ldx, st, sup_idx, sup_val, ctrl, nullptr, sh);
 }
 template <int T>
 __device__ __forceinline__ void xstep_start(const XstepArgs &a, int c, const float *__restrict__ V, int64_t ldv,
@@ -1252,7 +1335,7 @@ __device__ __forceinline__ void xstep_start(const XstepArgs &a, int c, const flo
   if (ctrl && threadIdx.x == 0) atomicAdd(&ctrl->n_full, 1);
   __syncthreads();
   if (!defer) {
-    xstep_full_global(a, c, V, ldv, X, ldx, st, sup_idx, sup_val, ctrl, fs.sh);
+    xstep_full_global<T == XT>(a, c, V, ldv, X, ldx, st, sup_idx, sup_val, ctrl, fs.sh);
     if (threadIdx.x == 0 && st.xfast) st.xfast[c] = 2;
   } else if (threadIdx.x == 0) {
     if (st.xfast) st.xfast[c] = 0;
@@ -1317,8 +1400,7 @@ __global__ void __launch_bounds__(XT, 2) k_g_xstep(const GProb *__restrict__ P, 
     StartState st = q.st;
     if (st.status[c] != ST_ACTIVE || st.xfast[c] != 0) continue;
     __syncthreads();   // (every thread has read the mark; shared memory is reused from start to start)
-    xstep_full_one(q.xa, c, q.V, q.ldX, q.X, q.ldX, st, q.sup_idx, q.sup_val, q.ctrl[parity], kSmem ? vsm : nullptr,
-                   sh);
+    xstep_full_one<kSmem, true>(q.xa, c, q.V, q.ldX, q.X, q.ldX, st, q.sup_idx, q.sup_val, q.ctrl[parity], vsm, sh);
     if (threadIdx.x == 0) st.xfast[c] = 2;
     __syncthreads();
   }
@@ -1547,7 +1629,7 @@ __global__ void __launch_bounds__(T) k_small_sweeps(XstepArgs xa, const float *_
     else __syncthreads();
     if (!xstep_fast_one<T>(xa, 0, v, 0, nullptr, 0, sl, load_state(sl, 0), li, lv, nullptr, fs)) {
       __syncthreads();
-      xstep_full_one(xa, 0, v, 0, nullptr, 0, sl, li, lv, nullptr, nullptr, fs.sh);
+      xstep_full_one<false, false>(xa, 0, v, 0, nullptr, 0, sl, li, lv, nullptr, nullptr, fs.sh);
       if (threadIdx.x == 0) ss.xfast = 2;
     }
     __syncthreads();
@@ -1609,34 +1691,52 @@ cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, const
                             sup_val, sweeps);
 }
 
+// The x-step of given v has no last threshold to start from, so its list costs a pass for the bound and one
+// for the list.  It pays, against the full pass of every start in one launch, for lambda_s with s up to 150
+// (above, the list often does not hold the active set), and for T_s and the Section 4.1 rule with few
+// selected entries: a 25th of v (a 10th when starts outnumber two per SM) and at most kFastMaxJ.  Whole
+// calls, full pass and list: one start, p = 1500, T_s, s = 200 28 and 31 us, s = 50 27 and 28; p = 6000, s = 500 33
+// and 39, s = 200 35 and 30; 1024 starts, p = 3000, s = 400 70 and 67, s = 500 68 and 86.  A fixed threshold is the
+// list's bound itself.
+bool xstep_list_pays(int form, double s, bool calibrate, int64_t p, int64_t r, int sms) {
+  if (uses_lam(form)) return s <= 150.0;
+  if (is_pen(form) && !calibrate) return true;
+  const int64_t need = (int64_t)s + (calibrate ? 1 : 0);
+  return need <= kFastMaxJ && need * (r <= 2 * (int64_t)sms ? 25 : 10) <= p;
+}
+
 cudaError_t launch_xstep(XstepArgs a, const float *V, int64_t ldv, int r, float *X, int64_t ldx,
                          StartState s, int *sup_idx, float *sup_val, Ctrl *ctrl, Ctrl *ctrl_read, int *act,
-                         int *rank, bool defer, int *flags, int nflags, cudaStream_t st) {
-  const int sms = sm_count(), d = defer ? 1 : 0;
+                         int *rank, XFull full, int *flags, int nflags, cudaStream_t st) {
+  const int sms = sm_count(), d = full == XFull::kAfter ? 1 : 0;
   if (sms < 1) return cudaErrorInvalidDevice;
-  int *al = defer ? nullptr : act;
+  int *al = d ? nullptr : act;
 #define SPCA_FAST(T)                                                                                             \
   k_xstep_fast<T><<<r, T, 0, st>>>(a, V, ldv, r, X, ldx, s, sup_idx, sup_val, ctrl, ctrl_read, al, rank, d, flags, nflags)
-  switch (fast_threads(r, a.p, sms)) {
-    case 1024: SPCA_FAST(1024); break;
-    case 512: SPCA_FAST(512); break;
-    case 256: SPCA_FAST(256); break;
-    default: SPCA_FAST(128); break;
+  cudaError_t e = cudaSuccess;
+  if (full != XFull::kAlone) {
+    switch (fast_threads(r, a.p, sms)) {
+      case 1024: SPCA_FAST(1024); break;
+      case 512: SPCA_FAST(512); break;
+      case 256: SPCA_FAST(256); break;
+      default: SPCA_FAST(128); break;
+    }
+    e = cudaGetLastError();
+    if (e != cudaSuccess || full == XFull::kInside) return e;
   }
 #undef SPCA_FAST
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || !defer) return e;
   // the full pass for the starts left: persistent CTAs (as many as fit), so that a sweep in which no
   // start needs it costs one short launch
   const size_t bytes = (size_t)a.p * sizeof(float);
+  const int every = full == XFull::kAlone ? 1 : 0;
   if (bytes <= (size_t)XSTEP_SMEM_MAX) {
     static const cudaError_t configured =
         cudaFuncSetAttribute(k_xstep<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, XSTEP_SMEM_MAX);
     if (configured != cudaSuccess) return configured;
     const int per_sm = bytes <= 100u * 1024u ? 2 : 1;
-    k_xstep<true><<<min(r, per_sm * sms), XT, bytes, st>>>(a, V, ldv, r, X, ldx, s, sup_idx, sup_val, ctrl);
+    k_xstep<true><<<min(r, per_sm * sms), XT, bytes, st>>>(a, V, ldv, r, X, ldx, s, sup_idx, sup_val, ctrl, every);
   } else {
-    k_xstep<false><<<min(r, 2 * sms), XT, 0, st>>>(a, V, ldv, r, X, ldx, s, sup_idx, sup_val, ctrl);
+    k_xstep<false><<<min(r, 2 * sms), XT, 0, st>>>(a, V, ldv, r, X, ldx, s, sup_idx, sup_val, ctrl, every);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess || !act) return e;

@@ -1048,16 +1048,19 @@ int spca_xstep(spca_handle *h, int form, double s, double gamma, int calibrate, 
   a.cap = 0; a.sparse_cap = (int)h->p;
   StartState st{};
   st.nnz = nnz; st.F = F; st.gamma = thr;
-  // starts that need the full pass are left to a kernel of their own (v in shared memory), but for short
-  // rows, whose full pass costs less inside the first kernel than a second launch (one start of p = 600:
-  // 46 -> 42 us a call; p = 3000: 51 -> 48 us)
-  // (and for an x over v but not in place, whose full pass needs v staged)
+  // starts that need the full pass take it inside the first kernel, whose CTAs are large while there is an SM
+  // for each (16 starts of p = 20011, lambda_s, s = 50, a few of them beyond the list: 112 us with a second launch,
+  // 91 so; none beyond it: 42 and 38), and else in a kernel of its own with v in shared memory, but for
+  // short rows.  An x over v but not in place needs v staged in any case.
   const float *v_end = V + (int64_t)(r - 1) * ldv + h->p, *x_end = X + (int64_t)(r - 1) * ldx + h->p;
   const bool overlap = X < v_end && V < x_end && !(X == V && ldx == ldv);
-  const bool defer = overlap || h->p > 8192 || xstep_may_need_full(form, s, a.calibrate != 0);
+  const bool apart = overlap || (r > h->sms && (h->p > 8192 || xstep_may_need_full(form, s, a.calibrate != 0)));
+  const XFull full = !xstep_list_pays(form, s, a.calibrate != 0, h->p, r, h->sms) ? XFull::kAlone
+                     : apart                                                      ? XFull::kAfter
+                                                                                  : XFull::kInside;
   RC(enter(h));
-  CK(timed(h, SPCA_K_XSTEP, defer ? 2 : 1, [&] {
-    return launch_xstep(a, V, ldv, r, X, ldx, st, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, defer,
+  CK(timed(h, SPCA_K_XSTEP, full == XFull::kAfter ? 2 : 1, [&] {
+    return launch_xstep(a, V, ldv, r, X, ldx, st, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, full,
                         nullptr, 0, h->stream);
   }));
   CK(cudaStreamSynchronize(h->stream));
@@ -1291,7 +1294,8 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
     // the stopped slots have their next starts)
     CK(timed(h, SPCA_K_XSTEP, pl.full ? (otf ? 2 : 3) : 1, [&] {
       return launch_xstep(xk, h->V, h->ldX, r, h->X, h->ldX, S, h->sup_idx, h->sup_val, nxt, cur,
-                          otf ? nullptr : h->act, h->rank, pl.full, sk.flags, sk.flags ? 2 * sk.slots : 0, st);
+                          otf ? nullptr : h->act, h->rank, pl.full ? XFull::kAfter : XFull::kInside, sk.flags,
+                          sk.flags ? 2 * sk.slots : 0, st);
     }));
     if (otf) {
       // stopped slots: archive their start, give them the next starts (Section 4.3)

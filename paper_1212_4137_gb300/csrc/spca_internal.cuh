@@ -587,6 +587,8 @@ cudaError_t launch_active_list(const int *status, const int *nnz, int r, int *ac
 inline bool xstep_may_need_full(int form, double s, bool target) {
   return is_pen(form) && !target ? true : s > (uses_lam(form) ? 150.0 : 500.0);
 }
+// whether the list pays in the x-step of given v (else the full pass of every start)
+bool xstep_list_pays(int form, double s, bool calibrate, int64_t p, int64_t r, int sms);
 // small problems (n p <= kSmallEntries, at most two starts per SM; x, u, y and v in shared memory): every
 // sweep of every start in one launch, a cluster of CTAs per start; sweeps = the most sweeps a start may run.
 // The lines: 20 sweeps of 1, 16 and 60 starts at n p = 1e6 321, 418 and 595 us (by sweeps 463, 544, 789), of
@@ -598,12 +600,15 @@ cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, const
                                 cudaStream_t st);
 // x-step (S3..S6), objective F, stopping rule, support lists, and (act given) the next sweep's active
 // list in *ctrl, which must be zero before; ctrl_read is cleared (see launch_active_list), and so are the
-// nflags ints at flags (the stream-K flags of the next contraction; null: none).  defer: a
-// second kernel runs the full pass of the starts that need it, with v in shared memory (else the
-// first one does, from global memory)
+// nflags ints at flags (the stream-K flags of the next contraction; null: none).
+enum class XFull {
+  kInside,   // the first kernel runs the full pass of the starts that need it, from global memory
+  kAfter,    // a second kernel does, with v in shared memory
+  kAlone     // that kernel alone, for every start (the x-step of given v: no list, flags or control words)
+};
 cudaError_t launch_xstep(XstepArgs a, const float *V, int64_t ldv, int r, float *X, int64_t ldx,
                          StartState s, int *sup_idx, float *sup_val, Ctrl *ctrl, Ctrl *ctrl_read, int *act,
-                         int *rank, bool defer, int *flags, int nflags, cudaStream_t st);
+                         int *rank, XFull full, int *flags, int nflags, cudaStream_t st);
 
 // a7: Table 1 objective in FP64 for every start, with u of each start into U, and the best start (of the
 // objective, or of the explained variance with use_ev); A^T in FP32, or (AT16 given) FP16 rows times their
