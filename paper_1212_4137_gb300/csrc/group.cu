@@ -618,7 +618,9 @@ int finish_members(spca_group *g, const std::vector<Member *> &list) {
     GCK(cudaMemcpyAsync(g->d_active, flags.data(), sizeof(int) * np, cudaMemcpyHostToDevice, st));
     done = g->d_active;   // (the counts it held have been read)
   }
-  GCK(launch_g_finish(g->dP, g->d_start_prob, g->R, np, g->max_n, g->max_p, done, st));
+  int max_chunks = 1;
+  for (const Member *m : list) max_chunks = std::max(max_chunks, finalise_chunks(m->n, m->r));
+  GCK(launch_g_finish(g->dP, g->d_start_prob, g->R, np, g->max_n, g->max_p, max_chunks, done, st));
   for (size_t k = 0; k < list.size(); ++k) {
     const Member &m = *list[k];
     const GProb &d = m.d;

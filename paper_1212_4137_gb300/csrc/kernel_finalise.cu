@@ -4,6 +4,7 @@
 // lower index), and y(x) and the support of the best x.
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "block_util.cuh"
 #include "spca_internal.cuh"
@@ -11,10 +12,21 @@
 namespace spca {
 
 namespace {
-constexpr int FT = 128;            // threads per CTA, four rows of A each
-constexpr int FR = 4 * FT;         // rows per chunk
+constexpr int FT = 128;            // threads per CTA, four rows of A each, or one
 }  // namespace
-int finalise_chunks(int64_t n) { return (int)((n + FR - 1) / FR); }
+// The rows of a chunk of an n-row problem of r starts: 4 FT where those chunks fill the chip, four on each of
+// about 150 SMs, and their threads (n > 2 FT), else FT.  A start's columns are one chain of loads and dependent
+// sums, twice as long for four rows of a thread as for one.  Supports of 9000 columns, four rows and one: n = 100, one
+// start 1044 and 342 us (524 before there were four); n = 2000, 16 starts 2621 and 801, 150 starts (600 chunks)
+// 2469 and 2010; n = 9000, 64 starts (1152) 2834 and 3645; n = 500, 1024 starts 2448 and 3163.
+// (By the problem's own starts and rows: in a group a problem has the same chunks alone and in any mix.)
+static __host__ __device__ inline int finalise_rows(int64_t n, int64_t r) {
+  return r * ((n + 4 * FT - 1) / (4 * FT)) >= 608 && n > 2 * FT ? 4 * FT : FT;
+}
+int finalise_chunks(int64_t n, int64_t r) {
+  const int rows = finalise_rows(n, r);
+  return (int)((n + rows - 1) / rows);
+}
 
 // argmax over r starts of f (or of the explained variance), ties to the lower index; written by other
 // CTAs of the same launch, so read from L2
@@ -43,18 +55,27 @@ __device__ __forceinline__ void best_body(const double *val, int r, int *best) {
   }
 }
 
-// four consecutive entries of a column of A (a row of A^T): FP32, or FP16 times the column's
+// R consecutive entries of a column of A (a row of A^T): FP32, or FP16 times the column's
 // power-of-two inverse scale (the 16-bit copy of a resident handle; exact in FP32)
-__device__ __forceinline__ float4 col4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
-__device__ __forceinline__ float4 col4(const __half *p) {
+template <int R>
+struct ColVec {
+  float v[R];
+};
+__device__ __forceinline__ void col_load(ColVec<4> &a, const float *p) {
+  const float4 t = __ldg(reinterpret_cast<const float4 *>(p));
+  a.v[0] = t.x; a.v[1] = t.y; a.v[2] = t.z; a.v[3] = t.w;
+}
+__device__ __forceinline__ void col_load(ColVec<4> &a, const __half *p) {
   const uint2 raw = __ldg(reinterpret_cast<const uint2 *>(p));
   const __half2 *h = reinterpret_cast<const __half2 *>(&raw);
-  const float2 a = __half22float2(h[0]), b = __half22float2(h[1]);
-  return make_float4(a.x, a.y, b.x, b.y);
+  const float2 lo = __half22float2(h[0]), hi = __half22float2(h[1]);
+  a.v[0] = lo.x; a.v[1] = lo.y; a.v[2] = hi.x; a.v[3] = hi.y;
 }
+__device__ __forceinline__ void col_load(ColVec<1> &a, const float *p) { a.v[0] = __ldg(p); }
+__device__ __forceinline__ void col_load(ColVec<1> &a, const __half *p) { a.v[0] = __half2float(__ldg(p)); }
 
 // Chunk b (of nch) of start c: u_i = sum_t x_{j_t} A[i, j_t] over the support (compensated FP32 pairs),
-// four rows per thread as one vector with eight columns' loads in flight, and the chunk's FP64 sum of
+// R rows per thread as one vector with eight columns' loads in flight, and the chunk's FP64 sum of
 // |u_i| or u_i^2, whichever the formulation's variance takes.  The start's last chunk then adds the
 // partial sums in a fixed order and gives f (Table 1) and the explained variance; the last start finds
 // the best one.  cnt: r + 1 zeroed counters, left zeroed.
@@ -63,7 +84,7 @@ __device__ __forceinline__ float4 col4(const __half *p) {
 // entry) and the gather through L2 bound it.
 // 1024 starts of 50 nonzeros, n = 5000: 156 us (a row per thread, one load in flight, both norms, and
 // three launches: 353 us); 12 members of a group: 42 us (342 us as launches of their own).
-template <typename T>
+template <int R, typename T>
 __device__ __forceinline__ void finalise_body(int form, const T *__restrict__ AT, const float *__restrict__ row_inv,
                                               int64_t ldat, int n, const int *__restrict__ sup_idx,
                                               const float *__restrict__ sup_val, int cap, const StartState &st, int r,
@@ -74,16 +95,14 @@ __device__ __forceinline__ void finalise_body(int form, const T *__restrict__ AT
   __shared__ float sinv[FT];
   __shared__ double red[32];
   __shared__ int state;
-  const int i4 = (b * FT + threadIdx.x) * 4;
+  const int i0 = (b * FT + threadIdx.x) * R;
   const int nnz = st.nnz[c];
   const int *gi = sup_idx + (int64_t)c * cap;
   const float *gv = sup_val + (int64_t)c * cap;
-  F32Pair acc[4];
-  auto step = [&](float x, float inv, const float4 &a) {
-    f32pair_fma(acc[0], x, a.x * inv);
-    f32pair_fma(acc[1], x, a.y * inv);
-    f32pair_fma(acc[2], x, a.z * inv);
-    f32pair_fma(acc[3], x, a.w * inv);
+  F32Pair acc[R];
+  auto step = [&](float x, float inv, const ColVec<R> &a) {
+#pragma unroll
+    for (int q = 0; q < R; ++q) f32pair_fma(acc[q], x, a.v[q] * inv);
   };
   for (int t0 = 0; t0 < nnz; t0 += FT) {
     __syncthreads();
@@ -95,26 +114,29 @@ __device__ __forceinline__ void finalise_body(int form, const T *__restrict__ AT
     }
     __syncthreads();
     const int m = min(FT, nnz - t0);
-    if (i4 < n) {              // (the columns are padded to a multiple of 8 rows)
-      const T *base = AT + i4;
+    if (i0 < n) {              // (the columns are padded to a multiple of 8 rows)
+      const T *base = AT + i0;
+      ColVec<R> a[8];
       int t = 0;
       for (; t + 8 <= m; t += 8) {
-        float4 a[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) a[q] = col4(base + (int64_t)sidx[t + q] * ldat);
+        for (int q = 0; q < 8; ++q) col_load(a[q], base + (int64_t)sidx[t + q] * ldat);
 #pragma unroll
         for (int q = 0; q < 8; ++q) step(sval[t + q], sinv[t + q], a[q]);
       }
-      for (; t < m; ++t) step(sval[t], sinv[t], col4(base + (int64_t)sidx[t] * ldat));
+      for (; t < m; ++t) {
+        col_load(a[0], base + (int64_t)sidx[t] * ldat);
+        step(sval[t], sinv[t], a[0]);
+      }
     }
   }
   const bool l1 = is_l1_var(form);
   double part = 0.0;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    if (i4 + q < n) {
+  for (int q = 0; q < R; ++q) {
+    if (i0 + q < n) {
       const double u = f32pair_value(acc[q]);
-      U[(int64_t)c * ldu + i4 + q] = (float)u;
+      U[(int64_t)c * ldu + i0 + q] = (float)u;
       part = l1 ? part + fabs(u) : fma(u, u, part);
     }
   }
@@ -153,29 +175,29 @@ __device__ __forceinline__ void finalise_body(int form, const T *__restrict__ AT
   if (state) best_body(use_ev ? st.ev : st.f, r, best);
 }
 
-template <typename T>
+template <int R, typename T>
 __global__ void __launch_bounds__(FT) k_finalise(int form, const T *__restrict__ AT, const float *__restrict__ row_inv,
                                                  int64_t ldat, int n, const int *__restrict__ sup_idx,
                                                  const float *__restrict__ sup_val, int cap, StartState st,
                                                  float *__restrict__ U, int64_t ldu, double *partials, int *cnt,
                                                  int use_ev, int *best) {
-  finalise_body(form, AT, row_inv, ldat, n, sup_idx, sup_val, cap, st, (int)gridDim.x, U, ldu, partials, cnt, use_ev,
-                best, (int)blockIdx.x, (int)blockIdx.y, (int)gridDim.y);
+  finalise_body<R>(form, AT, row_inv, ldat, n, sup_idx, sup_val, cap, st, (int)gridDim.x, U, ldu, partials, cnt,
+                   use_ev, best, (int)blockIdx.x, (int)blockIdx.y, (int)gridDim.y);
 }
 
 cudaError_t launch_finalise(int form, const float *AT, const __half *AT16, const float *at_inv, int64_t ldat, int n,
                             StartState s, int r, float *U, int64_t ldu, const int *sup_idx, const float *sup_val,
                             int cap, double *partials, int *cnt, int use_ev, int *best, cudaStream_t st) {
-  const int nch = finalise_chunks(n);
+  const int rows = finalise_rows(n, r), nch = finalise_chunks(n, r);
   if (nch > 65535) return cudaErrorInvalidValue;   // grid y limit
   const dim3 grid((unsigned)r, (unsigned)nch);
+  auto go = [&](auto kern, const auto *at, const float *inv) {
+    kern<<<grid, FT, 0, st>>>(form, at, inv, ldat, n, sup_idx, sup_val, cap, s, U, ldu, partials, cnt, use_ev, best);
+    return cudaGetLastError();
+  };
   if (AT16)
-    k_finalise<__half><<<grid, FT, 0, st>>>(form, AT16, at_inv, ldat, n, sup_idx, sup_val, cap, s, U, ldu, partials,
-                                            cnt, use_ev, best);
-  else
-    k_finalise<float><<<grid, FT, 0, st>>>(form, AT, nullptr, ldat, n, sup_idx, sup_val, cap, s, U, ldu, partials, cnt,
-                                           use_ev, best);
-  return cudaGetLastError();
+    return rows == FT ? go(k_finalise<1, __half>, AT16, at_inv) : go(k_finalise<4, __half>, AT16, at_inv);
+  return rows == FT ? go(k_finalise<1, float>, AT, nullptr) : go(k_finalise<4, float>, AT, nullptr);
 }
 
 // the same for the finishing members of a group (done[i] != 0; all when null), one launch
@@ -184,14 +206,22 @@ __global__ void __launch_bounds__(FT) k_g_finalise(const GProb *__restrict__ P, 
   const int i = prob[blockIdx.x];
   if (done && !done[i]) return;
   const GProb &q = P[i];
-  const int nch = (q.n + FR - 1) / FR, c = (int)blockIdx.x - q.start0;
+  const int rows = finalise_rows(q.n, q.r), nch = (q.n + rows - 1) / rows, c = (int)blockIdx.x - q.start0;
   if ((int)blockIdx.y >= nch) return;
-  if (q.AT16)
-    finalise_body(q.form, q.AT16, q.at_inv, q.ldAT, q.n, q.sup_idx, q.sup_val, q.p, q.st, q.r, q.U, q.ldU, q.partials,
-                  q.fin_cnt, q.use_ev, q.best, c, (int)blockIdx.y, nch);
-  else
-    finalise_body(q.form, q.AT32, static_cast<const float *>(nullptr), q.ldAT, q.n, q.sup_idx, q.sup_val, q.p, q.st,
-                  q.r, q.U, q.ldU, q.partials, q.fin_cnt, q.use_ev, q.best, c, (int)blockIdx.y, nch);
+  auto go = [&](auto rows_each, const auto *at, const float *inv) {
+    finalise_body<decltype(rows_each)::value>(q.form, at, inv, q.ldAT, q.n, q.sup_idx, q.sup_val, q.p, q.st, q.r, q.U,
+                                              q.ldU, q.partials, q.fin_cnt, q.use_ev, q.best, c, (int)blockIdx.y, nch);
+  };
+  using One = std::integral_constant<int, 1>;
+  using Four = std::integral_constant<int, 4>;
+  if (q.AT16) {
+    if (rows == FT) go(One{}, q.AT16, q.at_inv);
+    else go(Four{}, q.AT16, q.at_inv);
+  } else {
+    const float *none = nullptr;
+    if (rows == FT) go(One{}, q.AT32, none);
+    else go(Four{}, q.AT32, none);
+  }
 }
 
 // argmax over starts of f (or of the explained variance), ties to the lower index
@@ -294,11 +324,10 @@ __global__ void __launch_bounds__(OT_) k_g_best_outputs(const GProb *__restrict_
                     q.y_out, q.x_out, q.support_out, q.nnz_out, (int)blockIdx.x, (int)gridDim.x);
 }
 
-cudaError_t launch_g_finish(const GProb *P, const int *prob, int R, int np, int max_n, int max_p, const int *done,
-                            cudaStream_t st) {
-  const int nch = finalise_chunks(max_n);
-  if (nch > 65535) return cudaErrorInvalidValue;
-  k_g_finalise<<<dim3((unsigned)R, (unsigned)nch), FT, 0, st>>>(P, prob, done);
+cudaError_t launch_g_finish(const GProb *P, const int *prob, int R, int np, int max_n, int max_p, int max_chunks,
+                            const int *done, cudaStream_t st) {
+  if (max_chunks > 65535) return cudaErrorInvalidValue;
+  k_g_finalise<<<dim3((unsigned)R, (unsigned)max_chunks), FT, 0, st>>>(P, prob, done);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_g_best_outputs<<<dim3((unsigned)output_ctas(max_n, max_p), (unsigned)np), OT_, 0, st>>>(P, done);

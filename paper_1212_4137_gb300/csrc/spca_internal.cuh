@@ -459,7 +459,7 @@ struct GProb {
   int64_t ld0;
   uint64_t key;
   double gamma0;
-  // the finalise: scratch (r * finalise_chunks(n) doubles; r + 1 zeroed counters) and outputs
+  // the finalise: scratch (r * finalise_chunks(n, r) doubles; r + 1 zeroed counters) and outputs
   double *partials;
   int *fin_cnt;
   int use_ev, *best;
@@ -495,9 +495,10 @@ cudaError_t launch_copy_list(const CopyDesc *list, int count, cudaStream_t st);
 cudaError_t launch_g_ctrl(const GProb *P, int np, int parity, int *out, cudaStream_t st);
 cudaError_t launch_g_gather(const GProb *P, const int *prob, int R, int max_n, cudaStream_t st);
 cudaError_t launch_g_ystep(const GProb *P, const int *prob, int R, cudaStream_t st);
-// the finalise and the outputs of the members with done[i] != 0 (all when null)
-cudaError_t launch_g_finish(const GProb *P, const int *prob, int R, int np, int max_n, int max_p, const int *done,
-                            cudaStream_t st);
+// the finalise and the outputs of the members with done[i] != 0 (all when null); max_chunks: their most
+// finalise_chunks
+cudaError_t launch_g_finish(const GProb *P, const int *prob, int R, int np, int max_n, int max_p, int max_chunks,
+                            const int *done, cudaStream_t st);
 // (max_p: the longest v; max_p_small: the longest that fits in shared memory, 0 if none; any_large: some v does not;
 // defer: the full pass in kernels of its own, and no active lists, see launch_xstep)
 cudaError_t launch_g_xstep(const GProb *P, const int *prob, int R, int max_p, int max_p_small, bool any_large,
@@ -612,9 +613,9 @@ cudaError_t launch_xstep(XstepArgs a, const float *V, int64_t ldv, int r, float 
 
 // a7: Table 1 objective in FP64 for every start, with u of each start into U, and the best start (of the
 // objective, or of the explained variance with use_ev); A^T in FP32, or (AT16 given) FP16 rows times their
-// power-of-two inverse scale.  partials: r * finalise_chunks(n) doubles of scratch; cnt: r + 1 ints, zero
+// power-of-two inverse scale.  partials: r * finalise_chunks(n, r) doubles of scratch; cnt: r + 1 ints, zero
 // before and after
-int finalise_chunks(int64_t n);
+int finalise_chunks(int64_t n, int64_t r);
 cudaError_t launch_finalise(int form, const float *AT, const __half *AT16, const float *at_inv, int64_t ldat, int n,
                             StartState s, int r, float *U, int64_t ldu, const int *sup_idx, const float *sup_val,
                             int cap, double *partials, int *cnt, int use_ev, int *best, cudaStream_t st);
