@@ -1461,6 +1461,8 @@ cudaError_t launch_g_xstep(const GProb *P, const int *prob, int R, int max_p, in
 // What bounds a sweep is its chain of dependent steps (a round trip to L2 for u, then about 15 barriers).
 // 16 starts, n = 100, p = 500, 40 sweeps: 535 -> 235 us; n = 250, p = 1000, 20 sweeps 1250 -> 240 us
 // (one CTA per start, u by whole rows of A, u, y and v through memory before).
+// A start that has swept goes on from its support list and state: the sweeps may be cut into several launches,
+// with the same bits.
 
 // for every o < out: put(o, sum over k of w[k] M[row(k) ld + o]), row(k) = idx[k] or k: a thread per four
 // outputs and slice of the k (part: 4 T floats for the slices' sums)
@@ -1567,10 +1569,12 @@ __global__ void __launch_bounds__(T) k_small_sweeps(XstepArgs xa, const float *_
   float *as = vb + small_words<T>(n, p, ctas);
   const int pc = small_cols(p, ctas), j0 = rank * pc, mine = max(0, min(pc, p - j0));
   float *x = X + (int64_t)c * ldx;
-  // x^(0), the start's state, this CTA's columns of A
-  for (int j = threadIdx.x; j < p; j += T) {
-    lv[j] = x[j];
-    li[j] = j;
+  // x^(0), or the support list of a start that has swept; the start's state, this CTA's columns of A
+  const bool fresh = st.iters[c] == 0;
+  const int nnz0 = fresh ? p : st.nnz[c];
+  for (int j = threadIdx.x; j < nnz0; j += T) {
+    lv[j] = fresh ? x[j] : sup_val[(int64_t)c * p + j];
+    li[j] = fresh ? j : sup_idx[(int64_t)c * p + j];
   }
   if (a_smem) {
     for (int q = threadIdx.x; q < n * (pc / 4); q += T) {
@@ -1580,7 +1584,7 @@ __global__ void __launch_bounds__(T) k_small_sweeps(XstepArgs xa, const float *_
     }
   }
   if (threadIdx.x == 0) {
-    ss.status = st.status[c]; ss.iters = st.iters[c]; ss.nnz = p; ss.xfast = st.xfast[c];
+    ss.status = st.status[c]; ss.iters = st.iters[c]; ss.nnz = nnz0; ss.xfast = st.xfast[c];
     ss.F = st.F[c]; ss.F_prev = st.F_prev[c]; ss.gamma = st.gamma[c];
     ss.thr = st.thr[c]; ss.tprev = st.tprev[c];
   }
@@ -1591,7 +1595,7 @@ __global__ void __launch_bounds__(T) k_small_sweeps(XstepArgs xa, const float *_
   if (ss.status != ST_ACTIVE) return;   // (the same in every CTA of the cluster)
   for (int k = 0; k < sweeps; ++k) {
     float *v = vb + (ctas > 1 && (k & 1) ? p4 : 0);
-    small_product<T>(AT, ldat, k == 0 ? nullptr : li, lv, ss.nnz, n, part, [&](int i, float t) { u[i] = t; });
+    small_product<T>(AT, ldat, fresh && k == 0 ? nullptr : li, lv, ss.nnz, n, part, [&](int i, float t) { u[i] = t; });
     __syncthreads();
     // y-step
     if (threadIdx.x == 0) ss.iters += 1;

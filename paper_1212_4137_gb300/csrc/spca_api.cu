@@ -1351,18 +1351,22 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
   // engine keeps the per-sweep kernels)
   const bool small = P.engine == SPCA_ENGINE_AUTO && engine == SPCA_ENGINE_SIMT && !h->sparse && !otf && L == 0 &&
                      h->defl_k == 0 && h->A32 && small_sweeps_fit(h->n, h->p, r);
-  if (small) {
+  // (with a time limit in launches of check_every sweeps, between which the clock and the starts are looked at)
+  for (int64_t k0 = 0, piece = P.timeout_us > 0 ? check_every : max_iter; small && k0 < max_iter; k0 += piece) {
     CK(timed(h, SPCA_K_XSTEP, 1, [&] {
       return launch_small_sweeps(xa, h->A32, h->ldA, h->AT32, h->ldAT, n, p, h->X, h->ldX, S, h->sup_idx, h->sup_val, r,
-                                 max_iter, st);
+                                 (int)std::min<int64_t>(piece, max_iter - k0), st);
     }));
-    if (P.timeout_us > 0 && std::chrono::duration_cast<std::chrono::microseconds>(
-                                std::chrono::steady_clock::now() - t_start).count() > P.timeout_us) {
-      CK(cudaStreamSynchronize(st));
-      if (std::chrono::duration_cast<std::chrono::microseconds>(std::chrono::steady_clock::now() - t_start).count() >
-          P.timeout_us)
-        return fail(h, SPCA_E_TIMEOUT, "the solve ran past timeout_us%s");
-    }
+    if (P.timeout_us == 0) break;
+    int *status = reinterpret_cast<int *>(h->h_res + (reinterpret_cast<char *>(h->status) - h->res_block));
+    CK(read_flags());
+    CK(cudaMemcpyAsync(status, h->status, (size_t)r * sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    RC(check_flags());
+    if (std::chrono::duration_cast<std::chrono::microseconds>(std::chrono::steady_clock::now() - t_start).count() >
+        P.timeout_us)
+      return fail(h, SPCA_E_TIMEOUT, "the solve ran past timeout_us%s");
+    if (std::find(status, status + r, ST_ACTIVE) == status + r) break;
   }
   for (int k0 = 1; k0 <= max_total && rc == SPCA_OK && !small;) {
     // the first read-back comes early: after it the launches that dense x^(0) needed are dropped

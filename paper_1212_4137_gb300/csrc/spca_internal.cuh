@@ -591,7 +591,8 @@ inline bool xstep_may_need_full(int form, double s, bool target) {
 // whether the list pays in the x-step of given v (else the full pass of every start)
 bool xstep_list_pays(int form, double s, bool calibrate, int64_t p, int64_t r, int sms);
 // small problems (n p <= kSmallEntries, at most two starts per SM; x, u, y and v in shared memory): every
-// sweep of every start in one launch, a cluster of CTAs per start; sweeps = the most sweeps a start may run.
+// sweep of every start in one launch, a cluster of CTAs per start; sweeps = the most sweeps a start may run in
+// this launch (a start that is still active goes on in the next one).
 // The lines: 20 sweeps of 1, 16 and 60 starts at n p = 1e6 321, 418 and 595 us (by sweeps 463, 544, 789), of
 // 16 and 40 at 1.4e6 517 and 756 (564, 713); 300 starts at n p = 5e4 371 us (553), 1000 starts 1105 (730)
 constexpr int64_t kSmallEntries = int64_t(1) << 20;
