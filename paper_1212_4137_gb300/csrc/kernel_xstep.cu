@@ -1657,15 +1657,16 @@ __global__ void __launch_bounds__(T) k_small_sweeps(XstepArgs xa, const float *_
 }
 
 constexpr int kSmallT = 256, kSmallCtas = 8;
-bool small_sweeps_fit(int64_t n, int64_t p, int r) {
+bool small_sweeps_fit(int64_t n, int64_t p, int r, double support) {
   if (small_words<kSmallT>(n, p, kSmallCtas) * 4 > (int64_t)XSTEP_SMEM_MAX) return false;
+  if (n * p > kSmallAlways && (double)n * std::min(support, (double)p) > (double)kSmallReads) return false;
   return n * p <= kSmallEntries && r <= 2 * sm_count();
 }
 
 cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, const float *AT, int64_t ldat, int n, int p,
                                 float *X, int64_t ldx, StartState s, int *sup_idx, float *sup_val, int r, int sweeps,
                                 cudaStream_t st) {
-  if (!small_sweeps_fit(n, p, r) || lda % 8 != 0 || ldat % 8 != 0) return cudaErrorInvalidValue;
+  if (!small_sweeps_fit(n, p, r, 0.0) || lda % 8 != 0 || ldat % 8 != 0) return cudaErrorInvalidValue;
   static const cudaError_t configured =
       cudaFuncSetAttribute(k_small_sweeps<kSmallT>, cudaFuncAttributeMaxDynamicSharedMemorySize, XSTEP_SMEM_MAX);
   if (configured != cudaSuccess) return configured;

@@ -1349,8 +1349,10 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
   // a small dense matrix on the CUDA-core engine: every sweep of every start in one launch, since
   // the chain of launches of a sweep, not its work, would set the time (AUTO only: an explicit
   // engine keeps the per-sweep kernels)
+  // (lambda_s keeps about 2 s entries)
+  const double expected = uses_T(form) || target ? P.s : uses_lam(form) ? 2.0 * P.s : (double)p;
   const bool small = P.engine == SPCA_ENGINE_AUTO && engine == SPCA_ENGINE_SIMT && !h->sparse && !otf && L == 0 &&
-                     h->defl_k == 0 && h->A32 && small_sweeps_fit(h->n, h->p, r);
+                     h->defl_k == 0 && h->A32 && small_sweeps_fit(h->n, h->p, r, expected);
   // (with a time limit in launches of check_every sweeps, between which the clock and the starts are looked at)
   for (int64_t k0 = 0, piece = P.timeout_us > 0 ? check_every : max_iter; small && k0 < max_iter; k0 += piece) {
     CK(timed(h, SPCA_K_XSTEP, 1, [&] {

@@ -590,13 +590,17 @@ inline bool xstep_may_need_full(int form, double s, bool target) {
 }
 // whether the list pays in the x-step of given v (else the full pass of every start)
 bool xstep_list_pays(int form, double s, bool calibrate, int64_t p, int64_t r, int sms);
-// small problems (n p <= kSmallEntries, at most two starts per SM; x, u, y and v in shared memory): every
-// sweep of every start in one launch, a cluster of CTAs per start; sweeps = the most sweeps a start may run in
-// this launch (a start that is still active goes on in the next one).
+// small problems (n p <= kSmallEntries, at most two starts per SM; x, u, y and v in shared memory; support: the
+// nonzeros that x is expected to have): every sweep of every start in one launch, a cluster of CTAs per start;
+// sweeps = the most sweeps a start may run in this launch (a start that is still active goes on in the next one).
 // The lines: 20 sweeps of 1, 16 and 60 starts at n p = 1e6 321, 418 and 595 us (by sweeps 463, 544, 789), of
-// 16 and 40 at 1.4e6 517 and 756 (564, 713); 300 starts at n p = 5e4 371 us (553), 1000 starts 1105 (730)
-constexpr int64_t kSmallEntries = int64_t(1) << 20;
-bool small_sweeps_fit(int64_t n, int64_t p, int r);
+// 16 and 40 at 1.4e6 517 and 756 (564, 713); 300 starts at n p = 5e4 371 us (553), 1000 starts 1105 (730).
+// Every CTA of a start reads the whole support's rows for u, so above kSmallAlways n times the support counts:
+// 1000 x 1000, 1 and 16 starts, s = 250 572 and 674 us (853 by sweeps, 1 start), s = 1000 1110 and 1226 (714, 853);
+// 3000 x 300, one start, s = 112 616 (603), s = 300 1008 (604); 200 x 5000, s = 1250 982 (846), s = 5000 1882
+// (1226).  A fixed penalty may keep any number of entries.
+constexpr int64_t kSmallEntries = int64_t(1) << 20, kSmallAlways = int64_t(1) << 17, kSmallReads = int64_t(1) << 18;
+bool small_sweeps_fit(int64_t n, int64_t p, int r, double support);
 cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, const float *AT, int64_t ldat, int n, int p,
                                 float *X, int64_t ldx, StartState s, int *sup_idx, float *sup_val, int r, int sweeps,
                                 cudaStream_t st);
