@@ -85,6 +85,25 @@ int enter(spca_handle *h) {
   return SPCA_OK;
 }
 
+// whether kernels may use `ptr` as it is: memory of the current GPU, or managed memory.  (Another GPU's memory
+// needs peer access, which nothing here asks for; a copy does not need it.)
+bool own_memory(const void *ptr) {
+  cudaPointerAttributes at{};
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, ptr) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == dev);
+}
+// rows x cols floats between leading dimensions, one of the two sides being the caller's `ptr`
+cudaError_t copy_rows(const void *ptr, const float *src, int64_t lds, float *dst, int64_t ldd, int64_t cols, int rows,
+                      cudaStream_t st) {
+  if (own_memory(ptr)) return launch_copy_rows(src, lds, dst, ldd, cols, rows, st);
+  return cudaMemcpy2DAsync(dst, ldd * sizeof(float), src, lds * sizeof(float), (size_t)cols * sizeof(float), rows,
+                           cudaMemcpyDeviceToDevice, st);
+}
+
 cudaError_t drain_profile(spca_handle *h) {
   cudaError_t e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return e;
@@ -1081,7 +1100,7 @@ int spca_products(spca_handle *h, int form, int engine, const float *X, int64_t 
   RC(ensure_lr_coef(h, r));
   const int n = (int)h->n, p = (int)h->p;
   cudaStream_t st = h->stream;
-  CK(launch_copy_rows(X, ldx, h->X, h->ldX, p, r, st));
+  CK(copy_rows(X, X, ldx, h->X, h->ldX, p, r, st));
   CK(cudaMemsetAsync(h->status, 0xFF, (size_t)r * sizeof(int), st));   // every row active (-1)
   CK(cudaMemsetAsync(h->iters, 0, (size_t)r * sizeof(int), st));
   CK(cudaMemsetAsync(h->ctrl, 0, sizeof(Ctrl), st));
@@ -1089,8 +1108,8 @@ int spca_products(spca_handle *h, int form, int engine, const float *X, int64_t 
   RC(sweep_u_dense(h, eng, r, nullptr, &h->ctrl[0].active, r, lowp, h->sk));
   RC(sweep_lowrank_u(h, r, &h->ctrl[0].active, h->act));
   RC(sweep_y_v(h, eng, form, r, state_of(h), &h->ctrl[0].active, r, lowp, nullptr, false, h->sk));
-  CK(launch_copy_rows(h->U, h->ldU, U, ldu, n, r, st));
-  CK(launch_copy_rows(h->V, h->ldX, V, ldv, p, r, st));
+  CK(copy_rows(U, h->U, h->ldU, U, ldu, n, r, st));
+  CK(copy_rows(V, h->V, h->ldX, V, ldv, p, r, st));
   RC(read_dev_err(h));
   return SPCA_OK;
 }
@@ -1146,11 +1165,12 @@ int spca_solve(spca_handle *h, const spca_params *prm, const float *x0, spca_res
   if (x0) {
     x0src = x0;
     ld0 = p;
-    if (!P.x0_is_device) {
+    // (copied when the kernel that reads the starts cannot; on-the-fly replacement reads device x0 in place)
+    if (!P.x0_is_device || (!otf && !own_memory(x0))) {
       float *dst = otf ? h->otf_x0 : h->X;
       ld0 = otf ? p : h->ldX;
       CK(cudaMemcpy2DAsync(dst, ld0 * sizeof(float), x0, (size_t)p * sizeof(float), (size_t)p * sizeof(float), l,
-                           cudaMemcpyHostToDevice, st));
+                           P.x0_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
       x0src = dst;
     }
     CK(cudaMemsetAsync(h->flag, 0, sizeof(int), st));
