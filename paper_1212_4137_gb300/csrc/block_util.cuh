@@ -153,6 +153,14 @@ __device__ __forceinline__ void norm_and_inverse(float sumsq, float *hi, float *
   }
 }
 
+// ||w||_2 in FP64 from what norm_and_inverse gives, for the one thread that reports it: a Newton step on hi + lo,
+// within 1.4e-16 relative of FP64's square root (2^-52.7, over every FP32 sum of squares)
+__device__ __forceinline__ double norm_fp64(float sumsq, float hi, float lo) {
+  if (!(sumsq >= 1e-30f && sumsq <= 1e30f)) return sqrt((double)sumsq);
+  const double n = (double)hi + (double)lo;
+  return fma(fma(-n, n, (double)sumsq), 0.5 * (double)__frcp_rn(hi), n);
+}
+
 // order-preserving key of |v|: the IEEE bits without the sign (monotone for |v| >= 0)
 __device__ __forceinline__ uint32_t abs_key(float v) { return __float_as_uint(v) & 0x7fffffffu; }
 

@@ -364,7 +364,7 @@ __device__ void xstep_finish(const XstepArgs &a, int c, const float *vv, int len
   // ---- Table 3 value of the subproblem
   // (by the thread that uses it, below: FP64 is slow)
   auto value = [&]() -> double {
-    const double nrm = (double)nrm_hi + (double)nrm_lo;
+    const double nrm = norm_fp64(part, nrm_hi, nrm_lo);
     if (uses_lam(form)) return op.gam * a.sqrt_s + nrm;       // S4: lambda sqrt(s) + ||V||_2
     if (uses_U(form)) return (double)part - op.gam * (double)nnz;     // S5: ||U||^2 - gamma ||U||_0
     return nrm;                                                // S3: ||T_s(v)||_2, S6: ||V_gamma(v)||_2
@@ -1284,7 +1284,7 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
   }
   // ---- outputs, stopping rule (Section 2.2), control word for the next sweep
   if (threadIdx.x == 0) {
-    const double nrm = (double)nrm_hi + (double)nrm_lo;
+    const double nrm = norm_fp64(sumsq, nrm_hi, nrm_lo);
     double F;
     if (lam_form) F = gam * a.sqrt_s + nrm;                              // S4
     else if (uses_U(form)) F = (double)sumsq - gam * (double)nnz;        // S5
