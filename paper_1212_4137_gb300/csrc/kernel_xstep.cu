@@ -16,6 +16,7 @@
 // scheduling.
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "block_util.cuh"
 #include "spca_internal.cuh"
@@ -542,8 +543,8 @@ __global__ void __launch_bounds__(XT) k_xstep(XstepArgs a_in, const float *__res
 // memory.  The bound comes from
 //   - a fixed threshold itself (exact);
 //   - last sweep's threshold t: G = kGuess t (kGuessSteady t while t holds steady);
-//   - the maxima of 2048 disjoint subsets of v (one more pass), the same ones whatever the CTA's size: at
-//     least j entries lie at or above the j-th largest of them, and for j well below 2048 not many more do;
+//   - the maxima of 512 or 2048 disjoint subsets of v (one more pass), the same ones whatever the CTA's size: at
+//     least j entries lie at or above the j-th largest of them, and for j well below their number not many more;
 //   - 0 for a very short v: the list holds every nonzero entry.
 // A bound is checked before it is used: at least s (or s + 1) listed entries for the selections,
 // phi(G) < 0 for lambda_s (phi increases through its root); then the list holds every surviving
@@ -564,7 +565,8 @@ __global__ void __launch_bounds__(XT) k_xstep(XstepArgs a_in, const float *__res
 // 16 starts 57 -> 24 us; p = 20000, lambda_s, one start 44 -> 28 us (CUDA events, a few us included).
 constexpr int kFastCand = 1024;                // listed entries per start
 constexpr int kFastBins = 2048, kFastShift = 17;   // bins of 2^-6 octave below the largest |v_i|
-constexpr int kFastSubsets = 2048;             // disjoint subsets of v whose maxima bound the threshold
+constexpr int kFastSubsets = 2048;             // disjoint subsets of v whose maxima bound the threshold (or 512)
+constexpr int kCoarseJ = 170, kCoarseMaxJ = 200;   // j of the maxima of 512 subsets
 constexpr int kFastAllP = 64;                  // v up to this long: list every nonzero entry
 // j of the subset maxima: some 570 entries lie above the bound for 500, 36 in a segment, and rarely more than
 // the 64 that a segment may list (for 600 more than that in every other start)
@@ -594,7 +596,7 @@ struct FastShared {
       int wi[W * kWarpCap];
     } w;
     int rank[kFastCand];
-    uint4 maxima[kFastSubsets / 4];            // of the upper half of 1024 threads, see subset_bound
+    uint32_t maxima[kFastSubsets];
     struct {
       float val[kFastCand];                    // the surviving entries, in index order
       int idx[kFastCand];
@@ -615,36 +617,49 @@ struct FastShared {
 };
 
 // A row of v read as aligned 16-byte vectors wherever it starts: entry i is at q = i + sh of the aligned
-// base b, and a vector that crosses an end of the row is read entry by entry (0 outside).
+// base b.  The vectors at lo4 .. hi4 - 4 lie inside the row; the one at 0 (sh > 0) and the one at hi4 (end no
+// multiple of 4) cross an end.  Those are read entry by entry, once a pass and not at every load: an
+// x-step's warps stall for instructions more than for anything else, and that code at every load was a third of
+// a pass.
 struct Row {
   const float *b;
   int sh, end;                                 // valid q: sh .. end - 1
+  int lo4, hi4;
 };
 __device__ __forceinline__ Row row_of(const float *v, int p) {
   Row r;
   r.sh = (int)((reinterpret_cast<uintptr_t>(v) >> 2) & 3u);
   r.b = v - r.sh;
   r.end = p + r.sh;
+  r.lo4 = r.sh > 0 ? 4 : 0;
+  r.hi4 = r.end & ~3;
   return r;
 }
-// entries q .. q + 3 (q a multiple of 4), 0 from `hi` on
+// entries q .. q + 3 (q a multiple of 4) of a vector inside the row and below hi, else 0
 __device__ __forceinline__ float4 row_load(const Row &r, int q, int hi) {
-  if (q >= r.sh && q + 4 <= hi) return *reinterpret_cast<const float4 *>(r.b + q);
-  float4 t = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  if (q >= r.sh && q < hi) t.x = r.b[q];
-  if (q + 1 >= r.sh && q + 1 < hi) t.y = r.b[q + 1];
-  if (q + 2 >= r.sh && q + 2 < hi) t.z = r.b[q + 2];
-  if (q + 3 >= r.sh && q + 3 < hi) t.w = r.b[q + 3];
-  return t;
+  return q >= r.lo4 && q < min(hi, r.hi4) ? *reinterpret_cast<const float4 *>(r.b + q)
+                                          : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+}
+// entry q of the row, 0 outside
+__device__ __forceinline__ float row_entry(const Row &r, int q) { return q >= r.sh && q < r.end ? r.b[q] : 0.0f; }
+__device__ __forceinline__ float4 row_vector(const Row &r, int q) {
+  return make_float4(row_entry(r, q), row_entry(r, q + 1), row_entry(r, q + 2), row_entry(r, q + 3));
+}
+// where the vector over the row's end begins (-1: none, or it is the one over its beginning)
+__device__ __forceinline__ int row_last(const Row &r) { return r.hi4 < r.end && r.hi4 >= r.lo4 ? r.hi4 : -1; }
+// the entries of the vectors that cross an end, one for each of the first eight threads: its place, or -1
+__device__ __forceinline__ int edge_entry(const Row &r, int t) {
+  const int q = t < 4 ? t : row_last(r) + t - 4;
+  const bool is = t < 4 ? r.sh > 0 : t < 8 && row_last(r) >= 0;
+  return is && q >= r.sh && q < r.end ? q : -1;
 }
 
-// a lower bound of the j-th largest |v_i| from the maxima of 2048 subsets (the entries at q, q + 2048, ...
-// of the row): the lower edge of the histogram bin of the j-th largest maximum.  0 when the bins do not
-// resolve it.
+// a lower bound of the j-th largest |v_i| from the maxima of 512 or 2048 subsets: the lower edge of the
+// histogram bin of the j-th largest maximum.  0 when the bins do not resolve it.
 // lam_s > 0, for lambda_s: the maxima are a sample of v's largest entries, so phi over them tells, but for a
 // few percent, whether lambda_s lies above the bound.  If not for j, a larger one is taken (j becomes it), half as
-// much again each time; if not for kFastMaxJ either, kNoBound: the start's active set is longer than the list, as one
-// pass has shown.  (Sums over whole counts in a fixed order: not a matter of T.)
+// much again each time; if not for kFastMaxJ either, kNoBound: the start's active set is longer than the list, as
+// one pass has shown.  (Sums over whole counts in a fixed order: not a matter of T.)
 constexpr uint32_t kNoBound = 0xFFFFFFFFu;
 __device__ __forceinline__ int bin_of_rank(const unsigned *hist, int j) {
   // one warp: the first bin, from the largest down, whose running count reaches j (64 bins a step: the
@@ -671,7 +686,8 @@ __device__ __forceinline__ uint32_t bin_edge(uint32_t top, int bin) {
   const uint32_t down = (uint32_t)(bin + 1) << kFastShift;
   return bin >= kFastBins - 1 || down >= top ? 0u : top - down;
 }
-__device__ __forceinline__ bool root_above(const unsigned *hist, uint32_t top, int bin, float s, int p) {
+// (n_sub: the subsets that v's p entries are spread over)
+__device__ __forceinline__ bool root_above(const unsigned *hist, uint32_t top, int bin, float s, int p, int n_sub) {
   const uint32_t Gk = bin_edge(top, bin);
   if (Gk == 0u) return true;
   const int lane = threadIdx.x & 31;
@@ -689,17 +705,23 @@ __device__ __forceinline__ bool root_above(const unsigned *hist, uint32_t top, i
   w2 = warp_sum_f(w2);
   n = warp_sum_i(n);
   // of m entries above G, spread over subsets of q entries each, n are their subset's maximum
-  const float q = fmaxf(1.0f, (float)p / kFastSubsets), sub = (float)kFastSubsets;
+  const float sub = (float)n_sub, q = fmaxf(1.0f, (float)p / sub);
   const float m = sub * q * (1.0f - powf(1.0f - (float)n / sub, 1.0f / q));
   return s * w2 < 1.02f * (m / (float)n) * (w1 * w1);
 }
-template <int T>
-__device__ __forceinline__ uint32_t subset_bound(const Row &row, int &j, float lam_s, FastShared<T> &fs) {
+// The histogram of the subset maxima (fs.u.hist; the return value: the largest of them, bin 0): 2048 subsets
+// (kFine) or 512, the entries at q, q + 2048 or 512, ... of the row.  A thread has G groups of four subsets, load k
+// belonging to group k mod G; threads that share subsets meet in shared memory.
+template <int T, bool kFine>
+__device__ __forceinline__ uint32_t subset_maxima(const Row &row, FastShared<T> &fs) {
   constexpr int CH = T > 256 ? 4 : 8;          // loads in flight per thread
-  // the subsets of a thread: G groups of four, load k of it being group k mod G; with 1024 threads two
-  // threads share four
-  constexpr int G = kFastSubsets > 4 * T ? kFastSubsets / (4 * T) : 1;
+  constexpr int N = kFine ? kFastSubsets : kFastSubsets / 4, G = N > 4 * T ? N / (4 * T) : 1;
   static_assert(CH % G == 0, "a step covers whole rounds of the subsets");
+  uint32_t *sub = fs.a.maxima;
+  for (int b = threadIdx.x; b < kFastBins; b += T) {
+    fs.u.hist[b] = 0u;
+    if (b < N) sub[b] = 0u;
+  }
   uint32_t m[G][4];
 #pragma unroll
   for (int k = 0; k < G; ++k) m[k][0] = m[k][1] = m[k][2] = m[k][3] = 0u;
@@ -715,41 +737,55 @@ __device__ __forceinline__ uint32_t subset_bound(const Row &row, int &j, float l
       m[k % G][3] = max(m[k % G][3], abs_key(t[k].w));
     }
   }
-  for (int b = threadIdx.x; b < kFastBins; b += T) fs.u.hist[b] = 0u;
-  if (4 * T > kFastSubsets && threadIdx.x >= kFastSubsets / 4)
-    fs.a.maxima[threadIdx.x - kFastSubsets / 4] = make_uint4(m[0][0], m[0][1], m[0][2], m[0][3]);
+  __syncthreads();                             // (the zeros)
+#pragma unroll
+  for (int k = 0; k < G; ++k)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) atomicMax(&sub[(4 * (threadIdx.x + T * k) + e) & (N - 1)], m[k][e]);
+  const int q = edge_entry(row, (int)threadIdx.x);
+  if (q >= 0) atomicMax(&sub[q & (N - 1)], abs_key(row.b[q]));
+  __syncthreads();
   uint32_t all = 0u;
-#pragma unroll
-  for (int k = 0; k < G; ++k) all = max(all, max(max(m[k][0], m[k][1]), max(m[k][2], m[k][3])));
-  const uint32_t top = block_max_u(all, fs.sh.red_u);   // (barriers after the zeros and the shared maxima)
-  if (4 * T > kFastSubsets && threadIdx.x < kFastSubsets / 4) {
-    const uint4 o = fs.a.maxima[threadIdx.x];
-    m[0][0] = max(m[0][0], o.x); m[0][1] = max(m[0][1], o.y);
-    m[0][2] = max(m[0][2], o.z); m[0][3] = max(m[0][3], o.w);
-  }
-  if (threadIdx.x < kFastSubsets / 4) {
-#pragma unroll
-    for (int k = 0; k < G; ++k)
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        atomicAdd(&fs.u.hist[min((top - m[k][e]) >> kFastShift, (uint32_t)kFastBins - 1u)], 1u);
-  }
+  for (int b = threadIdx.x; b < N; b += T) all = max(all, sub[b]);
+  const uint32_t top = block_max_u(all, fs.sh.red_u);
+  for (int b = threadIdx.x; b < N; b += T)
+    atomicAdd(&fs.u.hist[min((top - sub[b]) >> kFastShift, (uint32_t)kFastBins - 1u)], 1u);
   __syncthreads();
-  if (threadIdx.x < 32) {
-    int jn = j, bin = bin_of_rank(fs.u.hist, jn);
-    while (lam_s > 0.0f && bin >= 0 && !root_above(fs.u.hist, top, bin, lam_s, row.end - row.sh)) {
-      const bool longer = jn < kFastMaxJ;
-      jn = min(kFastMaxJ, jn + jn / 2);
-      bin = longer ? bin_of_rank(fs.u.hist, jn) : -1;
+  return top;
+}
+template <int T>
+__device__ __noinline__ uint32_t subset_maxima_fine(const Row &row, FastShared<T> &fs) {
+  return subset_maxima<T, true>(row, fs);
+}
+
+template <int T>
+__device__ __forceinline__ uint32_t subset_bound(const Row &row, int &j, float lam_s, FastShared<T> &fs) {
+  // up to kCoarseJ the maxima of 512 subsets do (a list of 200 entries for j = 166, 173 with 2048), and the CTA
+  // saves three quarters of the updates of the histogram (1024 starts of p = 20011: 19 us); a lambda_s that lies
+  // lower than their limit takes the pass again with 2048
+  bool fine = j > kCoarseJ;
+  for (;;) {
+    const uint32_t top = fine ? subset_maxima_fine<T>(row, fs) : subset_maxima<T, false>(row, fs);
+    const int limit = fine ? kFastMaxJ : kCoarseMaxJ, n_sub = fine ? kFastSubsets : kFastSubsets / 4;
+    if (threadIdx.x < 32) {
+      int jn = j, bin = bin_of_rank(fs.u.hist, jn);
+      while (lam_s > 0.0f && bin >= 0 && !root_above(fs.u.hist, top, bin, lam_s, row.end - row.sh, n_sub)) {
+        const bool longer = jn < limit;
+        jn = min(limit, jn + jn / 2);
+        bin = longer ? bin_of_rank(fs.u.hist, jn) : -1;
+      }
+      if (threadIdx.x == 0) {
+        fs.sh.digit = bin;
+        fs.sh.rem = jn;
+      }
     }
-    if (threadIdx.x == 0) {
-      fs.sh.digit = bin;
-      fs.sh.rem = jn;
-    }
+    __syncthreads();
+    const int bin = fs.sh.digit;
+    j = fs.sh.rem;
+    if (bin >= 0 || fine) return bin < 0 ? kNoBound : bin_edge(top, bin);
+    fine = true;
+    __syncthreads();                 // (the result is read, and the histogram)
   }
-  __syncthreads();
-  j = fs.sh.rem;
-  return fs.sh.digit < 0 ? kNoBound : bin_edge(top, fs.sh.digit);
 }
 
 // An index segment of more than 1024 entries of v (a sixteenth, as list_above cuts it)
@@ -767,6 +803,8 @@ __device__ __forceinline__ bool first_segment_full(const Row &row, uint32_t Gk, 
     const float4 e = row_load(row, q, hi);
     n += (abs_key(e.x) > Gk) + (abs_key(e.y) > Gk) + (abs_key(e.z) > Gk) + (abs_key(e.w) > Gk);
   }
+  const int qe = edge_entry(row, (int)threadIdx.x);
+  if (qe >= 0 && qe < hi) n += abs_key(row.b[qe]) > Gk;
   return block_sum_i(n, reinterpret_cast<int *>(fs.sh.red_u)) > kFastSegCap;
 }
 
@@ -808,6 +846,11 @@ __device__ __forceinline__ bool list_above(const Row &row, uint32_t Gk, bool sum
   float4 e[CH], nx[CH];
 #pragma unroll
   for (int h = 0; h < CH; ++h) e[h] = row_load(row, lo + h * 128 + 4 * lane, hi);
+  if (lo == 0 && hi > 0 && row.sh > 0 && lane == 0) e[0] = row_vector(row, 0);
+  int at_end = row_last(row);                  // the vector over the row's end, if it is this lane's
+  float4 end_v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  if (at_end < lo || at_end >= hi || ((at_end - lo) & 127) != 4 * lane) at_end = -1;
+  if (at_end >= 0) end_v = row_vector(row, at_end);
   for (int base = lo; base < hi && !over; base += 128 * CH) {
 #pragma unroll
     for (int h = 0; h < CH; ++h) nx[h] = row_load(row, base + (CH + h) * 128 + 4 * lane, hi);
@@ -818,6 +861,7 @@ __device__ __forceinline__ bool list_above(const Row &row, uint32_t Gk, bool sum
         wc0 = wc;
       }
       ++chunk;
+      if (base + h * 128 + 4 * lane == at_end) e[h] = end_v;
       const float ev[4] = {e[h].x, e[h].y, e[h].z, e[h].w};
       if (sums) {
 #pragma unroll
@@ -1025,8 +1069,17 @@ __device__ __forceinline__ XState load_state(const StartState &st, int c) {
   return q;
 }
 
+// The form's family as a compile-time constant: the code of a family holds nothing of the others', and an
+// x-step's warps stall for instructions more than for anything else (16 sweeps' x-steps, without and with:
+// 16 starts of p = 4000, T_s, 236 and 204 us; of p = 100000, V_gamma, 446 and 365; one of 20000, T_s, 343 and 259).
+// kAny: groups, whose one launch serves members of every form.
+enum class XKind { kSelect, kLambda, kPenalty, kAny };
+inline XKind xstep_kind(int form) {
+  return uses_T(form) ? XKind::kSelect : uses_lam(form) ? XKind::kLambda : XKind::kPenalty;
+}
+
 // the x-step of start c (block-wide, T threads); false when it is left to the full pass
-template <int T>
+template <int T, XKind K>
 __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, const float *__restrict__ V, int64_t ldv,
                                                float *__restrict__ X, int64_t ldx, const StartState &st,
                                                const XState &q0, int *__restrict__ sup_idx,
@@ -1037,9 +1090,12 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
   const Row row = row_of(V + (int64_t)c * ldv, p);
   float *x = X ? X + (int64_t)c * ldx : nullptr;   // (null: the support list is all that is wanted)
   const unsigned lt_mask = (1u << lane) - 1u;
-  const bool lam_form = uses_lam(form), exact = is_pen(form) && !a.calibrate;
-  const bool keep_all = uses_T(form) && s_int >= p;
-  const int need = uses_T(form) ? s_int : (is_pen(form) && a.calibrate ? s_int + 1 : 1);
+  const bool t_form = K == XKind::kAny ? uses_T(form) : K == XKind::kSelect;
+  const bool lam_form = K == XKind::kAny ? uses_lam(form) : K == XKind::kLambda;
+  const bool pen_form = K == XKind::kAny ? is_pen(form) : K == XKind::kPenalty;
+  const bool exact = pen_form && !a.calibrate;
+  const bool keep_all = t_form && s_int >= p;
+  const int need = t_form ? s_int : (pen_form && a.calibrate ? s_int + 1 : 1);
   const bool all = p <= kFastAllP || (p <= kFastCand && keep_all);
   if (!all && !exact && (need > kFastMaxNeed || keep_all || need * kFastPerNeed > p)) return false;
   // j of the subset maxima: the active set of lambda_s has about 2 s entries where |v|'s tail is
@@ -1049,14 +1105,11 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
   const bool steady = q0.xfast == 1;
   // x is zero outside the last support list, once there is one (before: all of x is written)
   const bool listed = sup_idx && q0.iters > 1 && q0.nnz <= a.cap;
-  auto clear_x = [&] {
-    if (listed) {
-      const int nnz_old = q0.nnz;
-      const int *old = sup_idx + (int64_t)c * a.cap;
-      for (int t = threadIdx.x; t < nnz_old; t += T) x[old[t]] = 0.0f;
-      return;
-    }
-    // as aligned vectors, whatever the row's alignment
+  // (there, the old list's entries are cleared once the new one is made: their indices load meanwhile)
+  const int nnz_old = x && listed ? q0.nnz : 0;
+  const int *old = sup_idx + (int64_t)c * a.cap;
+  const int old0 = (int)threadIdx.x < nnz_old ? old[threadIdx.x] : -1;
+  auto clear_row = [&] {             // as aligned vectors, whatever the row's alignment
     const int sh = (int)((reinterpret_cast<uintptr_t>(x) >> 2) & 3u);
     float *xb = x - sh;
     for (int q = 4 * threadIdx.x; q < p + sh; q += 4 * T) {
@@ -1068,12 +1121,12 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
       }
     }
   };
-  // the zeros are stored while v is read, but for an x over v itself (the x-step of given v, in place), and
-  // for a fixed threshold, above which there may be any number of entries (and the full pass writes all of
-  // x): there once the list is made, which v is read for
+  // a whole row's zeros are stored while v is read, but for an x over v itself (the x-step of given v, in place),
+  // and for a fixed threshold, above which there may be any number of entries (and the full pass writes all
+  // of x): there once the list is made, which v is read for
   const float *vrow = V + (int64_t)c * ldv;
-  const bool late = (x < vrow + p && vrow < x + p) || (exact && !listed);
-  if (x && !late) clear_x();
+  const bool late = (x < vrow + p && vrow < x + p) || exact;
+  if (x && !listed && !late) clear_row();
 
   // ---- a bound, the list above it, and the check (block-uniform throughout)
   int buf = 0, ncand = 0;
@@ -1131,12 +1184,15 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
     }
     __syncthreads();                 // the lists are reused
   }
-  if (x && late) clear_x();          // (every thread has read its part of v: the list's barrier)
+  // (every thread has read its part of v: the list's barrier)
+  if (old0 >= 0) x[old0] = 0.0f;
+  for (int t = threadIdx.x + T; t < nnz_old; t += T) x[old[t]] = 0.0f;
+  if (x && !listed && late) clear_row();
 
   // ---- the operator on the list: which entries survive, as
   //   select: rank < need (T_s; ties at the threshold: the lower indices), or key above the threshold
   float tval = 0.0f, tnext = tprev;
-  const bool select = (uses_T(form) && !keep_all) || (is_pen(form) && a.calibrate);
+  const bool select = (t_form && !keep_all) || (pen_form && a.calibrate);
   const bool ranked = select && ncand >= need;
   uint32_t kmin = 0xFFFFFFFFu;       // the need-th largest key
   if (ranked) {
@@ -1168,7 +1224,7 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
     buf ^= 1;
     tval = __uint_as_float(kmin);
     tnext = tval;
-    if (uses_T(form) && above > need) {   // more entries tie at the threshold than fit: by index
+    if (t_form && above > need) {   // more entries tie at the threshold than fit: by index
       for (int t = threadIdx.x; t < ncand; t += T) {
         if (abs_key(fs.u.l.cv[t]) != kmin) continue;
         int order = 0;
@@ -1186,11 +1242,11 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
   } else {
     tnext = 0.0f;                    // at most s (or s + 1) nonzero entries: all of them; gamma = 0
   }
-  if (is_pen(form) && a.calibrate) gam = uses_U(form) ? (double)tval * (double)tval : (double)tval;
-  const bool soft = lam_form || uses_V(form);
+  if (pen_form && a.calibrate) gam = (pen_form && uses_U(form)) ? (double)tval * (double)tval : (double)tval;
+  const bool soft = lam_form || (pen_form && uses_V(form));
   // an entry survives when its key is above this one (lambda_s: |v| > lam in FP64)
   const uint32_t cut = lam_form && !lam0 ? __float_as_uint(__double2float_rd(lam))
-                       : ranked && !uses_T(form) ? kmin : 0u;
+                       : ranked && !t_form ? kmin : 0u;
 
   // ---- w, which takes the place of the list's values; the survivors are counted per 32 entries
   const int rounds = (ncand + T - 1) / T;
@@ -1201,7 +1257,7 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
       const float v = fs.u.l.cv[t];
       const uint32_t mine = abs_key(v);
       bool keep = mine > cut;
-      if (ranked && uses_T(form)) keep = fs.a.rank[t] < need;
+      if (ranked && t_form) keep = fs.a.rank[t] < need;
       if (keep) wq = soft ? copysignf(fabsf(v) - tval, v) : v;
     }
     const unsigned ball = __ballot_sync(0xffffffffu, wq != 0.0f);
@@ -1287,12 +1343,12 @@ __device__ __forceinline__ bool xstep_fast_one(const XstepArgs &a_in, int c, con
     const double nrm = norm_fp64(sumsq, nrm_hi, nrm_lo);
     double F;
     if (lam_form) F = gam * a.sqrt_s + nrm;                              // S4
-    else if (uses_U(form)) F = (double)sumsq - gam * (double)nnz;        // S5
+    else if ((pen_form && uses_U(form))) F = (double)sumsq - gam * (double)nnz;        // S5
     else F = nrm;                                                        // S3, S6
     if (st.F) st.F[c] = F;
     if (st.nnz) st.nnz[c] = nnz;
     if (st.gamma) st.gamma[c] = gam;
-    if (st.thr && is_pen(form) && a.calibrate) st.thr[c] = tval;
+    if (st.thr && pen_form && a.calibrate) st.thr[c] = tval;
     if (st.tprev) st.tprev[c] = tnext;
     if (st.xfast) {
       const bool near = tnext >= (1.0f - kSteady) * tprev && tnext <= (1.0f + kSteady) * tprev;
@@ -1326,12 +1382,12 @@ __device__ __noinline__ void xstep_full_global(const XstepArgs &a, int c, const 
                                                XShared &sh) {
   xstep_full_one<false, kOne>(a, c, V, ldv, X, ldx, st, sup_idx, sup_val, ctrl, nullptr, sh);
 }
-template <int T>
+template <int T, XKind K>
 __device__ __forceinline__ void xstep_start(const XstepArgs &a, int c, const float *__restrict__ V, int64_t ldv,
                                             float *__restrict__ X, int64_t ldx, const StartState &st,
                                             const XState &q0, int *__restrict__ sup_idx,
                                             float *__restrict__ sup_val, Ctrl *ctrl, bool defer, FastShared<T> &fs) {
-  if (xstep_fast_one<T>(a, c, V, ldv, X, ldx, st, q0, sup_idx, sup_val, ctrl, fs)) return;
+  if (xstep_fast_one<T, K>(a, c, V, ldv, X, ldx, st, q0, sup_idx, sup_val, ctrl, fs)) return;
   if (ctrl && threadIdx.x == 0) atomicAdd(&ctrl->n_full, 1);
   __syncthreads();
   if (!defer) {
@@ -1345,7 +1401,7 @@ __device__ __forceinline__ void xstep_start(const XstepArgs &a, int c, const flo
 
 // (CTAs per SM for the register budget: 7 x 152 of 128 threads hold 1024 starts at once)
 constexpr int fast_ctas(int t) { return t == 128 ? 7 : t == 256 ? 3 : 1; }
-template <int T>
+template <int T, XKind K>
 __global__ void __launch_bounds__(T, fast_ctas(T)) k_xstep_fast(XstepArgs a, const float *__restrict__ V, int64_t ldv,
                                                             int r, float *__restrict__ X, int64_t ldx, StartState st,
                                                             int *__restrict__ sup_idx, float *__restrict__ sup_val,
@@ -1357,7 +1413,7 @@ __global__ void __launch_bounds__(T, fast_ctas(T)) k_xstep_fast(XstepArgs a, con
     for (int i = threadIdx.x; i < nflags; i += T) flags[i] = 0;
   const int status = st.status ? st.status[c] : ST_ACTIVE;
   const XState q0 = load_state(st, c);
-  if (status == ST_ACTIVE) xstep_start<T>(a, c, V, ldv, X, ldx, st, q0, sup_idx, sup_val, ctrl, defer != 0, fs);
+  if (status == ST_ACTIVE) xstep_start<T, K>(a, c, V, ldv, X, ldx, st, q0, sup_idx, sup_val, ctrl, defer != 0, fs);
   if (act) last_makes_active_list(r, st.status, st.nnz, r, act, rank, ctrl, ctrl_read);
 }
 
@@ -1417,7 +1473,8 @@ __global__ void __launch_bounds__(T, fast_ctas(T)) k_g_xstep_fast(const GProb *_
   const int status = q.st.status[c];
   const XState q0 = load_state(q.st, c);
   if (status == ST_ACTIVE)
-    xstep_start<T>(q.xa, c, q.V, q.ldX, q.X, q.ldX, q.st, q0, q.sup_idx, q.sup_val, q.ctrl[parity], defer != 0, fs);
+    xstep_start<T, XKind::kAny>(q.xa, c, q.V, q.ldX, q.X, q.ldX, q.st, q0, q.sup_idx, q.sup_val, q.ctrl[parity],
+                                defer != 0, fs);
   if (!defer)
     last_makes_active_list(q.r, q.st.status, q.st.nnz, q.r, q.act, q.rank, q.ctrl[parity], q.ctrl[parity ^ 1]);
 }
@@ -1550,8 +1607,8 @@ __host__ __device__ inline int64_t small_words(int64_t n, int64_t p, int ctas) {
   return (ctas > 1 ? 4 : 3) * p4 + (a > b ? a : b);
 }
 
-template <int T>
-__global__ void __launch_bounds__(T) k_small_sweeps(XstepArgs xa, const float *__restrict__ A, int64_t lda,
+template <int T, XKind K>
+__global__ void __launch_bounds__(T, 1) k_small_sweeps(XstepArgs xa, const float *__restrict__ A, int64_t lda,
                                                     const float *__restrict__ AT, int64_t ldat, int n, int p,
                                                     int ctas, int a_smem, float *__restrict__ X, int64_t ldx,
                                                     StartState st, int *__restrict__ sup_idx,
@@ -1631,7 +1688,7 @@ __global__ void __launch_bounds__(T) k_small_sweeps(XstepArgs xa, const float *_
     }
     if (ctas > 1) cluster_barrier();
     else __syncthreads();
-    if (!xstep_fast_one<T>(xa, 0, v, 0, nullptr, 0, sl, load_state(sl, 0), li, lv, nullptr, fs)) {
+    if (!xstep_fast_one<T, K>(xa, 0, v, 0, nullptr, 0, sl, load_state(sl, 0), li, lv, nullptr, fs)) {
       __syncthreads();
       xstep_full_one<false, false>(xa, 0, v, 0, nullptr, 0, sl, li, lv, nullptr, nullptr, fs.sh);
       if (threadIdx.x == 0) ss.xfast = 2;
@@ -1663,13 +1720,15 @@ bool small_sweeps_fit(int64_t n, int64_t p, int r, double support) {
   return n * p <= kSmallEntries && r <= 2 * sm_count();
 }
 
+template <XKind K>
+static cudaError_t small_smem() {
+  return cudaFuncSetAttribute(k_small_sweeps<kSmallT, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, XSTEP_SMEM_MAX);
+}
+
 cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, const float *AT, int64_t ldat, int n, int p,
                                 float *X, int64_t ldx, StartState s, int *sup_idx, float *sup_val, int r, int sweeps,
                                 cudaStream_t st) {
   if (!small_sweeps_fit(n, p, r, 0.0) || lda % 8 != 0 || ldat % 8 != 0) return cudaErrorInvalidValue;
-  static const cudaError_t configured =
-      cudaFuncSetAttribute(k_small_sweeps<kSmallT>, cudaFuncAttributeMaxDynamicSharedMemorySize, XSTEP_SMEM_MAX);
-  if (configured != cudaSuccess) return configured;
   // CTAs per start, of at least 32 columns each: as many as are resident at once (a cluster lies in one GPC,
   // so of 152 SMs clusters of 8 reach 120 and clusters of 4 reach 144, at a CTA per SM; a second wave doubled
   // the time: 16 starts of p = 500 in clusters of 8 565 us, of 4 320)
@@ -1692,22 +1751,39 @@ cudaError_t launch_small_sweeps(XstepArgs xa, const float *A, int64_t lda, const
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_small_sweeps<kSmallT>, xa, A, lda, AT, ldat, n, p, ctas, a_smem, X, ldx, s, sup_idx,
-                            sup_val, sweeps);
+  auto go = [&](auto kern, cudaError_t configured) -> cudaError_t {
+    if (configured != cudaSuccess) return configured;
+    return cudaLaunchKernelEx(&cfg, kern, xa, A, lda, AT, ldat, n, p, ctas, a_smem, X, ldx, s, sup_idx, sup_val, sweeps);
+  };
+  // (function-local statics: configured once, thread-safe)
+  switch (xstep_kind(xa.form)) {
+    case XKind::kSelect: {
+      static const cudaError_t set = small_smem<XKind::kSelect>();
+      return go(k_small_sweeps<kSmallT, XKind::kSelect>, set);
+    }
+    case XKind::kLambda: {
+      static const cudaError_t set = small_smem<XKind::kLambda>();
+      return go(k_small_sweeps<kSmallT, XKind::kLambda>, set);
+    }
+    default: {
+      static const cudaError_t set = small_smem<XKind::kPenalty>();
+      return go(k_small_sweeps<kSmallT, XKind::kPenalty>, set);
+    }
+  }
 }
 
 // The x-step of given v has no last threshold to start from, so its list costs a pass for the bound and one
 // for the list.  It pays, against the full pass of every start in one launch, for lambda_s with s up to 150
 // (above, the list often does not hold the active set), and for T_s and the Section 4.1 rule with few
-// selected entries: a 25th of v (a 10th when starts outnumber two per SM) and at most kFastMaxJ.  Whole
+// selected entries: a 25th of v (a 13th when starts outnumber two per SM) and at most kFastMaxJ.  Whole
 // calls, full pass and list: one start, p = 1500, T_s, s = 200 28 and 31 us, s = 50 27 and 28; p = 6000, s = 500 33
-// and 39, s = 200 35 and 30; 1024 starts, p = 3000, s = 400 70 and 67, s = 500 68 and 86.  A fixed threshold is the
-// list's bound itself.
+// and 39, s = 200 35 and 30; 1024 starts, p = 3000, s = 200 66 and 44, s = 500 68 and 86; 600, p = 6000, s = 500 62
+// and 68.  A fixed threshold is the list's bound itself.
 bool xstep_list_pays(int form, double s, bool calibrate, int64_t p, int64_t r, int sms) {
   if (uses_lam(form)) return s <= 150.0;
   if (is_pen(form) && !calibrate) return true;
   const int64_t need = (int64_t)s + (calibrate ? 1 : 0);
-  return need <= kFastMaxJ && need * (r <= 2 * (int64_t)sms ? 25 : 10) <= p;
+  return need <= kFastMaxJ && need * (r <= 2 * (int64_t)sms ? 25 : 13) <= p;
 }
 
 cudaError_t launch_xstep(XstepArgs a, const float *V, int64_t ldv, int r, float *X, int64_t ldx,
@@ -1716,17 +1792,23 @@ cudaError_t launch_xstep(XstepArgs a, const float *V, int64_t ldv, int r, float 
   const int sms = sm_count(), d = full == XFull::kAfter ? 1 : 0;
   if (sms < 1) return cudaErrorInvalidDevice;
   int *al = d ? nullptr : act;
-#define SPCA_FAST(T)                                                                                             \
-  k_xstep_fast<T><<<r, T, 0, st>>>(a, V, ldv, r, X, ldx, s, sup_idx, sup_val, ctrl, ctrl_read, al, rank, d, flags, nflags)
   cudaError_t e = cudaSuccess;
   if (full != XFull::kAlone) {
+    auto go = [&](auto kern, int threads) {
+      kern<<<r, threads, 0, st>>>(a, V, ldv, r, X, ldx, s, sup_idx, sup_val, ctrl, ctrl_read, al, rank, d, flags, nflags);
+      return cudaGetLastError();
+    };
+    const XKind kind = xstep_kind(a.form);
+#define SPCA_FAST(T)                                                  \
+  (kind == XKind::kSelect   ? go(k_xstep_fast<T, XKind::kSelect>, T)  \
+   : kind == XKind::kLambda ? go(k_xstep_fast<T, XKind::kLambda>, T)  \
+                            : go(k_xstep_fast<T, XKind::kPenalty>, T))
     switch (fast_threads(r, a.p, sms)) {
-      case 1024: SPCA_FAST(1024); break;
-      case 512: SPCA_FAST(512); break;
-      case 256: SPCA_FAST(256); break;
-      default: SPCA_FAST(128); break;
+      case 1024: e = SPCA_FAST(1024); break;
+      case 512: e = SPCA_FAST(512); break;
+      case 256: e = SPCA_FAST(256); break;
+      default: e = SPCA_FAST(128); break;
     }
-    e = cudaGetLastError();
     if (e != cudaSuccess || full == XFull::kInside) return e;
   }
 #undef SPCA_FAST

@@ -63,10 +63,10 @@ def _check(lib, oracle, p, copies, form, s, calibrate, gamma, launches, V=None):
         assert abs(T[c] - ref.thr) <= 1e-6 * max(1.0, abs(ref.thr)), (c, T[c], ref.thr)
 
 
-# (p, copies of 6 rows, s, launches): a 25th of v up to two starts per SM (6 x 50 = 300), a 10th above
+# (p, copies of 6 rows, s, launches): a 25th of v up to two starts per SM (6 x 50 = 300), a 13th above
 # (6 x 51 = 306); at most 500 entries; past an SM for each start the full pass of long rows is a second launch
 @pytest.mark.parametrize("p,copies,s,launches", [(2500, 1, 100, 1), (2499, 1, 100, 1), (2500, 50, 101, 1),
-                                                 (2500, 51, 101, 1), (1000, 51, 100, 1), (999, 51, 100, 1),
+                                                 (2500, 51, 101, 1), (1300, 51, 100, 1), (1299, 51, 100, 1),
                                                  (20011, 1, 500, 1), (20011, 1, 501, 1), (20011, 60, 500, 2),
                                                  (20011, 60, 501, 1), (20011, 60, 450, 2), (20011, 1, 20011, 1),
                                                  (300, 1, 12, 1), (300, 1, 13, 1), (70, 1, 60, 1), (60, 60, 40, 1)])
