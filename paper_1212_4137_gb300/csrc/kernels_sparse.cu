@@ -21,7 +21,7 @@
 //   k_pack_t_h, k_spmm_h, k_spmm_wide_h
 //                   the same for y = +-1 (L1 variance), which FP16 holds exactly: 16 starts per
 //                   32-byte sector (slabs of 128 starts), products and sums in FP32;
-//   k_spmm_fix      a long row's segments' sums added in segment order;
+//   k_spmm_fix      a long row's segments' sums added in a fixed order, with the additions' errors;
 //   k_spmv_support  u = A x over the support of a sparse x: the support's columns (A^T's rows)
 //                   scattered into a shared-memory chunk of u, one column at a time in support
 //                   order, the FMA chain of each u_i in that order;
@@ -321,18 +321,59 @@ __global__ void __launch_bounds__(SPT, 3) k_spmm_wide(SpMat M, const SpItem *__r
   }
 }
 
-// block per long row: its segments' sums in segment order
-__global__ void __launch_bounds__(256) k_spmm_fix(const SpLong *__restrict__ longs, const float *__restrict__ part,
-                                                  int ldb, const int *__restrict__ count,
-                                                  const int *__restrict__ gate, const int *__restrict__ list,
-                                                  float *__restrict__ out, int64_t ldo) {
+// A block per long row: its segments' sums, every addition with its exact error: the segments are short, so a
+// long row has many, and their plain sum was most of the row's error (x of a 40000 x 20000 corpus was 8.7e-8
+// from its 64-bit value, 5.4e-8 with segments four times as long; now 3.3e-8).  256 / S starts at a time in S
+// slices of the segments, the fewer the starts the more slices (by the starts of the solve, so that a sum's order
+// does not change while they stop).
+constexpr int kFixThreads = 256;
+inline int fix_slices(int rmax) { return rmax <= 32 ? 8 : rmax <= 64 ? 4 : rmax <= 128 ? 2 : 1; }
+__global__ void __launch_bounds__(kFixThreads) k_spmm_fix(const SpLong *__restrict__ longs,
+                                                          const float *__restrict__ part, int ldb, int slices,
+                                                          const int *__restrict__ count, const int *__restrict__ gate,
+                                                          const int *__restrict__ list, float *__restrict__ out,
+                                                          int64_t ldo) {
   if (gate && *gate == 0) return;
+  __shared__ float2 sums[kFixThreads];
   const int cnt = *count;
   const SpLong L = longs[blockIdx.x];
-  for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
-    float s = 0.0f;
-    for (int g = 0; g < L.nseg; ++g) s += part[(int64_t)(L.seg0 + g) * ldb + k];
-    out[(int64_t)(list ? list[k] : k) * ldo + L.row] = s;
+  const int width = kFixThreads / slices, w = threadIdx.x / width, me = threadIdx.x % width;
+  auto add = [](float &s, float &lost, float v) {
+    const float t = s + v, z = t - s;
+    lost += (s - (t - z)) + (v - z);
+    s = t;
+  };
+  const int per = (L.nseg + slices - 1) / slices, g0 = min(L.nseg, w * per), g1 = min(L.nseg, g0 + per);
+  for (int k0 = 0; k0 < cnt; k0 += width) {
+    const int k = k0 + me;
+    float s = 0.0f, lost = 0.0f;
+    if (k < cnt) {
+      const float *v = part + (int64_t)(L.seg0 + g0) * ldb + k;
+      int g = g0;
+      for (; g + 8 <= g1; g += 8, v += 8 * (int64_t)ldb) {   // eight in pairs: one dependent step each eight
+        float x[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) x[q] = v[q * (int64_t)ldb];
+#pragma unroll
+        for (int h = 1; h < 8; h *= 2)
+#pragma unroll
+          for (int q = 0; q < 8; q += 2 * h) add(x[q], lost, x[q + h]);
+        add(s, lost, x[0]);
+      }
+      for (; g < g1; ++g, v += ldb) add(s, lost, *v);
+    }
+    if (slices > 1) {
+      __syncthreads();               // (the last round's sums are read)
+      sums[threadIdx.x] = make_float2(s, lost);
+      __syncthreads();
+      if (w > 0 || k >= cnt) continue;
+      for (int h = 1; h < slices; ++h) {
+        const float2 o = sums[h * width + me];
+        add(s, lost, o.x);
+        lost += o.y;
+      }
+    }
+    if (k < cnt) out[(int64_t)(list ? list[k] : k) * ldo + L.row] = s + lost;
   }
 }
 
@@ -359,7 +400,7 @@ cudaError_t launch_spmm(SpMat M, const SpPlan &P, const float *Bt, int ldb, cons
     if (e != cudaSuccess) return e;
   }
   if (P.nlong > 0) {
-    k_spmm_fix<<<P.nlong, 256, 0, st>>>(P.longs, part, ldb, count, gate, list, out, ldo);
+    k_spmm_fix<<<P.nlong, kFixThreads, 0, st>>>(P.longs, part, ldb, fix_slices(rmax), count, gate, list, out, ldo);
     return cudaGetLastError();
   }
   return cudaSuccess;
@@ -558,7 +599,7 @@ cudaError_t launch_spmm_h(SpMat M, const SpPlan &P, const float *Y, int64_t ldy,
     if (e != cudaSuccess) return e;
   }
   if (P.nlong > 0) {
-    k_spmm_fix<<<P.nlong, 256, 0, st>>>(P.longs, part, ldp, count, nullptr, list, out, ldo);
+    k_spmm_fix<<<P.nlong, kFixThreads, 0, st>>>(P.longs, part, ldp, fix_slices(rmax), count, nullptr, list, out, ldo);
     return cudaGetLastError();
   }
   return cudaSuccess;
