@@ -390,8 +390,9 @@ __device__ void xstep_finish(const XstepArgs &a, int c, const float *vv, int len
       const float w = (i < sg.hi) ? wval(vi, key, tie_keep) : 0.0f;
       const float xi = w * inv;
       if ((kOne || x) && i < sg.hi) x[i] = xi;
-      const unsigned nzb = __ballot_sync(0xffffffffu, xi != 0.0f);
-      if (gi && xi != 0.0f) {
+      // (listed by w, as nnz counts: x may underflow to 0 where w does not, and the list has nnz entries)
+      const unsigned nzb = __ballot_sync(0xffffffffu, w != 0.0f);
+      if (gi && w != 0.0f) {
         const int q = pos + __popc(nzb & lt_mask);
         if (q < a.cap) {
           gi[q] = i;
