@@ -133,7 +133,7 @@ typedef enum {
  *                its own work complete.  The handle runs its kernels on a stream of its own, so
  *                that the sweeps of a solve can be captured into CUDA graphs and replayed.
  * Errors: SPCA_E_INVALID (NULL pointers, n < 1, p < 1, lda < p, A not finite, unknown dtype),
- *         SPCA_E_UNSUPPORTED (n above 16,776,960 = 65535 * 256 rows: the finalise takes a dense
+ *         SPCA_E_UNSUPPORTED (n above 16,776,960 = 65535 * 256 rows: objectives take a dense
  *         A's rows in blocks of 256 on a grid dimension of at most 65535; SPCA_F64 storage;
  *         16- or 8-bit storage without tensor cores), SPCA_E_NOMEM, SPCA_E_CUDA.
  */

@@ -560,10 +560,10 @@ __global__ void __launch_bounds__(XT) k_xstep(XstepArgs a_in, const float *__res
 // of v from L2 or HBM, then about ten block barriers), so the chain is short: ranks are counted by
 // all threads at once instead of selected bit by bit by one warp, lambda_s takes a few monotone
 // steps instead of a bisection, and FP64 (1/64 of the FP32 rate) is left to single threads.
-// 1024 starts, p = 20011, lambda_s (spca_xstep, the whole call): 109 us, 387 us for the full pass in
+// 1024 starts, p = 20011, lambda_s (spca_xstep, the whole call): 119 us, 390 us for the full pass in
 // shared memory.  A solve's x-step and active list per sweep, before (filter, one-warp operator, full
 // pass and list: four launches) and now: p = 20000, T_s, 1024 starts 90 -> 46 us; p = 100000, V_gamma,
-// 16 starts 57 -> 24 us; p = 20000, lambda_s, one start 44 -> 28 us (CUDA events, a few us included).
+// 16 starts 57 -> 23 us; p = 20000, lambda_s, one start 44 -> 25 us (CUDA events, a few us included).
 constexpr int kFastCand = 1024;                // listed entries per start
 constexpr int kFastBins = 2048, kFastShift = 17;   // bins of 2^-6 octave below the largest |v_i|
 constexpr int kFastSubsets = 2048;             // disjoint subsets of v whose maxima bound the threshold (or 512)

@@ -97,8 +97,10 @@ struct XstepArgs {
   int calib_sweeps;
   int lowp_sweeps;
   int stop_enabled;
-  int ordered;         // ||w||^2 added in an order that does not depend on how the x-step found its
-                       // list (resident 16-bit matrices, whose every sweep rounds y to 11 bits)
+  int ordered;         // resident 16-bit matrices, whose every sweep rounds y to 11 bits (a last-bit
+                       // difference of ||w|| can end as 4e-5 in x): ||w||^2 is added over the list's
+                       // places where the list comes from the last threshold, else as the full pass
+                       // adds it, by index segment and lane
 };
 
 // the x-step switches of a start in its sweep `it` under XstepArgs::schedule (else as given)
@@ -173,9 +175,9 @@ struct SpMat {
   const float *val;
   int rows, cols;
 };
-// Work item of the SpMM: whole rows [row0, row1) (seg < 0), or the entries [nz0, nz1) of the long
-// row row0 whose sums go to partial slot seg.  Items hold at most kSpItemNnz entries and
-// kSpItemRows rows.
+// Work item of the SpMM: whole rows [row0, row1) (seg < 0), or a part of the long row row0 whose sums go
+// to partial slot seg; its entries are [nz0, nz1) either way.  Items hold at most kSpItemNnz entries
+// and kSpItemRows rows.
 struct SpItem {
   int row0, row1, seg, pad;
   int64_t nz0, nz1;
